@@ -89,8 +89,18 @@ inline bool uses_mma_match(const Problem& p) {
     return p.dtype == 1 && p.vec && p.r <= 2 && (long long)p.N * ((p.F + 15) / 16) < (1LL << 31);
 }
 
+// fp32 clips with 16-byte aligned rows and r <= 2 take the tiled fp32 kernel, which also takes the norms itself
+// (ttf_match_f32.cu).
+inline bool uses_f32_match(const Problem& p) {
+    return p.dtype == 0 && p.vec && p.r <= 2 && (long long)p.N * ((p.F + 3) / 4) < (1LL << 31);
+}
+cudaError_t launch_match_f32(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
+                             unsigned char* keep, cudaStream_t st);
+
 // The sweep stores per-token partial squared norms only for the kernels that read them.
-inline bool needs_sweep_norms(const Problem& p) { return !p.use_tc && (!uses_mma_match(p) || p.r == 2); }
+inline bool needs_sweep_norms(const Problem& p) {
+    return !p.use_tc && !uses_f32_match(p) && (!uses_mma_match(p) || p.r == 2);
+}
 
 // tcgen05 matching (ttf_match_tc.cu)
 bool tc_match_eligible(const Problem& p);

@@ -189,6 +189,7 @@ static cudaError_t launch_generic_t(const Problem& p, const Scratch& s, int* out
 
 cudaError_t launch_match(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                          unsigned char* keep, cudaStream_t st) {
+    if (uses_f32_match(p)) return launch_match_f32(p, s, out_anchor, shat, dst, keep, st);
     if (p.dtype == 0) return p.vec ? launch_generic_t<float, 4>(p, s, out_anchor, shat, dst, keep, st)
                                    : launch_generic_t<float, 1>(p, s, out_anchor, shat, dst, keep, st);
     if (p.use_tc) return launch_match_tc(p, s, out_anchor, shat, dst, keep, st);

@@ -30,6 +30,7 @@
 
 #include "ttf_internal.cuh"
 #include "ttf_async.cuh"
+#include "ttf_tensormap.cuh"
 
 #include <map>
 #include <mutex>
@@ -44,26 +45,6 @@ constexpr int kTcABytes = kTcM * 128;    // 16 KB
 constexpr int kTcThreads = 192;
 
 // ---- PTX wrappers -----------------------------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_4d(void* dst_smem, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        ::"r"(smem_u32(dst_smem)), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
-          "r"(smem_u32(bar))
-        : "memory");
-}
-// the same copy with an L2 cache policy (createpolicy) on the lines it reads
-__device__ __forceinline__ void tma_load_4d_hint(void* dst_smem, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                                 uint64_t* bar, uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
-        ::"r"(smem_u32(dst_smem)), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
-          "r"(smem_u32(bar)), "l"(policy)
-        : "memory");
-}
-__device__ __forceinline__ void tensormap_prefetch(const CUtensorMap* map) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
-}
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -435,18 +416,21 @@ static EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// X viewed as [F, H, W, C] (C innermost), one box of (64, bw, bh, bf) elements, 128-byte swizzle, zeros outside
-static bool make_map(CUtensorMap* m, const void* X, int F, int H, int W, int C, int bw, int bh, int bf) {
+bool make_tensor_map(CUtensorMap* m, const void* X, int dtype, int F, int H, int W, int C, int kc, int bw, int bh, int bf,
+                     bool swizzle128) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
+    const cuuint64_t es = dtype == 0 ? 4 : 2;
     const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)F};
-    const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-    const cuuint32_t box[4] = {(cuuint32_t)kTcKC, (cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bf};
+    const cuuint64_t strides[3] = {(cuuint64_t)C * es, (cuuint64_t)W * C * es, (cuuint64_t)H * W * C * es};
+    const cuuint32_t box[4] = {(cuuint32_t)kc, (cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bf};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(X), dims, strides, box, estr,
-               // (256-byte L2 promotion: the next stage reads the next 128 bytes of the same rows; 5 - 9 % faster than 128)
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return enc(m, dtype == 0 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(X),
+               dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+               // (256-byte L2 promotion: the next stage reads the next bytes of the same rows; 5 - 9 % faster than 128
+               // for the tcgen05 kernel)
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 bool tc_match_eligible(const Problem& p) {
@@ -478,8 +462,8 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
     static_assert((size_t)7 * ((S::WIN + 1) * kTcM + S::NCAND) * 4 <= (size_t)S::STAGES * S::STAGE || R == 2, "exchange rows must fit the ring");
     static_assert((size_t)3 * ((S::WIN + 1) * kTcM + S::NCAND) * 4 <= (size_t)S::STAGES * S::STAGE, "exchange rows must fit the ring");
     CUtensorMap mapA, mapB;
-    if (!make_map(&mapA, p.X, p.F, p.H, p.W, p.C, kTcWB, 1, kTcFR) ||
-        !make_map(&mapB, p.X, p.F, p.H, p.W, p.C, S::BW, S::SIDE, 1))
+    if (!make_tensor_map(&mapA, p.X, 1, p.F, p.H, p.W, p.C, kTcKC, kTcWB, 1, kTcFR, true) ||
+        !make_tensor_map(&mapB, p.X, 1, p.F, p.H, p.W, p.C, kTcKC, S::BW, S::SIDE, 1, true))
         return cudaErrorInvalidValue;
     const size_t smem = (size_t)S::STAGES * S::STAGE + 1024;
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R>), smem);
