@@ -143,12 +143,13 @@ int ttf_compress(const void* features, int F, int H, int W, int C, int r, float 
  * A batch of clips of one shape in one call (the long-video workload: the clips of a request processed
  * concurrently; Sec. 3 treats every clip independently, so this is scheduling only and each clip's results are
  * exactly those of ttf_compress).  features, out_tokens, out_count and out_pos_thw are HOST arrays of nclips
- * DEVICE pointers, read before the call returns.  The clips are spread round-robin over up to eight streams ("lanes")
+ * DEVICE pointers, read before the call returns.  Every kernel is launched once for a group of clips
+ * (half of the batch, at most 16), and the groups are spread round-robin over two streams ("lanes")
  * that the library keeps per device; these fork from `stream` and join it again through events, so the call is
- * asynchronous, ordered on `stream` like any other, and can be captured in a CUDA graph.  The kernels of one clip
- * leave much of the GPU idle while they ramp up and drain; with several clips in flight those gaps are filled
- * (ttf_set_schedule sets the number of lanes).  Within a lane the clips form a chain on two scratch blocks used in
- * turn: the sweep of a clip runs beside the gather of the clip before it.  The streams, their events and the scratch are created by
+ * asynchronous, ordered on `stream` like any other, and can be captured in a CUDA graph.  The kernels of one group
+ * leave part of the GPU idle while they ramp up and drain; the other lane's fill those gaps
+ * (ttf_set_schedule asks for a number of single clips in flight instead).  Within a lane the groups form a chain on two
+ * sets of scratch blocks used in turn: the sweep of a group runs beside the gather of the group before it.  The streams, their events and the scratch are created by
  * the first call on a device: make that call outside any stream capture.
  */
 int ttf_compress_batch(const void* const* features, int nclips, int F, int H, int W, int C, int r, float t,
@@ -166,8 +167,8 @@ int ttf_compress_batch(const void* const* features, int nclips, int F, int H, in
 int ttf_set_match_kernel(int which);
 
 /*
- * Schedule of ttf_compress_batch (the paper has no counterpart).  clips_in_flight bounds how many clips of a batch run
- * concurrently (lanes): 0 = automatic, 1 to 8, or TTF_SCHEDULE_PIPELINED.  Eq. (auto_anchor) needs all of X before any token can be matched,
+ * Schedule of ttf_compress_batch (the paper has no counterpart).  clips_in_flight: 0 = automatic (two groups of
+ * clips in flight, one launch per kernel and group), 1 to 8 = so many lanes of single clips, or TTF_SCHEDULE_PIPELINED.  Eq. (auto_anchor) needs all of X before any token can be matched,
  * so X is read twice; with few clips in flight the second read finds the clip in L2 but the kernels of one clip leave
  * much of the GPU idle while they ramp up and drain, with many the gaps are filled but the clips displace one another
  * in L2.  Results do not depend on it.  Process-wide; takes effect with the next call.

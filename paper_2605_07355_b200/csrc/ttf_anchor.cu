@@ -57,10 +57,12 @@ __device__ __forceinline__ float fold8(float (&v)[8], int lane) {
 // NORMS: also store the per-token partial squared norms (only the CUDA-core matching kernel reads them).
 template <typename T, int V, int LS, bool NORMS>
 __global__ void __launch_bounds__(kNormThreads)
-k_norm_sum(const T* __restrict__ X, int F, int N, int C, int nq,
+k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
            float* __restrict__ S, float* __restrict__ ssq, int* __restrict__ cnt, int* __restrict__ hdr,
-           int chain)
+           int chain, size_t sstride)
 {
+    const T* __restrict__ X = reinterpret_cast<const T*>(xs.X[blockIdx.y]);
+    S = clip_block(S, sstride); ssq = clip_block(ssq, sstride); cnt = clip_block(cnt, sstride); hdr = clip_block(hdr, sstride);
     using L = Loader<T, V>;
     constexpr int RG = kNormThreads / LS;
     constexpr int WPS = LS / 32;                    // warps across a slice = norm planes per slice
@@ -144,20 +146,19 @@ k_norm_sum(const T* __restrict__ X, int F, int N, int C, int nq,
     }
     if (q == 0 && tid == 0) cnt[k] = 0;             // survivor counters start at zero for the matching kernel
     if (blockIdx.x == 0 && tid == 0) hdr[HDR_ERROR] = 0;   // the error word reports on this call only
-    if (chain && blockIdx.x == 0) pdl_wait();
+    if (chain && blockIdx.x == 0 && blockIdx.y == 0) pdl_wait();
     trace_mark(hdr, 0, true);
 }
 
 template <typename T, int V>
 static cudaError_t launch_sum_t(const Problem& p, const Scratch& s, cudaStream_t st) {
-    const T* X = reinterpret_cast<const T*>(p.X);
     const unsigned blocks = (unsigned)((long long)p.F * p.nq);
-    const dim3 g(blocks), b(kNormThreads);
+    const dim3 g(blocks, p.nclips), b(kNormThreads);
     if (!needs_sweep_norms(p))
-        return launch_ex(true, 0, k_norm_sum<T, V, 32, false>, g, b, st, X, p.F, p.N, p.C, p.nq, s.S,
-                         s.ssq, s.cnt, s.hdr, p.chain);
-    return launch_ex(true, 0, k_norm_sum<T, V, 32, true>, g, b, st, X, p.F, p.N, p.C, p.nq, s.S, s.ssq,
-                     s.cnt, s.hdr, p.chain);
+        return launch_ex(true, 0, k_norm_sum<T, V, 32, false>, g, b, st, p.xs, p.F, p.N, p.C, p.nq, s.S,
+                         s.ssq, s.cnt, s.hdr, p.chain, p.sstride);
+    return launch_ex(true, 0, k_norm_sum<T, V, 32, true>, g, b, st, p.xs, p.F, p.N, p.C, p.nq, s.S, s.ssq,
+                     s.cnt, s.hdr, p.chain, p.sstride);
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -176,8 +177,11 @@ constexpr int kStatSub = 1;
 
 template <int V>
 __global__ void __launch_bounds__(kNormThreads)
-k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float* Gp, int* hdr, int* out_anchor)
+k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float* Gp, int* hdr, int* out_anchor,
+              size_t sstride)
 {
+    S = clip_block(S, sstride); Dp = clip_block(Dp, sstride); Qp = clip_block(Qp, sstride); Gp = clip_block(Gp, sstride);
+    hdr = clip_block(hdr, sstride);
     pdl_launch_dependents();
     trace_mark(hdr, 1, false);
     pdl_wait();                                      // the sweep's frame sums are complete and visible
@@ -317,8 +321,9 @@ constexpr int kStatClusterMaxF = 256;     // frames the cluster kernel takes (sh
 
 template <int SL>     // slices of 128 channels per CTA; FB = 16 / SL frames per thread and chunk (warp w owns frames w, w + 8, ...)
 __global__ void __launch_bounds__(kNormThreads)
-k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_anchor)
+k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_anchor, size_t sstride)
 {
+    S = clip_block(S, sstride); hdr = clip_block(hdr, sstride);
     constexpr int FB = 16 / SL;
     constexpr int CHUNK = kNormWarps * FB;           // frames per chunk: 32 / 64 / 128
     __shared__ float4 s_g[SL][kNormWarps][32];
@@ -441,21 +446,23 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
 template <int SL>
 static cudaError_t launch_stats_cluster_t(const Problem& p, const Scratch& s, int* out_anchor, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kStatCluster); cfg.blockDim = dim3(kNormThreads); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+    cfg.gridDim = dim3(kStatCluster, p.nclips); cfg.blockDim = dim3(kNormThreads); cfg.dynamicSmemBytes = 0; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = kStatCluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_frame_stats_cluster<SL>, (const float*)s.S, p.F, p.C, p.nsl, s.hdr, out_anchor);
+    return cudaLaunchKernelEx(&cfg, k_frame_stats_cluster<SL>, (const float*)s.S, p.F, p.C, p.nsl, s.hdr, out_anchor,
+                              p.sstride);
 }
 
 // What the sweep leaves behind besides its sums, for calls that need no sweep (a fixed anchor and a matching kernel
 // that takes the token norms itself): survivor counters at zero, error word cleared.
 __global__ void __launch_bounds__(256)
-k_begin_call(int F, int* __restrict__ cnt, int* __restrict__ hdr)
+k_begin_call(int F, int* __restrict__ cnt, int* __restrict__ hdr, size_t sstride)
 {
+    cnt = clip_block(cnt, sstride); hdr = clip_block(hdr, sstride);
     pdl_launch_dependents();
     pdl_wait();                                      // the previous call's gather may still read the counters
     for (int k = threadIdx.x; k < F; k += 256) cnt[k] = 0;
@@ -464,7 +471,7 @@ k_begin_call(int F, int* __restrict__ cnt, int* __restrict__ hdr)
 
 cudaError_t launch_norm_sum(const Problem& p, const Scratch& s, cudaStream_t st) {
     if (p.anchor_mode != 0 && !needs_sweep_norms(p))           // Eq. (auto_anchor) is not evaluated: no pass over X
-        return launch_ex(true, 0, k_begin_call, dim3(1), dim3(256), st, p.F, s.cnt, s.hdr);
+        return launch_ex(true, 0, k_begin_call, dim3(1, p.nclips), dim3(256), st, p.F, s.cnt, s.hdr, p.sstride);
     if (p.dtype == 0) return p.vec ? launch_sum_t<float, 4>(p, s, st) : launch_sum_t<float, 1>(p, s, st);
     return p.vec ? launch_sum_t<bf16_t, 8>(p, s, st) : launch_sum_t<bf16_t, 1>(p, s, st);
 }
@@ -485,10 +492,10 @@ cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anch
         return launch_stats_cluster_t<4>(p, s, out_anchor, st);
     }
     if (p.C % 4 == 0)
-        return launch_pdl(k_frame_stats<4>, dim3(p.nsl), dim3(kNormThreads), st, (const float*)s.S, p.F, p.C, p.nsl,
-                          s.Dp, s.Qp, s.Gp, s.hdr, out_anchor);
-    return launch_pdl(k_frame_stats<1>, dim3(p.nsl), dim3(kNormThreads), st, (const float*)s.S, p.F, p.C, p.nsl,
-                      s.Dp, s.Qp, s.Gp, s.hdr, out_anchor);
+        return launch_pdl(k_frame_stats<4>, dim3(p.nsl, p.nclips), dim3(kNormThreads), st, (const float*)s.S, p.F, p.C, p.nsl,
+                          s.Dp, s.Qp, s.Gp, s.hdr, out_anchor, p.sstride);
+    return launch_pdl(k_frame_stats<1>, dim3(p.nsl, p.nclips), dim3(kNormThreads), st, (const float*)s.S, p.F, p.C, p.nsl,
+                      s.Dp, s.Qp, s.Gp, s.hdr, out_anchor, p.sstride);
 }
 
 }  // namespace ttf

@@ -134,7 +134,7 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
     if (N >= (1LL << 31) || FN >= (1LL << 31)) return TTF_ERR_UNSUPPORTED;
     const long long esize = dtype == TTF_DTYPE_F32 ? 4 : 2;
     if ((double)FN * (double)C * (double)esize >= (double)(1LL << 46)) return TTF_ERR_UNSUPPORTED;
-    p->X = X; p->F = F; p->H = H; p->W = W; p->C = C; p->r = r; p->t = t; p->dtype = dtype;
+    p->X = X; p->xs.X[0] = X; p->nclips = 1; p->sstride = 0; p->F = F; p->H = H; p->W = W; p->C = C; p->r = r; p->t = t; p->dtype = dtype;
     p->N = (int)N;
     const long long row_bytes = (long long)C * esize;
     p->vec = (row_bytes % 16 == 0) && (reinterpret_cast<uintptr_t>(X) % 16 == 0);
@@ -217,7 +217,9 @@ static int clear_control_blocks(void* ws, size_t stride, int n, cudaStream_t st)
 // Checked build: the slack by which every index limit of the next calls is lowered (test hook, normally zero).
 #ifdef TTF_DEBUG
 static std::atomic<int> g_check_slack{0};
-__global__ void k_set_word(int* word, int value) { *word = value; }
+__global__ void k_set_word(int* word, int value, size_t stride) {
+    *reinterpret_cast<int*>(reinterpret_cast<uintptr_t>(word) + blockIdx.x * stride) = value;
+}
 #endif
 
 // steps shared by compress and query: norms + frame sums, anchor, matching + gate
@@ -225,7 +227,7 @@ static int run_front(const Problem& p, const Scratch& s, int* out_anchor, float*
                      unsigned char* keep, cudaStream_t st) {
     cudaError_t e;
 #ifdef TTF_DEBUG
-    k_set_word<<<1, 1, 0, st>>>(s.hdr + HDR_CHECK_SLACK, g_check_slack.load());
+    k_set_word<<<p.nclips, 1, 0, st>>>(s.hdr + HDR_CHECK_SLACK, g_check_slack.load(), p.sstride);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e);
 #endif
@@ -241,14 +243,19 @@ static int run_front(const Problem& p, const Scratch& s, int* out_anchor, float*
     return TTF_OK;
 }
 
-static int compress_impl(const Problem& p, void* ws, void* out_tokens, int* out_count, int* out_pos,
-                         cudaStream_t st) {
+static OutPtrs one_out(void* out_tokens, int* out_count, int* out_pos) {
+    OutPtrs o;
+    o.tokens[0] = out_tokens; o.count[0] = out_count; o.pos[0] = out_pos;
+    return o;
+}
+
+static int compress_impl(const Problem& p, void* ws, const OutPtrs& out, cudaStream_t st) {
     Scratch s;
     carve_scratch(p, ws, &s);
     int rc = run_front(p, s, nullptr, s.shat, s.dst, s.keep, st);
     if (rc != TTF_OK) return rc;
     cudaError_t e;
-    { ProfScope ps(st, PK_COMPACT); e = launch_compact(p, s, out_tokens, out_pos, out_count, st); }
+    { ProfScope ps(st, PK_COMPACT); e = launch_compact(p, s, out, st); }
     if (e != cudaSuccess) return cuda_fail(e);
     return TTF_OK;
 }
@@ -437,7 +444,7 @@ int ttf_compress_ws(const void* features, int F, int H, int W, int C, int r, flo
     if (rc != TTF_OK) return rc;
     rc = clear_control(p, workspace, (cudaStream_t)stream);
     if (rc != TTF_OK) return rc;
-    return compress_impl(p, workspace, out_tokens, out_count, out_pos_thw, (cudaStream_t)stream);
+    return compress_impl(p, workspace, one_out(out_tokens, out_count, out_pos_thw), (cudaStream_t)stream);
 }
 
 int ttf_compress(const void* features, int F, int H, int W, int C, int r, float t, int dtype,
@@ -451,7 +458,7 @@ int ttf_compress(const void* features, int F, int H, int W, int C, int r, float 
     void* ws = nullptr;
     rc = cached_scratch(s.bytes, (cudaStream_t)stream, &ws);
     if (rc != TTF_OK) return rc;
-    return compress_impl(p, ws, out_tokens, out_count, out_pos_thw, (cudaStream_t)stream);
+    return compress_impl(p, ws, one_out(out_tokens, out_count, out_pos_thw), (cudaStream_t)stream);
 }
 
 int ttf_query_ws(const void* features, int F, int H, int W, int C, int r, float t, int dtype,
@@ -523,7 +530,7 @@ int ttf_compress_ex(const void* features, int F, int H, int W, int C, int r, flo
     void* ws = nullptr;
     rc = cached_scratch(s.bytes, (cudaStream_t)stream, &ws);
     if (rc != TTF_OK) return rc;
-    return compress_impl(p, ws, out_tokens, out_count, out_pos_thw, (cudaStream_t)stream);
+    return compress_impl(p, ws, one_out(out_tokens, out_count, out_pos_thw), (cudaStream_t)stream);
 }
 
 int ttf_query_ex(const void* features, int F, int H, int W, int C, int r, float t, int dtype,
@@ -554,7 +561,7 @@ int ttf_compress_mean(const void* features, int F, int H, int W, int C, int r, f
     void* ws = nullptr;
     rc = cached_scratch(s.bytes, (cudaStream_t)stream, &ws);
     if (rc != TTF_OK) return rc;
-    rc = compress_impl(p, ws, out_tokens, out_count, out_pos_thw, (cudaStream_t)stream);
+    rc = compress_impl(p, ws, one_out(out_tokens, out_count, out_pos_thw), (cudaStream_t)stream);
     if (rc != TTF_OK) return rc;
     carve_scratch(p, ws, &s);
     cudaError_t e = launch_fuse_mean(p, s, out_tokens, (cudaStream_t)stream);
@@ -562,9 +569,9 @@ int ttf_compress_mean(const void* features, int F, int H, int W, int C, int r, f
 }
 
 // ---- batches on the library's own streams -----------------------------------------------------------------
-// The clips of a batch are independent, and the kernels of one clip leave most of the GPU idle while they ramp up
-// and drain, so a batch is spread round-robin over kBatchStreams internal streams per device that fork from the
-// caller's stream and join it again (events only: the call stays asynchronous and can be captured in a graph).
+// The clips of a batch are independent: they go through the kernels in groups (one launch covers a group), and the
+// groups are spread round-robin over up to kBatchStreams internal streams per device that fork from the caller's
+// stream and join it again (events only: the call stays asynchronous and can be captured in a graph).
 constexpr int kBatchStreams = 8;
 constexpr int kMatchedRing = 4;                  // events "clip n has been matched" of the pipelined schedule, used in turn
 struct BatchLanes {
@@ -596,8 +603,33 @@ static int batch_lanes(BatchLanes** out) {
     return TTF_OK;
 }
 
-// The clips of a lane form a chain on the lane's stream: sweep, statistics, matching, gather, next sweep, ... with two
-// scratch blocks used in turn, so that the sweep of a clip can run beside the gather of the clip before it.
+// How a batch is cut into launches: `group` clips per launch, `lanes` groups in flight.
+struct BatchPlan { int group, lanes; bool pipelined; };
+
+// Automatic: one launch of each kernel covers half of the batch (at most kMaxGroup clips), two halves in flight, so that
+// one half's kernels fill what the other's leave idle while they ramp up and drain.  Launches over single clips on
+// eight lanes were bound by the host for small clips (a clip of 1.2 MB: 16 clips 205 us, 63 us now; 7.2 MB: 12 clips
+// 162 -> 98 us) and were no faster for large ones (33 MB: 16 clips 304 -> 300 us; 67 MB: 517 -> 515; 268 MB, 8 clips:
+// 910 -> 911).  All clips in one launch, or one lane, leave the second half's ramp and tail uncovered (33 MB: 306 and
+// 330 us); more than two lanes of smaller groups gain nothing (within 2 % for every clip size measured).
+static BatchPlan plan_batch(const Problem& p, int nclips) {
+    BatchPlan b;
+    const int want = g_sched_lanes.load();
+    b.pipelined = want == TTF_SCHEDULE_PIPELINED && nclips >= 3 && p.anchor_mode == 0;
+    b.group = 1;
+    if (b.pipelined) { b.lanes = 2; return b; }
+    if (want >= 1 && want <= kBatchStreams) b.lanes = want;          // ttf_set_schedule: so many single clips in flight
+    else {
+        b.group = (nclips + 1) / 2 < kMaxGroup ? (nclips + 1) / 2 : kMaxGroup;
+        b.lanes = 2;
+    }
+    const int groups = (nclips + b.group - 1) / b.group;
+    if (b.lanes > groups) b.lanes = groups;
+    return b;
+}
+
+// The groups of a lane form a chain on the lane's stream: sweep, statistics, matching, gather, next sweep, ... with two
+// sets of scratch blocks used in turn, so that the sweep of a group can run beside the gather of the group before it.
 static int batch_on_streams(const void* const* features, int nclips, int F, int H, int W, int C, int r, float t,
                             int dtype, const ttf_options* options,
                             void* const* out_tokens, int* const* out_count, int* const* out_pos_thw, cudaStream_t st) {
@@ -605,31 +637,29 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
     BatchLanes* L = nullptr;
     int rc = batch_lanes(&L);
     if (rc != TTF_OK) return rc;
-    std::vector<Problem> ps(nclips);
+    // every clip is validated (and the largest scratch layout found) before anything is enqueued
+    Problem p0;
+    bool same_layout = true;                     // clips of one launch share the vector path or the scalar path
     size_t stride = 0;
     for (int n = 0; n < nclips; ++n) {
-        rc = make_problem(features[n], F, H, W, C, r, t, dtype, &ps[n]);
-        if (rc == TTF_OK) rc = apply_options(&ps[n], options);
+        Problem p;
+        rc = make_problem(features[n], F, H, W, C, r, t, dtype, &p);
+        if (rc == TTF_OK) rc = apply_options(&p, options);
         if (rc != TTF_OK) return rc;
         Scratch s;
-        carve_scratch(ps[n], nullptr, &s);
+        carve_scratch(p, nullptr, &s);
         if (s.bytes > stride) stride = s.bytes;
+        if (n == 0) p0 = p;
+        same_layout = same_layout && p.vec == p0.vec;
     }
-    int want = g_sched_lanes.load();
-    // Pipelined schedule (TTF_SCHEDULE_PIPELINED, automatic anchor only).  Eq. (auto_anchor) forces two passes over X;
-    // the second is free only while the clip is still in L2, which holds one 8B-shaped clip and most of a second.
-    // Two lanes in opposite phases: the matching kernels of consecutive clips are ordered one after the other, and a
-    // lane's next sweep starts when its previous clip has been matched (the chain below), so at any time one clip is
-    // matched out of L2 while the next one streams in.  The matching kernel marks the source rows it has read, and
-    // the gather what it reads and writes, as the first lines to leave L2; without that the incoming clip displaces
-    // exactly the rows that are still to be matched (they are the oldest lines).
-    const bool pipelined = want == TTF_SCHEDULE_PIPELINED && nclips >= 3 && ps[0].anchor_mode == 0;
-    if (pipelined) want = 2;
-    if (want < 1 || want > kBatchStreams) want = kBatchStreams;      // automatic: measured best for every clip shape so far
-    const int lanes = nclips < want ? nclips : want;
+    BatchPlan plan = plan_batch(p0, nclips);
+    if (!same_layout) plan.group = 1;
+    const int groups = (nclips + plan.group - 1) / plan.group;
+    const int lanes = groups < plan.lanes ? groups : plan.lanes;
+    const size_t set = (size_t)plan.group * stride;
     std::vector<void*> ws(lanes, nullptr);
     for (int i = 0; i < lanes; ++i) {            // (may allocate: before the fork, outside the event bracket)
-        rc = cached_scratch(2 * stride, L->s[i], &ws[i]);
+        rc = cached_scratch((groups > lanes ? 2 : 1) * set, L->s[i], &ws[i]);
         if (rc != TTF_OK) return rc;
     }
     cudaError_t e = cudaEventRecord(L->fork, st);
@@ -637,36 +667,54 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
     if (e != cudaSuccess) return cuda_fail(e);
     int first_rc = TTF_OK;
     std::vector<const int*> words;
-    for (int n = 0; n < nclips && first_rc == TTF_OK; ++n) {
-        const int lane = n % lanes, turn = n / lanes;
-        void* block = (char*)ws[lane] + (size_t)(turn & 1) * stride;
-        ps[n].overlapped = lanes;
-        ps[n].stream_once = pipelined ? 1 : 0;
-        ps[n].chain = turn > 0 ? 1 : 0;          // the lane's previous kernel is the gather of its previous clip
-        if (turn < 2) {
-            // the block may hold anything (another shape's data, or a failed call's counters): clear its control words
-            first_rc = clear_control(ps[n], block, L->s[lane]);
-            words.push_back(reinterpret_cast<const int*>(block));
-            if (first_rc != TTF_OK) break;
-            if (turn == 1) ps[n].chain = 0;      // (the memset sits between the gather and this sweep)
+    for (int q = 0; q < groups && first_rc == TTF_OK; ++q) {
+        const int lane = q % lanes, turn = q / lanes;
+        const int n0 = q * plan.group;
+        char* block = (char*)ws[lane] + (size_t)(turn & 1) * set;
+        cudaStream_t ls = L->s[lane];
+        Problem p;
+        make_problem(features[n0], F, H, W, C, r, t, dtype, &p);
+        apply_options(&p, options);
+        OutPtrs out;
+        p.nclips = nclips - n0 < plan.group ? nclips - n0 : plan.group;
+        p.sstride = stride;
+        for (int i = 0; i < p.nclips; ++i) {
+            p.xs.X[i] = features[n0 + i];
+            out.tokens[i] = out_tokens[n0 + i]; out.count[i] = out_count[n0 + i]; out.pos[i] = out_pos_thw[n0 + i];
         }
-        // (the lane's next clip, if there is one, is at turn + 1; its sweep is chained from turn 2 on)
-        ps[n].chain_next = (n + lanes < nclips && turn + 1 >= 2) ? 1 : 0;
-        if (!pipelined) {
-            first_rc = compress_impl(ps[n], block, out_tokens[n], out_count[n], out_pos_thw[n], L->s[lane]);
+        p.overlapped = lanes;
+        p.stream_once = plan.pipelined ? 1 : 0;
+        p.chain = turn > 0 ? 1 : 0;              // the lane's previous kernel is the gather of its previous group
+        if (turn < 2) {
+            // the blocks may hold anything (another shape's data, or a failed call's counters): clear their control words
+            first_rc = clear_control_blocks(block, stride, p.nclips, ls);
+            for (int i = 0; i < p.nclips; ++i) words.push_back(reinterpret_cast<const int*>(block + i * stride));
+            if (first_rc != TTF_OK) break;
+            if (turn == 1) p.chain = 0;          // (the memset sits between the gather and this sweep)
+        }
+        // (the lane's next group, if there is one, is at turn + 1; its sweep is chained from turn 2 on)
+        p.chain_next = (q + lanes < groups && turn + 1 >= 2) ? 1 : 0;
+        if (!plan.pipelined) {
+            first_rc = compress_impl(p, block, out, ls);
             continue;
         }
-        // the same kernels as compress_impl, with the matching kernel ordered after that of the clip before (which
-        // ran in the other lane)
+        // Pipelined schedule (TTF_SCHEDULE_PIPELINED, automatic anchor only).  Eq. (auto_anchor) forces two passes over X;
+        // the second is free only while the clip is still in L2, which holds one 8B-shaped clip and most of a second.
+        // Two lanes in opposite phases: the matching kernels of consecutive clips are ordered one after the other, and a
+        // lane's next sweep starts when its previous clip has been matched (the chain), so at any time one clip is
+        // matched out of L2 while the next one streams in.  The matching kernel marks the source rows it has read, and
+        // the gather what it reads and writes, as the first lines to leave L2; without that the incoming clip displaces
+        // exactly the rows that are still to be matched (they are the oldest lines).
+        // The same kernels as compress_impl, with the matching kernel ordered after that of the clip before (which
+        // ran in the other lane).
         Scratch sc;
-        carve_scratch(ps[n], block, &sc);
-        cudaStream_t ls = L->s[lane];
-        { ProfScope pr(ls, PK_NORM_SUM); e = launch_norm_sum(ps[n], sc, ls); }
-        if (e == cudaSuccess) { ProfScope pr(ls, PK_FRAME_STATS); e = launch_frame_stats(ps[n], sc, nullptr, ls); }
-        if (e == cudaSuccess && n > 0) e = cudaStreamWaitEvent(ls, L->matched[(n - 1) % kMatchedRing], 0);
-        if (e == cudaSuccess) { ProfScope pr(ls, PK_MATCH); e = launch_match(ps[n], sc, nullptr, sc.shat, sc.dst, sc.keep, ls); }
-        if (e == cudaSuccess) e = cudaEventRecord(L->matched[n % kMatchedRing], ls);
-        if (e == cudaSuccess) { ProfScope pr(ls, PK_COMPACT); e = launch_compact(ps[n], sc, out_tokens[n], out_pos_thw[n], out_count[n], ls); }
+        carve_scratch(p, block, &sc);
+        { ProfScope pr(ls, PK_NORM_SUM); e = launch_norm_sum(p, sc, ls); }
+        if (e == cudaSuccess) { ProfScope pr(ls, PK_FRAME_STATS); e = launch_frame_stats(p, sc, nullptr, ls); }
+        if (e == cudaSuccess && q > 0) e = cudaStreamWaitEvent(ls, L->matched[(q - 1) % kMatchedRing], 0);
+        if (e == cudaSuccess) { ProfScope pr(ls, PK_MATCH); e = launch_match(p, sc, nullptr, sc.shat, sc.dst, sc.keep, ls); }
+        if (e == cudaSuccess) e = cudaEventRecord(L->matched[q % kMatchedRing], ls);
+        if (e == cudaSuccess) { ProfScope pr(ls, PK_COMPACT); e = launch_compact(p, sc, out, ls); }
         if (e != cudaSuccess) first_rc = cuda_fail(e);
     }
     {   // the caller asks about the batch through its own stream: point it at the lanes' error words
@@ -735,7 +783,7 @@ int ttf_compress_segment(const void* features, int F, int H, int W, int C, int r
     void* ws = nullptr;
     rc = cached_scratch(s.bytes, (cudaStream_t)stream, &ws);
     if (rc != TTF_OK) return rc;
-    return compress_impl(p, ws, out_tokens, out_count, out_pos_thw, (cudaStream_t)stream);
+    return compress_impl(p, ws, one_out(out_tokens, out_count, out_pos_thw), (cudaStream_t)stream);
 }
 
 int ttf_restore(const void* compressed, size_t row_bytes, int F, int H, int W, const int* anchor,
@@ -986,21 +1034,39 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
     for (int n = 0; n < nclips; ++n)
         if (!features[n] || !out_tokens[n] || !out_count[n] || !out_pos_thw[n]) return TTF_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    std::vector<Problem> ps(nclips);
-    int want = g_sched_lanes.load();             // the kernels a batch call of these clips would launch
-    if (want < 1 || want > kBatchStreams) want = kBatchStreams;
+    std::vector<Problem> ps;                     // the launches a batch call of these clips would make
+    std::vector<OutPtrs> outs;
+    size_t stride = 0;
+    bool same_layout = true;
+    BatchPlan plan = {1, 1, false};
     for (int n = 0; n < nclips; ++n) {
-        int rc = make_problem(features[n], F, H, W, C, r, t, dtype, &ps[n]);
+        Problem p;
+        int rc = make_problem(features[n], F, H, W, C, r, t, dtype, &p);
         if (rc != TTF_OK) return rc;
-        ps[n].overlapped = nclips < want ? nclips : want;
-    }
-    Scratch s0;
-    carve_scratch(ps[0], nullptr, &s0);
-    size_t stride = s0.bytes;
-    for (int n = 1; n < nclips; ++n) {           // (the layout depends on the alignment of the clip)
-        Scratch sn;
-        carve_scratch(ps[n], nullptr, &sn);
+        Scratch sn;                              // (the layout depends on the alignment of the clip)
+        carve_scratch(p, nullptr, &sn);
         if (sn.bytes > stride) stride = sn.bytes;
+        if (n == 0) plan = plan_batch(p, nclips);
+        ps.push_back(p);
+        same_layout = same_layout && p.vec == ps[0].vec;
+    }
+    if (!same_layout) plan.group = 1;
+    {
+        std::vector<Problem> grouped;
+        for (int n0 = 0; n0 < nclips; n0 += plan.group) {
+            Problem p = ps[n0];
+            OutPtrs out;
+            p.nclips = nclips - n0 < plan.group ? nclips - n0 : plan.group;
+            p.sstride = stride;
+            p.overlapped = plan.lanes;
+            for (int i = 0; i < p.nclips; ++i) {
+                p.xs.X[i] = features[n0 + i];
+                out.tokens[i] = out_tokens[n0 + i]; out.count[i] = out_count[n0 + i]; out.pos[i] = out_pos_thw[n0 + i];
+            }
+            grouped.push_back(p);
+            outs.push_back(out);
+        }
+        ps.swap(grouped);
     }
     void* ws = nullptr;
     int rc = cached_scratch(stride * nclips, st, &ws);
@@ -1014,13 +1080,13 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
     for (int rep = 0; rep < reps && e == cudaSuccess; ++rep) {
         for (int stage = 0; stage < 4 && e == cudaSuccess; ++stage) {
             cudaEventRecord(ev[stage], st);
-            for (int n = 0; n < nclips && e == cudaSuccess; ++n) {
+            for (int n = 0; n < (int)ps.size() && e == cudaSuccess; ++n) {
                 Scratch s;
-                carve_scratch(ps[n], (char*)ws + stride * n, &s);
+                carve_scratch(ps[n], (char*)ws + stride * plan.group * n, &s);
                 if (stage == 0) e = launch_norm_sum(ps[n], s, st);
                 else if (stage == 1) e = launch_frame_stats(ps[n], s, nullptr, st);
                 else if (stage == 2) e = launch_match(ps[n], s, nullptr, s.shat, s.dst, s.keep, st);
-                else e = launch_compact(ps[n], s, out_tokens[n], out_pos_thw[n], out_count[n], st);
+                else e = launch_compact(ps[n], s, outs[n], st);
             }
         }
         cudaEventRecord(ev[4], st);

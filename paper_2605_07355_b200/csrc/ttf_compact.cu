@@ -17,8 +17,10 @@ namespace ttf {
 // exclusive scan of the effective per-frame counts (anchor frame counts as 0) for clips with more frames
 // than fit the shared-memory scan of the gather kernel
 __global__ void __launch_bounds__(1024)
-k_frame_prefix(const int* __restrict__ cnt, const int* __restrict__ hdr, int F, int acnt, int* __restrict__ prefix)
+k_frame_prefix(const int* __restrict__ cnt, const int* __restrict__ hdr, int F, int acnt, int* __restrict__ prefix,
+               size_t sstride)
 {
+    cnt = clip_block(cnt, sstride); hdr = clip_block(hdr, sstride); prefix = clip_block(prefix, sstride);
     __shared__ int s_warp[32];
     __shared__ int s_carry;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -75,13 +77,18 @@ constexpr int kCopyUnroll = 8;       // 16-byte units in flight per lane of the 
 constexpr int kBulkPiece = 8192;     // bytes per staging slot; longer rows go in pieces
 
 __global__ void __launch_bounds__(kCopyWarps * 32)
-k_compact_bulk(const unsigned char* __restrict__ X, size_t row_bytes, int F, int H, int W, int r,
+k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, int W, int r,
                int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
                const unsigned char* __restrict__ keep, const int* __restrict__ dst,
-               unsigned char* __restrict__ out_tokens, int* __restrict__ out_pos, int* __restrict__ out_count,
-               int* __restrict__ fuse_cnt, int ncopy_blocks, int NA, int acnt, int t_off, int pos_base,
-               int late_trigger, int wait_limit, int tx_extra, int stream_once)
+               const __grid_constant__ OutPtrs outs, int* __restrict__ fuse_cnt, int ncopy_blocks, int NA, int acnt, int t_off, int pos_base,
+               int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride)
 {
+    const unsigned char* __restrict__ X = reinterpret_cast<const unsigned char*>(xs.X[blockIdx.y]);
+    unsigned char* __restrict__ out_tokens = reinterpret_cast<unsigned char*>(outs.tokens[blockIdx.y]);
+    int* __restrict__ out_pos = outs.pos[blockIdx.y];
+    int* __restrict__ out_count = outs.count[blockIdx.y];
+    hdr = clip_block(hdr, sstride); cnt = clip_block(cnt, sstride); gprefix = clip_block(gprefix, sstride);
+    keep = clip_block(keep, sstride); dst = clip_block(dst, sstride); fuse_cnt = clip_block(fuse_cnt, sstride);
     extern __shared__ __align__(128) unsigned char stage[];     // [kCopyWarps][kBulkPiece]
     __shared__ uint64_t bar[kCopyWarps];
     const int N = H * W;
@@ -176,12 +183,19 @@ k_compact_bulk(const unsigned char* __restrict__ X, size_t row_bytes, int F, int
 
 template <int COPY_BYTES>
 __global__ void __launch_bounds__(kCopyWarps * 32)
-k_compact(const unsigned char* __restrict__ X, size_t row_bytes, int F, int H, int W, int r,
+k_compact(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, int W, int r,
           const int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
           const unsigned char* __restrict__ keep, const int* __restrict__ dst,
-          unsigned char* __restrict__ out_tokens, int* __restrict__ out_pos, int* __restrict__ out_count,
-          int* __restrict__ fuse_cnt, int ncopy_blocks, int NA, int acnt, int t_off, int pos_base, int late_trigger)
+          const __grid_constant__ OutPtrs outs,
+          int* __restrict__ fuse_cnt, int ncopy_blocks, int NA, int acnt, int t_off, int pos_base, int late_trigger,
+          size_t sstride)
 {
+    const unsigned char* __restrict__ X = reinterpret_cast<const unsigned char*>(xs.X[blockIdx.y]);
+    unsigned char* __restrict__ out_tokens = reinterpret_cast<unsigned char*>(outs.tokens[blockIdx.y]);
+    int* __restrict__ out_pos = outs.pos[blockIdx.y];
+    int* __restrict__ out_count = outs.count[blockIdx.y];
+    hdr = clip_block(hdr, sstride); cnt = clip_block(cnt, sstride); gprefix = clip_block(gprefix, sstride);
+    keep = clip_block(keep, sstride); dst = clip_block(dst, sstride); fuse_cnt = clip_block(fuse_cnt, sstride);
     using U = typename CopyUnit<COPY_BYTES>::type;
     const int N = H * W;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -246,22 +260,21 @@ cudaError_t launch_fuse_count(const Problem& p, const Scratch& s, const int* dst
     // bookkeeping only: the same kernel with zero copy CTAs
     const int nb = (p.N + kCopyWarps - 1) / kCopyWarps;
     k_compact<4><<<nb < 1024 ? nb : 1024, kCopyWarps * 32, 0, st>>>(
-        nullptr, 0, p.F, p.H, p.W, p.r, s.hdr, s.cnt, s.prefix, keep, dst, nullptr, nullptr, nullptr,
-        fuse_cnt, 0, p.N, 0, 0, 0, 0);
+        p.xs, 0, p.F, p.H, p.W, p.r, s.hdr, s.cnt, s.prefix, keep, dst, OutPtrs(), fuse_cnt, 0, p.N, 0, 0, 0, 0, 0);
     return cudaGetLastError();
 }
 
-cudaError_t launch_compact(const Problem& p, const Scratch& s, void* out_tokens, int* out_pos, int* out_count,
-                           cudaStream_t st) {
+cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& out, cudaStream_t st) {
     const size_t esize = p.dtype == 0 ? 4 : 2;
     const size_t row_bytes = (size_t)p.C * esize;
-    const bool vec = p.vec && (reinterpret_cast<uintptr_t>(out_tokens) % 16 == 0);
+    bool vec = p.vec;
+    for (int n = 0; n < p.nclips; ++n) vec = vec && reinterpret_cast<uintptr_t>(out.tokens[n]) % 16 == 0;
     // rows emitted as the anchor block / tokens the anchor frame adds to the flat walk: (N, 0) in the paper's order
     // (Eq. xprime_stack), (0, N) in natural order, (0, 0) for a streaming segment, which does not emit its anchor
     const int NA = (p.emit_anchor && !p.natural_order) ? p.N : 0;
     const int acnt = (p.emit_anchor && p.natural_order) ? p.N : 0;
     if (p.F > kWarpPrefixMaxF) {
-        k_frame_prefix<<<1, 1024, 0, st>>>(s.cnt, s.hdr, p.F, acnt, s.prefix);
+        k_frame_prefix<<<dim3(1, p.nclips), 1024, 0, st>>>(s.cnt, s.hdr, p.F, acnt, s.prefix, p.sstride);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -271,27 +284,25 @@ cudaError_t launch_compact(const Problem& p, const Scratch& s, void* out_tokens,
     int nfuse = (p.N + kCopyWarps - 1) / kCopyWarps;
     if (nfuse > sm_count()) nfuse = sm_count();
     const int grid = ncopy + nfuse;
-    const unsigned char* X = reinterpret_cast<const unsigned char*>(p.X);
-    unsigned char* out = reinterpret_cast<unsigned char*>(out_tokens);
-    const dim3 g(grid), b(kCopyWarps * 32);
+    const dim3 g(grid, p.nclips), b(kCopyWarps * 32);
     // the pre-scanned prefix of very long clips is read through plain loads: order that case by the stream
     const bool pdl = p.F <= kWarpPrefixMaxF;
     if (vec) {
         const size_t smem = (size_t)kCopyWarps * kBulkPiece;
         cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_compact_bulk), smem);
         if (e != cudaSuccess) return e;
-        return launch_ex(pdl, smem, k_compact_bulk, g, b, st, X, row_bytes, p.F, p.H, p.W, p.r, s.hdr,
+        return launch_ex(pdl, smem, k_compact_bulk, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, p.r, s.hdr,
                          (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, (const int*)s.dst, out,
-                         out_pos, out_count, s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next,
-                         wait_poll_limit(), wait_tx_extra(), p.stream_once);
+                         s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next,
+                         wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride);
     }
     if (esize == 4)
-        return launch_pdl_if(pdl, k_compact<4>, g, b, st, X, row_bytes, p.F, p.H, p.W, p.r, (const int*)s.hdr,
+        return launch_pdl_if(pdl, k_compact<4>, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, p.r, (const int*)s.hdr,
                           (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, (const int*)s.dst,
-                          out, out_pos, out_count, s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next);
-    return launch_pdl_if(pdl, k_compact<2>, g, b, st, X, row_bytes, p.F, p.H, p.W, p.r, (const int*)s.hdr,
+                          out, s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next, p.sstride);
+    return launch_pdl_if(pdl, k_compact<2>, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, p.r, (const int*)s.hdr,
                       (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, (const int*)s.dst,
-                      out, out_pos, out_count, s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next);
+                      out, s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next, p.sstride);
 }
 
 }  // namespace ttf

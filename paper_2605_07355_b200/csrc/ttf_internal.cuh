@@ -24,9 +24,18 @@ enum { HDR_ANCHOR = 0,          // anchor frame a*
        HDR_CHECK_INDEX = 10,    // that was out of range
        HDR_CHECK_LIMIT = 11 };
 
+constexpr int kMaxGroup = 16;          // clips one launch may cover
+
+// The clips of a launch: blockIdx.y is the clip, its scratch block lies blockIdx.y * sstride bytes after the first one's.
+struct ClipPtrs { const void* X[kMaxGroup]; };
+struct OutPtrs { void* tokens[kMaxGroup]; int* pos[kMaxGroup]; int* count[kMaxGroup]; };
+
 // Problem description handed to every launcher.
 struct Problem {
-    const void* X;      // [F, N, C]
+    const void* X;      // [F, N, C]: the first (or only) clip
+    ClipPtrs xs;        // all clips of the launch
+    int nclips;         // how many (1 unless the call is a batch)
+    size_t sstride;     // bytes between their scratch blocks
     int F, H, W, C, r;
     float t;
     int dtype;          // 0 fp32, 1 bf16
@@ -78,7 +87,7 @@ struct AnchorSrc {
     int fixed;          // >= 0: the anchor is this frame (first / last / explicit rule)
     int from_hdr;       // 1: an earlier kernel left it in hdr[HDR_ANCHOR]
     int* hdr;
-    int* out_anchor;    // optional user copy
+    int* out_anchor;    // optional user copy (single clips only)
 };
 
 inline AnchorSrc make_anchor_src(const Problem& p, const Scratch& s, int* out_anchor);
@@ -119,8 +128,7 @@ cudaError_t launch_match(const Problem& p, const Scratch& s, int* out_anchor, fl
                          unsigned char* keep, cudaStream_t st);
 cudaError_t launch_fuse_count(const Problem& p, const Scratch& s, const int* dst, const unsigned char* keep,
                               int* fuse_cnt, cudaStream_t st);
-cudaError_t launch_compact(const Problem& p, const Scratch& s, void* out_tokens, int* out_pos, int* out_count,
-                           cudaStream_t st);
+cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& out, cudaStream_t st);
 
 cudaError_t launch_restore(const void* comp, size_t row_bytes, int F, int N, const int* anchor,
                            const unsigned char* keep, const int* dst, void* out_full, int* row_index,
@@ -251,6 +259,16 @@ __device__ __forceinline__ bool in_bounds(int* hdr, int site, long long idx, lon
 #else
 __device__ __forceinline__ bool in_bounds(int*, int, long long, long long) { return true; }
 #endif
+
+// this CTA's clip: `p` points into the scratch block of the first clip of the launch
+template <typename T> __device__ __forceinline__ T* clip_block(T* p, size_t sstride) {
+    return reinterpret_cast<T*>(reinterpret_cast<uintptr_t>(p) + (size_t)blockIdx.y * sstride);
+}
+__device__ __forceinline__ AnchorSrc clip_block(AnchorSrc a, size_t sstride) {
+    a.Dp = clip_block(a.Dp, sstride); a.Qp = clip_block(a.Qp, sstride); a.Gp = clip_block(a.Gp, sstride);
+    a.hdr = clip_block(a.hdr, sstride);
+    return a;
+}
 
 struct bf16_t { uint16_t bits; };   // storage type only: all arithmetic is on the widened fp32 value
 

@@ -19,11 +19,14 @@ constexpr int kMatchWarps = 8;
 
 template <typename T, int V>
 __global__ void __launch_bounds__(kMatchWarps * 32)
-k_match_generic(const T* __restrict__ X, int F, int H, int W, int C, int r, float t, int fchunk, int nslice,
+k_match_generic(const __grid_constant__ ClipPtrs xs, int F, int H, int W, int C, int r, float t, int fchunk, int nslice,
                 AnchorSrc asrc, const float* __restrict__ ssq,
                 float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep,
-                int* __restrict__ cnt)
+                int* __restrict__ cnt, size_t sstride)
 {
+    const T* __restrict__ X = reinterpret_cast<const T*>(xs.X[blockIdx.y]);
+    asrc = clip_block(asrc, sstride); ssq = clip_block(ssq, sstride); cnt = clip_block(cnt, sstride);
+    shat = clip_block(shat, sstride); dst = clip_block(dst, sstride); keep = clip_block(keep, sstride);
     pdl_launch_dependents();
     pdl_wait();                                  // norms and the frame statistics are complete
     const int N = H * W;
@@ -127,11 +130,14 @@ __device__ __forceinline__ void match_mma_body(const bf16_t* __restrict__ X, int
 // r <= 1: 32 frames per CTA, norms from Gram diagonals, 96 registers (see TTF_MMA_BOUNDS)
 template <int MT, int NT>
 __global__ void TTF_MMA_BOUNDS
-k_match_mma(const bf16_t* __restrict__ X, int F, int H, int W, int C, int r, float t, AnchorSrc asrc,
+k_match_mma(const __grid_constant__ ClipPtrs xs, int F, int H, int W, int C, int r, float t, AnchorSrc asrc,
             float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
-            int stream_once)
+            int stream_once, size_t sstride)
 {
-    match_mma_body<MT, NT, true, kMmaStagesDefault>(X, F, H, W, C, r, t, asrc, nullptr, 0, shat, dst, keep, cnt, stream_once);
+    match_mma_body<MT, NT, true, kMmaStagesDefault>(reinterpret_cast<const bf16_t*>(xs.X[blockIdx.y]), F, H, W, C, r, t,
+                                                    clip_block(asrc, sstride), nullptr, 0, clip_block(shat, sstride),
+                                                    clip_block(dst, sstride), clip_block(keep, sstride),
+                                                    clip_block(cnt, sstride), stream_once);
 }
 
 // r = 2: the 25 candidate rows of a cell are as much data as 25 source rows, so a CTA takes 64 frames per cell to
@@ -140,11 +146,15 @@ k_match_mma(const bf16_t* __restrict__ X, int F, int H, int W, int C, int r, flo
 constexpr int kWideMT = 4;           // 64 frames per CTA
 constexpr int kWideStages = 2;       // cp.async stages per warp (the 64 x 32 accumulator tile leaves no room for more)
 __global__ void __launch_bounds__(kMmaWarps * 32, 2)
-k_match_mma_wide(const bf16_t* __restrict__ X, int F, int H, int W, int C, int r, float t, AnchorSrc asrc,
+k_match_mma_wide(const __grid_constant__ ClipPtrs xs, int F, int H, int W, int C, int r, float t, AnchorSrc asrc,
                  const float* __restrict__ ssq, int nslice,
-                 float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt)
+                 float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
+                 size_t sstride)
 {
-    match_mma_body<kWideMT, 4, false, kWideStages>(X, F, H, W, C, r, t, asrc, ssq, nslice, shat, dst, keep, cnt, 0);
+    match_mma_body<kWideMT, 4, false, kWideStages>(reinterpret_cast<const bf16_t*>(xs.X[blockIdx.y]), F, H, W, C, r, t,
+                                                   clip_block(asrc, sstride), clip_block(ssq, sstride), nslice,
+                                                   clip_block(shat, sstride), clip_block(dst, sstride),
+                                                   clip_block(keep, sstride), clip_block(cnt, sstride), 0);
 }
 
 template <int MT, int NT>
@@ -154,9 +164,9 @@ static cudaError_t launch_mma_t(const Problem& p, const Scratch& s, int* out_anc
     constexpr size_t smem = sizeof(uint4) * kMmaWarps * kMmaStagesDefault * (2 * MT + NT) * 32;
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_mma<MT, NT>), smem);
     if (e != cudaSuccess) return e;
-    return launch_ex(true, smem, k_match_mma<MT, NT>, dim3((unsigned)(chunks * p.N)),
-                     dim3(kMmaWarps * 32), st, reinterpret_cast<const bf16_t*>(p.X), p.F, p.H, p.W, p.C, p.r, p.t,
-                     make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, p.stream_once);
+    return launch_ex(true, smem, k_match_mma<MT, NT>, dim3((unsigned)(chunks * p.N), p.nclips),
+                     dim3(kMmaWarps * 32), st, p.xs, p.F, p.H, p.W, p.C, p.r, p.t,
+                     make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, p.stream_once, p.sstride);
 }
 
 static cudaError_t launch_mma_wide(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
@@ -165,9 +175,9 @@ static cudaError_t launch_mma_wide(const Problem& p, const Scratch& s, int* out_
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_mma_wide), smem);
     if (e != cudaSuccess) return e;
     const long long chunks = (p.F + 16 * kWideMT - 1) / (16 * kWideMT);
-    return launch_ex(true, smem, k_match_mma_wide, dim3((unsigned)(chunks * p.N)), dim3(kMmaWarps * 32),
-                     st, reinterpret_cast<const bf16_t*>(p.X), p.F, p.H, p.W, p.C, p.r, p.t,
-                     make_anchor_src(p, s, out_anchor), (const float*)s.ssq, p.nslice, shat, dst, keep, s.cnt);
+    return launch_ex(true, smem, k_match_mma_wide, dim3((unsigned)(chunks * p.N), p.nclips), dim3(kMmaWarps * 32),
+                     st, p.xs, p.F, p.H, p.W, p.C, p.r, p.t,
+                     make_anchor_src(p, s, out_anchor), (const float*)s.ssq, p.nslice, shat, dst, keep, s.cnt, p.sstride);
 }
 
 template <typename T, int V>
@@ -176,15 +186,15 @@ static cudaError_t launch_generic_t(const Problem& p, const Scratch& s, int* out
     // enough CTAs to fill the GPU a few times over: split the frames into chunks when the grid is small
     int fchunk = p.F;
     const long long want = 4LL * sm_count();
-    if ((long long)p.N < want) {
-        long long chunks = (want + p.N - 1) / p.N;
+    if ((long long)p.N * p.nclips < want) {
+        long long chunks = (want + (long long)p.N * p.nclips - 1) / ((long long)p.N * p.nclips);
         fchunk = (int)((p.F + chunks - 1) / chunks);
         if (fchunk < kMatchWarps) fchunk = kMatchWarps;
     }
     const long long nchunk = (p.F + fchunk - 1) / fchunk;
-    return launch_pdl(k_match_generic<T, V>, dim3((unsigned)(nchunk * p.N)), dim3(kMatchWarps * 32), st,
-                      reinterpret_cast<const T*>(p.X), p.F, p.H, p.W, p.C, p.r, p.t, fchunk, p.nslice,
-                      make_anchor_src(p, s, out_anchor), (const float*)s.ssq, shat, dst, keep, s.cnt);
+    return launch_pdl(k_match_generic<T, V>, dim3((unsigned)(nchunk * p.N), p.nclips), dim3(kMatchWarps * 32), st,
+                      p.xs, p.F, p.H, p.W, p.C, p.r, p.t, fchunk, p.nslice,
+                      make_anchor_src(p, s, out_anchor), (const float*)s.ssq, shat, dst, keep, s.cnt, p.sstride);
 }
 
 cudaError_t launch_match(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,

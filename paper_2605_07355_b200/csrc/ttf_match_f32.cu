@@ -52,13 +52,16 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, float ac
     return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
 }
 
-template <int R>
+template <int R, int G>
 __global__ void __launch_bounds__(F32Shape<R>::MAXW * 32)
-k_match_f32(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-            int F, int H, int W, int C, float t, AnchorSrc asrc,
+k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc,
             float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
-            int wait_limit, int tx_extra)
+            int wait_limit, int tx_extra, size_t sstride)
 {
+    const CUtensorMap& mapA = maps.a[blockIdx.y];
+    const CUtensorMap& mapB = maps.b[blockIdx.y];
+    asrc = clip_block(asrc, sstride); cnt = clip_block(cnt, sstride);
+    shat = clip_block(shat, sstride); dst = clip_block(dst, sstride); keep = clip_block(keep, sstride);
     using S = F32Shape<R>;
     extern __shared__ __align__(128) unsigned char f32_ring[];
     __shared__ uint64_t bar[S::STAGES];
@@ -191,30 +194,36 @@ k_match_f32(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 
 // Frames per CTA: 32 reads the window rows least often (41 rows per 32 at r = 1, 25 per 16), but a grid of fewer than
 // three CTAs per two SMs leaves SMs idle: then 16, then 8 (at least FW).
-template <int R>
+template <int R, int G>
 static cudaError_t launch_f32_t(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                 unsigned char* keep, cudaStream_t st) {
     using S = F32Shape<R>;
     int FR = 32;
-    while (FR > S::FW && (FR / 2 >= p.F || (long long)p.N * ((p.F + FR - 1) / FR) * 2 < 3LL * sm_count())) FR /= 2;
-    CUtensorMap mapA, mapB;
-    if (!make_tensor_map(&mapA, p.X, 0, p.F, p.H, p.W, p.C, kF32KC, 1, 1, FR, false) ||
-        !make_tensor_map(&mapB, p.X, 0, p.F, p.H, p.W, p.C, kF32KC, S::SIDE, S::SIDE, 1, false))
-        return cudaErrorInvalidValue;
+    while (FR > S::FW && (FR / 2 >= p.F || (long long)p.N * p.nclips * ((p.F + FR - 1) / FR) * 2 < 3LL * sm_count())) FR /= 2;
+    ClipMaps<G> maps;
+    for (int n = 0; n < p.nclips; ++n)
+        if (!make_tensor_map(&maps.a[n], p.xs.X[n], 0, p.F, p.H, p.W, p.C, kF32KC, 1, 1, FR, false) ||
+            !make_tensor_map(&maps.b[n], p.xs.X[n], 0, p.F, p.H, p.W, p.C, kF32KC, S::SIDE, S::SIDE, 1, false))
+            return cudaErrorInvalidValue;
     const size_t smem = (size_t)S::STAGES * (FR + S::WIN) * kF32Row;
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_f32<R>), (size_t)S::STAGES * (32 + S::WIN) * kF32Row);
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_f32<R, G>), (size_t)S::STAGES * (32 + S::WIN) * kF32Row);
     if (e != cudaSuccess) return e;
     const long long units = (long long)p.N * ((p.F + FR - 1) / FR);
-    return launch_ex(true, smem, k_match_f32<R>, dim3((unsigned)units), dim3(FR / S::FW * 32), st, mapA, mapB, p.F, p.H,
+    return launch_ex(true, smem, k_match_f32<R, G>, dim3((unsigned)units, p.nclips), dim3(FR / S::FW * 32), st, maps, p.F, p.H,
                      p.W, p.C, p.t, make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, wait_poll_limit(),
-                     wait_tx_extra());
+                     wait_tx_extra(), p.sstride);
 }
 
 cudaError_t launch_match_f32(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                              unsigned char* keep, cudaStream_t st) {
-    if (p.r == 0) return launch_f32_t<0>(p, s, out_anchor, shat, dst, keep, st);
-    if (p.r == 1) return launch_f32_t<1>(p, s, out_anchor, shat, dst, keep, st);
-    return launch_f32_t<2>(p, s, out_anchor, shat, dst, keep, st);
+    if (p.nclips > 1) {
+        if (p.r == 0) return launch_f32_t<0, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
+        if (p.r == 1) return launch_f32_t<1, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
+        return launch_f32_t<2, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
+    }
+    if (p.r == 0) return launch_f32_t<0, 1>(p, s, out_anchor, shat, dst, keep, st);
+    if (p.r == 1) return launch_f32_t<1, 1>(p, s, out_anchor, shat, dst, keep, st);
+    return launch_f32_t<2, 1>(p, s, out_anchor, shat, dst, keep, st);
 }
 
 }  // namespace ttf

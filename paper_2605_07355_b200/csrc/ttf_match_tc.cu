@@ -140,14 +140,17 @@ __device__ __forceinline__ float ssq8(const uint4& v, float acc) {
     return acc;
 }
 
-template <int R>
+template <int R, int G>
 __global__ void __launch_bounds__(kTcThreads)
-k_match_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-           int F, int H, int W, int C, float t, AnchorSrc asrc, int pieces,
+k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc, int pieces,
            float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
-           int wait_limit, int tx_extra, int stream_once)
+           int wait_limit, int tx_extra, int stream_once, size_t sstride)
 {
     using S = TcShape<R>;
+    const CUtensorMap& mapA = maps.a[blockIdx.y];
+    const CUtensorMap& mapB = maps.b[blockIdx.y];
+    asrc = clip_block(asrc, sstride); cnt = clip_block(cnt, sstride);
+    shat = clip_block(shat, sstride); dst = clip_block(dst, sstride); keep = clip_block(keep, sstride);
     extern __shared__ unsigned char dyn_raw[];
     __shared__ uint64_t bar_full[S::STAGES], bar_empty[S::STAGES], bar_acc;
     __shared__ uint32_t s_tmem;
@@ -455,23 +458,24 @@ int tc_match_pieces(const Problem& p) {
     return pieces;
 }
 
-template <int R>
+template <int R, int G>
 static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                unsigned char* keep, cudaStream_t st) {
     using S = TcShape<R>;
     static_assert((size_t)7 * ((S::WIN + 1) * kTcM + S::NCAND) * 4 <= (size_t)S::STAGES * S::STAGE || R == 2, "exchange rows must fit the ring");
     static_assert((size_t)3 * ((S::WIN + 1) * kTcM + S::NCAND) * 4 <= (size_t)S::STAGES * S::STAGE, "exchange rows must fit the ring");
-    CUtensorMap mapA, mapB;
-    if (!make_tensor_map(&mapA, p.X, 1, p.F, p.H, p.W, p.C, kTcKC, kTcWB, 1, kTcFR, true) ||
-        !make_tensor_map(&mapB, p.X, 1, p.F, p.H, p.W, p.C, kTcKC, S::BW, S::SIDE, 1, true))
-        return cudaErrorInvalidValue;
+    ClipMaps<G> maps;
+    for (int n = 0; n < p.nclips; ++n)
+        if (!make_tensor_map(&maps.a[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, kTcWB, 1, kTcFR, true) ||
+            !make_tensor_map(&maps.b[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, S::BW, S::SIDE, 1, true))
+            return cudaErrorInvalidValue;
     const size_t smem = (size_t)S::STAGES * S::STAGE + 1024;
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R>), smem);
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R, G>), smem);
     if (e != cudaSuccess) return e;
     const int pieces = tc_match_pieces(p);
     const long long tiles = (long long)tc_match_tiles(p);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(tiles * pieces)); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)(tiles * pieces), p.nclips); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -482,15 +486,20 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
         ++n;
     }
     cfg.attrs = attr; cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, k_match_tc<R>, mapA, mapB, p.F, p.H, p.W, p.C, p.t, make_anchor_src(p, s, out_anchor),
-                              pieces, shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(), p.stream_once);
+    return cudaLaunchKernelEx(&cfg, k_match_tc<R, G>, maps, p.F, p.H, p.W, p.C, p.t, make_anchor_src(p, s, out_anchor),
+                              pieces, shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride);
 }
 
 cudaError_t launch_match_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                             unsigned char* keep, cudaStream_t st) {
-    if (p.r == 0) return launch_tc_t<0>(p, s, out_anchor, shat, dst, keep, st);
-    if (p.r == 1) return launch_tc_t<1>(p, s, out_anchor, shat, dst, keep, st);
-    return launch_tc_t<2>(p, s, out_anchor, shat, dst, keep, st);
+    if (p.nclips > 1) {
+        if (p.r == 0) return launch_tc_t<0, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
+        if (p.r == 1) return launch_tc_t<1, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
+        return launch_tc_t<2, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
+    }
+    if (p.r == 0) return launch_tc_t<0, 1>(p, s, out_anchor, shat, dst, keep, st);
+    if (p.r == 1) return launch_tc_t<1, 1>(p, s, out_anchor, shat, dst, keep, st);
+    return launch_tc_t<2, 1>(p, s, out_anchor, shat, dst, keep, st);
 }
 
 }  // namespace ttf

@@ -3,9 +3,14 @@
 
 #include <cuda.h>
 
+#include "ttf_internal.cuh"
 #include "ttf_async.cuh"
 
 namespace ttf {
+
+// Tile copies of the source rows (a) and of the window rows (b) of every clip of a launch.  A kernel parameter, so a
+// launch over one clip has a type of its own: 256 bytes instead of 4 KB to hand over with every launch.
+template <int G> struct ClipMaps { CUtensorMap a[G], b[G]; };
 
 // Tile of (kc channels, bw cells, bh rows, bf frames) elements, zeros outside X; swizzle128: the 128-byte swizzle
 // (kc * element size must be 128 bytes), else rows of the tile are stored plainly.  dtype 0 fp32, 1 bf16.
