@@ -77,10 +77,9 @@ constexpr int kCopyUnroll = 8;       // 16-byte units in flight per lane of the 
 constexpr int kBulkPiece = 8192;     // bytes per staging slot; longer rows go in pieces
 
 __global__ void __launch_bounds__(kCopyWarps * 32)
-k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, int W, int r,
+k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, int W,
                int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
-               const unsigned char* __restrict__ keep, const int* __restrict__ dst,
-               const __grid_constant__ OutPtrs outs, int* __restrict__ fuse_cnt, int ncopy_blocks, int NA, int acnt, int t_off, int pos_base,
+               const unsigned char* __restrict__ keep, const __grid_constant__ OutPtrs outs, int NA, int acnt, int t_off, int pos_base,
                int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride)
 {
     const unsigned char* __restrict__ X = reinterpret_cast<const unsigned char*>(xs.X[blockIdx.y]);
@@ -88,7 +87,7 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     int* __restrict__ out_pos = outs.pos[blockIdx.y];
     int* __restrict__ out_count = outs.count[blockIdx.y];
     hdr = clip_block(hdr, sstride); cnt = clip_block(cnt, sstride); gprefix = clip_block(gprefix, sstride);
-    keep = clip_block(keep, sstride); dst = clip_block(dst, sstride); fuse_cnt = clip_block(fuse_cnt, sstride);
+    keep = clip_block(keep, sstride);
     extern __shared__ __align__(128) unsigned char stage[];     // [kCopyWarps][kBulkPiece]
     __shared__ uint64_t bar[kCopyWarps];
     const int N = H * W;
@@ -106,12 +105,8 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     if (late_trigger) pdl_launch_dependents();
     trace_mark(hdr, 6, false);
     const int a = __ldcg(hdr + HDR_ANCHOR);
-    if ((int)blockIdx.x >= ncopy_blocks) {       // bookkeeping CTAs: tokens fused into each anchor cell
-        fuse_count_cta(F, H, W, r, a, keep, dst, fuse_cnt, (int)blockIdx.x - ncopy_blocks, (int)gridDim.x - ncopy_blocks);
-        return;
-    }
     const int gw = blockIdx.x * kCopyWarps + w;
-    const int nw = ncopy_blocks * kCopyWarps;
+    const int nw = gridDim.x * kCopyWarps;
     int Lp = 0;
     if (gw == 0) {                               // L' = N + P (Eq. Lpre)
         int kk, bb;
@@ -181,21 +176,244 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     trace_mark(hdr, 3, true);
 }
 
-template <int COPY_BYTES>
-__global__ void __launch_bounds__(kCopyWarps * 32)
-k_compact(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, int W, int r,
-          const int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
-          const unsigned char* __restrict__ keep, const int* __restrict__ dst,
-          const __grid_constant__ OutPtrs outs,
-          int* __restrict__ fuse_cnt, int ncopy_blocks, int NA, int acnt, int t_off, int pos_base, int late_trigger,
-          size_t sstride)
+// The same for short rows, of which a warp moves many.  A CTA owns a contiguous range of output rows.  It packs the keep
+// flags of a window of tokens into bit words in shared memory together with the exclusive prefix of their population
+// counts, after which the source row of any output row of the window is found by a binary search and a select in shared
+// memory: the three dependent round trips (anchor, counts, flags) are paid once per window instead of once per row.
+// Clips of up to kGatherWindow tokens need no survivor counts: the window is the whole clip.  Longer ones enter the walk
+// at the frame that holds the CTA's first row and take as many windows as its range needs.
+//
+// A warp moves a batch of consecutive output rows at a time, through two slots in turn, so that the next batch is on its
+// way while this one lands: every lane issues the load of one row, and the batch leaves as one store, since the rows are
+// contiguous in the output.
+constexpr int kGatherSlot = 4096;                       // bytes of a staging slot; a warp has two
+constexpr int kGatherWords = 512;                       // bit words of a window
+constexpr int kGatherWindow = kGatherWords * 32;        // tokens
+constexpr int kGatherThreads = kCopyWarps * 32;
+
+// 32 keep flags (0 or 1 each) -> one bit each.  (The flags are masked first: a word that reaches past the end of the
+// array holds other bytes, whose higher bits would spill into its neighbours' in the product.)
+__device__ __forceinline__ unsigned pack_flags(const uint4& lo, const uint4& hi) {
+    const unsigned w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    unsigned bits = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) bits |= ((((w[e] & 0x01010101u) * 0x01020408u) >> 24) & 0xfu) << (4 * e);   // byte i -> bit i
+    return bits;
+}
+// position of the n-th (0-based) set bit; n < popcount(bits)
+__device__ __forceinline__ int select_bit(unsigned bits, int n) {
+    int at = 0;
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) {
+        const int c = __popc((bits >> at) & ((1u << h) - 1u));
+        if (n >= c) { n -= c; at += h; }
+    }
+    return at;
+}
+
+__global__ void __launch_bounds__(kGatherThreads)
+k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H, int W,
+               int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
+               const unsigned char* __restrict__ keep, const __grid_constant__ OutPtrs outs, int NA, int acnt, int t_off,
+               int pos_base, int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride)
 {
     const unsigned char* __restrict__ X = reinterpret_cast<const unsigned char*>(xs.X[blockIdx.y]);
     unsigned char* __restrict__ out_tokens = reinterpret_cast<unsigned char*>(outs.tokens[blockIdx.y]);
     int* __restrict__ out_pos = outs.pos[blockIdx.y];
     int* __restrict__ out_count = outs.count[blockIdx.y];
     hdr = clip_block(hdr, sstride); cnt = clip_block(cnt, sstride); gprefix = clip_block(gprefix, sstride);
-    keep = clip_block(keep, sstride); dst = clip_block(dst, sstride); fuse_cnt = clip_block(fuse_cnt, sstride);
+    keep = clip_block(keep, sstride);
+
+    extern __shared__ __align__(128) unsigned char stage[];     // [kCopyWarps][2][kGatherSlot]
+    __shared__ uint64_t bar[kCopyWarps][2];
+    __shared__ unsigned s_bits[kGatherWords];
+    __shared__ int s_pref[kGatherWords];
+    __shared__ int s_warp[kCopyWarps];
+    const int N = H * W, FN = F * N;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    if (!late_trigger) pdl_launch_dependents();  // (see k_compact_bulk)
+    trace_mark(hdr, 3, false);
+    if (lane == 0) { mbar_init(&bar[w][0], 1); mbar_init(&bar[w][1], 1); mbar_init_fence(); }
+    pdl_wait();                                  // keep flags and survivor counts are complete
+    if (late_trigger) pdl_launch_dependents();
+    trace_mark(hdr, 6, false);
+
+    // ---- window of the walk: bits and prefix of tokens [T0, T0 + kGatherWindow) ----------------------------------
+    constexpr int WPT = kGatherWords / kGatherThreads;          // consecutive words per thread
+    static_assert(kGatherWords % kGatherThreads == 0, "whole words per thread");
+    const int a = __ldcg(hdr + HDR_ANCHOR);
+    auto load_window = [&](int T0, int first) -> int {          // tokens before `first` do not count; returns the total
+        uint4 v[WPT][2];
+#pragma unroll
+        for (int u = 0; u < WPT; ++u) {
+            const int f = T0 + (tid * WPT + u) * 32;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                // (the flag array is 256-byte aligned and followed by other scratch: a load that starts inside it may
+                // run past its end by less than 16 bytes, which the masks below discard)
+                v[u][h] = (unsigned)(f + h * 16) < (unsigned)FN ? __ldcg(reinterpret_cast<const uint4*>(keep + f) + h)
+                                                                : make_uint4(0, 0, 0, 0);
+            }
+        }
+        auto below = [](int n) -> unsigned { return n <= 0 ? 0u : (n >= 32 ? 0xffffffffu : (1u << n) - 1u); };
+        unsigned b[WPT];
+        int mine = 0;
+#pragma unroll
+        for (int u = 0; u < WPT; ++u) {
+            const int f = T0 + (tid * WPT + u) * 32;
+            const unsigned anchor = below((a + 1) * N - f) & ~below(a * N - f);
+            b[u] = pack_flags(v[u][0], v[u][1]);
+            b[u] = acnt ? b[u] | anchor : b[u] & ~anchor;       // the anchor frame: all of its tokens, or none
+            b[u] &= f < 0 ? 0u : below(FN - f) & ~below(first - f);          // (f < 0: past 2^31, hence past the end)
+            mine += __popc(b[u]);
+        }
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int n = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += n;
+        }
+        __syncthreads();                                        // (the window before this one is done with)
+        if (lane == 31) s_warp[w] = incl;
+        __syncthreads();
+        int at = incl - mine, total = 0;
+#pragma unroll
+        for (int ww = 0; ww < kCopyWarps; ++ww) { if (ww < w) at += s_warp[ww]; total += s_warp[ww]; }
+#pragma unroll
+        for (int u = 0; u < WPT; ++u) {
+            s_bits[tid * WPT + u] = b[u];
+            s_pref[tid * WPT + u] = at;
+            at += __popc(b[u]);
+        }
+        __syncthreads();
+        return total;
+    };
+
+    // ---- this CTA's rows [j0, j1) of the output ------------------------------------------------------------------
+    const bool whole = FN <= kGatherWindow;
+    int k, before = 0, P, T0 = 0, in_window = 0;
+    if (whole) P = in_window = load_window(0, 0);
+    else { P = find_frame(cnt, gprefix, F, a, acnt, lane, -1, k, before); before = 0; }
+    const int Lp = NA + P;                       // L' = N + P (Eq. Lpre)
+    if (blockIdx.x == 0 && tid == 0) *reinterpret_cast<volatile int*>(out_count) = Lp;
+    const int per = (Lp + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int j0 = (int)min((long long)Lp, (long long)blockIdx.x * per), j1 = min(Lp, j0 + per);
+    // rows per batch: what fits a slot, but no more than leaves every warp of the CTA a batch
+    int R = min(32, kGatherSlot / row_bytes);
+    R = max(1, min(R, (per + kCopyWarps - 1) / kCopyWarps));
+
+    unsigned char* buf = stage + (size_t)w * 2 * kGatherSlot;
+    uint32_t phase = 0;                          // bit h: parity of slot h
+    bool gave_up = false;                        // (lane 0 decides; all lanes of the warp know)
+    const unsigned long long once = l2_evict_first_policy();
+
+    auto source = [&](int j) {
+        if (j < NA) return a * N + j;            // anchor rows first (Eq. xprime_stack)
+        const int n = j - NA - before;           // the n-th token of the window: word by binary search, then the bit
+        int lo = 0;
+#pragma unroll
+        for (int h = kGatherWords / 2; h > 0; h >>= 1) if (s_pref[lo + h] <= n) lo += h;
+        return T0 + lo * 32 + select_bit(s_bits[lo], n - s_pref[lo]);
+    };
+    // lanes 0 .. n-1 issue the loads of output rows jb .. jb + n - 1 into slot h and write their positions
+    auto issue = [&](int jb, int n, int h) {
+        if (lane == 0) {
+            bulk_wait_read<0>();                 // the store that used this slot has finished reading it
+            mbar_arrive_expect_tx(&bar[w][h], (uint32_t)(n * row_bytes) + (uint32_t)tx_extra);
+        }
+        __syncwarp();
+        if (lane < n) {
+            const int j = jb + lane, f = source(j);
+            const bool ok = in_bounds(hdr, 4, j, FN) && in_bounds(hdr, 4, f, FN);      // (checked build)
+            unsigned char* d = buf + h * kGatherSlot + lane * row_bytes;
+            // (a row the checked build refuses is replaced by row 0, so that the batch still completes)
+            const unsigned char* src = X + (size_t)(ok ? f : 0) * row_bytes;
+            if (stream_once) bulk_load_hint(d, src, (uint32_t)row_bytes, &bar[w][h], once);
+            else bulk_load(d, src, (uint32_t)row_bytes, &bar[w][h]);
+            if (ok) {                            // p_{k,i} = (k, y_i, x_i)  (Eq. compress_pos)
+                const int kk = f / N, i = f - kk * N, yy = i / W;
+                int* p = out_pos + (size_t)j * 3;
+                p[0] = pos_base + kk + t_off; p[1] = pos_base + yy; p[2] = pos_base + i - yy * W;
+            }
+        }
+    };
+    auto finish = [&](int jb, int n, int h) {    // the batch has landed: one store
+        if (lane == 0) {
+            if (!mbar_wait(&bar[w][h], (phase >> h) & 1, wait_limit)) {
+                mbar_wait(&bar[w][h], (phase >> h) & 1, wait_limit);     // one more bounded chance for the copies to land
+                gave_up = true;
+            } else if (in_bounds(hdr, 4, jb + n - 1, FN)) {
+                unsigned char* d = out_tokens + (size_t)jb * row_bytes;
+                if (stream_once) bulk_store_hint(d, buf + h * kGatherSlot, (uint32_t)(n * row_bytes), once);
+                else bulk_store(d, buf + h * kGatherSlot, (uint32_t)(n * row_bytes));
+                bulk_commit();
+            }
+        }
+        phase ^= 1u << h;
+        gave_up = __shfl_sync(0xffffffffu, gave_up ? 1 : 0, 0) != 0;
+    };
+    auto move_rows = [&](int ja, int jb) {       // rows [ja, jb) of the output, by the warps of the CTA in turn
+        int at = ja + w * R, h = 0;
+        if (at < jb && !gave_up) issue(at, min(R, jb - at), 0);
+        for (; at < jb && !gave_up; at += kCopyWarps * R) {
+            const int next = at + kCopyWarps * R;
+            if (next < jb) issue(next, min(R, jb - next), h ^ 1);
+            finish(at, min(R, jb - at), h);
+            h ^= 1;
+        }
+    };
+
+    if (whole) move_rows(j0, j1);
+    else {
+        move_rows(j0, min(j1, NA));
+        int e = max(j0, NA) - NA;                // next token of the walk this CTA emits
+        const int e1 = j1 - NA;
+        if (e < e1) {                            // (e, e1 and the counts are the same for all threads)
+            find_frame(cnt, gprefix, F, a, acnt, lane, e, k, before);
+            T0 = (k * N) & ~31;
+            in_window = load_window(T0, k * N);
+        }
+        while (e < e1) {
+            const int upto = min(e1, before + in_window);
+            move_rows(NA + e, NA + upto);
+            e = upto;
+            if (e >= e1 || T0 >= FN - kGatherWindow) break;      // (the second cannot happen when the counts match the flags)
+            before += in_window;
+            T0 += kGatherWindow;
+            in_window = load_window(T0, 0);
+        }
+    }
+
+    if (lane == 0) {
+        if (gave_up)                             // copies still on their way into this CTA's shared memory (bounded again)
+            for (int h = 0; h < 2; ++h) mbar_wait(&bar[w][h], (phase >> h) & 1, wait_limit);
+        bulk_wait<0>();                          // all rows of this warp are in global memory
+        if (gave_up) {                           // L' or -1: see k_compact_bulk
+            atomicExch(hdr + HDR_ERROR, 1);
+            __threadfence();
+            *reinterpret_cast<volatile int*>(out_count) = -1;
+        }
+        if (blockIdx.x == 0 && w == 0) {
+            __threadfence();
+            if (atomicAdd(hdr + HDR_ERROR, 0)) *reinterpret_cast<volatile int*>(out_count) = -1;
+        }
+    }
+    trace_mark(hdr, 3, true);
+}
+
+template <int COPY_BYTES>
+__global__ void __launch_bounds__(kCopyWarps * 32)
+k_compact(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, int W,
+          const int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
+          const unsigned char* __restrict__ keep, const __grid_constant__ OutPtrs outs, int NA, int acnt, int t_off,
+          int pos_base, int late_trigger, size_t sstride)
+{
+    const unsigned char* __restrict__ X = reinterpret_cast<const unsigned char*>(xs.X[blockIdx.y]);
+    unsigned char* __restrict__ out_tokens = reinterpret_cast<unsigned char*>(outs.tokens[blockIdx.y]);
+    int* __restrict__ out_pos = outs.pos[blockIdx.y];
+    int* __restrict__ out_count = outs.count[blockIdx.y];
+    hdr = clip_block(hdr, sstride); cnt = clip_block(cnt, sstride); gprefix = clip_block(gprefix, sstride);
+    keep = clip_block(keep, sstride);
     using U = typename CopyUnit<COPY_BYTES>::type;
     const int N = H * W;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -206,17 +424,11 @@ k_compact(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, i
     trace_mark(const_cast<int*>(hdr), 6, false);
     const int a = __ldcg(hdr + HDR_ANCHOR);
 
-    // ---- bookkeeping CTAs: tokens fused into each anchor cell ------------------------------------------------
-    if ((int)blockIdx.x >= ncopy_blocks) {
-        fuse_count_cta(F, H, W, r, a, keep, dst, fuse_cnt, (int)blockIdx.x - ncopy_blocks, (int)gridDim.x - ncopy_blocks);
-        return;
-    }
-
     // ---- output-driven gather, one warp per output row, no block-level synchronisation -----------------------
     // frame search: the frame that holds the e-th preserved source token (flat order, anchor frame skipped)
     // and the number of preserved tokens before that frame.  Returns the total P when e is past the end.
     const int gw = blockIdx.x * kCopyWarps + w;            // global warp index
-    const int nw = ncopy_blocks * kCopyWarps;
+    const int nw = gridDim.x * kCopyWarps;
     if (gw == 0) {                                         // L' = N + P (Eq. Lpre)
         int kk, bb;
         const int P = find_frame(cnt, gprefix, F, a, acnt, lane, -1, kk, bb);
@@ -255,13 +467,20 @@ k_compact(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, i
     trace_mark(const_cast<int*>(hdr), 3, true);
 }
 
+// tokens fused into each anchor cell (ttf_query)
+__global__ void __launch_bounds__(kCopyWarps * 32)
+k_fuse_count(int F, int H, int W, int r, const int* hdr, const unsigned char* keep, const int* dst, int* fuse_cnt)
+{
+    pdl_launch_dependents();
+    pdl_wait();
+    fuse_count_cta(F, H, W, r, __ldcg(hdr + HDR_ANCHOR), keep, dst, fuse_cnt, (int)blockIdx.x, (int)gridDim.x);
+}
+
 cudaError_t launch_fuse_count(const Problem& p, const Scratch& s, const int* dst, const unsigned char* keep,
                               int* fuse_cnt, cudaStream_t st) {
-    // bookkeeping only: the same kernel with zero copy CTAs
     const int nb = (p.N + kCopyWarps - 1) / kCopyWarps;
-    k_compact<4><<<nb < 1024 ? nb : 1024, kCopyWarps * 32, 0, st>>>(
-        p.xs, 0, p.F, p.H, p.W, p.r, s.hdr, s.cnt, s.prefix, keep, dst, OutPtrs(), fuse_cnt, 0, p.N, 0, 0, 0, 0, 0);
-    return cudaGetLastError();
+    return launch_pdl(k_fuse_count, dim3(nb < 1024 ? nb : 1024), dim3(kCopyWarps * 32), st, p.F, p.H, p.W, p.r,
+                      (const int*)s.hdr, keep, dst, fuse_cnt);
 }
 
 cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& out, cudaStream_t st) {
@@ -278,31 +497,46 @@ cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& ou
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    // enough warps for one output row each at the usual two-thirds removal (a warp loops when there are more)
+    // enough warps for one output row each at the usual two-thirds removal, at most three CTAs per SM and clip (a warp
+    // loops when there are more)
     const long long want = ((long long)p.F * p.N / 3 + p.N + kCopyWarps - 1) / kCopyWarps;
-    const int ncopy = (int)(want < 3LL * sm_count() ? (want < 1 ? 1 : want) : 3LL * sm_count());
-    int nfuse = (p.N + kCopyWarps - 1) / kCopyWarps;
-    if (nfuse > sm_count()) nfuse = sm_count();
-    const int grid = ncopy + nfuse;
-    const dim3 g(grid, p.nclips), b(kCopyWarps * 32);
+    int grid = (int)(want < 3LL * sm_count() ? (want < 1 ? 1 : want) : 3LL * sm_count());
+    const dim3 b(kCopyWarps * 32);
     // the pre-scanned prefix of very long clips is read through plain loads: order that case by the stream
     const bool pdl = p.F <= kWarpPrefixMaxF;
+    // Short rows in batches: up to half a slot always, up to a slot where the clip is one window of flags.  Measured, us
+    // per pass with one row per warp at a time / with batches: 128 x 32 x 32 x 64 (128-byte rows) 89.3 / 44.1,
+    // 128 x 24 x 24 x 256 58.5 / 39.6, 64 x 24 x 24 x 512 43.7 / 35.6, 64 x 32 x 32 x 1024 93.2 / 80.9; 4096-byte rows:
+    // 32 x 16 x 16 (one window) 29.3 / 28.5, 128 x 16 x 16 (two windows) 74.6 / 78.4; 2320-byte rows, one window
+    // 23.2 / 21.7.  Longer rows keep every warp's slot full by themselves.
+    if (vec && (row_bytes <= kGatherSlot / 2 || (row_bytes <= kGatherSlot && (long long)p.F * p.N <= kGatherWindow))) {
+        constexpr size_t smem = (size_t)kCopyWarps * 2 * kGatherSlot;
+        cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_compact_rows), smem);
+        if (e != cudaSuccess) return e;
+        long long most = 3LL * sm_count() / p.nclips;
+        if (most < 1) most = 1;
+        if (grid > most) grid = (int)most;
+        return launch_ex(pdl, smem, k_compact_rows, dim3(grid, p.nclips), b, st, p.xs, (int)row_bytes, p.F, p.H, p.W, s.hdr,
+                         (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt,
+                         p.pos_t_offset, p.pos_base, p.chain_next, wait_poll_limit(), wait_tx_extra(), p.stream_once,
+                         p.sstride);
+    }
+    const dim3 g(grid, p.nclips);
     if (vec) {
         const size_t smem = (size_t)kCopyWarps * kBulkPiece;
         cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_compact_bulk), smem);
         if (e != cudaSuccess) return e;
-        return launch_ex(pdl, smem, k_compact_bulk, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, p.r, s.hdr,
-                         (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, (const int*)s.dst, out,
-                         s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next,
-                         wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride);
+        return launch_ex(pdl, smem, k_compact_bulk, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, s.hdr, (const int*)s.cnt,
+                         (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt, p.pos_t_offset, p.pos_base,
+                         p.chain_next, wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride);
     }
     if (esize == 4)
-        return launch_pdl_if(pdl, k_compact<4>, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, p.r, (const int*)s.hdr,
-                          (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, (const int*)s.dst,
-                          out, s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next, p.sstride);
-    return launch_pdl_if(pdl, k_compact<2>, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, p.r, (const int*)s.hdr,
-                      (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, (const int*)s.dst,
-                      out, s.fuse_cnt, ncopy, NA, acnt, p.pos_t_offset, p.pos_base, p.chain_next, p.sstride);
+        return launch_pdl_if(pdl, k_compact<4>, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, (const int*)s.hdr,
+                             (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt,
+                             p.pos_t_offset, p.pos_base, p.chain_next, p.sstride);
+    return launch_pdl_if(pdl, k_compact<2>, g, b, st, p.xs, row_bytes, p.F, p.H, p.W, (const int*)s.hdr,
+                         (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt,
+                         p.pos_t_offset, p.pos_base, p.chain_next, p.sstride);
 }
 
 }  // namespace ttf

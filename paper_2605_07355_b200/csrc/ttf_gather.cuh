@@ -69,8 +69,11 @@ __device__ __forceinline__ int find_frame(const int* __restrict__ cnt, const int
 #pragma unroll
         for (int q = 0; q < kScanChunks; ++q) {
             const int k = base + q * 32 + lane;
-            c[q] = k < F ? (k == a ? acnt : __ldcg(cnt + k)) : 0;
+            c[q] = k < F ? __ldcg(cnt + k) : 0;            // (unconditional: the load need not wait for the anchor word)
         }
+#pragma unroll
+        for (int q = 0; q < kScanChunks; ++q)
+            if (base + q * 32 + lane == a) c[q] = acnt;
 #pragma unroll
         for (int q = 0; q < kScanChunks; ++q) {
             int incl = c[q];
