@@ -1,4 +1,5 @@
-"""Thin Python binding of libttf_b200.so: argument marshalling only.
+"""Thin Python binding of libttf_b200.so: argument marshalling only (ctypes, and _marshal.so, plain C, for the entry
+points that are called per clip).
 
 Function names and argument order follow include/ttf.h.  Tensors are torch tensors (device memory and
 streams come from PyTorch); every step of the pass runs in the library's CUDA kernels.  There is no CPU
@@ -37,16 +38,13 @@ class TTFOptions(ctypes.Structure):
                 ("pos_base", ctypes.c_int)]
 
 
-def _options(anchor_mode: int, anchor_frame: int, order: int, pos_base: int):
-    """NULL when everything is at its default, else a ttf_options by reference"""
-    if not (anchor_mode or anchor_frame or order or pos_base):
-        return None
-    return ctypes.byref(TTFOptions(int(anchor_mode), int(anchor_frame), int(order), int(pos_base)))
-
 TTF_STATIC_SCRATCH_BYTES = 8 << 20
 KERNEL_KINDS = ["norm_sum", "frame_stats", "match", "compact", "fuse_count"]
 
 _lib = None
+_fast = None                     # _marshal, bound to the library's functions
+_FAST_FUNCTIONS = ["ttf_compress", "ttf_compress_ws", "ttf_compress_ex", "ttf_compress_segment", "ttf_compress_batch",
+                   "ttf_compress_batch_ex", "ttf_query", "ttf_query_ws", "ttf_query_ex", "ttf_restore", "ttf_stats"]
 
 
 class TTFError(RuntimeError):
@@ -133,6 +131,20 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _marshal():
+    """The C marshalling module, bound to the library (both loaded on the first call)."""
+    global _fast
+    if _fast is None:
+        L = lib()
+        try:
+            from . import _marshal as m
+        except ImportError as e:
+            raise FileNotFoundError("_marshal.so not found: build it with `python -m paper_2605_07355_b200.build`") from e
+        m.bind(*[ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _FAST_FUNCTIONS])
+        _fast = m
+    return _fast
+
+
 def _dtype_code(x: torch.Tensor) -> int:
     if x.dtype == torch.float32:
         return TTF_DTYPE_F32
@@ -150,13 +162,31 @@ def _check_features(x: torch.Tensor, device: str):
         raise ValueError("features must be a CUDA tensor")
     if device == "cpu" and x.is_cuda:
         raise ValueError("features must be a host tensor")
-    return tuple(int(v) for v in x.shape)
+    return x.shape
 
 
 def _stream_ptr(stream) -> int:
     if stream is None:
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
+
+
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _elsewhere(x: torch.Tensor):
+    """None when the tensor's device is the current one, else a context that makes it so."""
+    i = x.get_device()
+    return None if i < 0 or i == _current_device() else torch.cuda.device(i)
+
+
+def _stream_of(x: torch.Tensor, stream) -> int:
+    return _current_raw_stream(x.get_device()) if stream is None else _stream_ptr(stream)
+
+
+def _addr(t: Optional[torch.Tensor]) -> int:
+    return 0 if t is None else t.data_ptr()
 
 
 def _p(t: Optional[torch.Tensor]):
@@ -178,29 +208,28 @@ def ttf_compress(features: torch.Tensor, r: int, t: float, out_tokens: Optional[
     """ttf_compress / ttf_compress_ws (ttf_compress_ex when any option is given).  Returns (out_tokens [F*H*W, C], out_count int32[1],
     out_pos_thw int32 [F*H*W, 3]); only the first out_count rows are defined.  Does not synchronise."""
     F, H, W, C = _check_features(features, "cuda")
-    dev = features.device
+    there = _elsewhere(features)
+    if there is not None:
+        with there:
+            return ttf_compress(features, r, t, out_tokens, out_count, out_pos_thw, workspace, stream, anchor_mode,
+                                anchor_frame, order, pos_base)
     n = F * H * W
     if out_tokens is None:
-        out_tokens = torch.empty((n, C), dtype=features.dtype, device=dev)
+        out_tokens = features.new_empty((n, C))
     if out_count is None:
-        out_count = torch.empty(1, dtype=torch.int32, device=dev)
+        out_count = features.new_empty(1, dtype=torch.int32)
     if out_pos_thw is None:
-        out_pos_thw = torch.empty((n, 3), dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
-        sp = _stream_ptr(stream)
-        opt = _options(anchor_mode, anchor_frame, order, pos_base)
-        if opt is not None:
-            if workspace is not None:
-                raise ValueError("the entry point with options uses the library's own scratch")
-            rc = lib().ttf_compress_ex(_p(features), F, H, W, C, int(r), float(t), _dtype_code(features), opt,
-                                       _p(out_tokens), _p(out_count), _p(out_pos_thw), sp)
-        elif workspace is None:
-            rc = lib().ttf_compress(_p(features), F, H, W, C, int(r), float(t), _dtype_code(features),
-                                    _p(out_tokens), _p(out_count), _p(out_pos_thw), sp)
-        else:
-            rc = lib().ttf_compress_ws(_p(features), F, H, W, C, int(r), float(t), _dtype_code(features),
-                                       _p(out_tokens), _p(out_count), _p(out_pos_thw),
-                                       _p(workspace), workspace.numel() * workspace.element_size(), sp)
+        out_pos_thw = features.new_empty((n, 3), dtype=torch.int32)
+    fast, sp, dt = _fast or _marshal(), _stream_of(features, stream), _dtype_code(features)
+    if workspace is None:
+        rc = fast.compress(features.data_ptr(), F, H, W, C, int(r), float(t), dt, int(anchor_mode), int(anchor_frame),
+                           int(order), int(pos_base), out_tokens.data_ptr(), out_count.data_ptr(), out_pos_thw.data_ptr(), sp)
+    elif anchor_mode or anchor_frame or order or pos_base:
+        raise ValueError("the entry point with options uses the library's own scratch")
+    else:
+        rc = fast.compress_ws(features.data_ptr(), F, H, W, C, int(r), float(t), dt, out_tokens.data_ptr(),
+                              out_count.data_ptr(), out_pos_thw.data_ptr(), workspace.data_ptr(),
+                              workspace.numel() * workspace.element_size(), sp)
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_compress")
     return out_tokens, out_count, out_pos_thw
@@ -307,29 +336,30 @@ def ttf_compress_batch(features, r: int, t: float, out_tokens=None, out_count=No
     feats = list(features)
     if not feats:
         raise ValueError("empty batch")
-    F, H, W, C = _check_features(feats[0], "cuda")
-    dev, dt = feats[0].device, feats[0].dtype
+    first = feats[0]
+    shape, dev, dt = _check_features(first, "cuda"), first.get_device(), first.dtype
     for x in feats[1:]:
-        if _check_features(x, "cuda") != (F, H, W, C) or x.dtype != dt or x.device != dev:
+        if _check_features(x, "cuda") != shape or x.dtype != dt or x.get_device() != dev:
             raise ValueError("all clips of a batch must have the same shape, dtype and device")
+    there = _elsewhere(first)
+    if there is not None:
+        with there:
+            return ttf_compress_batch(feats, r, t, out_tokens, out_count, out_pos_thw, stream, anchor_mode, anchor_frame,
+                                      order, pos_base)
+    F, H, W, C = shape
     n, B = F * H * W, len(feats)
     if out_tokens is None:
-        out_tokens = [torch.empty((n, C), dtype=dt, device=dev) for _ in range(B)]
+        out_tokens = [first.new_empty((n, C)) for _ in range(B)]
     if out_count is None:
-        out_count = [torch.empty(1, dtype=torch.int32, device=dev) for _ in range(B)]
+        out_count = [first.new_empty(1, dtype=torch.int32) for _ in range(B)]
     if out_pos_thw is None:
-        out_pos_thw = [torch.empty((n, 3), dtype=torch.int32, device=dev) for _ in range(B)]
+        out_pos_thw = [first.new_empty((n, 3), dtype=torch.int32) for _ in range(B)]
     if not (len(out_tokens) == len(out_count) == len(out_pos_thw) == B):
         raise ValueError("one output of each kind per clip")
-    arr = lambda ts: (ctypes.c_void_p * B)(*[t_.data_ptr() for t_ in ts])
-    opt = _options(anchor_mode, anchor_frame, order, pos_base)
-    with torch.cuda.device(dev):
-        if opt is None:
-            rc = lib().ttf_compress_batch(arr(feats), B, F, H, W, C, int(r), float(t), _dtype_code(feats[0]),
-                                          arr(out_tokens), arr(out_count), arr(out_pos_thw), _stream_ptr(stream))
-        else:
-            rc = lib().ttf_compress_batch_ex(arr(feats), B, F, H, W, C, int(r), float(t), _dtype_code(feats[0]), opt,
-                                             arr(out_tokens), arr(out_count), arr(out_pos_thw), _stream_ptr(stream))
+    rc = (_fast or _marshal()).compress_batch(
+        [x.data_ptr() for x in feats], F, H, W, C, int(r), float(t), _dtype_code(first), int(anchor_mode),
+        int(anchor_frame), int(order), int(pos_base), [x.data_ptr() for x in out_tokens],
+        [x.data_ptr() for x in out_count], [x.data_ptr() for x in out_pos_thw], _stream_of(first, stream))
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_compress_batch")
     return out_tokens, out_count, out_pos_thw
@@ -340,31 +370,35 @@ def ttf_query(features: torch.Tensor, r: int, t: float, workspace: Optional[torc
               anchor_frame: int = 0) -> dict:
     """ttf_query / ttf_query_ws (ttf_query_ex when an anchor rule other than auto is given).  Returns the requested device tensors.  Does not synchronise."""
     F, H, W, C = _check_features(features, "cuda")
-    dev = features.device
+    there = _elsewhere(features)
+    if there is not None:
+        with there:
+            return ttf_query(features, r, t, workspace, stream, want, anchor_mode, anchor_frame)
     n = F * H * W
-    out = {
-        "anchor": torch.empty(1, dtype=torch.int32, device=dev) if "anchor" in want else None,
-        "keep": torch.empty(n, dtype=torch.uint8, device=dev) if "keep" in want else None,
-        "dst": torch.empty(n, dtype=torch.int32, device=dev) if "dst" in want else None,
-        "best_sim": torch.empty(n, dtype=torch.float32, device=dev) if "best_sim" in want else None,
-        "fuse_cnt": torch.empty(H * W, dtype=torch.int32, device=dev) if "fuse_cnt" in want else None,
-    }
-    args = [_p(features), F, H, W, C, int(r), float(t), _dtype_code(features), _p(out["anchor"]), _p(out["keep"]),
-            _p(out["dst"]), _p(out["best_sim"]), _p(out["fuse_cnt"])]
-    with torch.cuda.device(dev):
-        sp = _stream_ptr(stream)
-        opt = _options(anchor_mode, anchor_frame, 0, 0)
-        if opt is not None:
-            if workspace is not None:
-                raise ValueError("the entry point with options uses the library's own scratch")
-            rc = lib().ttf_query_ex(*args[:8], opt, *args[8:], sp)
-        elif workspace is None:
-            rc = lib().ttf_query(*args, sp)
-        else:
-            rc = lib().ttf_query_ws(*args, _p(workspace), workspace.numel() * workspace.element_size(), sp)
+    out = {}
+    if "anchor" in want:
+        out["anchor"] = features.new_empty(1, dtype=torch.int32)
+    if "keep" in want:
+        out["keep"] = features.new_empty(n, dtype=torch.uint8)
+    if "dst" in want:
+        out["dst"] = features.new_empty(n, dtype=torch.int32)
+    if "best_sim" in want:
+        out["best_sim"] = features.new_empty(n, dtype=torch.float32)
+    if "fuse_cnt" in want:
+        out["fuse_cnt"] = features.new_empty(H * W, dtype=torch.int32)
+    outs = [_addr(out.get(k)) for k in ("anchor", "keep", "dst", "best_sim", "fuse_cnt")]
+    fast, sp, dt = _fast or _marshal(), _stream_of(features, stream), _dtype_code(features)
+    if workspace is None:
+        rc = fast.query(features.data_ptr(), F, H, W, C, int(r), float(t), dt, int(anchor_mode), int(anchor_frame), 0, 0,
+                        *outs, sp)
+    elif anchor_mode or anchor_frame:
+        raise ValueError("the entry point with options uses the library's own scratch")
+    else:
+        rc = fast.query_ws(features.data_ptr(), F, H, W, C, int(r), float(t), dt, *outs, workspace.data_ptr(),
+                           workspace.numel() * workspace.element_size(), sp)
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_query")
-    return {k: v for k, v in out.items() if v is not None}
+    return out
 
 
 def ttf_query_static(features: torch.Tensor, r: int, t: float, out: dict, stream=None) -> dict:
@@ -388,14 +422,17 @@ def ttf_compress_segment(features: torch.Tensor, r: int, t: float, frame_base: i
     """ttf_compress_segment: frame 0 is the rolling anchor, frames 1.. are compressed against it; returns
     (out_tokens [(F-1)*H*W, C], out_count int32[1] = P, out_pos_thw [(F-1)*H*W, 3])."""
     F, H, W, C = _check_features(features, "cuda")
-    dev = features.device
+    there = _elsewhere(features)
+    if there is not None:
+        with there:
+            return ttf_compress_segment(features, r, t, frame_base, stream)
     n = max(1, (F - 1) * H * W)
-    out_tokens = torch.empty((n, C), dtype=features.dtype, device=dev)
-    out_count = torch.empty(1, dtype=torch.int32, device=dev)
-    out_pos = torch.empty((n, 3), dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
-        rc = lib().ttf_compress_segment(_p(features), F, H, W, C, int(r), float(t), _dtype_code(features),
-                                        int(frame_base), _p(out_tokens), _p(out_count), _p(out_pos), _stream_ptr(stream))
+    out_tokens = features.new_empty((n, C))
+    out_count = features.new_empty(1, dtype=torch.int32)
+    out_pos = features.new_empty((n, 3), dtype=torch.int32)
+    rc = (_fast or _marshal()).compress_segment(features.data_ptr(), F, H, W, C, int(r), float(t), _dtype_code(features),
+                                                int(frame_base), out_tokens.data_ptr(), out_count.data_ptr(),
+                                                out_pos.data_ptr(), _stream_of(features, stream))
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_compress_segment")
     return out_tokens, out_count, out_pos
@@ -406,13 +443,17 @@ def ttf_restore(compressed: torch.Tensor, F: int, H: int, W: int, anchor: torch.
     """ttf_restore: returns (out_full [F*H*W, ...row shape], row_index int32 [F*H*W])."""
     if not compressed.is_contiguous():
         raise ValueError("compressed must be contiguous")
-    dev = compressed.device
-    row_bytes = compressed[0].numel() * compressed.element_size()
-    out = torch.empty((F * H * W,) + tuple(compressed.shape[1:]), dtype=compressed.dtype, device=dev)
-    idx = torch.empty(F * H * W, dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
-        rc = lib().ttf_restore(_p(compressed), row_bytes, F, H, W, _p(anchor), _p(keep), _p(dst), _p(out), _p(idx),
-                               _stream_ptr(stream))
+    there = _elsewhere(compressed)
+    if there is not None:
+        with there:
+            return ttf_restore(compressed, F, H, W, anchor, keep, dst, stream)
+    if compressed.shape[0] == 0:
+        raise IndexError("compressed has no rows")
+    row_bytes = compressed.numel() // compressed.shape[0] * compressed.element_size()
+    out = compressed.new_empty((F * H * W,) + tuple(compressed.shape[1:]))
+    idx = compressed.new_empty(F * H * W, dtype=torch.int32)
+    rc = (_fast or _marshal()).restore(compressed.data_ptr(), row_bytes, F, H, W, anchor.data_ptr(), keep.data_ptr(),
+                                       dst.data_ptr(), out.data_ptr(), idx.data_ptr(), _stream_of(compressed, stream))
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_restore")
     return out, idx
@@ -432,10 +473,13 @@ def ttf_sim_histogram(best_sim: torch.Tensor, anchor: torch.Tensor, F: int, H: i
 def ttf_stats(best_sim: torch.Tensor, keep: torch.Tensor, anchor: torch.Tensor, F: int, H: int, W: int, t: float,
               band: float = 1e-4, stream=None) -> torch.Tensor:
     """ttf_stats: int64 [3] on the device = (P preserved, fused, in-band source tokens).  Does not synchronise."""
-    dev = best_sim.device
-    out = torch.empty(3, dtype=torch.int64, device=dev)
-    with torch.cuda.device(dev):
-        rc = lib().ttf_stats(_p(best_sim), _p(keep), _p(anchor), F, H, W, float(t), float(band), _p(out), _stream_ptr(stream))
+    there = _elsewhere(best_sim)
+    if there is not None:
+        with there:
+            return ttf_stats(best_sim, keep, anchor, F, H, W, t, band, stream)
+    out = best_sim.new_empty(3, dtype=torch.int64)
+    rc = (_fast or _marshal()).stats(best_sim.data_ptr(), keep.data_ptr(), anchor.data_ptr(), F, H, W, float(t),
+                                     float(band), out.data_ptr(), _stream_of(best_sim, stream))
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_stats")
     return out
