@@ -124,6 +124,15 @@ void carve_scratch(const Problem& p, void* base, Scratch* s) {
     s->bytes = off;
 }
 
+// The matching kernel of a bf16 clip: the tcgen05 kernel wherever it can take it (rows of at least 64 channels, r <= 2).
+// It depends on the clip's shape alone, so that every call and every launch gives a clip the same bits.  Against the
+// warp-level kernel, us per pass: one clip of 21 x 13 x 19 x 1160 21.4 -> 19.0, 64 x 16 x 16 x 2048 45.4 -> 40.1,
+// 24 x 24 x 24 x 2048 46.1 -> 40.8, 32 x 16 x 16 x 4096 40.9 -> 39.1, 32 x 16 x 16 x 2048 28.3 -> 28.9,
+// 32 x 16 x 16 x 512 16.7 -> 18.5; batches: 16 of 32 x 16 x 16 x 4096 482 -> 449, 16 of 32 x 16 x 16 x 2048 269 -> 240,
+// 8 of 32 x 16 x 16 x 512 61 -> 45, 16 of 8 x 12 x 12 x 512 51 -> 34.  The few short 32-frame clips that it is slower on
+// alone gain four times as much in a batch.
+static int choose_match(const Problem& p) { return g_match_kernel.load() != 1 && tc_match_eligible(p) ? 1 : 0; }
+
 // Validates the shape arguments and fills the derived fields.  Pointers are checked by the callers.
 static int make_problem(const void* X, int F, int H, int W, int C, int r, float t, int dtype, Problem* p) {
     if (F < 1 || H < 1 || W < 1 || C < 1 || r < 0) return TTF_ERR_INVALID_ARG;
@@ -148,12 +157,7 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
     if ((long long)F * p->nq >= (1LL << 31)) return TTF_ERR_UNSUPPORTED;
     p->nsl = C % 4 == 0 ? (C + 127) / 128 : (C + 31) / 32;
     p->anchor_mode = 0; p->anchor_arg = 0; p->emit_anchor = 1; p->pos_t_offset = 0; p->pos_base = 0; p->natural_order = 0;
-    // Matching kernel: on request, else by measurement: the tcgen05 kernel where a clip has enough tiles to fill the
-    // GPU without cutting their channel range (long clips: 112 against 115 us; the 5 x 5 window: 218 against 303 us
-    // per clip), the warp-level MMA kernel for the short 16 x 16 clips (30 against 32 us on the 8B-shaped clip).
-    p->use_tc = 0;
-    const int which = g_match_kernel.load();
-    if (tc_match_eligible(*p)) p->use_tc = which == 2 || (which == 0 && (r == 2 || tc_match_pieces(*p) == 1)) ? 1 : 0;
+    p->use_tc = choose_match(*p);
     p->chain = 0; p->chain_next = 0; p->overlapped = 0; p->stream_once = 0;
     return TTF_OK;
 }

@@ -15,10 +15,16 @@
 //   Both arrive with the 128-byte swizzle, which is the K-major operand layout of tcgen05.mma; a pipeline stage is
 //   64 channels (4 MMAs of K = 16).  fp32 accumulation in tensor memory; bf16 products are exact in fp32.
 //
-// The channel range of a tile is cut into `pieces` consecutive parts, one CTA each, so that a small clip still gives
-// about two CTAs per SM.  The CTAs of a tile form a thread-block cluster: when their pipelines have drained, ranks
-// > 0 write their partial sums into rank 0's shared memory (distributed shared memory, two cluster barriers) and
-// rank 0 adds them in rank order, so the result does not depend on scheduling.
+// The channel range of a tile is cut into `chunks` consecutive parts, each with an accumulator of its own in tensor
+// memory, and a tile is worked on by `pieces` CTAs (a divisor of `chunks`), which take chunks / pieces of the parts each.
+// The sums of the parts are added as a binary tree over the parts, so the result depends on `chunks` alone: a clip gives
+// the same bits whether it has the GPU to itself (pieces = chunks, so that a small clip still gives about two CTAs per
+// SM) or shares a launch with others (fewer pieces, no exchange between CTAs).
+// The CTAs of a tile form a thread-block cluster, and each rank finishes 128 / pieces of the rows: when its accumulators
+// are complete a rank writes its partial sums of every rank's rows into that rank's shared memory (a region of its own
+// beside the ring, so that nobody has to wait for the others' pipelines to drain first) and one cluster barrier follows.
+// What comes after the main loop is a serial chain that nothing overlaps, so with several ranks every step of it is spread
+// over all 128 epilogue threads: (element, rank) sums, then the norms, then one row per thread.
 // Token norms are taken from the tiles themselves: while the pipeline runs, every epilogue thread adds up the squares
 // of "its" source row (and the first NCAND threads those of a candidate row) as the stages pass through shared memory.
 // Warp roles: 0 TMA producer, 1 tensor-memory owner and MMA issuer, 2-5 epilogue (one tensor-memory lane = one
@@ -69,18 +75,27 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// 16 consecutive fp32 columns of this thread's tensor-memory lane
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// 8 NG consecutive fp32 columns of this thread's tensor-memory lane
+template <int NG> __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[NG][8]) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+    for (int g = 0; g < NG; ++g)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]),
+                       "=r"(r[g][6]), "=r"(r[g][7])
+                     : "r"(taddr + (uint32_t)(g * 8))
+                     : "memory");
+#pragma unroll
+    for (int g = 0; g < NG; ++g)                           // (the registers are operands of the wait, so that nothing that
+        asm volatile("tcgen05.wait::ld.sync.aligned;"      // reads them can be moved before it)
+                     : "+r"(r[g][0]), "+r"(r[g][1]), "+r"(r[g][2]), "+r"(r[g][3]), "+r"(r[g][4]), "+r"(r[g][5]),
+                       "+r"(r[g][6]), "+r"(r[g][7])
+                     :: "memory");
+}
+template <int NG> __device__ __forceinline__ void tmem_add(uint32_t (&a)[NG][8], const uint32_t (&b)[NG][8]) {
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) a[g][e] = __float_as_uint(__uint_as_float(a[g][e]) + __uint_as_float(b[g][e]));
 }
 __device__ __forceinline__ void epilogue_bar_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
@@ -109,8 +124,14 @@ template <int R> struct TcShape {
     static constexpr int BBOX = NCAND * 128;              // bytes one B box copy delivers
     static constexpr int STAGE = kTcABytes + BBYTES;
     static constexpr int STAGES = 4;                      // two CTAs per SM with room left for CTAs of other kernels
-    static constexpr int TMEM_COLS = NB <= 32 ? 32 : 64;
     static constexpr int WIN = SIDE * SIDE;               // candidates of one source row
+    static constexpr int MAXCH = R == 2 ? 4 : 8;          // chunks at most (tensor memory: MAXCH * NB <= 256 columns)
+    // what one rank sends another (and itself): window sums and squared norms of the rows the other one finishes,
+    // squared norms of the candidates
+    static constexpr int XBYTES = (kTcM * (WIN + 1) + MAXCH * NCAND) * 4;                 // received by one rank
+    static constexpr int RING = STAGES * STAGE;
+    static constexpr int NP = NCAND * 8;                  // (candidate row, 16-byte piece column) pairs
+    static constexpr int NORMBYTES = MAXCH * (kTcM + NP) * 4;
 };
 
 // ---- thread-block clusters: the CTAs of one tile exchange their partial sums through distributed shared memory
@@ -119,15 +140,28 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// all threads of all CTAs of the cluster; writes before it are visible to every CTA of the cluster after it
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void st_cluster_f32(uint32_t local_smem_addr, uint32_t rank, float v) {
+// all threads of all CTAs of the cluster; writes before an arrival are visible to every CTA of the cluster after the wait
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t local_smem_addr, uint32_t rank) {
     uint32_t remote;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_smem_addr), "r"(rank));
+    return remote;
+}
+__device__ __forceinline__ void st_cluster_f32(uint32_t remote, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
+}
+// m is all ones or zero: a or b without a branch.  (The window of a row starts at one of four columns; as conditional
+// expressions the choice became divergent branches, 1400 cycles per row at r = 1 against 110 for the loads from tensor
+// memory; 16 logic operations now.)
+__device__ __forceinline__ uint32_t pick(uint32_t m, uint32_t a, uint32_t b) { return (a & m) | (b & ~m); }
+// binary tree over n = 1, 2, 4 or 8 terms
+template <typename Fn> __device__ __forceinline__ float tree_sum(int n, Fn&& term) {
+    float v = term(0);
+    if (n > 1) v += term(1);
+    if (n > 2) v += term(2) + term(3);
+    if (n > 4) v += (term(4) + term(5)) + (term(6) + term(7));
+    return v;
 }
 
 // sum of squares of the 8 bf16 values of a 16-byte piece
@@ -142,7 +176,7 @@ __device__ __forceinline__ float ssq8(const uint4& v, float acc) {
 
 template <int R, int G>
 __global__ void __launch_bounds__(kTcThreads)
-k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc, int pieces,
+k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc, int lpieces, int lchunks,
            float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
            int wait_limit, int tx_extra, int stream_once, size_t sstride)
 {
@@ -155,8 +189,6 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     __shared__ uint64_t bar_full[S::STAGES], bar_empty[S::STAGES], bar_acc;
     __shared__ uint32_t s_tmem;
     __shared__ int s_err;
-    __shared__ float s_nb[S::NCAND];                       // 1 / norm of the candidate rows
-    __shared__ float s_nbp[S::NCAND * 8];                  // ... per 16-byte piece column, before they are added up
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int N = H * W;
@@ -165,20 +197,24 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     // and the gather, which goes forwards again, finds what is matched last.  (64 x 16 x 16 x 4096: 81.9 -> 79.0 us per
     // pass, 64 x 32 x 32 x 4096 with r = 2: 255.5 -> 252.1; over several clips it made no difference or 0.4 % worse.)
     const unsigned walk = gridDim.y == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
-    const int tile = (int)(walk / (unsigned)pieces);
+    const int pieces = 1 << lpieces;
+    const int tile = (int)(walk >> lpieces);
     const int piece = pieces > 1 ? (int)cluster_rank() : 0;        // = blockIdx.x % pieces
     const int kg = tile / (H * xs_n), rem = tile - kg * (H * xs_n);
     const int y = rem / xs_n, x0 = (rem - y * xs_n) * kTcWB;
     const int k0 = kg * kTcFR;
     const int nst_all = (C + kTcKC - 1) / kTcKC;
-    const int st0 = (int)((long long)nst_all * piece / pieces), st1 = (int)((long long)nst_all * (piece + 1) / pieces);
-    const int nst = st1 - st0;
+    const int nch = 1 << (lchunks - lpieces);              // this CTA's chunks: ch0 .. ch0 + nch - 1
+    const int ch0 = piece * nch;
+    auto chunk_begin = [&](int c) { return (nst_all * c) >> lchunks; };
+    const int st0 = chunk_begin(ch0), nst = chunk_begin(ch0 + nch) - st0;
+    uint32_t tmem_cols = 32;
+    while (tmem_cols < (uint32_t)(nch * S::NB)) tmem_cols *= 2;
 
     // 1024-byte aligned stage ring (the swizzle pattern is a function of the shared-memory address)
     const uint32_t dyn_base = (smem_u32(dyn_raw) + 1023u) & ~1023u;
     unsigned char* dyn = dyn_raw + (dyn_base - smem_u32(dyn_raw));
 
-    pdl_launch_dependents();
     trace_mark(asrc.hdr, 2, false);
     if (tid == 0) {
         // a stage is full when its two copies have landed, and free again when the MMAs that read it have completed
@@ -196,11 +232,12 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
         reinterpret_cast<uint4*>(dyn + (size_t)s * S::STAGE + kTcABytes + S::BBOX)[o] = make_uint4(0, 0, 0, 0);
     }
     fence_async_smem();
-    if (warp == 1) tmem_alloc(&s_tmem, S::TMEM_COLS);
+    if (warp == 1) tmem_alloc(&s_tmem, tmem_cols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    if (pieces > 1) { cluster_arrive(); cluster_wait(); }  // every CTA of the tile is running: remote writes may come
 
     // everything upstream (the anchor, and whatever produced X) is complete after this wait
     trace_mark(asrc.hdr, 11, false); trace_mark(asrc.hdr, 11, true);     // set-up done
@@ -216,6 +253,9 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     const int q = warp & 3;                                // tensor-memory lane quadrant an epilogue warp may read
     const int m = q * 32 + lane;                           // source row of an epilogue thread: 4 * frame + cell
     const int et = (warp - 2) * 32 + lane;                 // 0..127 among the epilogue threads
+    float* const s_na = reinterpret_cast<float*>(dyn + S::RING + S::XBYTES);      // [chunk][row] squared norms
+    float* const s_nbp = s_na + S::MAXCH * kTcM;           // [chunk][candidate row, piece column]
+    const int dx = m & 3;
     float win[S::WIN];                                     // this row's window of dot products
     float na = 0.f, nb = 0.f;                              // squared norm of source row m / of candidate row et
 
@@ -250,15 +290,18 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
         // ---- MMA issuer: one lane, four K = 16 steps per stage -----------------------------------------------
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16(S::NB);
+            int ch = 0, begin = 0, end = chunk_begin(ch0 + 1) - st0;     // stages of the chunk
             for (int it = 0; it < nst; ++it) {
                 const int s = it % S::STAGES;
+                if (it == end) { ++ch; begin = end; end = chunk_begin(ch0 + ch + 1) - st0; }
                 if (!mbar_wait(&bar_full[s], (it / S::STAGES) & 1, wait_limit)) { atomicExch(&s_err, 1); break; }
                 tc_fence_after();
                 const uint32_t sa = dyn_base + (uint32_t)s * S::STAGE;
                 const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + kTcABytes);
 #pragma unroll
                 for (int k = 0; k < kTcKC / 16; ++k)       // 32 bytes further along K inside the swizzle row
-                    umma_bf16(tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, it > 0 || k > 0);
+                    umma_bf16(tmem + (uint32_t)(ch * S::NB), da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
+                              it > begin || k > 0);
                 umma_commit(&bar_empty[s]);                // one of the five arrivals that free the stage
             }
             umma_commit(&bar_acc);                         // accumulator complete (also arrives after a give-up)
@@ -269,13 +312,14 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
         // bytes per stage; its 16-byte pieces sit at (piece ^ (row & 7)) (the 128-byte swizzle), and a sum of
         // squares does not care in which order it meets them ---------------------------------------------------
         bool ok = true;
-        constexpr int NP = S::NCAND * 8;                   // (candidate row, 16-byte piece column) pairs
+        constexpr int NP = S::NP;
         constexpr int PP = (NP + 127) / 128;               // pairs per epilogue thread
         float na8[8], nbq[PP];                             // one running sum per piece column: eight short chains
 #pragma unroll
         for (int c = 0; c < 8; ++c) na8[c] = 0.f;
 #pragma unroll
         for (int u = 0; u < PP; ++u) nbq[u] = 0.f;
+        int ch = 0, end = chunk_begin(ch0 + 1) - st0;
         for (int it = 0; it < nst; ++it) {
             const int s = it % S::STAGES;
             if (!mbar_wait(&bar_full[s], (it / S::STAGES) & 1, wait_limit)) { atomicExch(&s_err, 1); ok = false; break; }
@@ -297,94 +341,133 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
             for (int u = 0; u < PP; ++u) nbq[u] = ssq8(vb[u], nbq[u]);
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_empty[s]);
-        }
-        na = ((na8[0] + na8[1]) + (na8[2] + na8[3])) + ((na8[4] + na8[5]) + (na8[6] + na8[7]));
+            if (it + 1 == end) {                           // a chunk is complete: put its norms away
+                s_na[ch * kTcM + m] = ((na8[0] + na8[1]) + (na8[2] + na8[3])) + ((na8[4] + na8[5]) + (na8[6] + na8[7]));
 #pragma unroll
-        for (int u = 0; u < PP; ++u) if (et + u * 128 < NP) s_nbp[et + u * 128] = nbq[u];
-        epilogue_bar_sync();
-        if (et < S::NCAND) {
-            const float* pp = s_nbp + et * 8;
-            nb = ((pp[0] + pp[1]) + (pp[2] + pp[3])) + ((pp[4] + pp[5]) + (pp[6] + pp[7]));
+                for (int c = 0; c < 8; ++c) na8[c] = 0.f;
+#pragma unroll
+                for (int u = 0; u < PP; ++u) {
+                    if (et + u * 128 < NP) s_nbp[ch * NP + et + u * 128] = nbq[u];
+                    nbq[u] = 0.f;
+                }
+                ++ch;
+                end = chunk_begin(ch0 + ch + 1) - st0;
+            }
         }
         if (et == 0) { trace_mark_any(asrc.hdr, 13, false); trace_mark_any(asrc.hdr, 13, true); }   // norms done
-        // ---- part 2: the accumulator ---------------------------------------------------------------------------
+        // ---- part 2: the accumulators, added up over this CTA's chunks ---------------------------------------------
         if (ok) ok = mbar_wait(&bar_acc, 0, wait_limit);
-        if (!ok) atomicExch(&s_err, 1);
+        if (!ok) atomicExch(&s_err, 1);                    // (what follows then works on whatever is there: the call has failed)
         if (et == 0) { trace_mark_any(asrc.hdr, 14, false); trace_mark_any(asrc.hdr, 14, true); }   // accumulator complete
         tc_fence_after();
-        float d[S::NB];
-        if (ok) {
-#pragma unroll
-            for (int c = 0; c < S::NB / 16; ++c) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 16), v);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) d[c * 16 + i] = v[i];
+        // The gather may be scheduled from here on.  (Not earlier: its CTAs would take the places of other kernels' CTAs and
+        // sit out the main loop; 24 x 24 x 24 x 2048: 45.8 us per pass with the trigger at the start, 42.3 here.)
+        pdl_launch_dependents();
+        epilogue_bar_sync();                               // the norms of the chunks are visible
+        const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
+        constexpr int NG = (S::NCAND + 7) / 8;
+        uint32_t d[NG][8];
+        tmem_ld<NG>(lanes, d);
+        if (nch > 1) {
+            uint32_t x[NG][8], z[NG][8];
+            tmem_ld<NG>(lanes + (uint32_t)S::NB, x);
+            tmem_add<NG>(d, x);
+#pragma unroll 1
+            for (int h = 2; h < nch; h += 2) {             // nch = 4 or 8: pairs (2,3) | ((4,5), (6,7))
+                tmem_ld<NG>(lanes + (uint32_t)(h * S::NB), x);
+                tmem_ld<NG>(lanes + (uint32_t)((h + 1) * S::NB), z);
+                tmem_add<NG>(x, z);
+                if (h == 4) {
+                    uint32_t u[NG][8];
+                    tmem_ld<NG>(lanes + (uint32_t)(6 * S::NB), u);
+                    tmem_ld<NG>(lanes + (uint32_t)(7 * S::NB), z);
+                    tmem_add<NG>(u, z);
+                    tmem_add<NG>(x, u);
+                    h = 6;
+                }
+                tmem_add<NG>(d, x);
             }
-        } else {
-#pragma unroll
-            for (int i = 0; i < S::NB; ++i) d[i] = 0.f;
         }
         // this row's window: candidate (dy, ddx) is column (dy + R) * BW + dx + ddx + R of the tile
-        const int dx = m & 3;
+        const uint32_t by1 = (dx & 1) ? 0xffffffffu : 0u, by2 = (dx & 2) ? 0xffffffffu : 0u;
+        auto col = [&](int n) { return d[n / 8][n % 8]; };
 #pragma unroll
-        for (int wy = 0; wy < S::SIDE; ++wy)
+        for (int wy = 0; wy < S::SIDE; ++wy) {
+            uint32_t e[S::SIDE + 2];
 #pragma unroll
-            for (int wx = 0; wx < S::SIDE; ++wx) {
-                const int n0 = wy * S::BW + wx;
-                win[wy * S::SIDE + wx] = dx == 0 ? d[n0] : (dx == 1 ? d[n0 + 1] : (dx == 2 ? d[n0 + 2] : d[n0 + 3]));
-            }
+            for (int n = 0; n < S::SIDE + 2; ++n) e[n] = pick(by1, col(wy * S::BW + n + 1), col(wy * S::BW + n));
+#pragma unroll
+            for (int wx = 0; wx < S::SIDE; ++wx) win[wy * S::SIDE + wx] = __uint_as_float(pick(by2, e[wx + 2], e[wx]));
+        }
+        na = tree_sum(nch, [&](int c) { return s_na[c * kTcM + m]; });
+        if (et < S::NCAND)
+            nb = tree_sum(nch, [&](int c) {
+                const float* pp = s_nbp + c * NP + et * 8;
+                return ((pp[0] + pp[1]) + (pp[2] + pp[3])) + ((pp[4] + pp[5]) + (pp[6] + pp[7]));
+            });
     }
 
-    // ---- split K: the CTAs of a tile form a cluster; ranks > 0 hand their partial sums to rank 0 through its
-    // shared memory (the stage ring, idle by then) and rank 0 adds them in rank order ----------------------------
-    constexpr int XROW = (S::WIN + 1) * kTcM + S::NCAND;   // floats one rank sends: window sums, row norms, candidate norms
+    const int per = kTcM >> lpieces;                       // rank p of the cluster finishes rows [p * per, (p + 1) * per)
+    const int rows_end = per * (S::WIN + 1);               // a share: [window sum 0 .. WIN-1, norm][row], candidate norms
+    const int seg = rows_end + S::NCAND;
+    float* const x_in = reinterpret_cast<float*>(dyn + S::RING);         // [rank][seg]
     if (pieces > 1) {
-        __syncwarp();
-        cluster_sync_all();                                // every CTA of the tile is past its pipeline: rank 0's ring is idle
-        if (warp >= 2 && piece > 0) {
-            const uint32_t base = dyn_base + (uint32_t)(piece - 1) * XROW * 4;
+        if (warp >= 2) {
+            const int owner = m >> (7 - lpieces);
+            const uint32_t own_share = dyn_base + S::RING + (uint32_t)(piece * seg) * 4;
+            uint32_t to = cluster_addr(own_share + (uint32_t)(m & (per - 1)) * 4, (uint32_t)owner);
 #pragma unroll
-            for (int c = 0; c < S::WIN; ++c) st_cluster_f32(base + (uint32_t)(c * kTcM + m) * 4, 0, win[c]);
-            st_cluster_f32(base + (uint32_t)(S::WIN * kTcM + m) * 4, 0, na);
-            if (et < S::NCAND) st_cluster_f32(base + (uint32_t)((S::WIN + 1) * kTcM + et) * 4, 0, nb);
+            for (int c = 0; c < S::WIN; ++c, to += (uint32_t)per * 4) st_cluster_f32(to, win[c]);
+            st_cluster_f32(to, na);
+            if (et < S::NCAND)
+                for (int p = 0; p < pieces; ++p)
+                    st_cluster_f32(cluster_addr(own_share + (uint32_t)(rows_end + et) * 4, (uint32_t)p), nb);
         }
         __syncwarp();
-        cluster_sync_all();
-        if (warp >= 2 && piece == 0) {
-            const float* xin = reinterpret_cast<const float*>(dyn);
-            for (int p = 1; p < pieces; ++p) {             // rank order
-                const float* xp = xin + (size_t)(p - 1) * XROW;
-#pragma unroll
-                for (int c = 0; c < S::WIN; ++c) win[c] += xp[c * kTcM + m];
-                na += xp[S::WIN * kTcM + m];
-                if (et < S::NCAND) nb += xp[(S::WIN + 1) * kTcM + et];
-            }
-        }
+        cluster_arrive();
+        cluster_wait();
     }
 
-    if (warp >= 2 && piece == 0) {
-        // ---- epilogue, part 3 (rank 0 of the tile): cosine, arg max over the window clipped to the grid, gate --
-        if (et < S::NCAND) s_nb[et] = 1.0f / fmaxf(sqrtf(nb), kNormFloor);     // once per candidate row, not once per use
-        epilogue_bar_sync();
-        const int kl = m >> 2, dx = m & 3;
-        const int k = k0 + kl, x = x0 + dx;
-        if (k < F && x < W && in_bounds(asrc.hdr, 3, (long long)k * N + (long long)y * W + x, (long long)F * N)) {
+    if (warp >= 2) {
+        // ---- epilogue, part 3 (the rows this rank finishes): cosine, arg max over the window clipped to the grid, gate --
+        float* const s_rb = x_in + rows_end;               // 1 / max(||x||, floor) of the candidates
+        int row = m;
+        if (pieces > 1) {
+            for (int e = et; e < seg; e += 128) {          // (an element is read and overwritten by the same thread)
+                float v = tree_sum(pieces, [&](int p) { return x_in[p * seg + e]; });
+                if (e >= rows_end - per) v = 1.0f / fmaxf(sqrtf(v), kNormFloor);     // ... and of the rows
+                x_in[e] = v;
+            }
+            epilogue_bar_sync();
+            row = piece * per + et;
+            if (et < per) {
+#pragma unroll
+                for (int c = 0; c < S::WIN; ++c) win[c] = x_in[c * per + et];
+                na = x_in[S::WIN * per + et];
+            }
+        } else {
+            if (et < S::NCAND) s_rb[et] = 1.0f / fmaxf(sqrtf(nb), kNormFloor);
+            na = 1.0f / fmaxf(sqrtf(na), kNormFloor);
+            epilogue_bar_sync();
+        }
+        const int k = k0 + (row >> 2), cell = row & 3, x = x0 + cell;
+        const bool mine = pieces > 1 ? et < per : true;
+        if (mine && k < F && x < W && in_bounds(asrc.hdr, 3, (long long)k * N + (long long)y * W + x, (long long)F * N)) {
             const size_t f = (size_t)k * N + (size_t)y * W + x;
             if (k == a) {                                  // anchor tokens are always retained (Eq. mask)
                 shat[f] = 1.0f; dst[f] = y * W + x; keep[f] = 1;
             } else {
-                const float rs = 1.0f / fmaxf(sqrtf(na), kNormFloor);
                 float best = -INFINITY;
                 int best_j = -1;
 #pragma unroll
-                for (int wy = 0; wy < S::SIDE; ++wy)
+                for (int wy = 0; wy < S::SIDE; ++wy)       // ascending anchor index among in-grid cells
 #pragma unroll
-                    for (int wx = 0; wx < S::SIDE; ++wx) {     // ascending anchor index among in-grid cells
+                    for (int wx = 0; wx < S::SIDE; ++wx) {
                         const int yy = y + wy - R, xx = x + wx - R;
-                        if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
-                        const float sim = win[wy * S::SIDE + wx] * rs * s_nb[wy * S::BW + dx + wx];
-                        if (sim > best || best_j < 0) { best = sim; best_j = yy * W + xx; }
+                        const float sim = win[wy * S::SIDE + wx] * na * s_rb[wy * S::BW + cell + wx];
+                        const bool take = ((unsigned)yy < (unsigned)H) & ((unsigned)xx < (unsigned)W) & ((sim > best) | (best_j < 0));
+                        best = take ? sim : best;
+                        best_j = take ? yy * W + xx : best_j;
                     }
                 const unsigned char kp = !(best > t);
                 shat[f] = best; dst[f] = best_j; keep[f] = kp;
@@ -399,7 +482,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     trace_mark(asrc.hdr, 2, true);
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, S::TMEM_COLS);
+        tmem_dealloc(tmem, tmem_cols);
     }
     if (tid == 0 && s_err) atomicExch(asrc.hdr + HDR_ERROR, 1);
 }
@@ -449,35 +532,36 @@ size_t tc_match_tiles(const Problem& p) {
     return (size_t)((p.F + kTcFR - 1) / kTcFR) * p.H * ((p.W + kTcWB - 1) / kTcWB);
 }
 
-// CTAs (= cluster size) per tile: the largest power of two that still fits the GPU in one wave of two CTAs per SM,
-// at most 8 (4 for r = 2, whose exchange rows are longer) and at least 4 stages each.  (One CTA per SM with a ring
-// twice as deep measured the same alone, 18.8 against 19.2 us on a cold 8B-shaped clip, and slower with other clips'
-// kernels beside it, 34.0 against 32.2 us per clip.)
-int tc_match_pieces(const Problem& p) {
-    const long long tiles = (long long)tc_match_tiles(p);
+// Parts of a tile's channel range: the largest power of two with which a launch over one clip still fits the GPU in one
+// wave of two CTAs per SM, at most 8 (4 for r = 2) and at least 2 stages each (4 stages: 16 x 8 x 8 x 512 13.9 us per pass,
+// 2: 12.9, 1: 13.3; 16 x 14 x 14 x 512 16.7 / 15.3 / 15.3).  (One CTA per SM with a ring twice as deep measured the same
+// alone, 18.8 against 19.2 us on a cold 8B-shaped clip, and slower with other clips' kernels beside it, 34.0 against
+// 32.2 us per clip.)
+static int split_of(const Problem& p, long long tiles, int most) {
     const int nst = (p.C + kTcKC - 1) / kTcKC;
-    const int cap = p.r == 2 ? 4 : 8;
-    int pieces = 1;
-    while (pieces * 2 <= cap && tiles * (pieces * 2) <= 2LL * sm_count() && nst / (pieces * 2) >= 4) pieces *= 2;
-    return pieces;
+    int n = 1;
+    while (n * 2 <= most && tiles * (n * 2) <= 2LL * sm_count() && nst / (n * 2) >= 2) n *= 2;
+    return n;
 }
+int tc_match_chunks(const Problem& p) { return split_of(p, (long long)tc_match_tiles(p), p.r == 2 ? 4 : 8); }
 
 template <int R, int G>
 static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                unsigned char* keep, cudaStream_t st) {
     using S = TcShape<R>;
-    static_assert((size_t)7 * ((S::WIN + 1) * kTcM + S::NCAND) * 4 <= (size_t)S::STAGES * S::STAGE || R == 2, "exchange rows must fit the ring");
-    static_assert((size_t)3 * ((S::WIN + 1) * kTcM + S::NCAND) * 4 <= (size_t)S::STAGES * S::STAGE, "exchange rows must fit the ring");
     ClipMaps<G> maps;
     for (int n = 0; n < p.nclips; ++n)
         if (!make_tensor_map(&maps.a[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, kTcWB, 1, kTcFR, true) ||
             !make_tensor_map(&maps.b[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, S::BW, S::SIDE, 1, true))
             return cudaErrorInvalidValue;
-    const size_t smem = (size_t)S::STAGES * S::STAGE + 1024;
+    // (at least 80 KB: never three CTAs on one SM while others have one or none; r = 0 would fit three)
+    const size_t need = (size_t)S::RING + S::XBYTES + S::NORMBYTES + 1024, smem = need < 80 * 1024 ? 80 * 1024 : need;
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R, G>), smem);
     if (e != cudaSuccess) return e;
-    const int pieces = tc_match_pieces(p);
     const long long tiles = (long long)tc_match_tiles(p);
+    const int chunks = tc_match_chunks(p);
+    const int pieces = split_of(p, tiles * p.nclips, chunks);      // CTAs (= cluster size) per tile
+    auto log2_of = [](int n) { int l = 0; while ((1 << l) < n) ++l; return l; };
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles * pieces), p.nclips); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -491,7 +575,7 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
     }
     cfg.attrs = attr; cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, k_match_tc<R, G>, maps, p.F, p.H, p.W, p.C, p.t, make_anchor_src(p, s, out_anchor),
-                              pieces, shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride);
+                              log2_of(pieces), log2_of(chunks), shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride);
 }
 
 cudaError_t launch_match_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,

@@ -1,0 +1,36 @@
+"""The tcgen05 matching kernel at the edges of its tiles (strips of 4 cells, 32 frames, stages of 64 channels, a tile's
+channel range in 1 to 8 chunks over as many CTAs), against the CPU oracle; and the same bits whether the chunks of a tile
+are summed by one CTA or by several."""
+import pytest
+import torch
+
+import paper_2605_07355_b200 as P
+from tests.parity import check_clip, to_device
+from tests.test_gpu_parity import corr_clip
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("r", [0, 1, 2])
+@pytest.mark.parametrize("shape", [(1, 3, 4, 64), (5, 4, 5, 128), (31, 3, 7, 200), (32, 2, 9, 264), (33, 5, 3, 520), (3, 6, 8, 1032),
+                                   (65, 1, 4, 1160), (9, 16, 17, 2056)])
+def test_tile_edges(shape, r):
+    X = corr_clip(*shape, seed=sum(shape) + r, dtype="bf16")
+    check_clip(X, r, 0.6)
+    check_clip(X, r, 0.6, anchor_mode=2)
+
+
+@pytest.mark.parametrize("shape,r,clips", [((6, 8, 8, 1024), 1, 24), ((32, 8, 8, 512), 1, 16), ((9, 7, 6, 576), 0, 32),
+                                           ((20, 9, 8, 1160), 2, 12)])
+def test_bits_do_not_depend_on_the_split(shape, r, clips):
+    """thresholds that are the similarity of some token, bit for bit: the strict gate flips on any difference"""
+    X = to_device(corr_clip(*shape, seed=sum(shape), dtype="bf16"))
+    q = P.ttf_query(X, r, 0.6)
+    sims = torch.sort(q["best_sim"][q["best_sim"] < 1.0]).values
+    for t in sims[:: max(1, sims.numel() // 8)].tolist():
+        one = P.ttf_compress(X, r, t)
+        toks, cnts, poss = P.ttf_compress_batch([X] * clips, r, t)
+        torch.cuda.synchronize()
+        L = int(one[1])
+        assert all(int(c) == L for c in cnts)
+        assert all(torch.equal(p[:L], one[2][:L]) for p in poss)
