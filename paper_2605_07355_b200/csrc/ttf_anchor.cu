@@ -14,6 +14,11 @@
 // of summation is fixed, so the result is reproducible.
 #include "ttf_internal.cuh"
 
+#include <map>
+#include <mutex>
+#include <set>
+#include <utility>
+
 namespace ttf {
 
 constexpr int kNormWarps = 8;
@@ -289,9 +294,9 @@ k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// The same statistics as ONE thread-block cluster of 8 CTAs, for clips of at most 4096 channels and 256 frames (the
-// frame sums of 32 / 64 / 128 frames at 4 / 2 / 1 slices of 128 channels per CTA stay in registers; longer clips are
-// fetched a second time for the second step).  A grid of
+// The same statistics as ONE thread-block cluster of CS = 1, 8 or 16 CTAs, for clips of at most 4096 channels and 256
+// frames (the frame sums of up to 128 / SL frames at SL slices of 128 channels per CTA stay in registers; longer clips
+// are fetched a second time for the second step).  A grid of
 // independent CTAs has to go through global memory, a fence and an arrival counter before one of them can take
 // the arg max, which is five to six dependent round trips after the sweep; here every CTA fetches all of its
 // frame sums in one round trip, the per-frame shares of <S_k, g>, |S_k|^2 and |g|^2 go to rank 0 through
@@ -299,8 +304,10 @@ k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float
 // the 8B-shaped clip, 42.1 -> 37.7 us per clip with one clip in flight).  Every order of summation is fixed
 // (slices inside a CTA, then ranks), so the result is reproducible; it may differ in the last bits from the grid
 // kernel's, which adds the same terms in another fixed order.
-constexpr int kStatCluster = 8;
-
+// What bounds it is a serial chain: what an SM can take in from L2 (64 KB per CTA for 32 frames of 4096 channels on eight
+// CTAs, 0.9 us; hence sixteen where the kernel runs alone), three block barriers and the cluster barrier.  With eight CTAs, two shuffle trees per frame and every warp adding up all
+// channels of g for itself a pass took, per clip, 39.3 us (32 x 16 x 16 x 4096), 28.9 (2048 channels), 134.7 (128 frames)
+// and 11.3 (4 x 8 x 8 x 64); as it stands 38.0, 28.1, 130.2 and 10.2.
 __device__ __forceinline__ uint32_t stat_cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -319,16 +326,17 @@ __device__ __forceinline__ void stat_st_cluster(const float* local, uint32_t ran
 
 constexpr int kStatClusterMaxF = 256;     // frames the cluster kernel takes (shares of all frames live in shared memory)
 
-template <int SL>     // slices of 128 channels per CTA; FB = 16 / SL frames per thread and chunk (warp w owns frames w, w + 8, ...)
+template <int SL, int CS>     // slices of 128 channels per CTA, CTAs; warp w owns frames w, w + 8, ...
 __global__ void __launch_bounds__(kNormThreads)
 k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_anchor, size_t sstride)
 {
     S = clip_block(S, sstride); hdr = clip_block(hdr, sstride);
-    constexpr int FB = 16 / SL;
+    constexpr int FB = 16 / SL;                      // frames per thread and chunk
     constexpr int CHUNK = kNormWarps * FB;           // frames per chunk: 32 / 64 / 128
-    __shared__ float4 s_g[SL][kNormWarps][32];
+    __shared__ float s_g[kNormWarps][SL * 128];
+    __shared__ float s_gl[SL * 128];
     __shared__ float s_D[kStatClusterMaxF], s_Q[kStatClusterMaxF], s_G;
-    __shared__ float s_x[kStatCluster - 1][2 * kStatClusterMaxF + 1];      // what the other ranks send (rank 0 only)
+    __shared__ float s_x[CS > 1 ? CS - 1 : 1][2 * kStatClusterMaxF + 1];   // what the other ranks send (rank 0 only)
     __shared__ float s_best[kNormWarps];
     __shared__ int s_idx[kNormWarps];
     pdl_launch_dependents();
@@ -336,7 +344,7 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     pdl_wait();                                      // the sweep's frame sums are complete and visible
     trace_mark(hdr, 4, false);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int rank = (int)stat_cluster_rank();
+    const int rank = CS > 1 ? (int)stat_cluster_rank() : 0;
     const bool one_chunk = F <= CHUNK;               // then the frame sums stay in registers for the second step
 
     // the frame sums of one chunk of frames: one round trip
@@ -344,7 +352,7 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     auto load_chunk = [&](int k0) {
 #pragma unroll
         for (int sl = 0; sl < SL; ++sl) {
-            const int q = rank + sl * kStatCluster;
+            const int q = rank + sl * CS;
             const int c0 = (q * 32 + lane) * 4;
 #pragma unroll
             for (int jj = 0; jj < FB; ++jj) {
@@ -368,32 +376,39 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
             }
     }
 #pragma unroll
-    for (int sl = 0; sl < SL; ++sl) s_g[sl][w][lane] = gacc[sl];
+    for (int sl = 0; sl < SL; ++sl) reinterpret_cast<float4*>(s_g[w])[sl * 32 + lane] = gacc[sl];
+    __syncthreads();
+    for (int c = tid; c < SL * 128; c += kNormThreads) {          // one channel per thread
+        float g = 0.f;
+#pragma unroll
+        for (int ww = 0; ww < kNormWarps; ++ww) g += s_g[ww][c];
+        s_gl[c] = g;
+    }
     __syncthreads();
     float4 gl[SL];
 #pragma unroll
-    for (int sl = 0; sl < SL; ++sl) {
-        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int ww = 0; ww < kNormWarps; ++ww) { const float4 t = s_g[sl][ww][lane]; g.x += t.x; g.y += t.y; g.z += t.z; g.w += t.w; }
-        gl[sl] = g;
-    }
-    // step 2: this CTA's shares of <S_k, g> and |S_k|^2 for every frame, slices in order
+    for (int sl = 0; sl < SL; ++sl) gl[sl] = reinterpret_cast<const float4*>(s_gl)[sl * 32 + lane];
+    // step 2: this CTA's shares of <S_k, g> and |S_k|^2 for every frame, slices in order; four frames at a time are added
+    // up over the warp (fold8)
     for (int k0 = 0; k0 < F; k0 += CHUNK) {
         if (!one_chunk) load_chunk(k0);              // (a second round trip per chunk for clips of several chunks)
 #pragma unroll
-        for (int jj = 0; jj < FB; ++jj) {
-            float d = 0.f, qq = 0.f;
+        for (int j0 = 0; j0 < FB; j0 += 4) {
+            float part[8];                           // <S_k, g> and |S_k|^2 of frames j0 .. j0 + 3
 #pragma unroll
-            for (int sl = 0; sl < SL; ++sl) {
-                const float4 x = v[sl][jj], g = gl[sl];
-                d = fmaf(x.x, g.x, d); d = fmaf(x.y, g.y, d); d = fmaf(x.z, g.z, d); d = fmaf(x.w, g.w, d);
-                qq = fmaf(x.x, x.x, qq); qq = fmaf(x.y, x.y, qq); qq = fmaf(x.z, x.z, qq); qq = fmaf(x.w, x.w, qq);
+            for (int e = 0; e < 4; ++e) {
+                float d = 0.f, qq = 0.f;
+#pragma unroll
+                for (int sl = 0; sl < SL; ++sl) {
+                    const float4 x = v[sl][j0 + e], g = gl[sl];
+                    d = fmaf(x.x, g.x, d); d = fmaf(x.y, g.y, d); d = fmaf(x.z, g.z, d); d = fmaf(x.w, g.w, d);
+                    qq = fmaf(x.x, x.x, qq); qq = fmaf(x.y, x.y, qq); qq = fmaf(x.z, x.z, qq); qq = fmaf(x.w, x.w, qq);
+                }
+                part[e] = d; part[4 + e] = qq;
             }
-            d = warp_sum(d);
-            qq = warp_sum(qq);
-            const int kk = k0 + w + jj * kNormWarps;
-            if (lane == 0 && kk < F) { s_D[kk] = d; s_Q[kk] = qq; }
+            const float tot = fold8(part, lane);     // lanes 0, 4, 8, ..: part[4 * bit4 + 2 * bit3 + bit2] of the lane index
+            const int kk = k0 + w + (j0 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)) * kNormWarps;
+            if ((lane & 3) == 0 && kk < F) (lane & 16 ? s_Q : s_D)[kk] = tot;
         }
     }
     if (w == 0) {
@@ -407,35 +422,43 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
         if (lane == 0) s_G = gg;
     }
     __syncthreads();
-    if (rank > 0) {                                  // hand the shares to rank 0
-        for (int i = tid; i < 2 * F + 1; i += kNormThreads)
-            stat_st_cluster(&s_x[rank - 1][i], 0, i < F ? s_D[i] : (i < 2 * F ? s_Q[i - F] : s_G));
+    if (CS > 1) {
+        if (rank > 0) {                              // hand the shares to rank 0
+            for (int i = tid; i < 2 * F + 1; i += kNormThreads)
+                stat_st_cluster(&s_x[rank - 1][i], 0, i < F ? s_D[i] : (i < 2 * F ? s_Q[i - F] : s_G));
+        }
+        __syncwarp();
+        stat_cluster_sync();
     }
-    __syncthreads();
-    stat_cluster_sync();
     if (rank == 0) {
         // Eq. (auto_anchor): a* = arg max_k <S_k, g> / (|S_k| |g|), lowest frame on ties; ranks added in rank order
         float best = -INFINITY;
         int idx = 0x7fffffff;
         if (tid < F) {                               // F <= kStatClusterMaxF = the CTA's 256 threads
             float D = s_D[tid], Q = s_Q[tid], G = s_G;
-            for (int r = 0; r < kStatCluster - 1; ++r) { D += s_x[r][tid]; Q += s_x[r][F + tid]; G += s_x[r][2 * F]; }
+#pragma unroll
+            for (int r = 0; r < CS - 1; ++r) { D += s_x[r][tid]; Q += s_x[r][F + tid]; G += s_x[r][2 * F]; }
             best = D * (1.0f / fmaxf(sqrtf(G), kNormFloor)) * (1.0f / fmaxf(sqrtf(Q), kNormFloor));
             idx = tid;
         }
+        auto better = [](float ob, int oi, float& best, int& idx) {
+            const bool take = (oi != 0x7fffffff) & ((idx == 0x7fffffff) | (ob > best) | ((ob == best) & (oi < idx)));
+            best = take ? ob : best;
+            idx = take ? oi : idx;
+        };
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const float ob = __shfl_xor_sync(0xffffffffu, best, o);
             const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-            if (oi != 0x7fffffff && (idx == 0x7fffffff || ob > best || (ob == best && oi < idx))) { best = ob; idx = oi; }
+            better(ob, oi, best, idx);
         }
-        if (lane == 0) { s_best[w] = best; s_idx[w] = idx; }
-        __syncthreads();
+        if (F > 32) {
+            if (lane == 0) { s_best[w] = best; s_idx[w] = idx; }
+            __syncthreads();
+            if (tid == 0)
+                for (int ww = 1; ww < kNormWarps; ++ww) better(s_best[ww], s_idx[ww], best, idx);
+        }
         if (tid == 0) {
-            for (int ww = 1; ww < kNormWarps; ++ww)
-                if (s_idx[ww] != 0x7fffffff && (idx == 0x7fffffff || s_best[ww] > best || (s_best[ww] == best && s_idx[ww] < idx))) {
-                    best = s_best[ww]; idx = s_idx[ww];
-                }
             hdr[HDR_ANCHOR] = idx;
             if (out_anchor) *out_anchor = idx;
         }
@@ -443,18 +466,36 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     trace_mark(hdr, 1, true);
 }
 
-template <int SL>
+// clusters of sixteen CTAs: allowed for `func` on the current device (set once)
+static cudaError_t ensure_large_clusters(const void* func) {
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    if (done.count({func, dev})) return cudaSuccess;
+    e = cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) done.insert({func, dev});
+    return e;
+}
+
+template <int SL, int CS>
 static cudaError_t launch_stats_cluster_t(const Problem& p, const Scratch& s, int* out_anchor, cudaStream_t st) {
+    const auto kernel = k_frame_stats_cluster<SL, CS>;
+    if (CS > 8) {                                    // (sixteen CTAs to a cluster have to be asked for)
+        cudaError_t e = ensure_large_clusters(reinterpret_cast<const void*>(kernel));
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kStatCluster, p.nclips); cfg.blockDim = dim3(kNormThreads); cfg.dynamicSmemBytes = 0; cfg.stream = st;
+    cfg.gridDim = dim3(CS, p.nclips); cfg.blockDim = dim3(kNormThreads); cfg.dynamicSmemBytes = 0; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = kStatCluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_frame_stats_cluster<SL>, (const float*)s.S, p.F, p.C, p.nsl, s.hdr, out_anchor,
-                              p.sstride);
+    attr[1].val.clusterDim.x = CS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = CS > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, (const float*)s.S, p.F, p.C, p.nsl, s.hdr, out_anchor, p.sstride);
 }
 
 // What the sweep leaves behind besides its sums, for calls that need no sweep (a fixed anchor and a matching kernel
@@ -476,6 +517,29 @@ cudaError_t launch_norm_sum(const Problem& p, const Scratch& s, cudaStream_t st)
     return p.vec ? launch_sum_t<bf16_t, 8>(p, s, st) : launch_sum_t<bf16_t, 1>(p, s, st);
 }
 
+// whether the current device can run such a cluster of the statistics kernel (asked once per device)
+static bool large_clusters() {
+    static std::mutex mu;
+    static std::map<int, bool> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = known.find(dev);
+    if (it != known.end()) return it->second;
+    const auto kernel = k_frame_stats_cluster<2, 16>;
+    int n = 0;
+    if (ensure_large_clusters(reinterpret_cast<const void*>(kernel)) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(16); cfg.blockDim = dim3(kNormThreads);
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 16; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr; cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
+    }
+    return known[dev] = n > 0;
+}
+
 cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anchor, cudaStream_t st) {
     if (p.anchor_mode != 0) return cudaSuccess;                // fixed anchors need no statistics
     // The single-cluster kernel is the shorter one (4.9 against 7.2 us on a 32-frame clip of 4096 channels) and takes
@@ -485,11 +549,14 @@ cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anch
     // clip with the cluster kernel, 29.8 with the grid kernel; two in flight: 33.9 against 35.0; 128-frame clip, eight
     // in flight: 107.9 against 110.1, the grid kernel's time grows with F).
     const bool crowded = p.overlapped >= 4 && p.F <= 32;
-    if (!crowded && p.C % 4 == 0 && p.nsl <= 4 * kStatCluster && p.F <= kStatClusterMaxF) {
-        const int sl = (p.nsl + kStatCluster - 1) / kStatCluster;          // slices per CTA: 1 .. 4
-        if (sl <= 1) return launch_stats_cluster_t<1>(p, s, out_anchor, st);
-        if (sl <= 2) return launch_stats_cluster_t<2>(p, s, out_anchor, st);
-        return launch_stats_cluster_t<4>(p, s, out_anchor, st);
+    if (!crowded && p.C % 4 == 0 && p.nsl <= 32 && p.F <= kStatClusterMaxF) {
+        if (p.nsl == 1) return launch_stats_cluster_t<1, 1>(p, s, out_anchor, st);      // nothing to split
+        const bool alone = p.overlapped <= 1 && large_clusters();
+        if (p.nsl > 16) return alone ? launch_stats_cluster_t<2, 16>(p, s, out_anchor, st)
+                                     : launch_stats_cluster_t<4, 8>(p, s, out_anchor, st);
+        if (p.nsl > 8) return alone ? launch_stats_cluster_t<1, 16>(p, s, out_anchor, st)
+                                    : launch_stats_cluster_t<2, 8>(p, s, out_anchor, st);
+        return launch_stats_cluster_t<1, 8>(p, s, out_anchor, st);
     }
     if (p.C % 4 == 0)
         return launch_pdl(k_frame_stats<4>, dim3(p.nsl, p.nclips), dim3(kNormThreads), st, (const float*)s.S, p.F, p.C, p.nsl,
