@@ -7,18 +7,19 @@ namespace ttf {
 constexpr int kXThreads = 256;
 
 // Number of non-zero flags in keep[lo, hi): bytes up to the first 16-byte boundary, 16 flags per load from there,
-// bytes again at the end.  Every thread of the CTA takes part; the caller adds the per-thread counts up.
-__device__ __forceinline__ int count_flags(const unsigned char* __restrict__ keep, size_t lo, size_t hi, int tid) {
+// bytes again at the end.  Every thread of the CTA takes part; the caller adds the per-thread counts up.  (L2-coherent
+// loads: the flags may come from a kernel that still ran when this one was scheduled.)
+__device__ __forceinline__ int count_flags(const unsigned char* keep, size_t lo, size_t hi, int tid) {
     if (lo >= hi) return 0;
     int c = 0;
     const uintptr_t base = reinterpret_cast<uintptr_t>(keep);
     size_t head = lo + ((16 - ((base + lo) & 15)) & 15);          // first index whose address is 16-byte aligned
     if (head > hi) head = hi;
     const size_t nvec = (hi - head) / 16, tail = head + nvec * 16;
-    for (size_t f = lo + tid; f < head; f += kXThreads) c += keep[f] ? 1 : 0;
+    for (size_t f = lo + tid; f < head; f += kXThreads) c += __ldcg(keep + f) ? 1 : 0;
     const uint4* v = reinterpret_cast<const uint4*>(keep + head);
     for (size_t u = tid; u < nvec; u += kXThreads) {
-        const uint4 q = __ldg(v + u);
+        const uint4 q = __ldcg(v + u);
         // a flag is any non-zero byte: fold each byte's bits into its lowest one
         unsigned w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
@@ -28,7 +29,7 @@ __device__ __forceinline__ int count_flags(const unsigned char* __restrict__ kee
             c += __popc(b & 0x01010101u);
         }
     }
-    for (size_t f = tail + tid; f < hi; f += kXThreads) c += keep[f] ? 1 : 0;
+    for (size_t f = tail + tid; f < hi; f += kXThreads) c += __ldcg(keep + f) ? 1 : 0;
     return c;
 }
 
@@ -74,57 +75,122 @@ k_restore_index(const int* __restrict__ anchor, const unsigned char* __restrict_
     }
 }
 
-// One warp per output row; a lane keeps up to eight loads in flight before it stores them, so a row of 8 KB moves
-// in two rounds.  Rows of retained tokens are read once (consecutive tokens sit in consecutive compressed rows);
-// the N anchor rows are read again and again and stay in L2.
-template <typename U>
-__global__ void __launch_bounds__(kXThreads)
-k_restore_copy(const unsigned char* __restrict__ comp, size_t row_bytes, long long rows,
-               const int* __restrict__ row_index, unsigned char* __restrict__ out)
-{
+// Rows f = first, first + step, ... < end of the output by one warp; `row(f)` is the compressed row that stands for token
+// f.  A lane keeps up to eight loads in flight before it stores them, so a row of 8 KB moves in two rounds.  Rows of
+// retained tokens are read once (consecutive tokens sit in consecutive compressed rows); the N anchor rows are read again
+// and again and stay in L2.
+template <typename U, typename Row>
+__device__ __forceinline__ void restore_rows(const unsigned char* comp, size_t row_bytes, long long first,
+                                             long long end, long long step, unsigned char* out, int lane,
+                                             Row&& row) {
     constexpr int kInFlight = 8;
-    const int lane = threadIdx.x & 31;
-    const long long gw = (long long)blockIdx.x * (kXThreads / 32) + (threadIdx.x >> 5);
-    const long long nw = (long long)gridDim.x * (kXThreads / 32);
     const int units = (int)(row_bytes / sizeof(U));
-    pdl_wait();                                  // row_index is complete
-    for (long long f = gw; f < rows; f += nw) {
-        const U* src = reinterpret_cast<const U*>(comp + (size_t)__ldcg(row_index + f) * row_bytes);
+    for (long long f = first; f < end; f += step) {
+        const U* src = reinterpret_cast<const U*>(comp + (size_t)row(f) * row_bytes);
         U* d = reinterpret_cast<U*>(out + (size_t)f * row_bytes);
         int u = lane;
         for (; u + (kInFlight - 1) * 32 < units; u += kInFlight * 32) {
             U v[kInFlight];
 #pragma unroll
-            for (int e = 0; e < kInFlight; ++e) v[e] = src[u + e * 32];
+            for (int e = 0; e < kInFlight; ++e) v[e] = __ldcg(src + u + e * 32);
 #pragma unroll
             for (int e = 0; e < kInFlight; ++e) d[u + e * 32] = v[e];
         }
-        for (; u < units; u += 32) d[u] = src[u];
+        for (; u < units; u += 32) d[u] = __ldcg(src + u);
     }
 }
 
 template <typename U>
-static cudaError_t launch_restore_copy(const unsigned char* c, size_t row_bytes, long long rows, const int* row_index,
-                                       unsigned char* o, cudaStream_t st) {
+__global__ void __launch_bounds__(kXThreads)
+k_restore_copy(const unsigned char* __restrict__ comp, size_t row_bytes, long long rows,
+               const int* __restrict__ row_index, unsigned char* __restrict__ out)
+{
+    const long long gw = (long long)blockIdx.x * (kXThreads / 32) + (threadIdx.x >> 5);
+    const long long nw = (long long)gridDim.x * (kXThreads / 32);
+    pdl_wait();                                  // row_index is complete
+    restore_rows<U>(comp, row_bytes, gw, rows, nw, out, threadIdx.x & 31, [&](long long f) { return __ldcg(row_index + f); });
+}
+
+// Both steps in one launch, for clips of up to kRestoreWhole tokens: a CTA owns a contiguous range of tokens, counts the
+// preserved tokens before it (16 flags per load: one round trip), ranks its own 256 at a time, and copies their rows from
+// the indices in shared memory.  With a kernel of its own for the indices (5.2 us) a 32 x 16 x 16 clip of 4096 bf16
+// channels took 23.7 us, 19.1 now (its 90 MB at the copy rate: 13.8); in longer clips the flags that every CTA reads would
+// outweigh the launch.
+constexpr int kRestoreWhole = 1 << 16;
+
+template <typename U>
+__global__ void __launch_bounds__(kXThreads)
+k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int* anchor, const unsigned char* keep,
+          const int* dst, int per, unsigned char* out, int* row_index)
+{
+    __shared__ int s_warp[kXThreads / 32];
+    __shared__ int s_row[kXThreads];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int f0 = blockIdx.x * per, f1 = min(FN, f0 + per);
+    pdl_launch_dependents();
+    pdl_wait();                                  // the caller's kernels before this one
+    const int a = __ldcg(anchor), a0 = a * N, a1 = a0 + N;
+    // preserved source tokens before f0 (the anchor frame does not count)
+    int c = count_flags(keep, 0, (size_t)min(f0, a0), tid);
+    if (f0 > a1) c += count_flags(keep, (size_t)a1, (size_t)f0, tid);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) s_warp[w] = c;
+    __syncthreads();
+    int run = N;
+#pragma unroll
+    for (int ww = 0; ww < kXThreads / 32; ++ww) run += s_warp[ww];
+    for (int b0 = f0; b0 < f1; b0 += kXThreads) {
+        const int f = b0 + tid;
+        const bool in = f < f1, own = f >= a0 && f < a1;
+        const bool kp = in && !own && __ldcg(keep + f);
+        const unsigned m = __ballot_sync(0xffffffffu, kp);
+        __syncthreads();                         // (the indices of the round before this one, and s_warp, are done with)
+        if (lane == 0) s_warp[w] = __popc(m);
+        __syncthreads();
+        int off = 0, total = 0;
+#pragma unroll
+        for (int ww = 0; ww < kXThreads / 32; ++ww) { off += ww < w ? s_warp[ww] : 0; total += s_warp[ww]; }
+        if (in) {
+            const int r = own ? f - a0 : (kp ? run + off + __popc(m & ((1u << lane) - 1)) : __ldcg(dst + f));
+            s_row[tid] = r;
+            row_index[f] = r;
+        }
+        run += total;
+        __syncthreads();
+        restore_rows<U>(comp, row_bytes, b0 + w, min(f1, b0 + kXThreads), kXThreads / 32, out, lane,
+                        [&](long long g) { return s_row[(int)g - b0]; });
+    }
+}
+
+template <typename U>
+static cudaError_t launch_restore_t(const unsigned char* c, size_t row_bytes, int F, int N, const int* anchor,
+                                    const unsigned char* keep, const int* dst, unsigned char* o, int* row_index,
+                                    cudaStream_t st) {
+    const long long rows = (long long)F * N;
     long long blocks = (rows + kXThreads / 32 - 1) / (kXThreads / 32);
     if (blocks > 8LL * sm_count()) blocks = 8LL * sm_count();
+    if (rows <= kRestoreWhole) {
+        const int per = (int)((rows + blocks - 1) / blocks);
+        return launch_pdl(k_restore<U>, dim3((unsigned)((rows + per - 1) / per)), dim3(kXThreads), st, c, row_bytes, (int)rows,
+                          N, anchor, keep, dst, per, o, row_index);
+    }
+    k_restore_index<<<F, kXThreads, 0, st>>>(anchor, keep, dst, F, N, row_index);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     return launch_pdl(k_restore_copy<U>, dim3((unsigned)blocks), dim3(kXThreads), st, c, row_bytes, rows, row_index, o);
 }
 
 cudaError_t launch_restore(const void* comp, size_t row_bytes, int F, int N, const int* anchor,
                            const unsigned char* keep, const int* dst, void* out_full, int* row_index,
                            cudaStream_t st) {
-    k_restore_index<<<F, kXThreads, 0, st>>>(anchor, keep, dst, F, N, row_index);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long long rows = (long long)F * N;
     const unsigned char* c = reinterpret_cast<const unsigned char*>(comp);
     unsigned char* o = reinterpret_cast<unsigned char*>(out_full);
     const uintptr_t al = reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(out_full) | row_bytes;
-    if (al % 16 == 0) return launch_restore_copy<uint4>(c, row_bytes, rows, row_index, o, st);
-    if (al % 4 == 0) return launch_restore_copy<uint32_t>(c, row_bytes, rows, row_index, o, st);
-    if (al % 2 == 0) return launch_restore_copy<uint16_t>(c, row_bytes, rows, row_index, o, st);
-    return launch_restore_copy<unsigned char>(c, row_bytes, rows, row_index, o, st);
+    if (al % 16 == 0) return launch_restore_t<uint4>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);
+    if (al % 4 == 0) return launch_restore_t<uint32_t>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);
+    if (al % 2 == 0) return launch_restore_t<uint16_t>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);
+    return launch_restore_t<unsigned char>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);
 }
 
 // Histogram of the best-match similarities of the source tokens over `bins` equal bins of [-1, 1]

@@ -120,3 +120,21 @@ def test_stats_match_oracle(name, band):
     assert P.ttf_reduction_ratio(int(st[0]), F, N) == rho
     toks, cnt, pos = P.ttf_compress(to_device(X), s.r, s.t)
     assert int(cnt.item()) == N + Pn                                  # L' = N + P (Eq. Lpre)
+
+
+@pytest.mark.parametrize("shape", [(2, 3, 3, 16), (9, 16, 16, 24), (64, 32, 32, 8), (65, 32, 32, 8), (300, 5, 7, 33), (3, 127, 129, 8)])
+def test_restore_one_and_two_launches(shape):
+    """clips around the size up to which index and copy are one launch, ranges of several rounds, odd rows"""
+    F, H, W, C = shape
+    N = H * W
+    X = corr_clip(F, H, W, C, seed=sum(shape), dtype="bf16", sigma=0.6)
+    Xd = to_device(X)
+    for mode in (0, 2):
+        q = P.ttf_query(Xd, 1, 0.6, anchor_mode=mode)
+        toks, cnt, _ = P.ttf_compress(Xd, 1, 0.6, anchor_mode=mode)
+        torch.cuda.synchronize()
+        full, idx = P.ttf_restore(toks[:int(cnt)], F, H, W, q["anchor"], q["keep"], q["dst"])
+        torch.cuda.synchronize()
+        keep, dst, a = q["keep"].cpu().numpy(), q["dst"].cpu().numpy(), int(q["anchor"])
+        ref_full, ref_idx = O.restore(to_bits(toks[:int(cnt)]), keep, dst, F, N, a)
+        assert (idx.cpu().numpy() == ref_idx).all() and (to_bits(full) == ref_full).all()
