@@ -341,8 +341,8 @@ int ttf_query_static(const void* features, int F, int H, int W, int C, int r, fl
  * device time in milliseconds and the number of launches; `kinds` is the length of both arrays
  * (TTF_KERNEL_KINDS covers all).  Kinds: 0 frame-sum (and norm) sweep, 1 frame statistics of the anchor rule,
  * 2 windowed match + gate (its prologue takes the anchor arg max), 3 compaction gather (with the frame-count
- * prefix of clips longer than 1024 frames), 4 fuse-count bookkeeping of ttf_query.  Profiling is process-wide
- * and meant for benchmarks; leave it off otherwise.
+ * prefix of clips longer than 1024 frames), 4 nothing any more (the matching kernel counts the fused tokens of
+ * ttf_query).  Profiling is process-wide and meant for benchmarks; leave it off otherwise.
  */
 #define TTF_KERNEL_KINDS 5
 int ttf_profile_begin(void);

@@ -13,6 +13,8 @@
 // <S_k, g>, |S_k|^2 and |g|^2 (the factors 1/N and 1/(FN) of Eq. auto_anchor cancel in a cosine).  Every order
 // of summation is fixed, so the result is reproducible.
 #include "ttf_internal.cuh"
+#include "ttf_async.cuh"
+#include "ttf_cluster.cuh"
 
 #include <map>
 #include <mutex>
@@ -166,6 +168,13 @@ static cudaError_t launch_sum_t(const Problem& p, const Scratch& s, cudaStream_t
                      s.cnt, s.hdr, p.chain, p.sstride);
 }
 
+// The query's counts of fused tokens start at zero for the matching kernel: cleared by the kernel between the sweep and it
+// (all CTAs of the grid; a parameter more in the sweep cost it a CTA per SM in registers, 37.8 -> 39.5 us per pass).
+__device__ __forceinline__ void clear_counts(int* fuse_cnt, int N) {
+    if (!fuse_cnt) return;
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) fuse_cnt[j] = 0;
+}
+
 // ---------------------------------------------------------------------------------------------------------
 constexpr int kStatFB = 4;           // frames per thread held in registers (8 warps x 4 = 32 frames)
 
@@ -183,7 +192,7 @@ constexpr int kStatSub = 1;
 template <int V>
 __global__ void __launch_bounds__(kNormThreads)
 k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float* Gp, int* hdr, int* out_anchor,
-              size_t sstride)
+              size_t sstride, int* fuse_cnt, int N)
 {
     S = clip_block(S, sstride); Dp = clip_block(Dp, sstride); Qp = clip_block(Qp, sstride); Gp = clip_block(Gp, sstride);
     hdr = clip_block(hdr, sstride);
@@ -191,6 +200,7 @@ k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float
     trace_mark(hdr, 1, false);
     pdl_wait();                                      // the sweep's frame sums are complete and visible
     trace_mark(hdr, 4, false);
+    clear_counts(fuse_cnt, N);
     const int q = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     constexpr int NV = kStatSub * V;                 // channels per lane
@@ -308,27 +318,11 @@ k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float
 // CTAs, 0.9 us; hence sixteen where the kernel runs alone), three block barriers and the cluster barrier.  With eight CTAs, two shuffle trees per frame and every warp adding up all
 // channels of g for itself a pass took, per clip, 39.3 us (32 x 16 x 16 x 4096), 28.9 (2048 channels), 134.7 (128 frames)
 // and 11.3 (4 x 8 x 8 x 64); as it stands 38.0, 28.1, 130.2 and 10.2.
-__device__ __forceinline__ uint32_t stat_cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void stat_cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void stat_st_cluster(const float* local, uint32_t rank, float v) {
-    uint32_t remote;
-    const uint32_t l = static_cast<uint32_t>(__cvta_generic_to_shared(local));
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(l), "r"(rank));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
-}
-
 constexpr int kStatClusterMaxF = 256;     // frames the cluster kernel takes (shares of all frames live in shared memory)
 
 template <int SL, int CS>     // slices of 128 channels per CTA, CTAs; warp w owns frames w, w + 8, ...
 __global__ void __launch_bounds__(kNormThreads)
-k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_anchor, size_t sstride)
+k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_anchor, size_t sstride, int* fuse_cnt, int N)
 {
     S = clip_block(S, sstride); hdr = clip_block(hdr, sstride);
     constexpr int FB = 16 / SL;                      // frames per thread and chunk
@@ -344,8 +338,10 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     pdl_wait();                                      // the sweep's frame sums are complete and visible
     trace_mark(hdr, 4, false);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int rank = CS > 1 ? (int)stat_cluster_rank() : 0;
+    const int rank = CS > 1 ? (int)cluster_rank() : 0;
     const bool one_chunk = F <= CHUNK;               // then the frame sums stay in registers for the second step
+
+    clear_counts(fuse_cnt, N);
 
     // the frame sums of one chunk of frames: one round trip
     float4 v[SL][FB];
@@ -425,10 +421,12 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     if (CS > 1) {
         if (rank > 0) {                              // hand the shares to rank 0
             for (int i = tid; i < 2 * F + 1; i += kNormThreads)
-                stat_st_cluster(&s_x[rank - 1][i], 0, i < F ? s_D[i] : (i < 2 * F ? s_Q[i - F] : s_G));
+                st_cluster_f32(cluster_addr(smem_u32(&s_x[rank - 1][i]), 0),
+                               i < F ? s_D[i] : (i < 2 * F ? s_Q[i - F] : s_G));
         }
         __syncwarp();
-        stat_cluster_sync();
+        cluster_arrive();
+        cluster_wait();
     }
     if (rank == 0) {
         // Eq. (auto_anchor): a* = arg max_k <S_k, g> / (|S_k| |g|), lowest frame on ties; ranks added in rank order
@@ -495,24 +493,27 @@ static cudaError_t launch_stats_cluster_t(const Problem& p, const Scratch& s, in
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = CS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = CS > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, (const float*)s.S, p.F, p.C, p.nsl, s.hdr, out_anchor, p.sstride);
+    return cudaLaunchKernelEx(&cfg, kernel, (const float*)s.S, p.F, p.C, p.nsl, s.hdr, out_anchor, p.sstride,
+                              p.fuse_cnt, p.N);
 }
 
 // What the sweep leaves behind besides its sums, for calls that need no sweep (a fixed anchor and a matching kernel
 // that takes the token norms itself): survivor counters at zero, error word cleared.
 __global__ void __launch_bounds__(256)
-k_begin_call(int F, int* __restrict__ cnt, int* __restrict__ hdr, size_t sstride)
+k_begin_call(int F, int* __restrict__ cnt, int* __restrict__ hdr, size_t sstride, int* fuse_cnt, int N)
 {
     cnt = clip_block(cnt, sstride); hdr = clip_block(hdr, sstride);
     pdl_launch_dependents();
     pdl_wait();                                      // the previous call's gather may still read the counters
     for (int k = threadIdx.x; k < F; k += 256) cnt[k] = 0;
+    clear_counts(fuse_cnt, N);
     if (threadIdx.x == 0) hdr[HDR_ERROR] = 0;
 }
 
 cudaError_t launch_norm_sum(const Problem& p, const Scratch& s, cudaStream_t st) {
     if (p.anchor_mode != 0 && !needs_sweep_norms(p))           // Eq. (auto_anchor) is not evaluated: no pass over X
-        return launch_ex(true, 0, k_begin_call, dim3(1, p.nclips), dim3(256), st, p.F, s.cnt, s.hdr, p.sstride);
+        return launch_ex(true, 0, k_begin_call, dim3(1, p.nclips), dim3(256), st, p.F, s.cnt, s.hdr, p.sstride,
+                         p.fuse_cnt, p.N);
     if (p.dtype == 0) return p.vec ? launch_sum_t<float, 4>(p, s, st) : launch_sum_t<float, 1>(p, s, st);
     return p.vec ? launch_sum_t<bf16_t, 8>(p, s, st) : launch_sum_t<bf16_t, 1>(p, s, st);
 }
@@ -560,9 +561,9 @@ cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anch
     }
     if (p.C % 4 == 0)
         return launch_pdl(k_frame_stats<4>, dim3(p.nsl, p.nclips), dim3(kNormThreads), st, (const float*)s.S, p.F, p.C, p.nsl,
-                          s.Dp, s.Qp, s.Gp, s.hdr, out_anchor, p.sstride);
+                          s.Dp, s.Qp, s.Gp, s.hdr, out_anchor, p.sstride, p.fuse_cnt, p.N);
     return launch_pdl(k_frame_stats<1>, dim3(p.nsl, p.nclips), dim3(kNormThreads), st, (const float*)s.S, p.F, p.C, p.nsl,
-                      s.Dp, s.Qp, s.Gp, s.hdr, out_anchor, p.sstride);
+                      s.Dp, s.Qp, s.Gp, s.hdr, out_anchor, p.sstride, p.fuse_cnt, p.N);
 }
 
 }  // namespace ttf

@@ -120,7 +120,6 @@ void carve_scratch(const Problem& p, void* base, Scratch* s) {
     s->shat = (float*)take(sizeof(float) * FN);
     s->dst = (int*)take(sizeof(int) * FN);
     s->keep = (unsigned char*)take(FN);
-    s->fuse_cnt = (int*)take(sizeof(int) * p.N);
     s->bytes = off;
 }
 
@@ -158,7 +157,7 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
     p->nsl = C % 4 == 0 ? (C + 127) / 128 : (C + 31) / 32;
     p->anchor_mode = 0; p->anchor_arg = 0; p->emit_anchor = 1; p->pos_t_offset = 0; p->pos_base = 0; p->natural_order = 0;
     p->use_tc = choose_match(*p);
-    p->chain = 0; p->chain_next = 0; p->overlapped = 0; p->stream_once = 0;
+    p->fuse_cnt = nullptr; p->chain = 0; p->chain_next = 0; p->overlapped = 0; p->stream_once = 0;
     return TTF_OK;
 }
 
@@ -271,14 +270,13 @@ static int query_impl(const Problem& p, void* ws, int* out_anchor, unsigned char
     float* shat = out_sim ? out_sim : s.shat;
     int* dst = out_dst ? out_dst : s.dst;
     unsigned char* keep = out_keep ? out_keep : s.keep;
-    int rc = run_front(p, s, out_anchor, shat, dst, keep, st);
-    if (rc != TTF_OK) return rc;
-    if (out_fuse) {
-        cudaError_t e;
-        { ProfScope ps(st, PK_FUSE_COUNT); e = launch_fuse_count(p, s, dst, keep, out_fuse, st); }
+    Problem q = p;
+    q.fuse_cnt = out_fuse;                       // counted by the matching kernel
+    if (out_fuse && p.anchor_mode != 0 && needs_sweep_norms(p)) {        // no kernel between the sweep and the matching kernel
+        cudaError_t e = cudaMemsetAsync(out_fuse, 0, sizeof(int) * (size_t)p.N, st);
         if (e != cudaSuccess) return cuda_fail(e);
     }
-    return TTF_OK;
+    return run_front(q, s, out_anchor, shat, dst, keep, st);
 }
 
 // ---- host-buffer entry point: staging buffers per device -------------------------------------------------

@@ -1,5 +1,4 @@
-// Token Compression and Positional Alignment (Eqs. xprime_stack, mask, compress_pos, Lpre), plus the
-// bookkeeping of identity replacement (how many source tokens each anchor cell absorbed).
+// Token Compression and Positional Alignment (Eqs. xprime_stack, mask, compress_pos, Lpre).
 //
 // The output position of a preserved source token is N plus the number of preserved source tokens before it
 // in flat (k, i) order.  That exclusive prefix is taken in two levels: the per-frame survivor counts written
@@ -465,22 +464,6 @@ k_compact(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, i
         }
     }
     trace_mark(const_cast<int*>(hdr), 3, true);
-}
-
-// tokens fused into each anchor cell (ttf_query)
-__global__ void __launch_bounds__(kCopyWarps * 32)
-k_fuse_count(int F, int H, int W, int r, const int* hdr, const unsigned char* keep, const int* dst, int* fuse_cnt)
-{
-    pdl_launch_dependents();
-    pdl_wait();
-    fuse_count_cta(F, H, W, r, __ldcg(hdr + HDR_ANCHOR), keep, dst, fuse_cnt, (int)blockIdx.x, (int)gridDim.x);
-}
-
-cudaError_t launch_fuse_count(const Problem& p, const Scratch& s, const int* dst, const unsigned char* keep,
-                              int* fuse_cnt, cudaStream_t st) {
-    const int nb = (p.N + kCopyWarps - 1) / kCopyWarps;
-    return launch_pdl(k_fuse_count, dim3(nb < 1024 ? nb : 1024), dim3(kCopyWarps * 32), st, p.F, p.H, p.W, p.r,
-                      (const int*)s.hdr, keep, dst, fuse_cnt);
 }
 
 cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& out, cudaStream_t st) {

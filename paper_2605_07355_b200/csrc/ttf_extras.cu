@@ -1,6 +1,8 @@
 // Extensions the paper sketches in its Discussion: TTF-R restoration through dst(k,i) (D4) and the empirical
 // distribution of the best-match similarities that an adaptive threshold would look at (D1).
 #include "ttf_internal.cuh"
+#include "ttf_async.cuh"
+#include "ttf_cluster.cuh"
 
 namespace ttf {
 
@@ -226,41 +228,97 @@ cudaError_t launch_sim_histogram(const float* sim, const int* anchor, int F, int
 // tokens whose best similarity lies within `band` of the threshold (the decisions rounding could flip).
 // out[0] = P (preserved source tokens), out[1] = fused source tokens, out[2] = in-band source tokens.  The band test
 // is taken in double on the stored fp32 values, so the counts are exact functions of the arrays.  Integer atomics.
+struct TokenCounts { int c[3]; };                // P, fused, in band
+
+__device__ __forceinline__ void count_token(TokenCounts& n, bool source, bool kept, float sim, float t, float band) {
+    n.c[0] += source && kept;
+    n.c[1] += source && !kept;
+    n.c[2] += source && fabs((double)sim - (double)t) < (double)band;
+}
+// sums over the CTA, to threads 0 .. 2 (count i in thread i); s_part: [3][warps]
+template <int WARPS> __device__ __forceinline__ int counts_of_block(TokenCounts& n, int (&s_part)[3][WARPS]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) n.c[q] += __shfl_xor_sync(0xffffffffu, n.c[q], o);
+        if (lane == 0) s_part[q][w] = n.c[q];
+    }
+    __syncthreads();
+    int v = 0;
+    if (threadIdx.x < 3)
+        for (int ww = 0; ww < WARPS; ++ww) v += s_part[threadIdx.x][ww];
+    return v;
+}
+
+// Clips of up to kStatsWhole tokens: one cluster of eight CTAs, whose counts meet in the shared memory of rank 0.  (A grid
+// of independent CTAs needs its three words cleared first: a memset before the kernel, 5 us of 37 for the query and the
+// counts of a 48 x 14 x 14 clip of 2048 channels.)
+constexpr int kStatsCtas = 8, kStatsThreads = 512;
+constexpr long long kStatsWhole = 1 << 18;
+
+__global__ void __cluster_dims__(kStatsCtas, 1, 1) __launch_bounds__(kStatsThreads)
+k_stats_cluster(const float* sim, const unsigned char* keep, const int* anchor, int N, int total, float t, float band,
+                long long* out)
+{
+    __shared__ int s_part[3][kStatsThreads / 32];
+    __shared__ int s_in[kStatsCtas][3];
+    pdl_launch_dependents();
+    pdl_wait();                                  // (what the kernel before this one wrote is read with L2-coherent loads)
+    const int a0 = __ldcg(anchor) * N, a1 = a0 + N;
+    const int rank = (int)cluster_rank();
+    TokenCounts n = {{0, 0, 0}};
+    constexpr int kInFlight = 4, kStride = kStatsCtas * kStatsThreads;
+    for (int f0 = rank * kStatsThreads + (int)threadIdx.x; f0 < total; f0 += kInFlight * kStride) {
+        unsigned char kp[kInFlight];
+        float s[kInFlight];
+#pragma unroll
+        for (int u = 0; u < kInFlight; ++u) {
+            const int f = min(f0 + u * kStride, total - 1);
+            kp[u] = __ldcg(keep + f);
+            s[u] = __ldcg(sim + f);
+        }
+#pragma unroll
+        for (int u = 0; u < kInFlight; ++u) {
+            const int f = f0 + u * kStride;
+            count_token(n, f < total && (f < a0 || f >= a1), kp[u] != 0, s[u], t, band);
+        }
+    }
+    const int v = counts_of_block(n, s_part);
+    if (threadIdx.x < 3) st_cluster_u32(cluster_addr(smem_u32(&s_in[rank][threadIdx.x]), 0), (uint32_t)v);
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    if (rank == 0 && threadIdx.x < 3) {
+        long long sum = 0;
+#pragma unroll
+        for (int r = 0; r < kStatsCtas; ++r) sum += s_in[r][threadIdx.x];
+        out[threadIdx.x] = sum;
+    }
+}
+
 __global__ void __launch_bounds__(kXThreads)
 k_stats(const float* __restrict__ sim, const unsigned char* __restrict__ keep, const int* __restrict__ anchor, int N,
         long long total, float t, float band, unsigned long long* __restrict__ out)
 {
     __shared__ int s_part[3][kXThreads / 32];
     const int a = *anchor;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int c[3] = {0, 0, 0};
+    TokenCounts n = {{0, 0, 0}};
     const long long stride = (long long)gridDim.x * kXThreads;
-    for (long long f = (long long)blockIdx.x * kXThreads + threadIdx.x; f < total; f += stride) {
-        if (f / N == a) continue;
-        const bool kp = keep[f] != 0;
-        c[0] += kp ? 1 : 0;
-        c[1] += kp ? 0 : 1;
-        c[2] += fabs((double)sim[f] - (double)t) < (double)band ? 1 : 0;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(0xffffffffu, c[q], o);
-        if (lane == 0) s_part[q][w] = c[q];
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        unsigned long long v = 0;
-        for (int ww = 0; ww < kXThreads / 32; ++ww) v += (unsigned long long)s_part[threadIdx.x][ww];
-        if (v) atomicAdd(out + threadIdx.x, v);
-    }
+    for (long long f = (long long)blockIdx.x * kXThreads + threadIdx.x; f < total; f += stride)
+        count_token(n, f / N != a, keep[f] != 0, sim[f], t, band);
+    const int v = counts_of_block(n, s_part);
+    if (threadIdx.x < 3 && v) atomicAdd(out + threadIdx.x, (unsigned long long)v);
 }
 
 cudaError_t launch_stats(const float* sim, const unsigned char* keep, const int* anchor, int F, int N, float t, float band,
                          long long* out, cudaStream_t st) {
+    const long long total = (long long)F * N;
+    if (total <= kStatsWhole)
+        return launch_pdl(k_stats_cluster, dim3(kStatsCtas), dim3(kStatsThreads), st, sim, keep, anchor, N, (int)total, t, band,
+                          out);
     cudaError_t e = cudaMemsetAsync(out, 0, 3 * sizeof(long long), st);
     if (e != cudaSuccess) return e;
-    const long long total = (long long)F * N;
     long long blocks = (total + kXThreads - 1) / kXThreads;
     if (blocks > 2LL * sm_count()) blocks = 2LL * sm_count();
     k_stats<<<(unsigned)blocks, kXThreads, 0, st>>>(sim, keep, anchor, N, total, t, band,

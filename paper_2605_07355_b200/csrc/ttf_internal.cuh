@@ -53,6 +53,8 @@ struct Problem {
     int pos_base;       // added to all three coordinates of every emitted position
     int natural_order;  // 1: all retained tokens in ascending flat index (the anchor rows where they fall)
     int use_tc;         // 1: the matching step runs on tcgen05 (ttf_match_tc.cu)
+    int* fuse_cnt;      // [N] the query's counts of tokens fused into each anchor cell, or NULL: zeroed between the
+                        // sweep and the matching kernel, which counts (single clips only)
     int chain;          // 1: the kernel before this call's sweep in the stream is the gather of the library's previous
                         // clip, which works on another scratch block: the sweep may run beside it
     int chain_next;     // 1: the kernel after this call's gather is such a sweep
@@ -74,7 +76,6 @@ struct Scratch {
     float* shat;        // [F*N] best similarity (Eq. argmax)
     int* dst;           // [F*N] best anchor cell (Eq. dst)
     unsigned char* keep;// [F*N] retention mask (Eq. mask)
-    int* fuse_cnt;      // [N]   tokens fused into each anchor cell
     size_t bytes;       // total, multiple of 256
 };
 
@@ -126,8 +127,6 @@ cudaError_t launch_norm_sum(const Problem& p, const Scratch& s, cudaStream_t st)
 cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anchor, cudaStream_t st);
 cudaError_t launch_match(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                          unsigned char* keep, cudaStream_t st);
-cudaError_t launch_fuse_count(const Problem& p, const Scratch& s, const int* dst, const unsigned char* keep,
-                              int* fuse_cnt, cudaStream_t st);
 cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& out, cudaStream_t st);
 
 cudaError_t launch_restore(const void* comp, size_t row_bytes, int F, int N, const int* anchor,
@@ -239,6 +238,16 @@ __device__ __forceinline__ void trace_mark(int*, int, bool) {}
 __device__ __forceinline__ unsigned long long trace_now() { return 0; }
 __device__ __forceinline__ void trace_acc(int*, int, unsigned long long) {}
 #endif
+
+// The gate of one source token (Eq. gating): a token is fused only when its best similarity exceeds t strictly, a NaN keeps
+// it.  Integer counts: order-independent.
+__device__ __forceinline__ void gate_token(float best, int best_j, float t, size_t f, float* shat, int* dst,
+                                           unsigned char* keep, int* cnt_k, int* fuse_cnt) {
+    const bool kp = !(best > t);
+    shat[f] = best; dst[f] = best_j; keep[f] = kp ? 1 : 0;
+    if (kp) atomicAdd(cnt_k, 1);
+    else if (fuse_cnt) atomicAdd(fuse_cnt + best_j, 1);
+}
 
 // Checked build (-DTTF_DEBUG): every global store whose index a kernel computes is guarded by in_bounds().  An
 // index outside [0, limit) raises the status word of the call's scratch to 2, leaves (site, index, limit) of the first

@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(kMatchWarps * 32)
 k_match_generic(const __grid_constant__ ClipPtrs xs, int F, int H, int W, int C, int r, float t, int fchunk, int nslice,
                 AnchorSrc asrc, const float* __restrict__ ssq,
                 float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep,
-                int* __restrict__ cnt, size_t sstride)
+                int* __restrict__ cnt, size_t sstride, int* fuse_cnt)
 {
     const T* __restrict__ X = reinterpret_cast<const T*>(xs.X[blockIdx.y]);
     asrc = clip_block(asrc, sstride); ssq = clip_block(ssq, sstride); cnt = clip_block(cnt, sstride);
@@ -83,9 +83,7 @@ k_match_generic(const __grid_constant__ ClipPtrs xs, int F, int H, int W, int C,
             }
         }
         if (lane == 0 && in_bounds(asrc.hdr, 2, (long long)f, (long long)FN)) {
-            const unsigned char kp = !(best > t);
-            shat[f] = best; dst[f] = best_j; keep[f] = kp;
-            if (kp) atomicAdd(&cnt[k], 1);   // integer count: order-independent
+            gate_token(best, best_j, t, f, shat, dst, keep, cnt + k, fuse_cnt);
         }
     }
 }
@@ -97,7 +95,7 @@ __device__ __forceinline__ void match_mma_body(const bf16_t* __restrict__ X, int
                                                const AnchorSrc& asrc, const float* ssq, int nslice,
                                                float* __restrict__ shat, int* __restrict__ dst,
                                                unsigned char* __restrict__ keep, int* __restrict__ cnt,
-                                               int stream_once)
+                                               int stream_once, int* fuse_cnt)
 {
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     const int N = H * W;
@@ -123,7 +121,7 @@ __device__ __forceinline__ void match_mma_body(const bf16_t* __restrict__ X, int
         trace_mark(asrc.hdr, 4, true);
         return a;
     };
-    match_mma_unit<MT, NT, GRAM, ST>(X, F, H, W, C, r, t, anchor_fn, i, k0, ssq, nslice, shat, dst, keep, cnt, asrc.hdr, dyn_smem, stream_once);
+    match_mma_unit<MT, NT, GRAM, ST>(X, F, H, W, C, r, t, anchor_fn, i, k0, ssq, nslice, shat, dst, keep, cnt, asrc.hdr, dyn_smem, stream_once, fuse_cnt);
     trace_mark(asrc.hdr, 2, true);
 }
 
@@ -132,12 +130,12 @@ template <int MT, int NT>
 __global__ void TTF_MMA_BOUNDS
 k_match_mma(const __grid_constant__ ClipPtrs xs, int F, int H, int W, int C, int r, float t, AnchorSrc asrc,
             float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
-            int stream_once, size_t sstride)
+            int stream_once, size_t sstride, int* fuse_cnt)
 {
     match_mma_body<MT, NT, true, kMmaStagesDefault>(reinterpret_cast<const bf16_t*>(xs.X[blockIdx.y]), F, H, W, C, r, t,
                                                     clip_block(asrc, sstride), nullptr, 0, clip_block(shat, sstride),
                                                     clip_block(dst, sstride), clip_block(keep, sstride),
-                                                    clip_block(cnt, sstride), stream_once);
+                                                    clip_block(cnt, sstride), stream_once, fuse_cnt);
 }
 
 // r = 2: the 25 candidate rows of a cell are as much data as 25 source rows, so a CTA takes 64 frames per cell to
@@ -149,12 +147,12 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 2)
 k_match_mma_wide(const __grid_constant__ ClipPtrs xs, int F, int H, int W, int C, int r, float t, AnchorSrc asrc,
                  const float* __restrict__ ssq, int nslice,
                  float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
-                 size_t sstride)
+                 size_t sstride, int* fuse_cnt)
 {
     match_mma_body<kWideMT, 4, false, kWideStages>(reinterpret_cast<const bf16_t*>(xs.X[blockIdx.y]), F, H, W, C, r, t,
                                                    clip_block(asrc, sstride), clip_block(ssq, sstride), nslice,
                                                    clip_block(shat, sstride), clip_block(dst, sstride),
-                                                   clip_block(keep, sstride), clip_block(cnt, sstride), 0);
+                                                   clip_block(keep, sstride), clip_block(cnt, sstride), 0, fuse_cnt);
 }
 
 template <int MT, int NT>
@@ -166,7 +164,8 @@ static cudaError_t launch_mma_t(const Problem& p, const Scratch& s, int* out_anc
     if (e != cudaSuccess) return e;
     return launch_ex(true, smem, k_match_mma<MT, NT>, dim3((unsigned)(chunks * p.N), p.nclips),
                      dim3(kMmaWarps * 32), st, p.xs, p.F, p.H, p.W, p.C, p.r, p.t,
-                     make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, p.stream_once, p.sstride);
+                     make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, p.stream_once, p.sstride,
+                     p.fuse_cnt);
 }
 
 static cudaError_t launch_mma_wide(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
@@ -177,7 +176,7 @@ static cudaError_t launch_mma_wide(const Problem& p, const Scratch& s, int* out_
     const long long chunks = (p.F + 16 * kWideMT - 1) / (16 * kWideMT);
     return launch_ex(true, smem, k_match_mma_wide, dim3((unsigned)(chunks * p.N), p.nclips), dim3(kMmaWarps * 32),
                      st, p.xs, p.F, p.H, p.W, p.C, p.r, p.t,
-                     make_anchor_src(p, s, out_anchor), (const float*)s.ssq, p.nslice, shat, dst, keep, s.cnt, p.sstride);
+                     make_anchor_src(p, s, out_anchor), (const float*)s.ssq, p.nslice, shat, dst, keep, s.cnt, p.sstride, p.fuse_cnt);
 }
 
 template <typename T, int V>
@@ -194,7 +193,7 @@ static cudaError_t launch_generic_t(const Problem& p, const Scratch& s, int* out
     const long long nchunk = (p.F + fchunk - 1) / fchunk;
     return launch_pdl(k_match_generic<T, V>, dim3((unsigned)(nchunk * p.N), p.nclips), dim3(kMatchWarps * 32), st,
                       p.xs, p.F, p.H, p.W, p.C, p.r, p.t, fchunk, p.nslice,
-                      make_anchor_src(p, s, out_anchor), (const float*)s.ssq, shat, dst, keep, s.cnt, p.sstride);
+                      make_anchor_src(p, s, out_anchor), (const float*)s.ssq, shat, dst, keep, s.cnt, p.sstride, p.fuse_cnt);
 }
 
 cudaError_t launch_match(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,

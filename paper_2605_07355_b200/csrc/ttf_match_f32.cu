@@ -56,7 +56,7 @@ template <int R, int G>
 __global__ void __launch_bounds__(F32Shape<R>::MAXW * 32)
 k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc,
             float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
-            int wait_limit, int tx_extra, size_t sstride)
+            int wait_limit, int tx_extra, size_t sstride, int* fuse_cnt)
 {
     const CUtensorMap& mapA = maps.a[blockIdx.y];
     const CUtensorMap& mapB = maps.b[blockIdx.y];
@@ -184,9 +184,7 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
                 const float sim = sum[lane * S::WIN + c] * rs * sum[S::FW * S::WIN + S::FW + c];
                 if (sim > best || best_j < 0) { best = sim; best_j = yy * W + xx; }
             }
-            const unsigned char kp = !(best > t);
-            shat[f] = best; dst[f] = best_j; keep[f] = kp;
-            if (kp) atomicAdd(&cnt[k], 1);
+            gate_token(best, best_j, t, f, shat, dst, keep, cnt + k, fuse_cnt);
         }
     }
     trace_mark(asrc.hdr, 2, true);
@@ -211,7 +209,7 @@ static cudaError_t launch_f32_t(const Problem& p, const Scratch& s, int* out_anc
     const long long units = (long long)p.N * ((p.F + FR - 1) / FR);
     return launch_ex(true, smem, k_match_f32<R, G>, dim3((unsigned)units, p.nclips), dim3(FR / S::FW * 32), st, maps, p.F, p.H,
                      p.W, p.C, p.t, make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, wait_poll_limit(),
-                     wait_tx_extra(), p.sstride);
+                     wait_tx_extra(), p.sstride, p.fuse_cnt);
 }
 
 cudaError_t launch_match_f32(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,

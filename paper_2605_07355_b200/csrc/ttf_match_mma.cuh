@@ -135,7 +135,7 @@ __device__ __forceinline__ void match_mma_unit(const bf16_t* __restrict__ X, int
                                                AnchorFn anchor_fn, int i, int k0, const float* ssq, int nslice,
                                                float* __restrict__ shat, int* __restrict__ dst,
                                                unsigned char* __restrict__ keep, int* __restrict__ cnt,
-                                               int* hdr, unsigned char* dyn_smem, int stream_once)
+                                               int* hdr, unsigned char* dyn_smem, int stream_once, int* fuse_cnt)
 {
     constexpr int kMmaStages = ST;
     constexpr int FR = 16 * MT;      // frames per CTA
@@ -298,9 +298,7 @@ __device__ __forceinline__ void match_mma_unit(const bf16_t* __restrict__ X, int
                     const float s = s_dot[tid][c] * rs * s_ra[c];
                     if (s > best || best_j < 0) { best = s; best_j = j; }
                 }
-                const unsigned char kp = !(best > t);
-                shat[f] = best; dst[f] = best_j; keep[f] = kp;
-                if (kp) atomicAdd(&cnt[k], 1);
+                gate_token(best, best_j, t, f, shat, dst, keep, cnt + k, fuse_cnt);
             }
         }
     }

@@ -36,6 +36,7 @@
 
 #include "ttf_internal.cuh"
 #include "ttf_async.cuh"
+#include "ttf_cluster.cuh"
 #include "ttf_tensormap.cuh"
 
 #include <map>
@@ -134,23 +135,6 @@ template <int R> struct TcShape {
     static constexpr int NORMBYTES = MAXCH * (kTcM + NP) * 4;
 };
 
-// ---- thread-block clusters: the CTAs of one tile exchange their partial sums through distributed shared memory
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// all threads of all CTAs of the cluster; writes before an arrival are visible to every CTA of the cluster after the wait
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t local_smem_addr, uint32_t rank) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_smem_addr), "r"(rank));
-    return remote;
-}
-__device__ __forceinline__ void st_cluster_f32(uint32_t remote, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
-}
 // m is all ones or zero: a or b without a branch.  (The window of a row starts at one of four columns; as conditional
 // expressions the choice became divergent branches, 1400 cycles per row at r = 1 against 110 for the loads from tensor
 // memory; 16 logic operations now.)
@@ -178,7 +162,7 @@ template <int R, int G>
 __global__ void __launch_bounds__(kTcThreads)
 k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc, int lpieces, int lchunks,
            float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
-           int wait_limit, int tx_extra, int stream_once, size_t sstride)
+           int wait_limit, int tx_extra, int stream_once, size_t sstride, int* fuse_cnt)
 {
     using S = TcShape<R>;
     const CUtensorMap& mapA = maps.a[blockIdx.y];
@@ -469,9 +453,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
                         best = take ? sim : best;
                         best_j = take ? yy * W + xx : best_j;
                     }
-                const unsigned char kp = !(best > t);
-                shat[f] = best; dst[f] = best_j; keep[f] = kp;
-                if (kp) atomicAdd(&cnt[k], 1);
+                gate_token(best, best_j, t, f, shat, dst, keep, cnt + k, fuse_cnt);
             }
         }
     }
@@ -575,7 +557,7 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
     }
     cfg.attrs = attr; cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, k_match_tc<R, G>, maps, p.F, p.H, p.W, p.C, p.t, make_anchor_src(p, s, out_anchor),
-                              log2_of(pieces), log2_of(chunks), shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride);
+                              log2_of(pieces), log2_of(chunks), shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride, p.fuse_cnt);
 }
 
 cudaError_t launch_match_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,

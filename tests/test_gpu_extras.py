@@ -138,3 +138,17 @@ def test_restore_one_and_two_launches(shape):
         keep, dst, a = q["keep"].cpu().numpy(), q["dst"].cpu().numpy(), int(q["anchor"])
         ref_full, ref_idx = O.restore(to_bits(toks[:int(cnt)]), keep, dst, F, N, a)
         assert (idx.cpu().numpy() == ref_idx).all() and (to_bits(full) == ref_full).all()
+
+
+@pytest.mark.parametrize("F,N", [(1, 1), (3, 5), (7, 585), (9, 4096), (256, 1024), (257, 1024)])
+def test_stats_over_sizes(F, N):
+    """one token, less than a block, one cluster up to its largest clip, the grid beyond it; anchor first, inside, last"""
+    rng = np.random.default_rng(F * N)
+    sim = rng.uniform(-1, 1, F * N).astype(np.float32)
+    sim[rng.random(F * N) < 0.01] = np.nan
+    keep = (rng.random(F * N) < 0.4).astype(np.uint8)
+    for a in sorted({0, F // 2, F - 1}):
+        got = P.ttf_stats(torch.from_numpy(sim).cuda(), torch.from_numpy(keep).cuda(),
+                          torch.tensor([a], dtype=torch.int32, device="cuda"), F, N, 1, 0.3, 0.05)
+        Pn, fused, in_band, _ = O.stats(sim, keep, F, N, a, 0.3, 0.05)
+        assert got.tolist() == [Pn, fused, in_band]
