@@ -1,9 +1,10 @@
 // Anchor Frame Selection (Eq. auto_anchor) and per-token norms: one streaming sweep over X plus a small
 // statistics kernel whose last CTA takes the arg max (resolve_anchor).
 //
-// k_norm_sum.  A CTA owns (frame k, channel slice q); a slice is LS = 32 lanes x one 16-byte load (512 bytes
-// of every token row; the CTAs of neighbouring slices run side by side, so DRAM sees whole rows).  The
-// 256 / LS row groups (warps) of a CTA walk the tokens of the frame interleaved, eight tokens per thread in
+// k_norm_sum.  A CTA owns (frame k, channel slice q); a slice is LS lanes x one 16-byte load (512 bytes
+// of every token row with LS = 32, less where a clip would make too few CTAs; the CTAs of neighbouring slices run side by
+// side, so DRAM sees whole rows).  The
+// 256 / LS row groups of a CTA walk the tokens of the frame interleaved, eight tokens per thread in
 // flight and the next eight prefetched.  A thread keeps running sums of its channels; the row groups are combined through
 // shared memory in a fixed order and give the frame sum S_k[slice] (= N x mean token of frame k) directly.
 // The squared norm of every token restricted to one warp's 32 lanes is reduced with a 9-shuffle fold and
@@ -60,7 +61,7 @@ __device__ __forceinline__ float fold8(float (&v)[8], int lane) {
     return r;
 }
 
-// LS: lanes across a slice (32 or 64); RG = 256 / LS row groups walk the tokens interleaved.
+// LS: lanes across a slice (4 to 32); RG = 256 / LS row groups walk the tokens interleaved.
 // NORMS: also store the per-token partial squared norms (only the CUDA-core matching kernel reads them).
 template <typename T, int V, int LS, bool NORMS>
 __global__ void __launch_bounds__(kNormThreads)
@@ -72,7 +73,6 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     S = clip_block(S, sstride); ssq = clip_block(ssq, sstride); cnt = clip_block(cnt, sstride); hdr = clip_block(hdr, sstride);
     using L = Loader<T, V>;
     constexpr int RG = kNormThreads / LS;
-    constexpr int WPS = LS / 32;                    // warps across a slice = norm planes per slice
     pdl_launch_dependents();
     // This kernel may be scheduled while the kernel before it in the stream still runs.  Normally that kernel may be
     // anything (the previous call's gather, which shares the scratch, or an upstream kernel that still writes X), so
@@ -87,14 +87,13 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     const int k = blockIdx.x / nq, q = blockIdx.x - k * nq;
     const int tid = threadIdx.x, lane = tid & 31;
     const int ls = tid & (LS - 1), rg = tid / LS;
-    const int wcol = ls >> 5;
     const size_t FN = (size_t)F * N;
     const int c0 = (q * LS + ls) * V;
     const bool active = c0 < C;                     // C is a multiple of V on the vector path
     const T* base = X + (size_t)k * N * C + c0;
-    float* plane = ssq + (size_t)(q * WPS + wcol) * FN + (size_t)k * N;
+    float* plane = ssq + (size_t)q * FN + (size_t)k * N;           // (NORMS: LS = 32, one plane per slice)
 
-    __shared__ float sm[RG][LS * V];
+    __shared__ float sm[kNormWarps][LS * V];
     float col[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) col[v] = 0.f;
@@ -140,14 +139,20 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     }
 
 #pragma unroll
-    for (int v = 0; v < V; ++v) sm[rg][ls * V + v] = col[v];
+    for (int o = LS; o < 32; o <<= 1)               // the row groups of a warp
+#pragma unroll
+        for (int v = 0; v < V; ++v) col[v] += __shfl_xor_sync(0xffffffffu, col[v], o);
+    if (lane < LS) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) sm[tid >> 5][ls * V + v] = col[v];
+    }
     __syncthreads();
     for (int idx = tid; idx < LS * V; idx += kNormThreads) {
         const int c = q * LS * V + idx;
         if (c < C) {
             float s = 0.f;
 #pragma unroll
-            for (int r2 = 0; r2 < RG; ++r2) s += sm[r2][idx];
+            for (int r2 = 0; r2 < kNormWarps; ++r2) s += sm[r2][idx];
             if (in_bounds(hdr, 1, (long long)k * C + c, (long long)F * C)) S[(size_t)k * C + c] = s;
         }
     }
@@ -157,15 +162,30 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     trace_mark(hdr, 0, true);
 }
 
+template <typename T, int V, int LS, bool NORMS>
+static cudaError_t launch_sum_ls(const Problem& p, const Scratch& s, cudaStream_t st) {
+    const int nq = (p.C + LS * V - 1) / (LS * V);
+    return launch_ex(true, 0, k_norm_sum<T, V, LS, NORMS>, dim3((unsigned)((long long)p.F * nq), p.nclips), dim3(kNormThreads),
+                     st, p.xs, p.F, p.N, p.C, nq, s.S, s.ssq, s.cnt, s.hdr, p.chain, p.sstride);
+}
+
 template <typename T, int V>
 static cudaError_t launch_sum_t(const Problem& p, const Scratch& s, cudaStream_t st) {
-    const unsigned blocks = (unsigned)((long long)p.F * p.nq);
-    const dim3 g(blocks, p.nclips), b(kNormThreads);
-    if (!needs_sweep_norms(p))
-        return launch_ex(true, 0, k_norm_sum<T, V, 32, false>, g, b, st, p.xs, p.F, p.N, p.C, p.nq, s.S,
-                         s.ssq, s.cnt, s.hdr, p.chain, p.sstride);
-    return launch_ex(true, 0, k_norm_sum<T, V, 32, true>, g, b, st, p.xs, p.F, p.N, p.C, p.nq, s.S, s.ssq,
-                     s.cnt, s.hdr, p.chain, p.sstride);
+    if (needs_sweep_norms(p)) return launch_sum_ls<T, V, 32, true>(p, s, st);
+    // Width of a slice: a warp across (512 bytes of a row), unless the launch then has fewer than two CTAs per SM: half or a
+    // quarter of a warp, with as many more rows in flight per warp.  Us per pass, 32 lanes / at most 16 / at most 8 / at most
+    // 4: 4 x 32 x 32 x 256 21.7 / 17.8 / 15.9 / 14.7, 4 x 32 x 32 x 1024 28.0 / 25.2 / 22.6 / 22.3, 8 x 24 x 24 x 2048
+    // 31.7 / 28.1 / 26.4 / 28.6, 32 x 16 x 16 x 1024 20.7 / 19.2 / 18.2 / 18.3, 16 x 8 x 8 x 512 12.2 / 12.5 / 12.3 / 12.8;
+    // with 512 CTAs as they are (32 x 16 x 16 x 4096) narrower slices gain nothing (37.9 / 38.2), and a batch of eight
+    // 24 x 20 x 20 x 1024 has enough of them together (86.4 against 89.9 with narrow slices).
+    if constexpr (V > 1) {
+        const long long rows = (long long)p.F * p.nclips, enough = 2LL * sm_count();
+        if (rows * p.nq < enough) {
+            if (rows * ((p.C + 16 * V - 1) / (16 * V)) >= enough) return launch_sum_ls<T, V, 16, false>(p, s, st);
+            return launch_sum_ls<T, V, 8, false>(p, s, st);
+        }
+    }
+    return launch_sum_ls<T, V, 32, false>(p, s, st);
 }
 
 // The query's counts of fused tokens start at zero for the matching kernel: cleared by the kernel between the sweep and it
