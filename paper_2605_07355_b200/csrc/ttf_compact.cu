@@ -180,7 +180,7 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
 // counts, after which the source row of any output row of the window is found by a binary search and a select in shared
 // memory: the three dependent round trips (anchor, counts, flags) are paid once per window instead of once per row.
 // Clips of up to kGatherWindow tokens need no survivor counts: the window is the whole clip.  Longer ones enter the walk
-// at the frame that holds the CTA's first row and take as many windows as its range needs.
+// at the frame that holds the CTA's first row and take as many windows, of a size that suits the range, as it needs.
 //
 // A warp moves a batch of consecutive output rows at a time, through two slots in turn, so that the next batch is on its
 // way while this one lands: every lane issues the load of one row, and the batch leaves as one store, since the rows are
@@ -210,12 +210,15 @@ __device__ __forceinline__ int select_bit(unsigned bits, int n) {
     return at;
 }
 
+// WHOLE: the clip is one window.  Else the windows are `words` * 32 tokens.
+template <bool WHOLE>
 __global__ void __launch_bounds__(kGatherThreads)
 k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H, int W,
                int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
                const unsigned char* __restrict__ keep, const __grid_constant__ OutPtrs outs, int NA, int acnt, int t_off,
-               int pos_base, int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride)
+               int pos_base, int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride, int window_words)
 {
+    const int words = WHOLE ? kGatherWords : window_words;
     const unsigned char* __restrict__ X = reinterpret_cast<const unsigned char*>(xs.X[blockIdx.y]);
     unsigned char* __restrict__ out_tokens = reinterpret_cast<unsigned char*>(outs.tokens[blockIdx.y]);
     int* __restrict__ out_pos = outs.pos[blockIdx.y];
@@ -228,6 +231,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
     __shared__ unsigned s_bits[kGatherWords];
     __shared__ int s_pref[kGatherWords];
     __shared__ int s_warp[kCopyWarps];
+    __shared__ int s_frames[WHOLE ? 1 : kWarpPrefixMaxF + 4];
     const int N = H * W, FN = F * N;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     if (!late_trigger) pdl_launch_dependents();  // (see k_compact_bulk)
@@ -237,7 +241,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
     if (late_trigger) pdl_launch_dependents();
     trace_mark(hdr, 6, false);
 
-    // ---- window of the walk: bits and prefix of tokens [T0, T0 + kGatherWindow) ----------------------------------
+    // ---- window of the walk: bits and prefix of tokens [T0, T0 + 32 words) ------------------------------------------
     constexpr int WPT = kGatherWords / kGatherThreads;          // consecutive words per thread
     static_assert(kGatherWords % kGatherThreads == 0, "whole words per thread");
     const int a = __ldcg(hdr + HDR_ANCHOR);
@@ -250,7 +254,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
             for (int h = 0; h < 2; ++h) {
                 // (the flag array is 256-byte aligned and followed by other scratch: a load that starts inside it may
                 // run past its end by less than 16 bytes, which the masks below discard)
-                v[u][h] = (unsigned)(f + h * 16) < (unsigned)FN ? __ldcg(reinterpret_cast<const uint4*>(keep + f) + h)
+                v[u][h] = (WHOLE || tid * WPT < words) && (unsigned)(f + h * 16) < (unsigned)FN ? __ldcg(reinterpret_cast<const uint4*>(keep + f) + h)
                                                                 : make_uint4(0, 0, 0, 0);
             }
         }
@@ -263,7 +267,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
             const unsigned anchor = below((a + 1) * N - f) & ~below(a * N - f);
             b[u] = pack_flags(v[u][0], v[u][1]);
             b[u] = acnt ? b[u] | anchor : b[u] & ~anchor;       // the anchor frame: all of its tokens, or none
-            b[u] &= f < 0 ? 0u : below(FN - f) & ~below(first - f);          // (f < 0: past 2^31, hence past the end)
+            b[u] &= f < 0 || (!WHOLE && tid * WPT >= words) ? 0u : below(FN - f) & ~below(first - f);          // (f < 0: past 2^31, hence past the end)
             mine += __popc(b[u]);
         }
         int incl = mine;
@@ -280,8 +284,10 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
         for (int ww = 0; ww < kCopyWarps; ++ww) { if (ww < w) at += s_warp[ww]; total += s_warp[ww]; }
 #pragma unroll
         for (int u = 0; u < WPT; ++u) {
-            s_bits[tid * WPT + u] = b[u];
-            s_pref[tid * WPT + u] = at;
+            if (WHOLE || tid * WPT < words) {
+                s_bits[tid * WPT + u] = b[u];
+                s_pref[tid * WPT + u] = at;
+            }
             at += __popc(b[u]);
         }
         __syncthreads();
@@ -289,10 +295,10 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
     };
 
     // ---- this CTA's rows [j0, j1) of the output ------------------------------------------------------------------
-    const bool whole = FN <= kGatherWindow;
+    const bool in_smem = F <= kWarpPrefixMaxF;   // (else the pre-scanned array)
     int k, before = 0, P, T0 = 0, in_window = 0;
-    if (whole) P = in_window = load_window(0, 0);
-    else { P = find_frame(cnt, gprefix, F, a, acnt, lane, -1, k, before); before = 0; }
+    if (WHOLE) P = in_window = load_window(0, 0);      // (no survivor counts needed)
+    else P = in_smem ? frame_prefix_cta(cnt, F, a, acnt, s_frames, s_warp) : __ldcg(gprefix + F);
     const int Lp = NA + P;                       // L' = N + P (Eq. Lpre)
     if (blockIdx.x == 0 && tid == 0) *reinterpret_cast<volatile int*>(out_count) = Lp;
     const int per = (Lp + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -311,7 +317,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
         const int n = j - NA - before;           // the n-th token of the window: word by binary search, then the bit
         int lo = 0;
 #pragma unroll
-        for (int h = kGatherWords / 2; h > 0; h >>= 1) if (s_pref[lo + h] <= n) lo += h;
+        for (int h = kGatherWords / 2; h > 0; h >>= 1) if ((WHOLE || h < words) && s_pref[lo + h] <= n) lo += h;
         return T0 + lo * 32 + select_bit(s_bits[lo], n - s_pref[lo]);
     };
     // lanes 0 .. n-1 issue the loads of output rows jb .. jb + n - 1 into slot h and write their positions
@@ -362,13 +368,14 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
         }
     };
 
-    if (whole) move_rows(j0, j1);
+    if (WHOLE) move_rows(j0, j1);
     else {
         move_rows(j0, min(j1, NA));
         int e = max(j0, NA) - NA;                // next token of the walk this CTA emits
         const int e1 = j1 - NA;
         if (e < e1) {                            // (e, e1 and the counts are the same for all threads)
-            find_frame(cnt, gprefix, F, a, acnt, lane, e, k, before);
+            if (in_smem) { k = frame_of(s_frames, F, e); before = s_frames[k]; }
+            else find_frame(cnt, gprefix, F, a, acnt, lane, e, k, before);
             T0 = (k * N) & ~31;
             in_window = load_window(T0, k * N);
         }
@@ -376,9 +383,9 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
             const int upto = min(e1, before + in_window);
             move_rows(NA + e, NA + upto);
             e = upto;
-            if (e >= e1 || T0 >= FN - kGatherWindow) break;      // (the second cannot happen when the counts match the flags)
+            if (e >= e1 || T0 >= FN - words * 32) break;      // (the second cannot happen when the counts match the flags)
             before += in_window;
-            T0 += kGatherWindow;
+            T0 += words * 32;
             in_window = load_window(T0, 0);
         }
     }
@@ -494,15 +501,25 @@ cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& ou
     // 23.2 / 21.7.  Longer rows keep every warp's slot full by themselves.
     if (vec && (row_bytes <= kGatherSlot / 2 || (row_bytes <= kGatherSlot && (long long)p.F * p.N <= kGatherWindow))) {
         constexpr size_t smem = (size_t)kCopyWarps * 2 * kGatherSlot;
-        cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_compact_rows), smem);
-        if (e != cudaSuccess) return e;
         long long most = 3LL * sm_count() / p.nclips;
         if (most < 1) most = 1;
         if (grid > most) grid = (int)most;
-        return launch_ex(pdl, smem, k_compact_rows, dim3(grid, p.nclips), b, st, p.xs, (int)row_bytes, p.F, p.H, p.W, s.hdr,
-                         (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt,
-                         p.pos_t_offset, p.pos_base, p.chain_next, wait_poll_limit(), wait_tx_extra(), p.stream_once,
-                         p.sstride);
+        // Clips beyond one window: windows of sixteen times the tokens that fall to a CTA (a window that holds too few rows
+        // costs another round trip), at least 512.  (Against windows of 16384 tokens and a count prefix per warp, us per pass:
+        // 64 x 24 x 24 x 512 32.3 -> 30.6, 64 x 32 x 32 x 1024 76.8 -> 75.2, 128 x 32 x 32 x 64 31.8 -> 29.8.  Clips of one
+        // window are better off without the counts: 32 x 16 x 16 x 2048 27.0 against 28.0.)
+        const long long FN = (long long)p.F * p.N;
+        int words = 16;
+        while (words < kGatherWords && words * 32LL < 16 * FN / grid) words *= 2;
+        auto launch = [&](auto kernel) {
+            cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+            if (e != cudaSuccess) return e;
+            return launch_ex(pdl, smem, kernel, dim3(grid, p.nclips), b, st, p.xs, (int)row_bytes, p.F, p.H, p.W, s.hdr,
+                             (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt,
+                             p.pos_t_offset, p.pos_base, p.chain_next, wait_poll_limit(), wait_tx_extra(), p.stream_once,
+                             p.sstride, words);
+        };
+        return FN <= kGatherWindow ? launch(k_compact_rows<true>) : launch(k_compact_rows<false>);
     }
     const dim3 g(grid, p.nclips);
     if (vec) {

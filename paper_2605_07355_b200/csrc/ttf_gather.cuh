@@ -8,6 +8,54 @@ namespace ttf {
 constexpr int kCopyWarps = 8;
 constexpr int kScanChunks = 4;       // frame counts per lane fetched at once by the warp-level frame search
 
+// Exclusive prefix of the survivor counts of all frames in shared memory, for clips of up to kWarpPrefixMaxF frames
+// (`pref`: [kWarpPrefixMaxF + 4]; pref[F] is the total, which is returned).  The anchor frame counts `acnt` tokens.  By all
+// threads of a CTA of 256.  (Not for the gather with one row per warp at a time: its warps do better without a barrier
+// before their first copy, 37.8 against 38.7 us per pass on 32 x 16 x 16 x 4096, 247 against 255 on 64 x 32 x 32 x 4096.)
+__device__ __forceinline__ int frame_prefix_cta(const int* cnt, int F, int a, int acnt, int* pref, int* s_warp) {
+    static_assert(kWarpPrefixMaxF == 4 * kCopyWarps * 32, "four frames per thread");
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, k = tid * 4;
+    // (the counts are 256-byte aligned and followed by other scratch: a load that starts inside may run past their end)
+    int4 v = k < F ? __ldcg(reinterpret_cast<const int4*>(cnt + k)) : make_int4(0, 0, 0, 0);
+    int c[4] = {v.x, v.y, v.z, v.w};
+    int mine = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        c[e] = k + e >= F ? 0 : (k + e == a ? acnt : c[e]);
+        mine += c[e];
+    }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += n;
+    }
+    if (lane == 31) s_warp[w] = incl;
+    __syncthreads();
+    int at = incl - mine, total = 0;
+#pragma unroll
+    for (int ww = 0; ww < kCopyWarps; ++ww) { at += ww < w ? s_warp[ww] : 0; total += s_warp[ww]; }
+    if (k <= F) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { pref[k + e] = at; at += c[e]; }
+    }
+    if (F == kWarpPrefixMaxF && tid == 0) pref[F] = total;
+    __syncthreads();
+    return total;
+}
+
+// Frame that holds the e-th token of the walk (e < pref[F]).
+__device__ __forceinline__ int frame_of(const int* pref, int F, int e) {
+    int lo = 0, hi = F;                              // pref[lo] <= e < pref[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        const bool up = pref[mid] <= e;
+        lo = up ? mid : lo;
+        hi = up ? hi : mid;
+    }
+    return lo;
+}
+
 // Frame search of the gather: the frame that holds the e-th token of the flat walk and the number of walked tokens
 // before that frame.  The walk visits the preserved tokens of the source frames in flat order; the anchor frame
 // contributes `acnt` tokens: 0 when its rows are emitted as a block of their own (Eq. xprime_stack), N in natural
