@@ -564,7 +564,7 @@ def main():
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": max(3, args.warmup), "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": spec.dtype, "accumulate": "f32", "data": "synthetic",
-            "config": workload_config(spec, t, nclips, f"{lanes} (library: ttf_compress_batch)" if args.streams == 0 else nstreams,
+            "config": workload_config(spec, t, nclips, f"{lanes if args.lanes else '2 groups of clips'} (library: ttf_compress_batch)" if args.streams == 0 else nstreams,
                                       tokens_step, args.anchor, use_graph, args.match_kernel),
             "step_ms": step_ms,
             "clips_per_s": clips_per_s, "rho": rho, "count_mean": avg_count,
