@@ -685,7 +685,13 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
             out.tokens[i] = out_tokens[n0 + i]; out.count[i] = out_count[n0 + i]; out.pos[i] = out_pos_thw[n0 + i];
         }
         p.overlapped = lanes;
-        p.stream_once = plan.pipelined ? 1 : 0;
+        // When the sweep of a group is done, L2 holds the last clip or two of it: the matching kernel starts with those, and it
+        // and the gather mark what they have read (and the gather what it writes) as the first to go.  16 clips of
+        // 32 x 16 x 16 x 4096 447.0 -> 444.4 us, 4 of them 127.0 -> 123.8, 16 of 32 x 16 x 16 x 2048 238.8 -> 236.3, 8 of
+        // 24 x 20 x 20 x 1024 86.8 -> 85.3.  Not for clips that are larger than L2 by themselves (8 of 268 MB: 880 -> 884),
+        // nor without a sweep (184.1 -> 184.6) or on the fp32 kernel, which has no hints (167.0 -> 167.3).
+        const bool fits_l2 = (double)p.F * p.N * p.C * 2 < 128.0 * (1 << 20);
+        p.stream_once = plan.pipelined || (p.nclips > 1 && fits_l2 && p.use_tc && p.anchor_mode == 0) ? 1 : 0;
         p.chain = turn > 0 ? 1 : 0;              // the lane's previous kernel is the gather of its previous group
         if (turn < 2) {
             // the blocks may hold anything (another shape's data, or a failed call's counters): clear their control words

@@ -59,8 +59,9 @@ struct Problem {
                         // clip, which works on another scratch block: the sweep may run beside it
     int chain_next;     // 1: the kernel after this call's gather is such a sweep
     int overlapped;     // clips whose kernels run beside one another: the lanes of a batch (0 or 1: this call runs alone)
-    int stream_once;    // 1: the matching kernel marks the lines of the source rows it reads as the first to leave L2
-                        // (the pipelined schedule: the next clip streams into L2 while this one is matched)
+    int stream_once;    // 1: the matching kernel marks the lines of the source rows it reads as the first to leave L2, and the
+                        // gather its lines (the pipelined schedule: the next clip streams into L2 while this one is matched;
+                        // a group: the clips that the sweep left in L2 are matched first, backwards)
 };
 
 // Device pointers carved out of one scratch allocation.
@@ -270,14 +271,16 @@ __device__ __forceinline__ bool in_bounds(int*, int, long long, long long) { ret
 #endif
 
 // this CTA's clip: `p` points into the scratch block of the first clip of the launch
-template <typename T> __device__ __forceinline__ T* clip_block(T* p, size_t sstride) {
-    return reinterpret_cast<T*>(reinterpret_cast<uintptr_t>(p) + (size_t)blockIdx.y * sstride);
+template <typename T> __device__ __forceinline__ T* clip_block(T* p, size_t sstride, unsigned clip) {
+    return reinterpret_cast<T*>(reinterpret_cast<uintptr_t>(p) + (size_t)clip * sstride);
 }
-__device__ __forceinline__ AnchorSrc clip_block(AnchorSrc a, size_t sstride) {
-    a.Dp = clip_block(a.Dp, sstride); a.Qp = clip_block(a.Qp, sstride); a.Gp = clip_block(a.Gp, sstride);
-    a.hdr = clip_block(a.hdr, sstride);
+template <typename T> __device__ __forceinline__ T* clip_block(T* p, size_t sstride) { return clip_block(p, sstride, blockIdx.y); }
+__device__ __forceinline__ AnchorSrc clip_block(AnchorSrc a, size_t sstride, unsigned clip) {
+    a.Dp = clip_block(a.Dp, sstride, clip); a.Qp = clip_block(a.Qp, sstride, clip); a.Gp = clip_block(a.Gp, sstride, clip);
+    a.hdr = clip_block(a.hdr, sstride, clip);
     return a;
 }
+__device__ __forceinline__ AnchorSrc clip_block(AnchorSrc a, size_t sstride) { return clip_block(a, sstride, blockIdx.y); }
 
 struct bf16_t { uint16_t bits; };   // storage type only: all arithmetic is on the widened fp32 value
 

@@ -165,10 +165,12 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
            int wait_limit, int tx_extra, int stream_once, size_t sstride, int* fuse_cnt)
 {
     using S = TcShape<R>;
-    const CUtensorMap& mapA = maps.a[blockIdx.y];
-    const CUtensorMap& mapB = maps.b[blockIdx.y];
-    asrc = clip_block(asrc, sstride); cnt = clip_block(cnt, sstride);
-    shat = clip_block(shat, sstride); dst = clip_block(dst, sstride); keep = clip_block(keep, sstride);
+    const bool backwards = gridDim.y == 1 || stream_once;
+    const unsigned clip = backwards ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+    const CUtensorMap& mapA = maps.a[clip];
+    const CUtensorMap& mapB = maps.b[clip];
+    asrc = clip_block(asrc, sstride, clip); cnt = clip_block(cnt, sstride, clip);
+    shat = clip_block(shat, sstride, clip); dst = clip_block(dst, sstride, clip); keep = clip_block(keep, sstride, clip);
     extern __shared__ unsigned char dyn_raw[];
     __shared__ uint64_t bar_full[S::STAGES], bar_empty[S::STAGES], bar_acc;
     __shared__ uint32_t s_tmem;
@@ -179,8 +181,8 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     const int xs_n = (W + kTcWB - 1) / kTcWB;
     // A launch over one clip walks its tiles backwards: the sweep has gone forwards, so what it read last is still in L2,
     // and the gather, which goes forwards again, finds what is matched last.  (64 x 16 x 16 x 4096: 81.9 -> 79.0 us per
-    // pass, 64 x 32 x 32 x 4096 with r = 2: 255.5 -> 252.1; over several clips it made no difference or 0.4 % worse.)
-    const unsigned walk = gridDim.y == 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    // pass, 64 x 32 x 32 x 4096 with r = 2: 255.5 -> 252.1.)  Over several clips it needs the L2 hints of stream_once as well.
+    const unsigned walk = backwards ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
     const int pieces = 1 << lpieces;
     const int tile = (int)(walk >> lpieces);
     const int piece = pieces > 1 ? (int)cluster_rank() : 0;        // = blockIdx.x % pieces
