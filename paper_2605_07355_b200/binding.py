@@ -185,6 +185,16 @@ def _stream_of(x: torch.Tensor, stream) -> int:
     return _current_raw_stream(x.get_device()) if stream is None else _stream_ptr(stream)
 
 
+def _check_operands(name: str, first: torch.Tensor, *others) -> None:
+    """The first tensor of an entry point without _check_features decides the device, so it must be on one; the others must
+    be memory a kernel can read (a NULL is the library's to refuse)."""
+    if not first.is_cuda:
+        raise ValueError(f"{name} must be a CUDA tensor, got one on {first.device}")
+    for t in others:
+        if t is not None and not t.is_cuda and not t.is_pinned():
+            raise ValueError(f"the arrays that go with {name} must be CUDA tensors, got one on {t.device}")
+
+
 def _addr(t: Optional[torch.Tensor]) -> int:
     return 0 if t is None else t.data_ptr()
 
@@ -443,6 +453,7 @@ def ttf_restore(compressed: torch.Tensor, F: int, H: int, W: int, anchor: torch.
     """ttf_restore: returns (out_full [F*H*W, ...row shape], row_index int32 [F*H*W])."""
     if not compressed.is_contiguous():
         raise ValueError("compressed must be contiguous")
+    _check_operands("compressed", compressed, anchor, keep, dst)
     there = _elsewhere(compressed)
     if there is not None:
         with there:
@@ -452,8 +463,8 @@ def ttf_restore(compressed: torch.Tensor, F: int, H: int, W: int, anchor: torch.
     row_bytes = compressed.numel() // compressed.shape[0] * compressed.element_size()
     out = compressed.new_empty((F * H * W,) + tuple(compressed.shape[1:]))
     idx = compressed.new_empty(F * H * W, dtype=torch.int32)
-    rc = (_fast or _marshal()).restore(compressed.data_ptr(), row_bytes, F, H, W, anchor.data_ptr(), keep.data_ptr(),
-                                       dst.data_ptr(), out.data_ptr(), idx.data_ptr(), _stream_of(compressed, stream))
+    rc = (_fast or _marshal()).restore(compressed.data_ptr(), row_bytes, F, H, W, _addr(anchor), _addr(keep),
+                                       _addr(dst), out.data_ptr(), idx.data_ptr(), _stream_of(compressed, stream))
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_restore")
     return out, idx
@@ -473,12 +484,13 @@ def ttf_sim_histogram(best_sim: torch.Tensor, anchor: torch.Tensor, F: int, H: i
 def ttf_stats(best_sim: torch.Tensor, keep: torch.Tensor, anchor: torch.Tensor, F: int, H: int, W: int, t: float,
               band: float = 1e-4, stream=None) -> torch.Tensor:
     """ttf_stats: int64 [3] on the device = (P preserved, fused, in-band source tokens).  Does not synchronise."""
+    _check_operands("best_sim", best_sim, keep, anchor)
     there = _elsewhere(best_sim)
     if there is not None:
         with there:
             return ttf_stats(best_sim, keep, anchor, F, H, W, t, band, stream)
     out = best_sim.new_empty(3, dtype=torch.int64)
-    rc = (_fast or _marshal()).stats(best_sim.data_ptr(), keep.data_ptr(), anchor.data_ptr(), F, H, W, float(t),
+    rc = (_fast or _marshal()).stats(best_sim.data_ptr(), _addr(keep), _addr(anchor), F, H, W, float(t),
                                      float(band), out.data_ptr(), _stream_of(best_sim, stream))
     if rc != TTF_OK:
         raise TTFError(rc, "ttf_stats")
