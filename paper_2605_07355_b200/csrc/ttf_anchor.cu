@@ -354,6 +354,7 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     __shared__ float s_best[kNormWarps];
     __shared__ int s_idx[kNormWarps];
     pdl_launch_dependents();
+    if (CS > 1) cluster_arrive();                    // this CTA runs: the others may write into it
     trace_mark(hdr, 1, false);
     pdl_wait();                                      // the sweep's frame sums are complete and visible
     trace_mark(hdr, 4, false);
@@ -439,6 +440,7 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     }
     __syncthreads();
     if (CS > 1) {
+        cluster_wait();                              // every CTA has started
         if (rank > 0) {                              // hand the shares to rank 0
             for (int i = tid; i < 2 * F + 1; i += kNormThreads)
                 st_cluster_f32(cluster_addr(smem_u32(&s_x[rank - 1][i]), 0),

@@ -264,6 +264,7 @@ k_stats_cluster(const float* sim, const unsigned char* keep, const int* anchor, 
     __shared__ int s_part[3][kStatsThreads / 32];
     __shared__ int s_in[kStatsCtas][3];
     pdl_launch_dependents();
+    cluster_arrive();                            // this CTA runs: the others may write into it
     pdl_wait();                                  // (what the kernel before this one wrote is read with L2-coherent loads)
     const int a0 = __ldcg(anchor) * N, a1 = a0 + N;
     const int rank = (int)cluster_rank();
@@ -285,6 +286,8 @@ k_stats_cluster(const float* sim, const unsigned char* keep, const int* anchor, 
         }
     }
     const int v = counts_of_block(n, s_part);
+    __syncwarp();
+    cluster_wait();                              // every CTA has started
     if (threadIdx.x < 3) st_cluster_u32(cluster_addr(smem_u32(&s_in[rank][threadIdx.x]), 0), (uint32_t)v);
     __syncwarp();
     cluster_arrive();
