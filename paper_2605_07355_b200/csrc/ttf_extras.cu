@@ -55,7 +55,7 @@ k_restore_index(const int* __restrict__ anchor, const unsigned char* __restrict_
     // preserved source tokens in the frames before this one (the anchor frame does not count)
     const size_t before = (size_t)k * N;
     int c = count_flags(keep, 0, before, tid);
-    if (a < k) c -= count_flags(keep, (size_t)a * N, (size_t)(a + 1) * N, tid);
+    if (a >= 0 && a < k) c -= count_flags(keep, (size_t)a * N, (size_t)(a + 1) * N, tid);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (lane == 0) s_warp[w] = c;
@@ -131,7 +131,10 @@ k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int*
     const int f0 = blockIdx.x * per, f1 = min(FN, f0 + per);
     pdl_launch_dependents();
     pdl_wait();                                  // the caller's kernels before this one
-    const int a = __ldcg(anchor), a0 = a * N, a1 = a0 + N;
+    // the anchor frame's tokens: [a0, a1), none of the clip's for an anchor outside it
+    const int a = __ldcg(anchor);
+    const bool inside = (unsigned)a < (unsigned)(FN / N);
+    const int a0 = inside ? a * N : FN, a1 = inside ? a0 + N : FN;
     // preserved source tokens before f0 (the anchor frame does not count)
     int c = count_flags(keep, 0, (size_t)min(f0, a0), tid);
     if (f0 > a1) c += count_flags(keep, (size_t)a1, (size_t)f0, tid);
@@ -266,7 +269,9 @@ k_stats_cluster(const float* sim, const unsigned char* keep, const int* anchor, 
     pdl_launch_dependents();
     cluster_arrive();                            // this CTA runs: the others may write into it
     pdl_wait();                                  // (what the kernel before this one wrote is read with L2-coherent loads)
-    const int a0 = __ldcg(anchor) * N, a1 = a0 + N;
+    const int a = __ldcg(anchor);                // (outside the clip: no token is the anchor frame's)
+    const bool inside = (unsigned)a < (unsigned)(total / N);
+    const int a0 = inside ? a * N : 0, a1 = inside ? a0 + N : 0;
     const int rank = (int)cluster_rank();
     TokenCounts n = {{0, 0, 0}};
     constexpr int kInFlight = 4, kStride = kStatsCtas * kStatsThreads;

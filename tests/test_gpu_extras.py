@@ -152,3 +152,23 @@ def test_stats_over_sizes(F, N):
                           torch.tensor([a], dtype=torch.int32, device="cuda"), F, N, 1, 0.3, 0.05)
         Pn, fused, in_band, _ = O.stats(sim, keep, F, N, a, 0.3, 0.05)
         assert got.tolist() == [Pn, fused, in_band]
+
+
+@pytest.mark.parametrize("shape", [(4, 8, 8), (65, 32, 32)])             # restore in one launch and in two
+@pytest.mark.parametrize("anchor", [-1, 65, 1 << 29, -(1 << 29)])
+def test_an_anchor_outside_the_clip_excludes_no_frame(shape, anchor):
+    """-1 and frames past the end: every kept token has a row of its own behind the N anchor rows, every token is counted"""
+    F, H, W = shape
+    N = H * W
+    rng = np.random.default_rng(7)
+    keep = (rng.random(F * N) < 0.4).astype(np.uint8)
+    dst = rng.integers(0, N, F * N, dtype=np.int32)
+    sim = rng.uniform(-1, 1, F * N).astype(np.float32)
+    comp = torch.arange(N + int(keep.sum()), dtype=torch.int32, device="cuda").view(-1, 1).repeat(1, 4)
+    dev = lambda x: torch.from_numpy(x).cuda()
+    a = torch.tensor([anchor], dtype=torch.int32, device="cuda")
+    full, idx = P.ttf_restore(comp, F, H, W, a, dev(keep), dev(dst))
+    ref = np.where(keep != 0, N + np.cumsum(keep) - keep, dst)
+    assert (idx.cpu().numpy() == ref).all() and (full[:, 0].cpu().numpy() == ref).all()
+    got = P.ttf_stats(dev(sim), dev(keep), a, F, H, W, 0.3, 0.05).tolist()
+    assert got == [int(keep.sum()), int(F * N - keep.sum()), int((np.abs(sim.astype(np.float64) - np.float64(np.float32(0.3))) < np.float64(np.float32(0.05))).sum())]
