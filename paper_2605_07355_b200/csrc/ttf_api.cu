@@ -165,6 +165,7 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
 struct CacheEntry {
     void* ptr = nullptr; size_t bytes = 0;
     std::vector<const int*> status_words;        // header blocks the most recent call on this stream used
+    int status_index = HDR_ERROR;                // ... and the word of each that tells how it went
 };
 static std::mutex g_mu;
 static std::map<std::pair<int, cudaStream_t>, CacheEntry> g_scratch;
@@ -193,6 +194,7 @@ static int cached_scratch(size_t bytes, cudaStream_t st, void** out) {
     }
     *out = ce.ptr;
     ce.status_words.assign(1, reinterpret_cast<const int*>(ce.ptr));
+    ce.status_index = HDR_ERROR;
     return TTF_OK;
 }
 
@@ -345,11 +347,11 @@ const char* ttf_status_string(int status) {
 
 int ttf_last_cuda_error(void) { return tl_cuda_error; }
 
-static int read_status_words(const std::vector<const int*>& words, int* host_status) {
+static int read_status_words(const std::vector<const int*>& words, int index, int* host_status) {
     *host_status = TTF_OK;
     for (const int* hdr : words) {
         int v = 0;
-        cudaError_t e = cudaMemcpy(&v, hdr + HDR_ERROR, sizeof(int), cudaMemcpyDeviceToHost);
+        cudaError_t e = cudaMemcpy(&v, hdr + index, sizeof(int), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(e);
         if (v == 2) *host_status = TTF_ERR_BOUNDS;                   // (checked build only)
         else if (v && *host_status == TTF_OK) *host_status = TTF_ERR_TIMEOUT;
@@ -366,12 +368,13 @@ int ttf_last_device_status(ttf_stream_t stream, int* host_status) {
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
     std::vector<const int*> words;
+    int index = HDR_ERROR;
     {
         std::lock_guard<std::mutex> lk(g_mu);
         auto it = g_scratch.find(std::make_pair(dev, st));
-        if (it != g_scratch.end()) words = it->second.status_words;
+        if (it != g_scratch.end()) { words = it->second.status_words; index = it->second.status_index; }
     }
-    return read_status_words(words, host_status);     // no call of the library on this stream yet: TTF_OK
+    return read_status_words(words, index, host_status);     // no call of the library on this stream yet: TTF_OK
 }
 
 int ttf_workspace_status(const void* workspace, ttf_stream_t stream, int* host_status) {
@@ -383,7 +386,7 @@ int ttf_workspace_status(const void* workspace, ttf_stream_t stream, int* host_s
         int rc = static_scratch_address(&ws);
         if (rc != TTF_OK) return rc;
     }
-    return read_status_words(std::vector<const int*>(1, reinterpret_cast<const int*>(ws)), host_status);
+    return read_status_words(std::vector<const int*>(1, reinterpret_cast<const int*>(ws)), HDR_ERROR, host_status);
 }
 
 #ifdef TTF_TRACE
@@ -729,7 +732,9 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         int dev = 0;
         if (cudaGetDevice(&dev) == cudaSuccess) {
             std::lock_guard<std::mutex> lk(g_mu);
-            g_scratch[std::make_pair(dev, st)].status_words = words;
+            CacheEntry& ce = g_scratch[std::make_pair(dev, st)];
+            ce.status_words = words;
+            ce.status_index = HDR_BATCH_ERROR;   // (groups that use the same blocks in turn clear the other word)
         }
     }
     // always join, also after a failed launch, so that the caller's stream (or capture) is whole again

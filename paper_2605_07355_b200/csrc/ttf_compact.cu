@@ -163,7 +163,7 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
         // warp that gave up raises the error word first and writes -1 afterwards.  Whichever order the two run in, -1
         // is what stays: either the -1 lands after L', or warp 0 sees the error word and writes -1 itself.
         if (gave_up) {
-            atomicExch(hdr + HDR_ERROR, 1);
+            report_give_up(hdr);
             __threadfence();
             *reinterpret_cast<volatile int*>(out_count) = -1;
         }
@@ -395,7 +395,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
             for (int h = 0; h < 2; ++h) mbar_wait(&bar[w][h], (phase >> h) & 1, wait_limit);
         bulk_wait<0>();                          // all rows of this warp are in global memory
         if (gave_up) {                           // L' or -1: see k_compact_bulk
-            atomicExch(hdr + HDR_ERROR, 1);
+            report_give_up(hdr);
             __threadfence();
             *reinterpret_cast<volatile int*>(out_count) = -1;
         }

@@ -19,6 +19,7 @@ enum { HDR_ANCHOR = 0,          // anchor frame a*
        HDR_DONE_ALL = 1,        // arrival counter of the statistics CTAs (zero between calls)
        HDR_ERROR = 2,           // 1: a bounded wait of this call gave up; 2: a checked build caught an index outside its
                                 // array (cleared by the first kernel of every call)
+       HDR_BATCH_ERROR = 3,     // the same, kept until the block is cleared: the clips of a batch that share a block report here
        HDR_CHECK_SLACK = 8,     // checked build: every limit is lowered by this much (test hook; zero otherwise)
        HDR_CHECK_SITE = 9,      // checked build: kernel site, index (clamped to 31 bits) and limit of the first index
        HDR_CHECK_INDEX = 10,    // that was out of range
@@ -250,6 +251,12 @@ __device__ __forceinline__ void gate_token(float best, int best_j, float t, size
     else if (fuse_cnt) atomicAdd(fuse_cnt + best_j, 1);
 }
 
+// a bounded wait of this call has run out
+__device__ __forceinline__ void report_give_up(int* hdr) {
+    atomicExch(hdr + HDR_ERROR, 1);
+    atomicExch(hdr + HDR_BATCH_ERROR, 1);
+}
+
 // Checked build (-DTTF_DEBUG): every global store whose index a kernel computes is guarded by in_bounds().  An
 // index outside [0, limit) raises the status word of the call's scratch to 2, leaves (site, index, limit) of the first
 // offender in the header, and the caller skips the access: nothing traps, the context stays usable, and the host
@@ -260,6 +267,7 @@ __device__ __forceinline__ bool in_bounds(int* hdr, int site, long long idx, lon
     limit -= __ldcg(hdr + HDR_CHECK_SLACK);
     if (idx >= 0 && idx < limit) return true;
     if (atomicCAS(hdr + HDR_ERROR, 0, 2) == 0) {
+        atomicExch(hdr + HDR_BATCH_ERROR, 2);
         hdr[HDR_CHECK_SITE] = site;
         hdr[HDR_CHECK_INDEX] = (int)(idx < 0 ? -1 : (idx > 0x7fffffffLL ? 0x7fffffffLL : idx));
         hdr[HDR_CHECK_LIMIT] = (int)(limit > 0x7fffffffLL ? 0x7fffffffLL : limit);

@@ -143,7 +143,7 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
         // copies still land in this CTA's shared memory: wait (bounded again) for the stages issued last
         for (int it = issued > S::STAGES ? issued - S::STAGES : 0; it < issued; ++it)
             mbar_wait(&bar[it % S::STAGES], (it / S::STAGES) & 1, wait_limit);
-        atomicExch(asrc.hdr + HDR_ERROR, 1);
+        report_give_up(asrc.hdr);
     }
     pdl_launch_dependents();                               // (not at the start: the gather's CTAs would take the place
                                                            // of other clips' kernels while this one runs)

@@ -468,7 +468,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
         tc_fence_after();
         tmem_dealloc(tmem, tmem_cols);
     }
-    if (tid == 0 && s_err) atomicExch(asrc.hdr + HDR_ERROR, 1);
+    if (tid == 0 && s_err) report_give_up(asrc.hdr);
 }
 
 // ---- host side: tensor maps and launch ------------------------------------------------------------------------

@@ -92,3 +92,34 @@ def test_status_of_caller_owned_and_built_in_scratch():
     P.ttf_query_static(Xd, 1, 0.7, out)
     assert P.ttf_workspace_status(None) == B.TTF_OK
     assert P.ttf_last_device_status(torch.cuda.Stream()) == B.TTF_OK      # a stream the library has never seen
+
+
+def test_a_batch_reports_a_clip_whose_scratch_block_a_later_clip_used():
+    """one lane, five clips on two scratch blocks in turn: the first gives up, the others, 2 bytes off a 16-byte boundary,
+    take the kernels without bounded waits and come out right"""
+    F, H, W, C = 4, 5, 5, 64
+    X = corr_clip(F, H, W, C, seed=81, dtype="bf16")
+    Xs = [to_device(X)]
+    for _ in range(4):
+        buf = torch.zeros(X.size + 8, dtype=torch.bfloat16, device="cuda")
+        Xs.append(buf[1:1 + X.size].view(F, H, W, C))
+        Xs[-1].copy_(Xs[0])
+    L = int(P.ttf_compress(Xs[0], 1, 0.7)[1])
+    st = torch.cuda.Stream()
+    P.ttf_set_schedule(1)
+    try:
+        P.ttf_compress_batch(Xs, 1, 0.7, stream=st)
+        assert P.ttf_last_device_status(st) == B.TTF_OK
+        P.ttf_debug_set_wait(32, 16)
+        try:
+            _, cnts, _ = P.ttf_compress_batch(Xs, 1, 0.7, stream=st)
+            assert P.ttf_last_device_status(st) == B.TTF_ERR_TIMEOUT
+            assert [int(c) for c in cnts] == [-1] + [L] * 4
+        finally:
+            P.ttf_debug_set_wait()
+        _, cnts, _ = P.ttf_compress_batch(Xs, 1, 0.7, stream=st)
+        assert P.ttf_last_device_status(st) == B.TTF_OK and [int(c) for c in cnts] == [L] * 5
+        P.ttf_compress(Xs[0], 1, 0.7, stream=st)
+        assert P.ttf_last_device_status(st) == B.TTF_OK
+    finally:
+        P.ttf_set_schedule(0)
