@@ -148,9 +148,12 @@ int ttf_compress(const void* features, int F, int H, int W, int C, int r, float 
  * that the library keeps per device; these fork from `stream` and join it again through events, so the call is
  * asynchronous, ordered on `stream` like any other, and can be captured in a CUDA graph.  The kernels of one group
  * leave part of the GPU idle while they ramp up and drain; the other lane's fill those gaps
- * (ttf_set_schedule asks for a number of single clips in flight instead).  Within a lane the groups form a chain on two
- * sets of scratch blocks used in turn: the sweep of a group runs beside the gather of the group before it.  The streams, their events and the scratch are created by
- * the first call on a device: make that call outside any stream capture.
+ * (ttf_set_schedule asks for a number of single clips in flight instead; a lane then chains its clips on two scratch
+ * blocks used in turn: the sweep of a clip runs beside the gather of the clip before it).  The streams, their events and
+ * the scratch are created by the first call on a device: make that call outside any stream capture.  The scratch (the
+ * blocks of 16 clips for 8 clips or more, of 32 for more than 16) grows with larger batches; a capture, which cannot
+ * allocate, and a device without memory left work in smaller groups on what there is.  Scratch that a graph was captured
+ * with stays valid until a larger clip arrives or ttf_release is called.
  */
 int ttf_compress_batch(const void* const* features, int nclips, int F, int H, int W, int C, int r, float t,
                        int dtype, void* const* out_tokens, int* const* out_count, int* const* out_pos_thw,

@@ -164,39 +164,59 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
 // ---- scratch cache: one block per (device, stream), grown on demand -------------------------------------
 struct CacheEntry {
     void* ptr = nullptr; size_t bytes = 0;
+    size_t unit = 0;                             // scratch of the largest clip seen on this stream
+    std::vector<void*> outgrown;                 // smaller blocks of the same clips, which captured graphs may still use
     std::vector<const int*> status_words;        // header blocks the most recent call on this stream used
     int status_index = HDR_ERROR;                // ... and the word of each that tells how it went
 };
 static std::mutex g_mu;
 static std::map<std::pair<int, cudaStream_t>, CacheEntry> g_scratch;
 
-static int cached_scratch(size_t bytes, cudaStream_t st, void** out) {
+// `bytes` of scratch for a call on `st`; `unit` is the scratch of one of its clips.  The block moves when a larger clip
+// arrives.  A block that is too small because the call has more clips than those before it is kept beside its successor:
+// a graph captured with fewer clips of the same shape points into it.  (Every successor is at least twice as large, so all
+// of them together stay below the current block; a larger clip or ttf_release gives them back.)
+static int cached_scratch(size_t bytes, size_t unit, cudaStream_t st, void** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
     std::lock_guard<std::mutex> lk(g_mu);
     CacheEntry& ce = g_scratch[std::make_pair(dev, st)];
     if (ce.bytes < bytes) {
-        if (ce.ptr) {
-            // earlier calls on this stream may still read the old block
+        if (ce.ptr && unit > ce.unit) {
+            // earlier calls on this stream may still read the old blocks
             e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) return cuda_fail(e);
             cudaFree(ce.ptr);
+            for (void* q : ce.outgrown) cudaFree(q);
             ce.ptr = nullptr; ce.bytes = 0;
+            ce.outgrown.clear();
             ce.status_words.clear();
         }
-        e = cudaMalloc(&ce.ptr, bytes);
-        if (e != cudaSuccess) { ce.ptr = nullptr; return cuda_fail(e); }
-        ce.bytes = bytes;
+        if (bytes < 2 * ce.bytes) bytes = 2 * ce.bytes;
+        void* fresh = nullptr;
+        e = cudaMalloc(&fresh, bytes);
+        if (e != cudaSuccess) return cuda_fail(e);
+        if (ce.ptr) ce.outgrown.push_back(ce.ptr);
+        ce.ptr = fresh; ce.bytes = bytes;
         // the arrival counters must start at zero; the kernels leave them at zero after every call
         e = cudaMemsetAsync(ce.ptr, 0, bytes, st);
         if (e != cudaSuccess) return cuda_fail(e);
     }
+    if (ce.unit < unit) ce.unit = unit;
     *out = ce.ptr;
     ce.status_words.assign(1, reinterpret_cast<const int*>(ce.ptr));
     ce.status_index = HDR_ERROR;
     return TTF_OK;
 }
+static size_t scratch_held(cudaStream_t st) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lk(g_mu);
+    auto it = g_scratch.find(std::make_pair(dev, st));
+    return it == g_scratch.end() ? 0 : it->second.bytes;
+}
+static int cached_scratch(size_t bytes, cudaStream_t st, void** out) { return cached_scratch(bytes, bytes, st, out); }
 
 static int check_ws(const Problem& p, void* ws, size_t ws_bytes, Scratch* s) {
     carve_scratch(p, nullptr, s);
@@ -608,8 +628,9 @@ static int batch_lanes(BatchLanes** out) {
     return TTF_OK;
 }
 
-// How a batch is cut into launches: `group` clips per launch, `lanes` groups in flight.
-struct BatchPlan { int group, lanes; bool pipelined; };
+// How a batch is cut into launches: `group` clips per launch, `lanes` groups in flight, `sets` of `group` scratch blocks
+// per lane, `blocks` of scratch blocks to hold per lane.
+struct BatchPlan { int group, lanes, sets, blocks; bool pipelined; };
 
 // Automatic: one launch of each kernel covers half of the batch (at most kMaxGroup clips), two halves in flight, so that
 // one half's kernels fill what the other's leave idle while they ramp up and drain.  Launches over single clips on
@@ -617,24 +638,28 @@ struct BatchPlan { int group, lanes; bool pipelined; };
 // 162 -> 98 us) and were no faster for large ones (33 MB: 16 clips 304 -> 300 us; 67 MB: 517 -> 515; 268 MB, 8 clips:
 // 910 -> 911).  All clips in one launch, or one lane, leave the second half's ramp and tail uncovered (33 MB: 306 and
 // 330 us); more than two lanes of smaller groups gain nothing (within 2 % for every clip size measured).
+// Scratch: 16 blocks in all for eight clips or more, 32 for more than 16; so few sizes that the lanes' scratch soon stays
+// as it is, whatever the number of clips.
 static BatchPlan plan_batch(const Problem& p, int nclips) {
     BatchPlan b;
     const int want = g_sched_lanes.load();
     b.pipelined = want == TTF_SCHEDULE_PIPELINED && nclips >= 3 && p.anchor_mode == 0;
-    b.group = 1;
+    b.group = 1; b.sets = b.blocks = 2;
     if (b.pipelined) { b.lanes = 2; return b; }
     if (want >= 1 && want <= kBatchStreams) b.lanes = want;          // ttf_set_schedule: so many single clips in flight
     else {
         b.group = (nclips + 1) / 2 < kMaxGroup ? (nclips + 1) / 2 : kMaxGroup;
         b.lanes = 2;
+        b.sets = b.blocks = 1;
+        while (b.blocks < (nclips >= 8 && b.group < 8 ? 8 : b.group)) b.blocks *= 2;
     }
     const int groups = (nclips + b.group - 1) / b.group;
     if (b.lanes > groups) b.lanes = groups;
     return b;
 }
 
-// The groups of a lane form a chain on the lane's stream: sweep, statistics, matching, gather, next sweep, ... with two
-// sets of scratch blocks used in turn, so that the sweep of a group can run beside the gather of the group before it.
+// A lane takes its groups one after the other on its stream.  Lanes of single clips (two sets of scratch blocks used in
+// turn) chain them: the sweep of a clip runs beside the gather of the clip before it.
 static int batch_on_streams(const void* const* features, int nclips, int F, int H, int W, int C, int r, float t,
                             int dtype, const ttf_options* options,
                             void* const* out_tokens, int* const* out_count, int* const* out_pos_thw, cudaStream_t st) {
@@ -658,16 +683,28 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         same_layout = same_layout && p.vec == p0.vec;
     }
     BatchPlan plan = plan_batch(p0, nclips);
-    if (!same_layout) plan.group = 1;
-    const int groups = (nclips + plan.group - 1) / plan.group;
-    const int lanes = groups < plan.lanes ? groups : plan.lanes;
-    const size_t set = (size_t)plan.group * stride;
-    std::vector<void*> ws(lanes, nullptr);
-    for (int i = 0; i < lanes; ++i) {            // (may allocate: before the fork, outside the event bracket)
-        rc = cached_scratch((groups > lanes ? 2 : 1) * set, L->s[i], &ws[i]);
-        if (rc != TTF_OK) return rc;
+    if (!same_layout) { plan.group = 1; plan.sets = plan.blocks = 2; }
+    // Scratch (before the fork, outside the event bracket).  Where it cannot grow, inside a capture or for lack of memory, the
+    // groups are as large as what the lanes hold allows.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &capture);
+    if (e != cudaSuccess) return cuda_fail(e);
+    std::vector<void*> ws(plan.lanes, nullptr);
+    for (int i = 0; i < plan.lanes; ++i) {
+        const size_t held = scratch_held(L->s[i]) / stride;
+        int blocks = plan.blocks;
+        if (capture != cudaStreamCaptureStatusNone && held >= (size_t)plan.sets && held < (size_t)blocks) blocks = (int)held;
+        while ((rc = cached_scratch(blocks * stride, stride, L->s[i], &ws[i])) != TTF_OK) {
+            if (blocks == plan.sets) return rc;
+            cudaGetLastError();
+            blocks = blocks / 2 > plan.sets ? blocks / 2 : plan.sets;
+        }
+        if (plan.group > blocks / plan.sets) plan.group = blocks / plan.sets;
     }
-    cudaError_t e = cudaEventRecord(L->fork, st);
+    const int groups = (nclips + plan.group - 1) / plan.group;
+    const int lanes = plan.lanes;
+    const size_t set = (size_t)plan.group * stride;
+    e = cudaEventRecord(L->fork, st);
     for (int i = 0; i < lanes && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(L->s[i], L->fork, 0);
     if (e != cudaSuccess) return cuda_fail(e);
     int first_rc = TTF_OK;
@@ -675,7 +712,7 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
     for (int q = 0; q < groups && first_rc == TTF_OK; ++q) {
         const int lane = q % lanes, turn = q / lanes;
         const int n0 = q * plan.group;
-        char* block = (char*)ws[lane] + (size_t)(turn & 1) * set;
+        char* block = (char*)ws[lane] + (size_t)(turn % plan.sets) * set;
         cudaStream_t ls = L->s[lane];
         Problem p;
         make_problem(features[n0], F, H, W, C, r, t, dtype, &p);
@@ -695,16 +732,16 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         // nor without a sweep (184.1 -> 184.6) or on the fp32 kernel, which has no hints (167.0 -> 167.3).
         const bool fits_l2 = (double)p.F * p.N * p.C * 2 < 128.0 * (1 << 20);
         p.stream_once = plan.pipelined || (p.nclips > 1 && fits_l2 && p.use_tc && p.anchor_mode == 0) ? 1 : 0;
-        p.chain = turn > 0 ? 1 : 0;              // the lane's previous kernel is the gather of its previous group
-        if (turn < 2) {
+        p.chain = plan.sets == 2 && turn > 0 ? 1 : 0;        // the lane's previous kernel is the gather of its previous clip
+        if (turn < plan.sets) {
             // the blocks may hold anything (another shape's data, or a failed call's counters): clear their control words
             first_rc = clear_control_blocks(block, stride, p.nclips, ls);
             for (int i = 0; i < p.nclips; ++i) words.push_back(reinterpret_cast<const int*>(block + i * stride));
             if (first_rc != TTF_OK) break;
             if (turn == 1) p.chain = 0;          // (the memset sits between the gather and this sweep)
         }
-        // (the lane's next group, if there is one, is at turn + 1; its sweep is chained from turn 2 on)
-        p.chain_next = (q + lanes < groups && turn + 1 >= 2) ? 1 : 0;
+        // (the lane's next clip, if there is one, is at turn + 1; its sweep is chained from turn 2 on)
+        p.chain_next = (plan.sets == 2 && q + lanes < groups && turn + 1 >= 2) ? 1 : 0;
         if (!plan.pipelined) {
             first_rc = compress_impl(p, block, out, ls);
             continue;
@@ -1051,7 +1088,7 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
     std::vector<OutPtrs> outs;
     size_t stride = 0;
     bool same_layout = true;
-    BatchPlan plan = {1, 1, false};
+    BatchPlan plan = {1, 1, 1, 1, false};
     for (int n = 0; n < nclips; ++n) {
         Problem p;
         int rc = make_problem(features[n], F, H, W, C, r, t, dtype, &p);
@@ -1146,6 +1183,7 @@ int ttf_release(void) {
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess && first == cudaSuccess) first = e;
         if (kv.second.ptr) cudaFree(kv.second.ptr);
+        for (void* q : kv.second.outgrown) cudaFree(q);
     }
     g_scratch.clear();
     for (auto& kv : g_staging) {

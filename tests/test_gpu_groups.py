@@ -37,3 +37,65 @@ def test_clips_of_different_alignment():
     outs = P.ttf_compress_batch(Xs, 1, 0.6)
     torch.cuda.synchronize()
     assert_same_as_single(Xs, 1, 0.6, outs)
+
+
+def outputs(X, n):
+    rows, C = X.shape[0] * X.shape[1] * X.shape[2], X.shape[3]
+    return ([torch.zeros((rows, C), dtype=X.dtype, device="cuda") for _ in range(n)],
+            [torch.zeros(1, dtype=torch.int32, device="cuda") for _ in range(n)],
+            [torch.zeros((rows, 3), dtype=torch.int32, device="cuda") for _ in range(n)])
+
+
+def captured(Xs, outs, st):
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        P.ttf_compress_batch(Xs, 1, 0.6, *outs, stream=st)
+    return g
+
+
+def assert_replays(g, Xs, outs):
+    for c in outs[1]:
+        c.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert_same_as_single(Xs, 1, 0.6, outs)
+
+
+def test_scratch_and_captures_after_eight_clips():
+    """batches of up to 16 clips take no more device memory than the one of eight, and a capture, which cannot allocate, takes
+    any number of clips"""
+    Xs = [to_device(corr_clip(16, 32, 32, 64, seed=700 + j, dtype="bf16")) for j in range(5)]
+    Xs = [Xs[j % 5] for j in range(33)]
+    outs = outputs(Xs[0], 33)
+    P.ttf_release()
+    assert_same_as_single(Xs[:8], 1, 0.6, P.ttf_compress_batch(Xs[:8], 1, 0.6))      # (loads the kernels for one clip, too)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for n in (9, 16):
+        P.ttf_compress_batch(Xs[:n], 1, 0.6, *[o[:n] for o in outs])
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == before
+    st = torch.cuda.Stream()
+    assert_replays(captured(Xs, outs, st), Xs, outs)
+    P.ttf_release()
+    P.ttf_compress_batch(Xs[:2], 1, 0.6)                     # one block per lane: single clips, one after the other
+    assert_replays(captured(Xs[:7], [o[:7] for o in outs], st), Xs[:7], [o[:7] for o in outs])
+    assert_same_as_single(Xs + Xs, 1, 0.6, P.ttf_compress_batch(Xs + Xs, 1, 0.6))    # several turns per lane
+
+
+def test_graphs_of_smaller_batches_stay_valid():
+    """every batch of the row is larger than the one before it; the graphs captured with the smaller ones are replayed after it"""
+    Xs = [to_device(corr_clip(4, 16, 16, 64, seed=720 + j, dtype="bf16")) for j in range(5)]
+    Xs = [Xs[j % 5] for j in range(20)]
+    P.ttf_release()
+    st = torch.cuda.Stream()
+    graphs = []
+    for n in (1, 2, 3, 5, 8, 20):
+        outs = outputs(Xs[0], n)
+        P.ttf_compress_batch(Xs[:n], 1, 0.6, *outs, stream=st)
+        torch.cuda.synchronize()
+        for g, m, o in graphs:
+            assert_replays(g, Xs[:m], o)
+        graphs.append((captured(Xs[:n], outs, st), n, outs))
+    for g, m, o in graphs:
+        assert_replays(g, Xs[:m], o)
