@@ -640,13 +640,18 @@ struct BatchPlan { int group, lanes, sets, blocks; bool pipelined; };
 // 330 us); more than two lanes of smaller groups gain nothing (within 2 % for every clip size measured).
 // Scratch: 16 blocks in all for eight clips or more, 32 for more than 16; so few sizes that the lanes' scratch soon stays
 // as it is, whatever the number of clips.
-static BatchPlan plan_batch(const Problem& p, int nclips) {
+// Clips that do not take the same path (one base or output pointer on a 16-byte boundary, another one off it) cannot share
+// a launch: single clips on all lanes, since the element-wise kernels of one clip alone leave much of the GPU idle (16 clips
+// of 32 x 16 x 16 x 1024, every second one 2 bytes off: 1247 us per batch on two lanes, 1080 on eight; 16 of 8 x 12 x 12 x 512, every
+// fourth one off, in a replayed graph: 238 and 140).
+static BatchPlan plan_batch(const Problem& p, int nclips, bool same_layout) {
     BatchPlan b;
     const int want = g_sched_lanes.load();
     b.pipelined = want == TTF_SCHEDULE_PIPELINED && nclips >= 3 && p.anchor_mode == 0;
     b.group = 1; b.sets = b.blocks = 2;
     if (b.pipelined) { b.lanes = 2; return b; }
     if (want >= 1 && want <= kBatchStreams) b.lanes = want;          // ttf_set_schedule: so many single clips in flight
+    else if (!same_layout) b.lanes = kBatchStreams;
     else {
         b.group = (nclips + 1) / 2 < kMaxGroup ? (nclips + 1) / 2 : kMaxGroup;
         b.lanes = 2;
@@ -670,6 +675,7 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
     // every clip is validated (and the largest scratch layout found) before anything is enqueued
     Problem p0;
     bool same_layout = true;                     // clips of one launch share the vector path or the scalar path
+    auto aligned = [&](int n) { return reinterpret_cast<uintptr_t>(out_tokens[n]) % 16 == 0; };
     size_t stride = 0;
     for (int n = 0; n < nclips; ++n) {
         Problem p;
@@ -680,10 +686,9 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         carve_scratch(p, nullptr, &s);
         if (s.bytes > stride) stride = s.bytes;
         if (n == 0) p0 = p;
-        same_layout = same_layout && p.vec == p0.vec;
+        same_layout = same_layout && p.vec == p0.vec && (!p.vec || aligned(n) == aligned(0));
     }
-    BatchPlan plan = plan_batch(p0, nclips);
-    if (!same_layout) { plan.group = 1; plan.sets = plan.blocks = 2; }
+    BatchPlan plan = plan_batch(p0, nclips, same_layout);
     // Scratch (before the fork, outside the event bracket).  Where it cannot grow, inside a capture or for lack of memory, the
     // groups are as large as what the lanes hold allows.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -1088,7 +1093,7 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
     std::vector<OutPtrs> outs;
     size_t stride = 0;
     bool same_layout = true;
-    BatchPlan plan = {1, 1, 1, 1, false};
+    auto aligned = [&](int n) { return reinterpret_cast<uintptr_t>(out_tokens[n]) % 16 == 0; };
     for (int n = 0; n < nclips; ++n) {
         Problem p;
         int rc = make_problem(features[n], F, H, W, C, r, t, dtype, &p);
@@ -1096,11 +1101,10 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
         Scratch sn;                              // (the layout depends on the alignment of the clip)
         carve_scratch(p, nullptr, &sn);
         if (sn.bytes > stride) stride = sn.bytes;
-        if (n == 0) plan = plan_batch(p, nclips);
         ps.push_back(p);
-        same_layout = same_layout && p.vec == ps[0].vec;
+        same_layout = same_layout && p.vec == ps[0].vec && (!p.vec || aligned(n) == aligned(0));
     }
-    if (!same_layout) plan.group = 1;
+    const BatchPlan plan = plan_batch(ps[0], nclips, same_layout);
     {
         std::vector<Problem> grouped;
         for (int n0 = 0; n0 < nclips; n0 += plan.group) {

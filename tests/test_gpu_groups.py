@@ -39,6 +39,15 @@ def test_clips_of_different_alignment():
     assert_same_as_single(Xs, 1, 0.6, outs)
 
 
+def test_outputs_of_different_alignment():
+    """21 clips, the token rows of every third 2 bytes off"""
+    Xs = [to_device(corr_clip(3, 4, 5, 64, seed=620 + j, dtype="bf16")) for j in range(21)]
+    toks, cnts, poss = outputs(Xs[0], 21)
+    for j in range(0, 21, 3):
+        toks[j] = torch.zeros(toks[j].numel() + 8, dtype=toks[j].dtype, device="cuda")[1:1 + toks[j].numel()].view(toks[j].shape)
+    assert_same_as_single(Xs, 1, 0.6, P.ttf_compress_batch(Xs, 1, 0.6, toks, cnts, poss))
+
+
 def outputs(X, n):
     rows, C = X.shape[0] * X.shape[1] * X.shape[2], X.shape[3]
     return ([torch.zeros((rows, C), dtype=X.dtype, device="cuda") for _ in range(n)],
