@@ -61,9 +61,12 @@ __device__ __forceinline__ float fold8(float (&v)[8], int lane) {
     return r;
 }
 
-// LS: lanes across a slice (4 to 32); RG = 256 / LS row groups walk the tokens interleaved.
+// LS: lanes across a slice (8, 16 or 32); RG = 256 / LS row groups walk the tokens interleaved.
+// CLS: a thread keeps CLS running sums, of every CLS-th of its tokens.  A sum over all tokens is the same tree whether 32
+// classes of tokens belong to 32 row groups of 8 lanes (CLS = 1), to 16 of 16 (2) or to 8 of 32 (4): class w + 8 J to warp w,
+// the J = 0..3 of a warp as (0 + 1) + (2 + 3), then the warps in order; likewise 16 classes.
 // NORMS: also store the per-token partial squared norms (only the CUDA-core matching kernel reads them).
-template <typename T, int V, int LS, bool NORMS>
+template <typename T, int V, int LS, bool NORMS, int CLS>
 __global__ void __launch_bounds__(kNormThreads)
 k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
            float* __restrict__ S, float* __restrict__ ssq, int* __restrict__ cnt, int* __restrict__ hdr,
@@ -86,7 +89,7 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     if (chain) trace_mark(hdr, 15, false);
     const int k = blockIdx.x / nq, q = blockIdx.x - k * nq;
     const int tid = threadIdx.x, lane = tid & 31;
-    const int ls = tid & (LS - 1), rg = tid / LS;
+    const int ls = tid & (LS - 1), rg = (tid >> 5) + kNormWarps * (lane / LS);
     const size_t FN = (size_t)F * N;
     const int c0 = (q * LS + ls) * V;
     const bool active = c0 < C;                     // C is a multiple of V on the vector path
@@ -94,9 +97,12 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     float* plane = ssq + (size_t)q * FN + (size_t)k * N;           // (NORMS: LS = 32, one plane per slice)
 
     __shared__ float sm[kNormWarps][LS * V];
-    float col[V];
+    static_assert(kBatch % CLS == 0, "whole rounds of the classes");
+    float col[CLS][V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) col[v] = 0.f;
+    for (int c = 0; c < CLS; ++c)
+#pragma unroll
+        for (int v = 0; v < V; ++v) col[c][v] = 0.f;
 
     // thread's tokens: rg, rg + RG, rg + 2 RG, ...; a batch is kBatch of them
     typename L::Raw cur[kBatch], nxt[kBatch];
@@ -119,7 +125,7 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
 #pragma unroll
             for (int v = 0; v < V; ++v) {
                 if (NORMS) s = fmaf(x[v], x[v], s);
-                col[v] += x[v];
+                col[u % CLS][v] += x[v];
             }
             ss[u] = s;
         }
@@ -139,12 +145,19 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     }
 
 #pragma unroll
-    for (int o = LS; o < 32; o <<= 1)               // the row groups of a warp
+    for (int o = LS; o < 32; o <<= 1)               // the row groups of a warp (the low bits of J)
 #pragma unroll
-        for (int v = 0; v < V; ++v) col[v] += __shfl_xor_sync(0xffffffffu, col[v], o);
+        for (int c = 0; c < CLS; ++c)
+#pragma unroll
+            for (int v = 0; v < V; ++v) col[c][v] += __shfl_xor_sync(0xffffffffu, col[c][v], o);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {                   // and of a thread (the high bits)
+        if (CLS == 2) col[0][v] += col[CLS / 2][v];
+        if (CLS == 4) col[0][v] = (col[0][v] + col[CLS / 4][v]) + (col[CLS / 2][v] + col[CLS - 1][v]);
+    }
     if (lane < LS) {
 #pragma unroll
-        for (int v = 0; v < V; ++v) sm[tid >> 5][ls * V + v] = col[v];
+        for (int v = 0; v < V; ++v) sm[tid >> 5][ls * V + v] = col[0][v];
     }
     __syncthreads();
     for (int idx = tid; idx < LS * V; idx += kNormThreads) {
@@ -162,10 +175,10 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
     trace_mark(hdr, 0, true);
 }
 
-template <typename T, int V, int LS, bool NORMS>
+template <typename T, int V, int LS, bool NORMS, int CLS = 1>
 static cudaError_t launch_sum_ls(const Problem& p, const Scratch& s, cudaStream_t st) {
     const int nq = (p.C + LS * V - 1) / (LS * V);
-    return launch_ex(true, 0, k_norm_sum<T, V, LS, NORMS>, dim3((unsigned)((long long)p.F * nq), p.nclips), dim3(kNormThreads),
+    return launch_ex(true, 0, k_norm_sum<T, V, LS, NORMS, CLS>, dim3((unsigned)((long long)p.F * nq), p.nclips), dim3(kNormThreads),
                      st, p.xs, p.F, p.N, p.C, nq, s.S, s.ssq, s.cnt, s.hdr, p.chain, p.sstride);
 }
 
@@ -178,12 +191,19 @@ static cudaError_t launch_sum_t(const Problem& p, const Scratch& s, cudaStream_t
     // 31.7 / 28.1 / 26.4 / 28.6, 32 x 16 x 16 x 1024 20.7 / 19.2 / 18.2 / 18.3, 16 x 8 x 8 x 512 12.2 / 12.5 / 12.3 / 12.8;
     // with 512 CTAs as they are (32 x 16 x 16 x 4096) narrower slices gain nothing (37.9 / 38.2), and a batch of eight
     // 24 x 20 x 20 x 1024 has enough of them together (86.4 against 89.9 with narrow slices).
+    // The order of summation is that of the width which the clip takes alone, so that the anchor does not depend on the launch:
+    // wider slices keep the sums of its classes apart (more registers, 0 - 4 % of a batch's time: eight 24 x 20 x 20 x 1024
+    // 83.8 -> 85.8 us, eight 32 x 16 x 16 x 1024 66.7 -> 67.4; with the narrow slices themselves 87.8 and
+    // 71.7).
     if constexpr (V > 1) {
-        const long long rows = (long long)p.F * p.nclips, enough = 2LL * sm_count();
-        if (rows * p.nq < enough) {
-            if (rows * ((p.C + 16 * V - 1) / (16 * V)) >= enough) return launch_sum_ls<T, V, 16, false>(p, s, st);
-            return launch_sum_ls<T, V, 8, false>(p, s, st);
-        }
+        const long long enough = 2LL * sm_count();
+        const int nq16 = (p.C + 16 * V - 1) / (16 * V);
+        auto width = [&](long long rows) { return rows * p.nq >= enough ? 32 : (rows * nq16 >= enough ? 16 : 8); };
+        const int alone = width(p.F), here = width((long long)p.F * p.nclips);
+        if (alone == 16) return here == 32 ? launch_sum_ls<T, V, 32, false, 2>(p, s, st) : launch_sum_ls<T, V, 16, false>(p, s, st);
+        if (alone == 8)
+            return here == 32 ? launch_sum_ls<T, V, 32, false, 4>(p, s, st)
+                 : here == 16 ? launch_sum_ls<T, V, 16, false, 2>(p, s, st) : launch_sum_ls<T, V, 8, false>(p, s, st);
     }
     return launch_sum_ls<T, V, 32, false>(p, s, st);
 }
@@ -331,9 +351,10 @@ k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float
 // the arg max, which is five to six dependent round trips after the sweep; here every CTA fetches all of its
 // frame sums in one round trip, the per-frame shares of <S_k, g>, |S_k|^2 and |g|^2 go to rank 0 through
 // distributed shared memory, and rank 0 takes the arg max after one cluster barrier (7.2 -> 4.8 us per launch on
-// the 8B-shaped clip, 42.1 -> 37.7 us per clip with one clip in flight).  Every order of summation is fixed
-// (slices inside a CTA, then ranks), so the result is reproducible; it may differ in the last bits from the grid
-// kernel's, which adds the same terms in another fixed order.
+// the 8B-shaped clip, 42.1 -> 37.7 us per clip with one clip in flight).  Every order of summation is fixed and a function of
+// the clip's shape: with more than eight slices the unit is one sixteenth of them (slices v, v + 16), two units v and v + 8
+// are added first and these pairs in order, whether eight CTAs hold a pair each or sixteen a unit each.  (The grid kernel
+// adds the same terms in an order of its own; which of the two a clip takes depends on its shape alone.)
 // What bounds it is a serial chain: what an SM can take in from L2 (64 KB per CTA for 32 frames of 4096 channels on eight
 // CTAs, 0.9 us; hence sixteen where the kernel runs alone), three block barriers and the cluster barrier.  With eight CTAs, two shuffle trees per frame and every warp adding up all
 // channels of g for itself a pass took, per clip, 39.3 us (32 x 16 x 16 x 4096), 28.9 (2048 channels), 134.7 (128 frames)
@@ -405,37 +426,45 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
     float4 gl[SL];
 #pragma unroll
     for (int sl = 0; sl < SL; ++sl) gl[sl] = reinterpret_cast<const float4*>(s_gl)[sl * 32 + lane];
-    // step 2: this CTA's shares of <S_k, g> and |S_k|^2 for every frame, slices in order; four frames at a time are added
-    // up over the warp (fold8)
+    // step 2: this CTA's shares of <S_k, g> and |S_k|^2 for every frame, eight sums at a time added up over the warp (fold8):
+    // four frames, or two frames of two units (even and odd slices of this CTA), which are then added
+    constexpr int U = CS == 8 && SL > 1 ? 2 : 1;     // units of this CTA
+    constexpr int FP = 4 / U;                        // frames per fold
     for (int k0 = 0; k0 < F; k0 += CHUNK) {
         if (!one_chunk) load_chunk(k0);              // (a second round trip per chunk for clips of several chunks)
 #pragma unroll
-        for (int j0 = 0; j0 < FB; j0 += 4) {
-            float part[8];                           // <S_k, g> and |S_k|^2 of frames j0 .. j0 + 3
+        for (int j0 = 0; j0 < FB; j0 += FP) {
+            float part[8];                           // [<S_k, g> or |S_k|^2][unit][frames j0 .. j0 + FP - 1]
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 float d = 0.f, qq = 0.f;
 #pragma unroll
-                for (int sl = 0; sl < SL; ++sl) {
-                    const float4 x = v[sl][j0 + e], g = gl[sl];
+                for (int sl = e / FP; sl < SL; sl += U) {
+                    const float4 x = v[sl][j0 + e % FP], g = gl[sl];
                     d = fmaf(x.x, g.x, d); d = fmaf(x.y, g.y, d); d = fmaf(x.z, g.z, d); d = fmaf(x.w, g.w, d);
                     qq = fmaf(x.x, x.x, qq); qq = fmaf(x.y, x.y, qq); qq = fmaf(x.z, x.z, qq); qq = fmaf(x.w, x.w, qq);
                 }
                 part[e] = d; part[4 + e] = qq;
             }
-            const float tot = fold8(part, lane);     // lanes 0, 4, 8, ..: part[4 * bit4 + 2 * bit3 + bit2] of the lane index
-            const int kk = k0 + w + (j0 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)) * kNormWarps;
-            if ((lane & 3) == 0 && kk < F) (lane & 16 ? s_Q : s_D)[kk] = tot;
+            float tot = fold8(part, lane);           // lanes 0, 4, 8, ..: part[4 * bit4 + 2 * bit3 + bit2] of the lane index
+            if (U == 2) tot += __shfl_xor_sync(0xffffffffu, tot, 8);
+            const int kk = k0 + w + (j0 + (U == 2 ? 0 : (lane >> 3) & 1) * 2 + ((lane >> 2) & 1)) * kNormWarps;
+            if ((lane & (U == 2 ? 11 : 3)) == 0 && kk < F) (lane & 16 ? s_Q : s_D)[kk] = tot;
         }
     }
     if (w == 0) {
         float gg = 0.f;
 #pragma unroll
-        for (int sl = 0; sl < SL; ++sl) {
-            const float4 g = gl[sl];
-            gg = fmaf(g.x, g.x, gg); gg = fmaf(g.y, g.y, gg); gg = fmaf(g.z, g.z, gg); gg = fmaf(g.w, g.w, gg);
+        for (int u = 0; u < U; ++u) {
+            float part = 0.f;
+#pragma unroll
+            for (int sl = u; sl < SL; sl += U) {
+                const float4 g = gl[sl];
+                part = fmaf(g.x, g.x, part); part = fmaf(g.y, g.y, part); part = fmaf(g.z, g.z, part); part = fmaf(g.w, g.w, part);
+            }
+            part = warp_sum(part);
+            gg = u == 0 ? part : gg + part;
         }
-        gg = warp_sum(gg);
         if (lane == 0) s_G = gg;
     }
     __syncthreads();
@@ -451,13 +480,20 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
         cluster_wait();
     }
     if (rank == 0) {
-        // Eq. (auto_anchor): a* = arg max_k <S_k, g> / (|S_k| |g|), lowest frame on ties; ranks added in rank order
+        // Eq. (auto_anchor): a* = arg max_k <S_k, g> / (|S_k| |g|), lowest frame on ties; ranks added in order
         float best = -INFINITY;
         int idx = 0x7fffffff;
         if (tid < F) {                               // F <= kStatClusterMaxF = the CTA's 256 threads
-            float D = s_D[tid], Q = s_Q[tid], G = s_G;
+            // what rank r holds, and with sixteen ranks what rank r + 8 holds added to it first
+            auto share = [&](int r, int i, float own) {
+                const float x = r == 0 ? own : s_x[r - 1][i];
+                return CS == 16 ? x + s_x[CS == 16 ? r + 7 : 0][i] : x;
+            };
+            float D = share(0, tid, s_D[tid]), Q = share(0, F + tid, s_Q[tid]), G = share(0, 2 * F, s_G);
 #pragma unroll
-            for (int r = 0; r < CS - 1; ++r) { D += s_x[r][tid]; Q += s_x[r][F + tid]; G += s_x[r][2 * F]; }
+            for (int r = 1; r < (CS < 8 ? CS : 8); ++r) {
+                D += share(r, tid, 0.f); Q += share(r, F + tid, 0.f); G += share(r, 2 * F, 0.f);
+            }
             best = D * (1.0f / fmaxf(sqrtf(G), kNormFloor)) * (1.0f / fmaxf(sqrtf(Q), kNormFloor));
             idx = tid;
         }
@@ -566,13 +602,9 @@ static bool large_clusters() {
 cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anchor, cudaStream_t st) {
     if (p.anchor_mode != 0) return cudaSuccess;                // fixed anchors need no statistics
     // The single-cluster kernel is the shorter one (4.9 against 7.2 us on a 32-frame clip of 4096 channels) and takes
-    // the call whenever it can, with one exception that was measured: short clips with four or more clips in flight.
-    // A cluster starts only when eight CTA slots of one GPC are free at the same moment, and on a GPU that is full of
-    // other clips' kernels that wait costs more than the kernel saves (8B-shaped clip, eight in flight: 30.3 us per
-    // clip with the cluster kernel, 29.8 with the grid kernel; two in flight: 33.9 against 35.0; 128-frame clip, eight
-    // in flight: 107.9 against 110.1, the grid kernel's time grows with F).
-    const bool crowded = p.overlapped >= 4 && p.F <= 32;
-    if (!crowded && p.C % 4 == 0 && p.nsl <= 32 && p.F <= kStatClusterMaxF) {
+    // every clip it can.  Sixteen CTAs where nothing runs beside the call, eight in a batch: a cluster starts only when all
+    // its places in one GPC are free at the same moment.
+    if (p.C % 4 == 0 && p.nsl <= 32 && p.F <= kStatClusterMaxF) {
         if (p.nsl == 1) return launch_stats_cluster_t<1, 1>(p, s, out_anchor, st);      // nothing to split
         const bool alone = p.overlapped <= 1 && large_clusters();
         if (p.nsl > 16) return alone ? launch_stats_cluster_t<2, 16>(p, s, out_anchor, st)
