@@ -642,7 +642,7 @@ struct BatchPlan { int group, lanes, sets, blocks; bool pipelined; };
 // as it is, whatever the number of clips.
 // Clips that do not take the same path (one base or output pointer on a 16-byte boundary, another one off it) cannot share
 // a launch: single clips on all lanes, since the element-wise kernels of one clip alone leave much of the GPU idle (16 clips
-// of 32 x 16 x 16 x 1024, every second one 2 bytes off: 1247 us per batch on two lanes, 1080 on eight; 16 of 8 x 12 x 12 x 512, every
+// of 32 x 16 x 16 x 1024, every second one 2 bytes off: 1247 us per batch on two lanes, 1027 on eight; 16 of 8 x 12 x 12 x 512, every
 // fourth one off, in a replayed graph: 238 and 140).
 static BatchPlan plan_batch(const Problem& p, int nclips, bool same_layout) {
     BatchPlan b;

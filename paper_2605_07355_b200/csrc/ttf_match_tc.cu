@@ -544,7 +544,11 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)tc_match_tiles(p);
     const int chunks = tc_match_chunks(p);
-    const int pieces = split_of(p, tiles * p.nclips, chunks);      // CTAs (= cluster size) per tile
+    // CTAs (= cluster size) per tile.  Three or more single clips in flight (ttf_set_schedule, clips that cannot share a launch)
+    // fill the GPU together: 16 clips of 32 x 16 x 16 x 4096 on eight lanes 497 -> 445 us, on three 512 -> 506 (on two 530 ->
+    // 507, but three clips, of which two share a launch, 98 -> 102).
+    const int beside = p.nclips == 1 && p.overlapped >= 3 ? p.overlapped : 1;
+    const int pieces = split_of(p, tiles * p.nclips * beside, chunks);
     auto log2_of = [](int n) { int l = 0; while ((1 << l) < n) ++l; return l; };
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles * pieces), p.nclips); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;

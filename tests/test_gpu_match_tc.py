@@ -29,8 +29,13 @@ def test_bits_do_not_depend_on_the_split(shape, r, clips):
     sims = torch.sort(q["best_sim"][q["best_sim"] < 1.0]).values
     for t in sims[:: max(1, sims.numel() // 8)].tolist():
         one = P.ttf_compress(X, r, t)
-        toks, cnts, poss = P.ttf_compress_batch([X] * clips, r, t)
-        torch.cuda.synchronize()
         L = int(one[1])
-        assert all(int(c) == L for c in cnts)
-        assert all(torch.equal(p[:L], one[2][:L]) for p in poss)
+        for lanes in (0, 8):                                 # groups, and single clips that count with their neighbours
+            P.ttf_set_schedule(lanes)
+            try:
+                toks, cnts, poss = P.ttf_compress_batch([X] * clips, r, t)
+            finally:
+                P.ttf_set_schedule(0)
+            torch.cuda.synchronize()
+            assert all(int(c) == L for c in cnts)
+            assert all(torch.equal(p[:L], one[2][:L]) for p in poss)
