@@ -9,8 +9,8 @@ namespace ttf {
 constexpr int kXThreads = 256;
 
 // Number of non-zero flags in keep[lo, hi): bytes up to the first 16-byte boundary, 16 flags per load from there,
-// bytes again at the end.  Every thread of the CTA takes part; the caller adds the per-thread counts up.  (L2-coherent
-// loads: the flags may come from a kernel that still ran when this one was scheduled.)
+// bytes again at the end.  Every thread of the CTA takes part; the caller adds the per-thread counts up.  (Plain loads, as for
+// the rows below: the CTAs of an SM read the same lines.  Past L1, restoring 128 x 32 x 32 tokens of 128 bytes took 24.5 us, 19.5 now.)
 __device__ __forceinline__ int count_flags(const unsigned char* keep, size_t lo, size_t hi, int tid) {
     if (lo >= hi) return 0;
     int c = 0;
@@ -18,10 +18,10 @@ __device__ __forceinline__ int count_flags(const unsigned char* keep, size_t lo,
     size_t head = lo + ((16 - ((base + lo) & 15)) & 15);          // first index whose address is 16-byte aligned
     if (head > hi) head = hi;
     const size_t nvec = (hi - head) / 16, tail = head + nvec * 16;
-    for (size_t f = lo + tid; f < head; f += kXThreads) c += __ldcg(keep + f) ? 1 : 0;
+    for (size_t f = lo + tid; f < head; f += kXThreads) c += keep[f] ? 1 : 0;
     const uint4* v = reinterpret_cast<const uint4*>(keep + head);
     for (size_t u = tid; u < nvec; u += kXThreads) {
-        const uint4 q = __ldcg(v + u);
+        const uint4 q = v[u];
         // a flag is any non-zero byte: fold each byte's bits into its lowest one
         unsigned w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
@@ -31,7 +31,7 @@ __device__ __forceinline__ int count_flags(const unsigned char* keep, size_t lo,
             c += __popc(b & 0x01010101u);
         }
     }
-    for (size_t f = tail + tid; f < hi; f += kXThreads) c += __ldcg(keep + f) ? 1 : 0;
+    for (size_t f = tail + tid; f < hi; f += kXThreads) c += keep[f] ? 1 : 0;
     return c;
 }
 
@@ -94,11 +94,11 @@ __device__ __forceinline__ void restore_rows(const unsigned char* comp, size_t r
         for (; u + (kInFlight - 1) * 32 < units; u += kInFlight * 32) {
             U v[kInFlight];
 #pragma unroll
-            for (int e = 0; e < kInFlight; ++e) v[e] = __ldcg(src + u + e * 32);
+            for (int e = 0; e < kInFlight; ++e) v[e] = src[u + e * 32];
 #pragma unroll
             for (int e = 0; e < kInFlight; ++e) d[u + e * 32] = v[e];
         }
-        for (; u < units; u += 32) d[u] = __ldcg(src + u);
+        for (; u < units; u += 32) d[u] = src[u];
     }
 }
 
@@ -115,9 +115,11 @@ k_restore_copy(const unsigned char* __restrict__ comp, size_t row_bytes, long lo
 
 // Both steps in one launch, for clips of up to kRestoreWhole tokens: a CTA owns a contiguous range of tokens, counts the
 // preserved tokens before it (16 flags per load: one round trip), ranks its own 256 at a time, and copies their rows from
-// the indices in shared memory.  With a kernel of its own for the indices (5.2 us) a 32 x 16 x 16 clip of 4096 bf16
-// channels took 23.7 us, 19.1 now (its 90 MB at the copy rate: 13.8); in longer clips the flags that every CTA reads would
-// outweigh the launch.
+// the indices in shared memory.  What bounds it is the traffic of long rows, and for short ones a chain of round trips.  Us
+// per call / in a replayed graph, with a launch for the indices -> in one: 4 x 16 x 16 x 64 bf16 channels 11.7 / 3.9 -> 8.9 /
+// 2.4, 32 x 16 x 16 x 64 11.7 / 4.9 -> 8.7 / 6.3, 32 x 16 x 16 x 4096 18.5 / 16.9 -> 15.3 / 15.2 (its 90 MB at the copy rate:
+// 13.8), 64 x 32 x 32 x 64 15.4 / 13.0 -> 14.1 / 14.0, x 1024 53.7 / 48.7 -> 45.5 / 45.4: the graph's time alone would draw the
+// line for short rows at 4096 tokens, a call's at 65536.  In longer clips the flags that every CTA reads outweigh the launch.
 constexpr int kRestoreWhole = 1 << 16;
 
 template <typename U>
@@ -131,6 +133,9 @@ k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int*
     const int f0 = blockIdx.x * per, f1 = min(FN, f0 + per);
     pdl_launch_dependents();
     pdl_wait();                                  // the caller's kernels before this one
+    // (what the first round needs of this CTA's tokens is asked for together with the anchor and the flags before them)
+    unsigned char next_keep = f0 + tid < f1 ? keep[f0 + tid] : (unsigned char)0;
+    int next_dst = f0 + tid < f1 ? dst[f0 + tid] : 0;
     // the anchor frame's tokens: [a0, a1), none of the clip's for an anchor outside it
     const int a = __ldcg(anchor);
     const bool inside = (unsigned)a < (unsigned)(FN / N);
@@ -148,7 +153,10 @@ k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int*
     for (int b0 = f0; b0 < f1; b0 += kXThreads) {
         const int f = b0 + tid;
         const bool in = f < f1, own = f >= a0 && f < a1;
-        const bool kp = in && !own && __ldcg(keep + f);
+        const bool kp = in && !own && next_keep;
+        const int to = next_dst;
+        next_keep = f + kXThreads < f1 ? keep[f + kXThreads] : (unsigned char)0;
+        next_dst = f + kXThreads < f1 ? dst[f + kXThreads] : 0;
         const unsigned m = __ballot_sync(0xffffffffu, kp);
         __syncthreads();                         // (the indices of the round before this one, and s_warp, are done with)
         if (lane == 0) s_warp[w] = __popc(m);
@@ -157,7 +165,7 @@ k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int*
 #pragma unroll
         for (int ww = 0; ww < kXThreads / 32; ++ww) { off += ww < w ? s_warp[ww] : 0; total += s_warp[ww]; }
         if (in) {
-            const int r = own ? f - a0 : (kp ? run + off + __popc(m & ((1u << lane) - 1)) : __ldcg(dst + f));
+            const int r = own ? f - a0 : (kp ? run + off + __popc(m & ((1u << lane) - 1)) : to);
             s_row[tid] = r;
             row_index[f] = r;
         }
