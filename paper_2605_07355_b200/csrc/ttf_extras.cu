@@ -264,9 +264,10 @@ template <int WARPS> __device__ __forceinline__ int counts_of_block(TokenCounts&
 
 // Clips of up to kStatsWhole tokens: one cluster of eight CTAs, whose counts meet in the shared memory of rank 0.  (A grid
 // of independent CTAs needs its three words cleared first: a memset before the kernel, 5 us of 37 for the query and the
-// counts of a 48 x 14 x 14 clip of 2048 channels.)
+// counts of a 48 x 14 x 14 clip of 2048 channels.)  The cluster's time grows with the clip, us in a replayed graph, cluster /
+// grid: 9408 tokens 1.9 / 5.9, 98304 3.5 / 5.9, 196608 5.5 / 5.9, 262144 6.6 / 6.2.
 constexpr int kStatsCtas = 8, kStatsThreads = 512;
-constexpr long long kStatsWhole = 1 << 18;
+constexpr long long kStatsWhole = 3 << 16;
 
 __global__ void __cluster_dims__(kStatsCtas, 1, 1) __launch_bounds__(kStatsThreads)
 k_stats_cluster(const float* sim, const unsigned char* keep, const int* anchor, int N, int total, float t, float band,

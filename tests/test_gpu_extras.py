@@ -140,7 +140,7 @@ def test_restore_one_and_two_launches(shape):
         assert (idx.cpu().numpy() == ref_idx).all() and (to_bits(full) == ref_full).all()
 
 
-@pytest.mark.parametrize("F,N", [(1, 1), (3, 5), (7, 585), (9, 4096), (256, 1024), (257, 1024)])
+@pytest.mark.parametrize("F,N", [(1, 1), (3, 5), (7, 585), (9, 4096), (192, 1024), (193, 1024), (256, 1024), (257, 1024)])
 def test_stats_over_sizes(F, N):
     """one token, less than a block, one cluster up to its largest clip, the grid beyond it; anchor first, inside, last"""
     rng = np.random.default_rng(F * N)
