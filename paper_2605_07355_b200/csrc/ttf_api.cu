@@ -731,12 +731,16 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         }
         p.overlapped = lanes;
         // When the sweep of a group is done, L2 holds the last clip or two of it: the matching kernel starts with those, and it
-        // and the gather mark what they have read (and the gather what it writes) as the first to go.  16 clips of
-        // 32 x 16 x 16 x 4096 447.0 -> 444.4 us, 4 of them 127.0 -> 123.8, 16 of 32 x 16 x 16 x 2048 238.8 -> 236.3, 8 of
-        // 24 x 20 x 20 x 1024 86.8 -> 85.3.  Not for clips that are larger than L2 by themselves (8 of 268 MB: 880 -> 884),
-        // nor without a sweep (184.1 -> 184.6) or on the fp32 kernel, which has no hints (167.0 -> 167.3).
-        const bool fits_l2 = (double)p.F * p.N * p.C * 2 < 128.0 * (1 << 20);
-        p.stream_once = plan.pipelined || (p.nclips > 1 && fits_l2 && p.use_tc && p.anchor_mode == 0) ? 1 : 0;
+        // and the gather mark what they have read as the first to go.  16 clips of 32 x 16 x 16 x 4096 430 -> 428 us, 4 of them
+        // 126 -> 123, 16 of 32 x 16 x 16 x 2048 230 -> 228, 8 of 24 x 20 x 20 x 1024 87.2 -> 86.2; larger clips, four of 134 MB
+        // 228 -> 223, of 201 MB 327 -> 323, but 8 of 268 MB 880 -> 884: up to 208 MB.  Not without a sweep (184.1 -> 184.6) or
+        // on the fp32 kernel, which has no hints (167.0 -> 167.3).  The rows that the gather writes are what the caller reads
+        // next, so they are marked only where a third of the batch, the usual share of kept rows, would not stay in L2 anyway
+        // (16 clips of 32 x 16 x 16 x 4096: 428 -> 425, with a copy of all kept rows behind it 592 -> 587; 4 of them: 122.8 ->
+        // 122.0, but 160.8 -> 162.0 with the copy).
+        const double clip_mb = (double)p.F * p.N * p.C * 2e-6;
+        const bool first_to_go = p.nclips > 1 && clip_mb < 208.0 && p.use_tc && p.anchor_mode == 0;
+        p.stream_once = plan.pipelined || (first_to_go && clip_mb * nclips / 3 > 126.0) ? 2 : (first_to_go ? 1 : 0);
         p.chain = plan.sets == 2 && turn > 0 ? 1 : 0;        // the lane's previous kernel is the gather of its previous clip
         if (turn < plan.sets) {
             // the blocks may hold anything (another shape's data, or a failed call's counters): clear their control words

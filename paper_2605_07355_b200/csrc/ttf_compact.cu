@@ -116,8 +116,8 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     const int pieces = (int)((row_bytes + kBulkPiece - 1) / kBulkPiece);
     uint32_t phase = 0;
     bool gave_up = false;
-    // pipelined schedule: neither the rows read here nor the rows written are needed in L2 again, while the clip
-    // that is being matched and the one streaming in are: their lines are the first to go
+    // the rows read here are not needed in L2 again, while the clip that is being matched and the one streaming in are: their
+    // lines are the first to go; those of the rows written, which the caller reads next, only where they would not stay anyway
     const unsigned long long once = l2_evict_first_policy();
     for (int j = gw; ; j += nw) {
         int f;
@@ -150,7 +150,7 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
                     break;
                 }
                 ++phase;
-                if (stream_once) bulk_store_hint(out_tokens + (size_t)j * row_bytes + off, buf, bytes, once);
+                if (stream_once == 2) bulk_store_hint(out_tokens + (size_t)j * row_bytes + off, buf, bytes, once);
                 else bulk_store(out_tokens + (size_t)j * row_bytes + off, buf, bytes);
                 bulk_commit();
             }
@@ -349,7 +349,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
                 gave_up = true;
             } else if (in_bounds(hdr, 4, jb + n - 1, FN)) {
                 unsigned char* d = out_tokens + (size_t)jb * row_bytes;
-                if (stream_once) bulk_store_hint(d, buf + h * kGatherSlot, (uint32_t)(n * row_bytes), once);
+                if (stream_once == 2) bulk_store_hint(d, buf + h * kGatherSlot, (uint32_t)(n * row_bytes), once);
                 else bulk_store(d, buf + h * kGatherSlot, (uint32_t)(n * row_bytes));
                 bulk_commit();
             }

@@ -60,9 +60,9 @@ struct Problem {
                         // clip, which works on another scratch block: the sweep may run beside it
     int chain_next;     // 1: the kernel after this call's gather is such a sweep
     int overlapped;     // clips whose kernels run beside one another: the lanes of a batch (0 or 1: this call runs alone)
-    int stream_once;    // 1: the matching kernel marks the lines of the source rows it reads as the first to leave L2, and the
-                        // gather its lines (the pipelined schedule: the next clip streams into L2 while this one is matched;
-                        // a group: the clips that the sweep left in L2 are matched first, backwards)
+    int stream_once;    // 1: the matching kernel and the gather mark the lines of the rows they have read as the first to leave L2
+                        // (the pipelined schedule: the next clip streams into L2 while this one is matched; a group: the
+                        // clips that the sweep left in L2 are matched first, backwards); 2: the gather also those it writes
 };
 
 // Device pointers carved out of one scratch allocation.
