@@ -663,6 +663,36 @@ static BatchPlan plan_batch(const Problem& p, int nclips, bool same_layout) {
     return b;
 }
 
+// The launches over one group of a batch's clips, n0 and those that follow it (the clips have been validated).
+struct GroupLaunch { Problem p; OutPtrs out; };
+static GroupLaunch group_launch(const BatchPlan& plan, const Problem& like, const ttf_options* options, size_t stride,
+                                const void* const* features, int nclips, int n0, void* const* out_tokens,
+                                int* const* out_count, int* const* out_pos_thw) {
+    GroupLaunch g;
+    Problem& p = g.p;
+    make_problem(features[n0], like.F, like.H, like.W, like.C, like.r, like.t, like.dtype, &p);
+    apply_options(&p, options);
+    p.nclips = nclips - n0 < plan.group ? nclips - n0 : plan.group;
+    p.sstride = stride;
+    for (int i = 0; i < p.nclips; ++i) {
+        p.xs.X[i] = features[n0 + i];
+        g.out.tokens[i] = out_tokens[n0 + i]; g.out.count[i] = out_count[n0 + i]; g.out.pos[i] = out_pos_thw[n0 + i];
+    }
+    p.overlapped = plan.lanes;
+    // When the sweep of a group is done, L2 holds the last clip or two of it: the matching kernel starts with those, and it
+    // and the gather mark what they have read as the first to go.  16 clips of 32 x 16 x 16 x 4096 430 -> 428 us, 4 of them
+    // 126 -> 123, 16 of 32 x 16 x 16 x 2048 230 -> 228, 8 of 24 x 20 x 20 x 1024 87.2 -> 86.2; larger clips, four of 134 MB
+    // 228 -> 223, of 201 MB 327 -> 323, but 8 of 268 MB 880 -> 884: up to 208 MB.  Not without a sweep (184.1 -> 184.6) or
+    // on the fp32 kernel, which has no hints (167.0 -> 167.3).  The rows that the gather writes are what the caller reads
+    // next, so they are marked only where a third of the batch, the usual share of kept rows, would not stay in L2 anyway
+    // (16 clips of 32 x 16 x 16 x 4096: 428 -> 425, with a copy of all kept rows behind it 592 -> 587; 4 of them: 122.8 ->
+    // 122.0, but 160.8 -> 162.0 with the copy).
+    const double clip_mb = (double)p.F * p.N * p.C * 2e-6;
+    const bool first_to_go = p.nclips > 1 && clip_mb < 208.0 && p.use_tc && p.anchor_mode == 0;
+    p.stream_once = plan.pipelined || (first_to_go && clip_mb * nclips / 3 > 126.0) ? 2 : (first_to_go ? 1 : 0);
+    return g;
+}
+
 // A lane takes its groups one after the other on its stream.  Lanes of single clips (two sets of scratch blocks used in
 // turn) chain them: the sweep of a clip runs beside the gather of the clip before it.
 static int batch_on_streams(const void* const* features, int nclips, int F, int H, int W, int C, int r, float t,
@@ -719,28 +749,9 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         const int n0 = q * plan.group;
         char* block = (char*)ws[lane] + (size_t)(turn % plan.sets) * set;
         cudaStream_t ls = L->s[lane];
-        Problem p;
-        make_problem(features[n0], F, H, W, C, r, t, dtype, &p);
-        apply_options(&p, options);
-        OutPtrs out;
-        p.nclips = nclips - n0 < plan.group ? nclips - n0 : plan.group;
-        p.sstride = stride;
-        for (int i = 0; i < p.nclips; ++i) {
-            p.xs.X[i] = features[n0 + i];
-            out.tokens[i] = out_tokens[n0 + i]; out.count[i] = out_count[n0 + i]; out.pos[i] = out_pos_thw[n0 + i];
-        }
-        p.overlapped = lanes;
-        // When the sweep of a group is done, L2 holds the last clip or two of it: the matching kernel starts with those, and it
-        // and the gather mark what they have read as the first to go.  16 clips of 32 x 16 x 16 x 4096 430 -> 428 us, 4 of them
-        // 126 -> 123, 16 of 32 x 16 x 16 x 2048 230 -> 228, 8 of 24 x 20 x 20 x 1024 87.2 -> 86.2; larger clips, four of 134 MB
-        // 228 -> 223, of 201 MB 327 -> 323, but 8 of 268 MB 880 -> 884: up to 208 MB.  Not without a sweep (184.1 -> 184.6) or
-        // on the fp32 kernel, which has no hints (167.0 -> 167.3).  The rows that the gather writes are what the caller reads
-        // next, so they are marked only where a third of the batch, the usual share of kept rows, would not stay in L2 anyway
-        // (16 clips of 32 x 16 x 16 x 4096: 428 -> 425, with a copy of all kept rows behind it 592 -> 587; 4 of them: 122.8 ->
-        // 122.0, but 160.8 -> 162.0 with the copy).
-        const double clip_mb = (double)p.F * p.N * p.C * 2e-6;
-        const bool first_to_go = p.nclips > 1 && clip_mb < 208.0 && p.use_tc && p.anchor_mode == 0;
-        p.stream_once = plan.pipelined || (first_to_go && clip_mb * nclips / 3 > 126.0) ? 2 : (first_to_go ? 1 : 0);
+        GroupLaunch g = group_launch(plan, p0, options, stride, features, nclips, n0, out_tokens, out_count, out_pos_thw);
+        Problem& p = g.p;
+        const OutPtrs& out = g.out;
         p.chain = plan.sets == 2 && turn > 0 ? 1 : 0;        // the lane's previous kernel is the gather of its previous clip
         if (turn < plan.sets) {
             // the blocks may hold anything (another shape's data, or a failed call's counters): clear their control words
@@ -1093,8 +1104,7 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
     for (int n = 0; n < nclips; ++n)
         if (!features[n] || !out_tokens[n] || !out_count[n] || !out_pos_thw[n]) return TTF_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    std::vector<Problem> ps;                     // the launches a batch call of these clips would make
-    std::vector<OutPtrs> outs;
+    Problem p0;
     size_t stride = 0;
     bool same_layout = true;
     auto aligned = [&](int n) { return reinterpret_cast<uintptr_t>(out_tokens[n]) % 16 == 0; };
@@ -1105,27 +1115,13 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
         Scratch sn;                              // (the layout depends on the alignment of the clip)
         carve_scratch(p, nullptr, &sn);
         if (sn.bytes > stride) stride = sn.bytes;
-        ps.push_back(p);
-        same_layout = same_layout && p.vec == ps[0].vec && (!p.vec || aligned(n) == aligned(0));
+        if (n == 0) p0 = p;
+        same_layout = same_layout && p.vec == p0.vec && (!p.vec || aligned(n) == aligned(0));
     }
-    const BatchPlan plan = plan_batch(ps[0], nclips, same_layout);
-    {
-        std::vector<Problem> grouped;
-        for (int n0 = 0; n0 < nclips; n0 += plan.group) {
-            Problem p = ps[n0];
-            OutPtrs out;
-            p.nclips = nclips - n0 < plan.group ? nclips - n0 : plan.group;
-            p.sstride = stride;
-            p.overlapped = plan.lanes;
-            for (int i = 0; i < p.nclips; ++i) {
-                p.xs.X[i] = features[n0 + i];
-                out.tokens[i] = out_tokens[n0 + i]; out.count[i] = out_count[n0 + i]; out.pos[i] = out_pos_thw[n0 + i];
-            }
-            grouped.push_back(p);
-            outs.push_back(out);
-        }
-        ps.swap(grouped);
-    }
+    const BatchPlan plan = plan_batch(p0, nclips, same_layout);
+    std::vector<GroupLaunch> gs;                 // the launches a batch call of these clips would make
+    for (int n0 = 0; n0 < nclips; n0 += plan.group)
+        gs.push_back(group_launch(plan, p0, nullptr, stride, features, nclips, n0, out_tokens, out_count, out_pos_thw));
     void* ws = nullptr;
     int rc = cached_scratch(stride * nclips, st, &ws);
     if (rc != TTF_OK) return rc;
@@ -1138,13 +1134,14 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
     for (int rep = 0; rep < reps && e == cudaSuccess; ++rep) {
         for (int stage = 0; stage < 4 && e == cudaSuccess; ++stage) {
             cudaEventRecord(ev[stage], st);
-            for (int n = 0; n < (int)ps.size() && e == cudaSuccess; ++n) {
+            for (int n = 0; n < (int)gs.size() && e == cudaSuccess; ++n) {
+                const Problem& p = gs[n].p;
                 Scratch s;
-                carve_scratch(ps[n], (char*)ws + stride * plan.group * n, &s);
-                if (stage == 0) e = launch_norm_sum(ps[n], s, st);
-                else if (stage == 1) e = launch_frame_stats(ps[n], s, nullptr, st);
-                else if (stage == 2) e = launch_match(ps[n], s, nullptr, s.shat, s.dst, s.keep, st);
-                else e = launch_compact(ps[n], s, outs[n], st);
+                carve_scratch(p, (char*)ws + stride * plan.group * n, &s);
+                if (stage == 0) e = launch_norm_sum(p, s, st);
+                else if (stage == 1) e = launch_frame_stats(p, s, nullptr, st);
+                else if (stage == 2) e = launch_match(p, s, nullptr, s.shat, s.dst, s.keep, st);
+                else e = launch_compact(p, s, gs[n].out, st);
             }
         }
         cudaEventRecord(ev[4], st);

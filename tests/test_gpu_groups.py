@@ -108,3 +108,17 @@ def test_graphs_of_smaller_batches_stay_valid():
         graphs.append((captured(Xs[:n], outs, st), n, outs))
     for g, m, o in graphs:
         assert_replays(g, Xs[:m], o)
+
+
+def test_bench_counts_the_launches_of_a_step():
+    """each kernel once per group of a batch, once per clip where clips go alone; no statistics for a fixed anchor"""
+    from bench import count_launches
+    Xs = [to_device(corr_clip(4, 5, 6, 64, seed=740, dtype="bf16"))] * 16
+    assert count_launches(lambda: P.ttf_compress_batch(Xs, 1, 0.6)) == 2 * 4
+    assert count_launches(lambda: P.ttf_compress_batch(Xs, 1, 0.6, anchor_mode=1)) == 2 * 3
+    assert count_launches(lambda: P.ttf_compress(Xs[0], 1, 0.6)) == 4
+    P.ttf_set_schedule(3)
+    try:
+        assert count_launches(lambda: P.ttf_compress_batch(Xs, 1, 0.6)) == 16 * 4
+    finally:
+        P.ttf_set_schedule(0)
