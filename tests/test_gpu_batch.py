@@ -25,7 +25,7 @@ def assert_same_as_single(Xs, r, t, outs):
 
 def test_batch_on_library_streams_matches_single_calls_and_oracle():
     s = clips.CONFIGS["vl2b_cal"]
-    Xn = [clips.make_clip(s, s.seed + j) for j in range(11)]         # 11 clips over 8 streams: ragged last round
+    Xn = [clips.make_clip(s, s.seed + j) for j in range(11)]         # groups of 6 and 5 clips on two lanes
     Xs = [to_device(x) for x in Xn]
     outs = P.ttf_compress_batch(Xs, s.r, s.t)
     torch.cuda.synchronize()

@@ -44,11 +44,11 @@ def test_copy_wait_runs_out_then_the_next_call_is_clean():
         check_clip(X, 1, 0.7, stream=st)                                 # and it still equals the oracle
 
 
-@pytest.mark.parametrize("C", [256, 2048])
+@pytest.mark.parametrize("C", [64, 256, 2048])
 def test_tensor_core_pipeline_gives_up_and_recovers(C):
     """the tcgen05 matching kernel under the same hook: its copy barriers never complete, so its MMA issuer, its
-    epilogue warps and then its producer run out of polls; the CTAs (alone for C = 256, in clusters of 8 for
-    C = 2048) still meet at their barriers, free their tensor memory and return; the query reports the time-out
+    epilogue warps and then its producer run out of polls; the CTAs (alone for C = 64, in clusters of 2 for C = 256
+    and of 8 for C = 2048) still meet at their barriers, free their tensor memory and return; the query reports the time-out
     and the next call is clean"""
     X = corr_clip(6, 6, 7, C, seed=79, dtype="bf16")
     Xd = to_device(X)
@@ -73,6 +73,29 @@ def test_tensor_core_pipeline_gives_up_and_recovers(C):
             check_clip(X, 1, 0.7, stream=st)
     finally:
         P.ttf_set_match_kernel(0)
+
+
+@pytest.mark.parametrize("r,clips", [(1, 24), (2, 24)])
+def test_tiles_of_one_cta_and_several_chunks_give_up_and_recover(r, clips):
+    """large launches: every tile is one CTA that sums all chunks of its channels (8 alone, 4 for r = 2) itself"""
+    X = corr_clip(6, 8, 8, 1024, seed=82, dtype="bf16")
+    Xs = [to_device(X)] * clips
+    st = torch.cuda.Stream()
+    ref = P.ttf_compress(Xs[0], r, 0.7, stream=st)
+    L = int(ref[1].item())
+    P.ttf_compress_batch(Xs, r, 0.7, stream=st)
+    assert P.ttf_last_device_status(st) == B.TTF_OK
+    P.ttf_debug_set_wait(32, 16)
+    try:
+        _, cnts, _ = P.ttf_compress_batch(Xs, r, 0.7, stream=st)
+        assert P.ttf_last_device_status(st) == B.TTF_ERR_TIMEOUT
+        assert all(int(c) == -1 for c in cnts)
+    finally:
+        P.ttf_debug_set_wait()
+    toks, cnts, poss = P.ttf_compress_batch(Xs, r, 0.7, stream=st)
+    assert P.ttf_last_device_status(st) == B.TTF_OK
+    for t, c, p in zip(toks, cnts, poss):
+        assert int(c) == L and torch.equal(t[:L], ref[0][:L]) and torch.equal(p[:L], ref[2][:L])
 
 
 def test_status_of_caller_owned_and_built_in_scratch():
