@@ -179,8 +179,8 @@ int ttf_set_match_kernel(int which);
  * lanes in opposite phases, so that one clip is matched out of L2 while the next one streams in; the matching kernel
  * and the gather mark the lines they are done with as the first to leave L2.  On the 8B-shaped clip this takes the DRAM
  * traffic of a clip from 170 MB to 133 MB (the matching pass is served by L2 for the most part), but the sweep, the
- * matching kernel and the gather slow one another down when they share the SMs and the pass is slower than with
- * eight clips in flight (32.6 against 29.8 us per clip), which is why it is not the default.
+ * matching kernel and the gather slow one another down when they share the SMs and the pass is slower than the
+ * default (36.0 against 26.7 us per clip, 16 clips), which is why it is not the default.
  */
 #define TTF_SCHEDULE_PIPELINED (-1)
 int ttf_set_schedule(int clips_in_flight);
@@ -343,9 +343,9 @@ int ttf_query_static(const void* features, int F, int H, int W, int C, int r, fl
  * on its own stream.  ttf_profile_end waits for those events and returns, per kernel kind, the summed
  * device time in milliseconds and the number of launches; `kinds` is the length of both arrays
  * (TTF_KERNEL_KINDS covers all).  Kinds: 0 frame-sum (and norm) sweep, 1 frame statistics of the anchor rule,
- * 2 windowed match + gate (its prologue takes the anchor arg max), 3 compaction gather (with the frame-count
- * prefix of clips longer than 1024 frames), 4 nothing any more (the matching kernel counts the fused tokens of
- * ttf_query).  Profiling is process-wide and meant for benchmarks; leave it off otherwise.
+ * 2 windowed match + gate, 3 compaction gather (with the frame-count
+ * prefix of clips longer than 1024 frames).  TTF_KERNEL_KINDS leaves room for one more, which stays zero.  Profiling is
+ * process-wide and meant for benchmarks; leave it off otherwise.
  */
 #define TTF_KERNEL_KINDS 5
 int ttf_profile_begin(void);
@@ -353,10 +353,10 @@ int ttf_profile_end(double* total_ms, long long* launches, int kinds);
 
 /*
  * Steady-state duration of each kernel of the pass (no counterpart in the paper).  For `reps` rounds, each of the
- * four kernels (kinds 0..3 above) is launched back to back for all `nclips` clips of the batch, each clip on its
- * own scratch block, with one pair of CUDA events around the group; ms_per_launch[kind] = group time / nclips,
- * averaged over the rounds.  With a batch larger than L2 every launch finds its clip cold in HBM, which is how a
- * kernel runs when several clips are in flight.  Arguments as ttf_compress_batch; the outputs are those of the
+ * four kernels (kinds 0..3 above) is launched back to back for all `nclips` clips of the batch as ttf_compress_batch
+ * would launch it (once per group of clips), each clip on its own scratch block, with one pair of CUDA events around
+ * all of them; ms_per_launch[kind] = that time / nclips, averaged over the rounds.  With a batch larger than L2 every
+ * launch finds its clips cold in HBM, which is how a kernel runs when several clips are in flight.  Arguments as ttf_compress_batch; the outputs are those of the
  * pass.  Synchronises `stream`.
  */
 int ttf_profile_stages(const void* const* features, int nclips, int F, int H, int W, int C, int r, float t,

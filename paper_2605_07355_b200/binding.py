@@ -39,7 +39,7 @@ class TTFOptions(ctypes.Structure):
 
 
 TTF_STATIC_SCRATCH_BYTES = 8 << 20
-KERNEL_KINDS = ["norm_sum", "frame_stats", "match", "compact", "fuse_count"]
+KERNEL_KINDS = ["norm_sum", "frame_stats", "match", "compact", "fuse_count"]     # (the last: no kernel any more, always zero)
 
 _lib = None
 _fast = None                     # _marshal, bound to the library's functions

@@ -356,9 +356,11 @@ k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float
 // are added first and these pairs in order, whether eight CTAs hold a pair each or sixteen a unit each.  (The grid kernel
 // adds the same terms in an order of its own; which of the two a clip takes depends on its shape alone.)
 // What bounds it is a serial chain: what an SM can take in from L2 (64 KB per CTA for 32 frames of 4096 channels on eight
-// CTAs, 0.9 us; hence sixteen where the kernel runs alone), three block barriers and the cluster barrier.  With eight CTAs, two shuffle trees per frame and every warp adding up all
-// channels of g for itself a pass took, per clip, 39.3 us (32 x 16 x 16 x 4096), 28.9 (2048 channels), 134.7 (128 frames)
-// and 11.3 (4 x 8 x 8 x 64); as it stands 38.0, 28.1, 130.2 and 10.2.
+// CTAs, 0.9 us; hence sixteen where the kernel runs alone), three block barriers and the cluster barrier.
+// With eight CTAs, two shuffle trees per frame and every warp adding up all channels of g for itself a pass took, in a
+// replayed graph, 39.3 us (32 x 16 x 16 x 4096), 28.9 (2048 channels), 134.7 (128 frames) and 11.3 (4 x 8 x 8 x 64) where it
+// took 38.0, 28.1, 130.2 and 10.2; the order of summation that eight and sixteen CTAs share added nothing (39.8 -> 39.6 and
+// 28.5 -> 28.3 per call).
 constexpr int kStatClusterMaxF = 256;     // frames the cluster kernel takes (shares of all frames live in shared memory)
 
 template <int SL, int CS>     // slices of 128 channels per CTA, CTAs; warp w owns frames w, w + 8, ...

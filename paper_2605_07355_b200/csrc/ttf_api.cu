@@ -71,14 +71,13 @@ int wait_poll_limit() { return g_wait_limit.load(); }
 int wait_tx_extra() { return g_wait_tx_extra.load(); }
 
 // ---- optional per-kernel timing: CUDA events recorded around every launch while profiling is on ---------
-enum { PK_NORM_SUM = 0, PK_FRAME_STATS = 1, PK_MATCH = 2, PK_COMPACT = 3, PK_FUSE_COUNT = 4, PK_KINDS = 5 };
+enum { PK_NORM_SUM = 0, PK_FRAME_STATS = 1, PK_MATCH = 2, PK_COMPACT = 3, PK_KINDS = 4 };
 struct ProfRecord { int kind; cudaEvent_t a, b; };
 static std::mutex g_prof_mu;
 static std::atomic<bool> g_prof_on{false};
 static std::vector<ProfRecord> g_prof;
 
-static const char* const kKindNames[PK_KINDS] = {"ttf sweep", "ttf frame statistics", "ttf matching", "ttf gather",
-                                                 "ttf fuse count"};
+static const char* const kKindNames[PK_KINDS] = {"ttf sweep", "ttf frame statistics", "ttf matching", "ttf gather"};
 
 // One scope per kernel launch: an NVTX range on the host side of the launch (a no-op unless a tool that listens is
 // attached) and, while profiling is on, a pair of CUDA events around it.
@@ -634,9 +633,8 @@ struct BatchPlan { int group, lanes, sets, blocks; bool pipelined; };
 
 // Automatic: one launch of each kernel covers half of the batch (at most kMaxGroup clips), two halves in flight, so that
 // one half's kernels fill what the other's leave idle while they ramp up and drain.  Launches over single clips on
-// eight lanes were bound by the host for small clips (a clip of 1.2 MB: 16 clips 205 us, 63 us now; 7.2 MB: 12 clips
-// 162 -> 98 us) and were no faster for large ones (33 MB: 16 clips 304 -> 300 us; 67 MB: 517 -> 515; 268 MB, 8 clips:
-// 910 -> 911).  All clips in one launch, or one lane, leave the second half's ramp and tail uncovered (33 MB: 306 and
+// eight lanes were bound by the host for small clips (a clip of 1.2 MB: 16 clips 300 us, 42 us now) and were no faster for large ones (33 MB: 16 clips 304 -> 300 us; 67 MB: 517 -> 515; 268 MB, 8 clips:
+// 910 -> 911, all with the warp-level matching kernel of the time).  All clips in one launch, or one lane, leave the second half's ramp and tail uncovered (33 MB: 306 and
 // 330 us); more than two lanes of smaller groups gain nothing (within 2 % for every clip size measured).
 // Scratch: 16 blocks in all for eight clips or more, 32 for more than 16; so few sizes that the lanes' scratch soon stays
 // as it is, whatever the number of clips.

@@ -11,7 +11,7 @@
 // fp32 pipes are within a few per cent of each other at r = 1 (68 against 89 cycles of an SM per warp and stage), and
 // both stay below what an SM takes in from L2 (FR + WIN rows per stage).  The CUDA-core kernel that it
 // replaced here gave a warp one token and read every window row again for every token: on a 32 x 16 x 16 clip of 1152
-// channels 67 us of a pass of 81.8 us; the pass takes 32.5 us now (no norms in the sweep either).
+// channels 67 us of a pass of 81.8 us; the pass takes 30.3 us now (no norms in the sweep either).
 #include <cuda.h>
 
 #include "ttf_internal.cuh"
