@@ -61,6 +61,13 @@ __device__ __forceinline__ float fold8(float (&v)[8], int lane) {
     return r;
 }
 
+// The control words of a block at the start of a call: the error word reports on this call only; a block that may hold anything
+// (fresh) also gets its arrival counter and the error word of its batch cleared.
+__device__ __forceinline__ void clear_words(int* hdr, bool fresh) {
+    hdr[HDR_ERROR] = 0;
+    if (fresh) { hdr[HDR_DONE_ALL] = 0; hdr[HDR_BATCH_ERROR] = 0; }
+}
+
 // LS: lanes across a slice (8, 16 or 32); RG = 256 / LS row groups walk the tokens interleaved.
 // CLS: a thread keeps CLS running sums, of every CLS-th of its tokens.  A sum over all tokens is the same tree whether 32
 // classes of tokens belong to 32 row groups of 8 lanes (CLS = 1), to 16 of 16 (2) or to 8 of 32 (4): class w + 8 J to warp w,
@@ -70,8 +77,9 @@ template <typename T, int V, int LS, bool NORMS, int CLS>
 __global__ void __launch_bounds__(kNormThreads)
 k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
            float* __restrict__ S, float* __restrict__ ssq, int* __restrict__ cnt, int* __restrict__ hdr,
-           int chain, size_t sstride)
+           int flags, size_t sstride)
 {
+    const bool chain = flags & 1;                   // (bit 0: chain, bit 1: fresh; see Problem)
     const T* __restrict__ X = reinterpret_cast<const T*>(xs.X[blockIdx.y]);
     S = clip_block(S, sstride); ssq = clip_block(ssq, sstride); cnt = clip_block(cnt, sstride); hdr = clip_block(hdr, sstride);
     using L = Loader<T, V>;
@@ -170,7 +178,7 @@ k_norm_sum(const __grid_constant__ ClipPtrs xs, int F, int N, int C, int nq,
         }
     }
     if (q == 0 && tid == 0) cnt[k] = 0;             // survivor counters start at zero for the matching kernel
-    if (blockIdx.x == 0 && tid == 0) hdr[HDR_ERROR] = 0;   // the error word reports on this call only
+    if (blockIdx.x == 0 && tid == 0) clear_words(hdr, flags & 2);
     if (chain && blockIdx.x == 0 && blockIdx.y == 0) pdl_wait();
     trace_mark(hdr, 0, true);
 }
@@ -179,7 +187,7 @@ template <typename T, int V, int LS, bool NORMS, int CLS = 1>
 static cudaError_t launch_sum_ls(const Problem& p, const Scratch& s, cudaStream_t st) {
     const int nq = (p.C + LS * V - 1) / (LS * V);
     return launch_ex(true, 0, k_norm_sum<T, V, LS, NORMS, CLS>, dim3((unsigned)((long long)p.F * nq), p.nclips), dim3(kNormThreads),
-                     st, p.xs, p.F, p.N, p.C, nq, s.S, s.ssq, s.cnt, s.hdr, p.chain, p.sstride);
+                     st, p.xs, p.F, p.N, p.C, nq, s.S, s.ssq, s.cnt, s.hdr, p.chain | (p.fresh << 1), p.sstride);
 }
 
 template <typename T, int V>
@@ -560,20 +568,20 @@ static cudaError_t launch_stats_cluster_t(const Problem& p, const Scratch& s, in
 // What the sweep leaves behind besides its sums, for calls that need no sweep (a fixed anchor and a matching kernel
 // that takes the token norms itself): survivor counters at zero, error word cleared.
 __global__ void __launch_bounds__(256)
-k_begin_call(int F, int* __restrict__ cnt, int* __restrict__ hdr, size_t sstride, int* fuse_cnt, int N)
+k_begin_call(int F, int* __restrict__ cnt, int* __restrict__ hdr, size_t sstride, int* fuse_cnt, int N, int fresh)
 {
     cnt = clip_block(cnt, sstride); hdr = clip_block(hdr, sstride);
     pdl_launch_dependents();
     pdl_wait();                                      // the previous call's gather may still read the counters
     for (int k = threadIdx.x; k < F; k += 256) cnt[k] = 0;
     clear_counts(fuse_cnt, N);
-    if (threadIdx.x == 0) hdr[HDR_ERROR] = 0;
+    if (threadIdx.x == 0) clear_words(hdr, fresh);
 }
 
 cudaError_t launch_norm_sum(const Problem& p, const Scratch& s, cudaStream_t st) {
     if (p.anchor_mode != 0 && !needs_sweep_norms(p))           // Eq. (auto_anchor) is not evaluated: no pass over X
         return launch_ex(true, 0, k_begin_call, dim3(1, p.nclips), dim3(256), st, p.F, s.cnt, s.hdr, p.sstride,
-                         p.fuse_cnt, p.N);
+                         p.fuse_cnt, p.N, p.fresh);
     if (p.dtype == 0) return p.vec ? launch_sum_t<float, 4>(p, s, st) : launch_sum_t<float, 1>(p, s, st);
     return p.vec ? launch_sum_t<bf16_t, 8>(p, s, st) : launch_sum_t<bf16_t, 1>(p, s, st);
 }

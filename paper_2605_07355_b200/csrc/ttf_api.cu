@@ -156,7 +156,7 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
     p->nsl = C % 4 == 0 ? (C + 127) / 128 : (C + 31) / 32;
     p->anchor_mode = 0; p->anchor_arg = 0; p->emit_anchor = 1; p->pos_t_offset = 0; p->pos_base = 0; p->natural_order = 0;
     p->use_tc = choose_match(*p);
-    p->fuse_cnt = nullptr; p->chain = 0; p->chain_next = 0; p->overlapped = 0; p->stream_once = 0;
+    p->fuse_cnt = nullptr; p->fresh = 0; p->chain = 0; p->chain_next = 0; p->overlapped = 0; p->stream_once = 0;
     return TTF_OK;
 }
 
@@ -168,19 +168,22 @@ struct CacheEntry {
     std::vector<const int*> status_words;        // header blocks the most recent call on this stream used
     int status_index = HDR_ERROR;                // ... and the word of each that tells how it went
 };
+typedef std::map<std::pair<int, cudaStream_t>, CacheEntry> ScratchCache;
 static std::mutex g_mu;
-static std::map<std::pair<int, cudaStream_t>, CacheEntry> g_scratch;
+static ScratchCache g_scratch;
+static ScratchCache g_batch_scratch;             // of small batches (batch_on_stream), apart from the scratch of other calls:
+                                                 // batches may be enqueued from several threads
 
 // `bytes` of scratch for a call on `st`; `unit` is the scratch of one of its clips.  The block moves when a larger clip
 // arrives.  A block that is too small because the call has more clips than those before it is kept beside its successor:
 // a graph captured with fewer clips of the same shape points into it.  (Every successor is at least twice as large, so all
 // of them together stay below the current block; a larger clip or ttf_release gives them back.)
-static int cached_scratch(size_t bytes, size_t unit, cudaStream_t st, void** out) {
+static int cached_scratch(size_t bytes, size_t unit, cudaStream_t st, void** out, ScratchCache& cache = g_scratch) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
     std::lock_guard<std::mutex> lk(g_mu);
-    CacheEntry& ce = g_scratch[std::make_pair(dev, st)];
+    CacheEntry& ce = cache[std::make_pair(dev, st)];
     if (ce.bytes < bytes) {
         if (ce.ptr && unit > ce.unit) {
             // earlier calls on this stream may still read the old blocks
@@ -208,12 +211,12 @@ static int cached_scratch(size_t bytes, size_t unit, cudaStream_t st, void** out
     ce.status_index = HDR_ERROR;
     return TTF_OK;
 }
-static size_t scratch_held(cudaStream_t st) {
+static size_t scratch_held(cudaStream_t st, ScratchCache& cache = g_scratch) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lk(g_mu);
-    auto it = g_scratch.find(std::make_pair(dev, st));
-    return it == g_scratch.end() ? 0 : it->second.bytes;
+    auto it = cache.find(std::make_pair(dev, st));
+    return it == cache.end() ? 0 : it->second.bytes;
 }
 static int cached_scratch(size_t bytes, cudaStream_t st, void** out) { return cached_scratch(bytes, bytes, st, out); }
 
@@ -627,6 +630,27 @@ static int batch_lanes(BatchLanes** out) {
     return TTF_OK;
 }
 
+// Batches of few bytes: groups of up to eight clips, one after the other on the caller's own stream.  What bounds such a
+// batch is the number of things that are enqueued: forking to two lanes and joining them again is two memsets and seven calls
+// on events besides the launches, and each edge between streams costs the GPU some microseconds.  Us per pass, lanes / own
+// stream: 6 clips of 4 x 8 x 10 x 1288 35.6 / 23.6, 7 of 26 x 8 x 10 x 120 34.1 / 20.0, 8 of 16 x 14 x 14 x 512 (26 MB)
+// 35.1 / 29.0, 4 of 24 x 16 x 16 x 1024 (50 MB) 40.0 / 30.9; with 67 MB in all 64.5 / 65.3 (8 of 8 x 16 x 16 x 2048), 48.7 /
+// 49.5, 44.3 / 36.9, 42.8 / 36.5; with 118 MB 73.8 / 81.2: the lanes fill each other's ramps.  Without a sweep (fixed anchors)
+// 25.7 MB 30.4 / 21.9, 67 MB 54.6 / 49.9 and 40.1 / 35.3, 134 MB 58.3 / 55.3, 157 MB 70.7 / 67.8, 201 MB 81.4 / 79.9, 335 MB
+// 132.6 / 135.7.  Nine to sixteen clips are two launches of each kernel, which do not overlap here: 14 MB 40.2 / 37.2, 28 MB
+// 40.1 / 39.4, 51 MB 49.7 / 62.3 (fixed anchors 32 MB 33.7 / 27.6, 51 MB 40.3 / 45.1), and in a replayed graph, where the
+// host's part is gone, 1.3 MB 18.2 / 23.7: not in a capture.
+constexpr int kInlineClips = 16, kInlineGroup = 8;
+constexpr size_t kInlineStreams = 64;            // streams that hold scratch for it; on further ones the lanes take the batch
+
+static bool takes_own_stream(const Problem& p, int nclips, bool same_layout, bool capturing, cudaStream_t st) {
+    if (st == cudaStreamPerThread) return false;                     // (one handle, another stream in every thread)
+    if (g_sched_lanes.load() != 0 || !same_layout || nclips > kInlineClips || (nclips > kInlineGroup && capturing)) return false;
+    const double mb = (double)p.F * p.N * p.C * (p.dtype == TTF_DTYPE_F32 ? 4e-6 : 2e-6) * nclips;
+    const bool sweep = p.anchor_mode == 0 || needs_sweep_norms(p);
+    return mb <= (nclips <= kInlineGroup ? (sweep ? 64.0 : 160.0) : (sweep ? 16.0 : 32.0));
+}
+
 // How a batch is cut into launches: `group` clips per launch, `lanes` groups in flight, `sets` of `group` scratch blocks
 // per lane, `blocks` of scratch blocks to hold per lane.
 struct BatchPlan { int group, lanes, sets, blocks; bool pipelined; };
@@ -642,7 +666,7 @@ struct BatchPlan { int group, lanes, sets, blocks; bool pipelined; };
 // a launch: single clips on all lanes, since the element-wise kernels of one clip alone leave much of the GPU idle (16 clips
 // of 32 x 16 x 16 x 1024, every second one 2 bytes off: 1247 us per batch on two lanes, 1027 on eight; 16 of 8 x 12 x 12 x 512, every
 // fourth one off, in a replayed graph: 238 and 140).
-static BatchPlan plan_batch(const Problem& p, int nclips, bool same_layout) {
+static BatchPlan plan_batch(const Problem& p, int nclips, bool same_layout, bool own_stream = false) {
     BatchPlan b;
     const int want = g_sched_lanes.load();
     b.pipelined = want == TTF_SCHEDULE_PIPELINED && nclips >= 3 && p.anchor_mode == 0;
@@ -650,7 +674,12 @@ static BatchPlan plan_batch(const Problem& p, int nclips, bool same_layout) {
     if (b.pipelined) { b.lanes = 2; return b; }
     if (want >= 1 && want <= kBatchStreams) b.lanes = want;          // ttf_set_schedule: so many single clips in flight
     else if (!same_layout) b.lanes = kBatchStreams;
-    else {
+    else if (own_stream) {
+        b.group = nclips <= kInlineGroup ? nclips : (nclips + 1) / 2;
+        b.lanes = b.sets = b.blocks = 1;
+        while (b.blocks < b.group) b.blocks *= 2;
+        return b;
+    } else {
         b.group = (nclips + 1) / 2 < kMaxGroup ? (nclips + 1) / 2 : kMaxGroup;
         b.lanes = 2;
         b.sets = b.blocks = 1;
@@ -691,15 +720,71 @@ static GroupLaunch group_launch(const BatchPlan& plan, const Problem& like, cons
     return g;
 }
 
+// The caller asks about a batch through its own stream: point that at the error words of the batch's blocks.
+static void report_batch(cudaStream_t st, const std::vector<const int*>& words) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lk(g_mu);
+    CacheEntry& ce = g_scratch[std::make_pair(dev, st)];
+    ce.status_words = words;
+    ce.status_index = HDR_BATCH_ERROR;           // (groups that use the same blocks in turn clear the other word)
+}
+
+// Scratch of the lanes of `plan`.  Where it cannot grow, inside a capture or for lack of memory, the groups become as large as
+// what the lanes hold allows.
+static int lanes_scratch(BatchLanes* L, BatchPlan* plan, size_t stride, bool capturing, std::vector<void*>* ws) {
+    ws->assign(plan->lanes, nullptr);
+    for (int i = 0; i < plan->lanes; ++i) {
+        const size_t held = scratch_held(L->s[i]) / stride;
+        int blocks = plan->blocks, rc;
+        if (capturing && held >= (size_t)plan->sets && held < (size_t)blocks) blocks = (int)held;
+        while ((rc = cached_scratch(blocks * stride, stride, L->s[i], &(*ws)[i])) != TTF_OK) {
+            if (blocks == plan->sets) return rc;
+            cudaGetLastError();
+            blocks = blocks / 2 > plan->sets ? blocks / 2 : plan->sets;
+        }
+        if (plan->group > blocks / plan->sets) plan->group = blocks / plan->sets;
+    }
+    return TTF_OK;
+}
+
+// `plan`: the groups on the stream.  Returns false, with nothing enqueued, where the stream has no scratch and cannot get it
+// (inside a capture, or for lack of memory).  The lanes get the scratch that the batch would take there too (`over_lanes`): a
+// later capture, which cannot allocate, may be on a stream that has none.
+static bool batch_on_stream(BatchLanes* L, const BatchPlan& plan, BatchPlan over_lanes, const Problem& like, const ttf_options* options, size_t stride, bool capturing,
+                            const void* const* features, int nclips, void* const* out_tokens, int* const* out_count,
+                            int* const* out_pos_thw, cudaStream_t st, int* rc) {
+    const size_t held = scratch_held(st, g_batch_scratch);
+    if (held < plan.blocks * stride) {
+        std::lock_guard<std::mutex> lk(g_mu);
+        if (capturing || (!held && g_batch_scratch.size() >= kInlineStreams)) return false;
+    }
+    void* ws = nullptr;
+    *rc = cached_scratch(plan.blocks * stride, stride, st, &ws, g_batch_scratch);
+    if (*rc != TTF_OK) {
+        cudaGetLastError();
+        return false;
+    }
+    std::vector<void*> unused;
+    if (!capturing && lanes_scratch(L, &over_lanes, stride, false, &unused) != TTF_OK) cudaGetLastError();
+    std::vector<const int*> words;
+    for (int i = 0; i < plan.group; ++i) words.push_back(reinterpret_cast<const int*>((char*)ws + i * stride));
+    report_batch(st, words);
+    for (int n0 = 0; n0 < nclips && *rc == TTF_OK; n0 += plan.group) {
+        GroupLaunch g = group_launch(plan, like, options, stride, features, nclips, n0, out_tokens, out_count, out_pos_thw);
+        g.p.fresh = n0 == 0 ? 1 : 0;             // (the blocks may hold another shape's data)
+        *rc = compress_impl(g.p, ws, g.out, st);
+    }
+    return true;
+}
+
 // A lane takes its groups one after the other on its stream.  Lanes of single clips (two sets of scratch blocks used in
 // turn) chain them: the sweep of a clip runs beside the gather of the clip before it.
 static int batch_on_streams(const void* const* features, int nclips, int F, int H, int W, int C, int r, float t,
                             int dtype, const ttf_options* options,
                             void* const* out_tokens, int* const* out_count, int* const* out_pos_thw, cudaStream_t st) {
     std::lock_guard<std::mutex> enqueue(g_lane_mu);
-    BatchLanes* L = nullptr;
-    int rc = batch_lanes(&L);
-    if (rc != TTF_OK) return rc;
+    int rc = TTF_OK;
     // every clip is validated (and the largest scratch layout found) before anything is enqueued
     Problem p0;
     bool same_layout = true;                     // clips of one launch share the vector path or the scalar path
@@ -716,24 +801,21 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         if (n == 0) p0 = p;
         same_layout = same_layout && p.vec == p0.vec && (!p.vec || aligned(n) == aligned(0));
     }
-    BatchPlan plan = plan_batch(p0, nclips, same_layout);
-    // Scratch (before the fork, outside the event bracket).  Where it cannot grow, inside a capture or for lack of memory, the
-    // groups are as large as what the lanes hold allows.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &capture);
     if (e != cudaSuccess) return cuda_fail(e);
-    std::vector<void*> ws(plan.lanes, nullptr);
-    for (int i = 0; i < plan.lanes; ++i) {
-        const size_t held = scratch_held(L->s[i]) / stride;
-        int blocks = plan.blocks;
-        if (capture != cudaStreamCaptureStatusNone && held >= (size_t)plan.sets && held < (size_t)blocks) blocks = (int)held;
-        while ((rc = cached_scratch(blocks * stride, stride, L->s[i], &ws[i])) != TTF_OK) {
-            if (blocks == plan.sets) return rc;
-            cudaGetLastError();
-            blocks = blocks / 2 > plan.sets ? blocks / 2 : plan.sets;
-        }
-        if (plan.group > blocks / plan.sets) plan.group = blocks / plan.sets;
-    }
+    const bool capturing = capture != cudaStreamCaptureStatusNone;
+    BatchLanes* L = nullptr;
+    rc = batch_lanes(&L);
+    if (rc != TTF_OK) return rc;
+    BatchPlan plan = plan_batch(p0, nclips, same_layout);
+    if (takes_own_stream(p0, nclips, same_layout, capturing, st) &&
+        batch_on_stream(L, plan_batch(p0, nclips, true, true), plan, p0, options, stride, capturing, features, nclips,
+                        out_tokens, out_count, out_pos_thw, st, &rc))
+        return rc;
+    std::vector<void*> ws;                       // (before the fork, outside the event bracket)
+    rc = lanes_scratch(L, &plan, stride, capturing, &ws);
+    if (rc != TTF_OK) return rc;
     const int groups = (nclips + plan.group - 1) / plan.group;
     const int lanes = plan.lanes;
     const size_t set = (size_t)plan.group * stride;
@@ -783,15 +865,7 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         if (e == cudaSuccess) { ProfScope pr(ls, PK_COMPACT); e = launch_compact(p, sc, out, ls); }
         if (e != cudaSuccess) first_rc = cuda_fail(e);
     }
-    {   // the caller asks about the batch through its own stream: point it at the lanes' error words
-        int dev = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess) {
-            std::lock_guard<std::mutex> lk(g_mu);
-            CacheEntry& ce = g_scratch[std::make_pair(dev, st)];
-            ce.status_words = words;
-            ce.status_index = HDR_BATCH_ERROR;   // (groups that use the same blocks in turn clear the other word)
-        }
-    }
+    report_batch(st, words);
     // always join, also after a failed launch, so that the caller's stream (or capture) is whole again
     for (int i = 0; i < lanes; ++i) {
         cudaError_t e2 = cudaEventRecord(L->join[i], L->s[i]);
@@ -1181,14 +1255,16 @@ int ttf_release(void) {
     int cur = 0;
     cudaGetDevice(&cur);
     cudaError_t first = cudaSuccess;
-    for (auto& kv : g_scratch) {
-        cudaSetDevice(kv.first.first);
-        cudaError_t e = cudaDeviceSynchronize();
-        if (e != cudaSuccess && first == cudaSuccess) first = e;
-        if (kv.second.ptr) cudaFree(kv.second.ptr);
-        for (void* q : kv.second.outgrown) cudaFree(q);
+    for (ScratchCache* cache : {&g_scratch, &g_batch_scratch}) {
+        for (auto& kv : *cache) {
+            cudaSetDevice(kv.first.first);
+            cudaError_t e = cudaDeviceSynchronize();
+            if (e != cudaSuccess && first == cudaSuccess) first = e;
+            if (kv.second.ptr) cudaFree(kv.second.ptr);
+            for (void* q : kv.second.outgrown) cudaFree(q);
+        }
+        cache->clear();
     }
-    g_scratch.clear();
     for (auto& kv : g_staging) {
         cudaSetDevice(kv.first);
         cudaError_t e = cudaDeviceSynchronize();

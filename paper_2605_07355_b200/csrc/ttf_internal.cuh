@@ -56,6 +56,7 @@ struct Problem {
     int use_tc;         // 1: the matching step runs on tcgen05 (ttf_match_tc.cu)
     int* fuse_cnt;      // [N] the query's counts of tokens fused into each anchor cell, or NULL: zeroed between the
                         // sweep and the matching kernel, which counts (single clips only)
+    int fresh;          // 1: the scratch blocks may hold anything: the first kernel clears their control words
     int chain;          // 1: the kernel before this call's sweep in the stream is the gather of the library's previous
                         // clip, which works on another scratch block: the sweep may run beside it
     int chain_next;     // 1: the kernel after this call's gather is such a sweep
