@@ -117,7 +117,6 @@ inline bool needs_sweep_norms(const Problem& p) {
 
 // tcgen05 matching (ttf_match_tc.cu)
 bool tc_match_eligible(const Problem& p);
-int tc_match_chunks(const Problem& p);
 size_t tc_match_tiles(const Problem& p);
 cudaError_t launch_match_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                             unsigned char* keep, cudaStream_t st);

@@ -2,15 +2,19 @@
 // clips on the fifth-generation tensor cores: TMA tensor tiles -> shared memory -> tcgen05.mma -> tensor memory.
 //
 // All tokens of a grid cell share their candidate set, and neighbouring cells share most of it, so the unit of
-// work is a TILE of 128 source rows = 32 frames x a strip of 4 cells of one grid row, against the
-// (2r+1) x (4+2r) anchor cells around the strip (18 for r = 1): one dense contraction
-//     D[128 x NB] = A[128 x C] . B[NB x C]^T,     NB = 16 / 32 / 48 >= (2r+1)(4+2r),
-// of which every source row uses its own (2r+1)^2 columns.  Operand traffic is (128 + 18) / 128 = 1.14 x |X| for
-// r = 1 instead of 41 / 32 when every cell fetches its own 9 candidates.
+// work is a TILE of 128 source rows = FR frames x WY grid rows x 4 cells (FR = 32 / WY, WY = 1, 2 or 4), against the
+// (WY+2r) x (4+2r) anchor cells around them: one dense contraction
+//     D[128 x NB] = A[128 x C] . B[NB x C]^T,     NB = 16 / 32 / 48 >= (WY+2r)(4+2r),
+// of which every source row uses its own (2r+1)^2 columns.  Operand traffic is (128 + 18) / 128 = 1.14 x |X| for 32 frames at
+// r = 1 instead of 41 / 32 when every cell fetches its own 9 candidates.  Frames that a clip does not have are rows of zeros:
+// they cost no traffic, but the stages, norms and epilogue of a whole tile, so clips of few frames take tiles of fewer frames
+// and more grid rows (tile_rows; against 32 frames throughout, us per pass: 8 clips of 8 x 32 x 32 x 1024 128 -> 76, 16 of
+// 8 x 16 x 16 x 1024 71 -> 46, 7 of 6 x 12 x 7 x 1944 25.4 -> 16.9, 6 of 48 x 14 x 14 x 1024 71.9 -> 64.6, one of
+// 9 x 16 x 16 x 4096 26.4 -> 22.8, of 5 x 29 x 13 x 1016 at r = 2 20.2 -> 18.4).
 //
-//   A tile:  box (64 channels, 4 cells, 1 row, 32 frames) of X viewed as [F, H, W, C]; row m = 4 * frame + cell.
-//   B tile:  box (64 channels, 4 + 2r cells, 2r + 1 rows, 1 frame) at frame a*, starting r cells up and left of the
-//            strip; cells outside the grid arrive as zeros and are left out of the arg max (window clipped to the
+//   A tile:  box (64 channels, 4 cells, WY rows, FR frames) of X viewed as [F, H, W, C]; row m = (frame, cell row, cell).
+//   B tile:  box (64 channels, 4 + 2r cells, WY + 2r rows, 1 frame) at frame a*, starting r cells up and left of the
+//            tile; cells outside the grid arrive as zeros and are left out of the arg max (window clipped to the
 //            grid, Eq. pi, with the duplicates of the clipping masked).
 //   Both arrive with the 128-byte swizzle, which is the K-major operand layout of tcgen05.mma; a pipeline stage is
 //   64 channels (4 MMAs of K = 16).  fp32 accumulation in tensor memory; bf16 products are exact in fp32.
@@ -45,8 +49,7 @@
 namespace ttf {
 
 constexpr int kTcWB = 4;                 // cells per strip
-constexpr int kTcFR = 32;                // frames per tile
-constexpr int kTcM = kTcWB * kTcFR;      // 128 source rows = tensor-memory lanes
+constexpr int kTcM = 128;                // source rows of a tile = tensor-memory lanes
 constexpr int kTcKC = 64;                // channels per stage (128 bytes: one swizzle row)
 constexpr int kTcABytes = kTcM * 128;    // 16 KB
 constexpr int kTcThreads = 192;
@@ -116,17 +119,18 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int NB) {
 }
 
 // ---- the kernel -------------------------------------------------------------------------------------------
-template <int R> struct TcShape {
+template <int R, int WY> struct TcShape {
+    static constexpr int FR = kTcM / (kTcWB * WY);        // frames per tile
     static constexpr int SIDE = 2 * R + 1;
-    static constexpr int BW = kTcWB + 2 * R;              // candidate cells per window row
-    static constexpr int NCAND = SIDE * BW;               // rows the B box delivers
+    static constexpr int BW = kTcWB + 2 * R, BH = WY + 2 * R;      // candidate cells: columns, rows
+    static constexpr int NCAND = BW * BH;                 // rows the B box delivers
     static constexpr int NB = (NCAND + 15) / 16 * 16;     // MMA N
     static constexpr int BBYTES = NB * 128;
     static constexpr int BBOX = NCAND * 128;              // bytes one B box copy delivers
     static constexpr int STAGE = kTcABytes + BBYTES;
     static constexpr int STAGES = 4;                      // two CTAs per SM with room left for CTAs of other kernels
     static constexpr int WIN = SIDE * SIDE;               // candidates of one source row
-    static constexpr int MAXCH = R == 2 ? 4 : 8;          // chunks at most (tensor memory: MAXCH * NB <= 256 columns)
+    static constexpr int MAXCH = NB > 32 ? 4 : 8;         // chunks at most (tensor memory: MAXCH * NB <= 256 columns)
     // what one rank sends another (and itself): window sums and squared norms of the rows the other one finishes,
     // squared norms of the candidates
     static constexpr int XBYTES = (kTcM * (WIN + 1) + MAXCH * NCAND) * 4;                 // received by one rank
@@ -158,13 +162,13 @@ __device__ __forceinline__ float ssq8(const uint4& v, float acc) {
     return acc;
 }
 
-template <int R, int G>
+template <int R, int WY, int G>
 __global__ void __launch_bounds__(kTcThreads)
 k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc, int lpieces, int lchunks,
            float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
            int wait_limit, int tx_extra, int stream_once, size_t sstride, int* fuse_cnt)
 {
-    using S = TcShape<R>;
+    using S = TcShape<R, WY>;
     const bool backwards = gridDim.y == 1 || stream_once;
     const unsigned clip = backwards ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
     const CUtensorMap& mapA = maps.a[clip];
@@ -186,9 +190,10 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     const int pieces = 1 << lpieces;
     const int tile = (int)(walk >> lpieces);
     const int piece = pieces > 1 ? (int)cluster_rank() : 0;        // = blockIdx.x % pieces
-    const int kg = tile / (H * xs_n), rem = tile - kg * (H * xs_n);
-    const int y = rem / xs_n, x0 = (rem - y * xs_n) * kTcWB;
-    const int k0 = kg * kTcFR;
+    const int ys_n = (H + WY - 1) / WY;
+    const int kg = tile / (ys_n * xs_n), rem = tile - kg * (ys_n * xs_n);
+    const int y0 = rem / xs_n * WY, x0 = rem % xs_n * kTcWB;
+    const int k0 = kg * S::FR;
     const int nst_all = (C + kTcKC - 1) / kTcKC;
     const int nch = 1 << (lchunks - lpieces);              // this CTA's chunks: ch0 .. ch0 + nch - 1
     const int ch0 = piece * nch;
@@ -213,8 +218,9 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
         tensormap_prefetch(&mapB);
     }
     // the B rows beyond the box (NCAND .. NB-1) are never written by a copy: zero them once
-    for (int i = tid; i < S::STAGES * (S::BBYTES - S::BBOX) / 16; i += kTcThreads) {
-        const int s = i / ((S::BBYTES - S::BBOX) / 16), o = i - s * ((S::BBYTES - S::BBOX) / 16);
+    constexpr int PAD = (S::BBYTES - S::BBOX) / 16;        // 16-byte pieces per stage
+    for (int i = tid; i < S::STAGES * PAD; i += kTcThreads) {
+        const int s = i / (PAD > 0 ? PAD : 1), o = i - s * PAD;
         reinterpret_cast<uint4*>(dyn + (size_t)s * S::STAGE + kTcABytes + S::BBOX)[o] = make_uint4(0, 0, 0, 0);
     }
     fence_async_smem();
@@ -237,11 +243,11 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
 
     // epilogue-thread state that outlives the role code
     const int q = warp & 3;                                // tensor-memory lane quadrant an epilogue warp may read
-    const int m = q * 32 + lane;                           // source row of an epilogue thread: 4 * frame + cell
+    const int m = q * 32 + lane;                           // source row of an epilogue thread: (frame, cell row, cell column)
     const int et = (warp - 2) * 32 + lane;                 // 0..127 among the epilogue threads
     float* const s_na = reinterpret_cast<float*>(dyn + S::RING + S::XBYTES);      // [chunk][row] squared norms
     float* const s_nbp = s_na + S::MAXCH * kTcM;           // [chunk][candidate row, piece column]
-    const int dx = m & 3;
+    const int dx = m & 3, dy = (m >> 2) & (WY - 1);
     float win[S::WIN];                                     // this row's window of dot products
     float na = 0.f, nb = 0.f;                              // squared norm of source row m / of candidate row et
 
@@ -259,9 +265,9 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
                 mbar_arrive_expect_tx(&bar_full[s], kTcABytes + S::BBOX + (uint32_t)tx_extra);   // (extra: test hook only)
                 // source rows are read by this tile alone: in a schedule that streams the next clip into L2 meanwhile,
                 // their lines are the ones to give up first (the candidate rows are shared with neighbouring tiles)
-                if (stream_once) tma_load_4d_hint(sa, &mapA, c0, x0, y, k0, &bar_full[s], once);
-                else tma_load_4d(sa, &mapA, c0, x0, y, k0, &bar_full[s]);
-                tma_load_4d(sa + kTcABytes, &mapB, c0, x0 - R, y - R, a, &bar_full[s]);
+                if (stream_once) tma_load_4d_hint(sa, &mapA, c0, x0, y0, k0, &bar_full[s], once);
+                else tma_load_4d(sa, &mapA, c0, x0, y0, k0, &bar_full[s]);
+                tma_load_4d(sa + kTcABytes, &mapB, c0, x0 - R, y0 - R, a, &bar_full[s]);
                 issued = it + 1;
             }
             trace_mark_any(asrc.hdr, 12, false); trace_mark_any(asrc.hdr, 12, true);   // all copies issued
@@ -363,7 +369,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
                 tmem_ld<NG>(lanes + (uint32_t)(h * S::NB), x);
                 tmem_ld<NG>(lanes + (uint32_t)((h + 1) * S::NB), z);
                 tmem_add<NG>(x, z);
-                if (h == 4) {
+                if (S::MAXCH > 4 && h == 4) {
                     uint32_t u[NG][8];
                     tmem_ld<NG>(lanes + (uint32_t)(6 * S::NB), u);
                     tmem_ld<NG>(lanes + (uint32_t)(7 * S::NB), z);
@@ -374,14 +380,19 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
                 tmem_add<NG>(d, x);
             }
         }
-        // this row's window: candidate (dy, ddx) is column (dy + R) * BW + dx + ddx + R of the tile
+        // this row's window: candidate (wy, wx) is column (dy + wy) * BW + dx + wx of the tile
         const uint32_t by1 = (dx & 1) ? 0xffffffffu : 0u, by2 = (dx & 2) ? 0xffffffffu : 0u;
-        auto col = [&](int n) { return d[n / 8][n % 8]; };
+        const uint32_t dy1 = (dy & 1) ? 0xffffffffu : 0u, dy2 = (dy & 2) ? 0xffffffffu : 0u;
+        auto col = [&](int yy, int n) { return d[(yy * S::BW + n) / 8][(yy * S::BW + n) % 8]; };
+        auto col2 = [&](int yy, int n) { return WY > 2 ? pick(dy2, col(yy + (WY > 2 ? 2 : 0), n), col(yy, n)) : col(yy, n); };
+        auto row_col = [&](int yy, int n) { return WY > 1 ? pick(dy1, col2(yy + (WY > 1 ? 1 : 0), n), col2(yy, n)) : col2(yy, n); };
 #pragma unroll
         for (int wy = 0; wy < S::SIDE; ++wy) {
-            uint32_t e[S::SIDE + 2];
+            uint32_t c[S::BW], e[S::SIDE + 2];
 #pragma unroll
-            for (int n = 0; n < S::SIDE + 2; ++n) e[n] = pick(by1, col(wy * S::BW + n + 1), col(wy * S::BW + n));
+            for (int n = 0; n < S::BW; ++n) c[n] = row_col(wy, n);
+#pragma unroll
+            for (int n = 0; n < S::SIDE + 2; ++n) e[n] = pick(by1, c[n + 1], c[n]);
 #pragma unroll
             for (int wx = 0; wx < S::SIDE; ++wx) win[wy * S::SIDE + wx] = __uint_as_float(pick(by2, e[wx + 2], e[wx]));
         }
@@ -436,9 +447,9 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
             na = 1.0f / fmaxf(sqrtf(na), kNormFloor);
             epilogue_bar_sync();
         }
-        const int k = k0 + (row >> 2), cell = row & 3, x = x0 + cell;
+        const int k = k0 + row / (kTcWB * WY), cell = row & 3, cy = (row >> 2) & (WY - 1), x = x0 + cell, y = y0 + cy;
         const bool mine = pieces > 1 ? et < per : true;
-        if (mine && k < F && x < W && in_bounds(asrc.hdr, 3, (long long)k * N + (long long)y * W + x, (long long)F * N)) {
+        if (mine && k < F && x < W && y < H && in_bounds(asrc.hdr, 3, (long long)k * N + (long long)y * W + x, (long long)F * N)) {
             const size_t f = (size_t)k * N + (size_t)y * W + x;
             if (k == a) {                                  // anchor tokens are always retained (Eq. mask)
                 shat[f] = 1.0f; dst[f] = y * W + x; keep[f] = 1;
@@ -450,7 +461,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
 #pragma unroll
                     for (int wx = 0; wx < S::SIDE; ++wx) {
                         const int yy = y + wy - R, xx = x + wx - R;
-                        const float sim = win[wy * S::SIDE + wx] * na * s_rb[wy * S::BW + cell + wx];
+                        const float sim = win[wy * S::SIDE + wx] * na * s_rb[(cy + wy) * S::BW + cell + wx];
                         const bool take = ((unsigned)yy < (unsigned)H) & ((unsigned)xx < (unsigned)W) & ((sim > best) | (best_j < 0));
                         best = take ? sim : best;
                         best_j = take ? yy * W + xx : best_j;
@@ -512,9 +523,22 @@ bool tc_match_eligible(const Problem& p) {
     return (long long)tc_match_tiles(p) * 8 < (1LL << 31);
 }
 
-size_t tc_match_tiles(const Problem& p) {
-    return (size_t)((p.F + kTcFR - 1) / kTcFR) * p.H * ((p.W + kTcWB - 1) / kTcWB);
+static size_t tiles_of(const Problem& p, int wy) {
+    const int fr = kTcM / (kTcWB * wy);
+    return (size_t)((p.F + fr - 1) / fr) * ((p.H + wy - 1) / wy) * ((p.W + kTcWB - 1) / kTcWB);
 }
+// Grid rows of a tile (1, 2 or 4, hence 32, 16 or 8 frames): the one with the fewest rows to fetch, padding and candidates
+// included.  (r = 2 with four rows would need 64 columns of 128 registers.)
+static int tile_rows(const Problem& p) {
+    int best = 1;
+    size_t least = 0;
+    for (int wy = 1; wy <= (p.r == 2 ? 2 : 4); wy *= 2) {
+        const size_t rows = tiles_of(p, wy) * (kTcM + (kTcWB + 2 * p.r) * (wy + 2 * p.r));
+        if (wy == 1 || rows < least) { least = rows; best = wy; }
+    }
+    return best;
+}
+size_t tc_match_tiles(const Problem& p) { return tiles_of(p, tile_rows(p)); }
 
 // Parts of a tile's channel range: the largest power of two with which a launch over one clip still fits the GPU in one
 // wave of two CTAs per SM, at most 8 (4 for r = 2) and at least 2 stages each (4 stages: 16 x 8 x 8 x 512 13.9 us per pass,
@@ -527,23 +551,23 @@ static int split_of(const Problem& p, long long tiles, int most) {
     while (n * 2 <= most && tiles * (n * 2) <= 2LL * sm_count() && nst / (n * 2) >= 2) n *= 2;
     return n;
 }
-int tc_match_chunks(const Problem& p) { return split_of(p, (long long)tc_match_tiles(p), p.r == 2 ? 4 : 8); }
 
-template <int R, int G>
+
+template <int R, int WY, int G>
 static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                unsigned char* keep, cudaStream_t st) {
-    using S = TcShape<R>;
+    using S = TcShape<R, WY>;
     ClipMaps<G> maps;
     for (int n = 0; n < p.nclips; ++n)
-        if (!make_tensor_map(&maps.a[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, kTcWB, 1, kTcFR, true) ||
-            !make_tensor_map(&maps.b[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, S::BW, S::SIDE, 1, true))
+        if (!make_tensor_map(&maps.a[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, kTcWB, WY, S::FR, true) ||
+            !make_tensor_map(&maps.b[n], p.xs.X[n], 1, p.F, p.H, p.W, p.C, kTcKC, S::BW, S::BH, 1, true))
             return cudaErrorInvalidValue;
     // (at least 80 KB: never three CTAs on one SM while others have one or none; r = 0 would fit three)
     const size_t need = (size_t)S::RING + S::XBYTES + S::NORMBYTES + 1024, smem = need < 80 * 1024 ? 80 * 1024 : need;
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R, G>), smem);
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R, WY, G>), smem);
     if (e != cudaSuccess) return e;
-    const long long tiles = (long long)tc_match_tiles(p);
-    const int chunks = tc_match_chunks(p);
+    const long long tiles = (long long)tiles_of(p, WY);
+    const int chunks = split_of(p, tiles, S::MAXCH);
     // CTAs (= cluster size) per tile.  Three or more single clips in flight (ttf_set_schedule, clips that cannot share a launch)
     // fill the GPU together: 16 clips of 32 x 16 x 16 x 4096 on eight lanes 497 -> 445 us, on three 512 -> 506 (on two 530 ->
     // 507, but three clips, of which two share a launch, 98 -> 102).
@@ -562,20 +586,29 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
         ++n;
     }
     cfg.attrs = attr; cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, k_match_tc<R, G>, maps, p.F, p.H, p.W, p.C, p.t, make_anchor_src(p, s, out_anchor),
+    return cudaLaunchKernelEx(&cfg, k_match_tc<R, WY, G>, maps, p.F, p.H, p.W, p.C, p.t, make_anchor_src(p, s, out_anchor),
                               log2_of(pieces), log2_of(chunks), shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(), p.stream_once, p.sstride, p.fuse_cnt);
 }
 
+template <int R, int G>
+static cudaError_t launch_tc_rows(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
+                                  unsigned char* keep, cudaStream_t st) {
+    const int wy = tile_rows(p);
+    if constexpr (R < 2) if (wy == 4) return launch_tc_t<R, 4, G>(p, s, out_anchor, shat, dst, keep, st);
+    return wy == 2 ? launch_tc_t<R, 2, G>(p, s, out_anchor, shat, dst, keep, st)
+                   : launch_tc_t<R, 1, G>(p, s, out_anchor, shat, dst, keep, st);
+}
+template <int G>
+static cudaError_t launch_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
+                             unsigned char* keep, cudaStream_t st) {
+    if (p.r == 0) return launch_tc_rows<0, G>(p, s, out_anchor, shat, dst, keep, st);
+    if (p.r == 1) return launch_tc_rows<1, G>(p, s, out_anchor, shat, dst, keep, st);
+    return launch_tc_rows<2, G>(p, s, out_anchor, shat, dst, keep, st);
+}
 cudaError_t launch_match_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                             unsigned char* keep, cudaStream_t st) {
-    if (p.nclips > 1) {
-        if (p.r == 0) return launch_tc_t<0, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
-        if (p.r == 1) return launch_tc_t<1, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
-        return launch_tc_t<2, kMaxGroup>(p, s, out_anchor, shat, dst, keep, st);
-    }
-    if (p.r == 0) return launch_tc_t<0, 1>(p, s, out_anchor, shat, dst, keep, st);
-    if (p.r == 1) return launch_tc_t<1, 1>(p, s, out_anchor, shat, dst, keep, st);
-    return launch_tc_t<2, 1>(p, s, out_anchor, shat, dst, keep, st);
+    return p.nclips > 1 ? launch_tc<kMaxGroup>(p, s, out_anchor, shat, dst, keep, st)
+                        : launch_tc<1>(p, s, out_anchor, shat, dst, keep, st);
 }
 
 }  // namespace ttf

@@ -39,3 +39,19 @@ def test_bits_do_not_depend_on_the_split(shape, r, clips):
             torch.cuda.synchronize()
             assert all(int(c) == L for c in cnts)
             assert all(torch.equal(p[:L], one[2][:L]) for p in poss)
+
+
+@pytest.mark.parametrize("r", [0, 1, 2])
+@pytest.mark.parametrize("shape", [(2, 4, 4, 64), (7, 5, 4, 136), (8, 4, 9, 512), (8, 7, 3, 1032), (9, 6, 5, 264), (15, 1, 6, 200), (16, 2, 8, 520),
+                                   (16, 9, 7, 1160), (17, 4, 4, 128), (24, 8, 5, 576), (40, 4, 7, 72), (48, 6, 3, 328)])
+def test_tiles_of_fewer_frames(shape, r):
+    """tiles of 8 and 16 frames over four and two grid rows: frames, rows and cells that end inside a tile"""
+    X = corr_clip(*shape, seed=sum(shape) + r, dtype="bf16")
+    check_clip(X, r, 0.6)
+    check_clip(X, r, 0.6, anchor_mode=1)
+
+
+@pytest.mark.parametrize("shape,r,clips", [((6, 8, 8, 1024), 1, 24), ((40, 8, 8, 1024), 1, 24), ((16, 16, 16, 1024), 2, 24)])
+def test_bits_of_tiles_of_fewer_frames(shape, r, clips):
+    """a tile as a cluster, and (the second and third) as one CTA that sums all chunks itself"""
+    test_bits_do_not_depend_on_the_split(shape, r, clips)
