@@ -553,6 +553,34 @@ static int split_of(const Problem& p, long long tiles, int most) {
 }
 
 
+// How many clusters of n CTAs run at the same time on the current device (asked once).  Two CTAs fit an SM, but the places of a
+// cluster lie in one GPC: 148 SMs hold 148 clusters of two, 71 of four, 33 of eight.  (The runtime is asked about a kernel of
+// the same shape that uses no tensor memory: for one that does it counts one CTA per SM, although two run.)
+__global__ void __launch_bounds__(kTcThreads) k_cluster_places(int* p) { if (p) *p = 0; }
+static long long cluster_places(int n) {
+    constexpr int kSmem = 100 * 1024;
+    static std::mutex mu;
+    static std::map<std::pair<int, int>, long long> known;
+    int dev = 0;
+    if (n == 1 || cudaGetDevice(&dev) != cudaSuccess) return 2LL * sm_count() / n;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = known.find({dev, n});
+    if (it != known.end()) return it->second;
+    int found = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = kSmem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = n; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_cluster_places), kSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&found, k_cluster_places, &cfg) != cudaSuccess || found < 1) {
+        cudaGetLastError();
+        found = 2 * sm_count() / n;
+    }
+    return known[{dev, n}] = found;
+}
+
 template <int R, int WY, int G>
 static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                unsigned char* keep, cudaStream_t st) {
@@ -572,7 +600,12 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
     // fill the GPU together: 16 clips of 32 x 16 x 16 x 4096 on eight lanes 497 -> 445 us, on three 512 -> 506 (on two 530 ->
     // 507, but three clips, of which two share a launch, 98 -> 102).
     const int beside = p.nclips == 1 && p.overlapped >= 3 ? p.overlapped : 1;
-    const int pieces = split_of(p, tiles * p.nclips * beside, chunks);
+    // Not more than run at the same time: the cluster that has to wait for a place costs the whole main loop once more (us per
+    // pass, 32 frames of 2048 channels: 71 tiles in fours 23.4, 72 in fours 30.9, in twos 27.2; 33 in eights 19.6, 34 in
+    // eights 23.8, in fours 20.6; 12 x 24 x 24 x 2048 28.8 -> 26.0).
+    const long long units = tiles * p.nclips * beside;
+    int pieces = split_of(p, units, chunks);
+    while (pieces > 1 && units > cluster_places(pieces)) pieces /= 2;
     auto log2_of = [](int n) { int l = 0; while ((1 << l) < n) ++l; return l; };
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles * pieces), p.nclips); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;

@@ -55,3 +55,9 @@ def test_tiles_of_fewer_frames(shape, r):
 def test_bits_of_tiles_of_fewer_frames(shape, r, clips):
     """a tile as a cluster, and (the second and third) as one CTA that sums all chunks itself"""
     test_bits_do_not_depend_on_the_split(shape, r, clips)
+
+
+@pytest.mark.parametrize("tiles", [33, 34, 71, 72, 148, 149])
+def test_as_many_clusters_as_run_at_once_and_one_more(tiles):
+    X = corr_clip(3, tiles * 4, 4, 256 if tiles < 100 else 128, seed=tiles, dtype="bf16")
+    check_clip(X, 1, 0.6)
