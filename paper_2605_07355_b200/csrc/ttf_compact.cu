@@ -11,6 +11,8 @@
 #include "ttf_async.cuh"
 #include "ttf_gather.cuh"
 
+#include <algorithm>
+
 namespace ttf {
 
 // exclusive scan of the effective per-frame counts (anchor frame counts as 0) for clips with more frames
@@ -175,7 +177,7 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     trace_mark(hdr, 3, true);
 }
 
-// The same for short rows, of which a warp moves many.  A CTA owns a contiguous range of output rows.  It packs the keep
+// The same with the rows of a CTA found together.  A CTA owns a contiguous range of output rows.  It packs the keep
 // flags of a window of tokens into bit words in shared memory together with the exclusive prefix of their population
 // counts, after which the source row of any output row of the window is found by a binary search and a select in shared
 // memory: the three dependent round trips (anchor, counts, flags) are paid once per window instead of once per row.
@@ -184,11 +186,23 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
 //
 // A warp moves a batch of consecutive output rows at a time, through two slots in turn, so that the next batch is on its
 // way while this one lands: every lane issues the load of one row, and the batch leaves as one store, since the rows are
-// contiguous in the output.
-constexpr int kGatherSlot = 4096;                       // bytes of a staging slot; a warp has two
+// contiguous in the output.  Rows longer than a slot go in pieces, a piece at a time.
+//
+// What bounds it where the GPU has nothing else to do is how soon the first copies are on their way: every CTA reads the same
+// flags at the same moment, and they queue on the same cache lines of L2 (clock counts from the wait to the packed bits: 1100
+// cycles with 29 CTAs on 1 KB of flags, 2150 with 141 on 3 KB, 2850 with 341 on 8 KB, 4250 with 444 on 13 KB; one row per
+// warp at a time, which has every warp read counts and flags for itself, 5400 before its first copy).  Hence ONE CTA per SM
+// there, and the slots as large as their sum may be: us per pass with three CTAs of 8 warps and 4 KB slots / one CTA of 16
+// warps and 4 KB slots / one of 8 warps and 8 KB slots (128 KB both), in a replayed graph: 24 x 20 x 15 x 248 15.7 / 13.6 /
+// 13.8, 32 x 16 x 16 x 2048 21.8 / 20.9 / 20.8, 64 x 32 x 32 x 1024 73.8 / 69.9 / 68.9, 128 x 32 x 32 x 64 27.7 / 27.7 / 28.6;
+// from rows of 8 KB one at a time 9 x 16 x 16 x 4096 with a fixed anchor 20.9 / 20.2 / 15.4, 32 x 16 x 16 x 4096 32.8 / 31.4 /
+// 30.9.  With 64 KB of slots 24 x 20 x 15 x 248 takes 16.8 and 32 x 16 x 16 x 4096 42.5, with 192 KB 13.7 and 32.7 (the
+// sweep of the next call finds less L1).  Windows of 32768 or 65536 tokens gain nothing (128 x 16 x 16 x 512 22.1 / 22.3,
+// 64 x 24 x 24 x 512 23.8 / 26.1).
+// Where other clips' kernels run beside it the CTAs are three per SM, and long rows go one at a time: the waits of one CTA
+// are filled by others (16 clips of 32 x 16 x 16 x 4096 448 us, 457 with one CTA per SM; 8 of 24 x 20 x 20 x 1024 84.6 / 87.4).
 constexpr int kGatherWords = 512;                       // bit words of a window
 constexpr int kGatherWindow = kGatherWords * 32;        // tokens
-constexpr int kGatherThreads = kCopyWarps * 32;
 
 // 32 keep flags (0 or 1 each) -> one bit each.  (The flags are masked first: a word that reaches past the end of the
 // array holds other bytes, whose higher bits would spill into its neighbours' in the product.)
@@ -210,14 +224,17 @@ __device__ __forceinline__ int select_bit(unsigned bits, int n) {
     return at;
 }
 
-// WHOLE: the clip is one window.  Else the windows are `words` * 32 tokens.
-template <bool WHOLE>
-__global__ void __launch_bounds__(kGatherThreads)
-k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H, int W,
+// WHOLE: the clip is one window.  Else the windows are `window_words` * 32 tokens.  NW: warps; `slot`: bytes of a staging slot, of
+// which a warp has two; `pieces` of a row, or `batch` rows at most to a slot.
+template <bool WHOLE, int NW>
+__global__ void __launch_bounds__(NW * 32)
+k_compact_rows(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int H, int W,
                int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
                const unsigned char* __restrict__ keep, const __grid_constant__ OutPtrs outs, int NA, int acnt, int t_off,
-               int pos_base, int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride, int window_words)
+               int pos_base, int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride, int window_words,
+               unsigned per_magic, int pieces, int batch, int slot)
 {
+    constexpr int kThreads = NW * 32;
     const int words = WHOLE ? kGatherWords : window_words;
     const unsigned char* __restrict__ X = reinterpret_cast<const unsigned char*>(xs.X[blockIdx.y]);
     unsigned char* __restrict__ out_tokens = reinterpret_cast<unsigned char*>(outs.tokens[blockIdx.y]);
@@ -226,11 +243,11 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
     hdr = clip_block(hdr, sstride); cnt = clip_block(cnt, sstride); gprefix = clip_block(gprefix, sstride);
     keep = clip_block(keep, sstride);
 
-    extern __shared__ __align__(128) unsigned char stage[];     // [kCopyWarps][2][kGatherSlot]
-    __shared__ uint64_t bar[kCopyWarps][2];
+    extern __shared__ __align__(128) unsigned char stage[];     // [NW][2][slot]
+    __shared__ uint64_t bar[NW][2];
     __shared__ unsigned s_bits[kGatherWords];
     __shared__ int s_pref[kGatherWords];
-    __shared__ int s_warp[kCopyWarps];
+    __shared__ int s_warp[NW];
     __shared__ int s_frames[WHOLE ? 1 : kWarpPrefixMaxF + 4];
     const int N = H * W, FN = F * N;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -242,8 +259,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
     trace_mark(hdr, 6, false);
 
     // ---- window of the walk: bits and prefix of tokens [T0, T0 + 32 words) ------------------------------------------
-    constexpr int WPT = kGatherWords / kGatherThreads;          // consecutive words per thread
-    static_assert(kGatherWords % kGatherThreads == 0, "whole words per thread");
+    constexpr int WPT = (kGatherWords + kThreads - 1) / kThreads;         // consecutive words per thread
     const int a = __ldcg(hdr + HDR_ANCHOR);
     auto load_window = [&](int T0, int first) -> int {          // tokens before `first` do not count; returns the total
         uint4 v[WPT][2];
@@ -254,7 +270,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
             for (int h = 0; h < 2; ++h) {
                 // (the flag array is 256-byte aligned and followed by other scratch: a load that starts inside it may
                 // run past its end by less than 16 bytes, which the masks below discard)
-                v[u][h] = (WHOLE || tid * WPT < words) && (unsigned)(f + h * 16) < (unsigned)FN ? __ldcg(reinterpret_cast<const uint4*>(keep + f) + h)
+                v[u][h] = tid * WPT < words && (unsigned)(f + h * 16) < (unsigned)FN ? __ldcg(reinterpret_cast<const uint4*>(keep + f) + h)
                                                                 : make_uint4(0, 0, 0, 0);
             }
         }
@@ -267,7 +283,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
             const unsigned anchor = below((a + 1) * N - f) & ~below(a * N - f);
             b[u] = pack_flags(v[u][0], v[u][1]);
             b[u] = acnt ? b[u] | anchor : b[u] & ~anchor;       // the anchor frame: all of its tokens, or none
-            b[u] &= f < 0 || (!WHOLE && tid * WPT >= words) ? 0u : below(FN - f) & ~below(first - f);          // (f < 0: past 2^31, hence past the end)
+            b[u] &= f < 0 || tid * WPT >= words ? 0u : below(FN - f) & ~below(first - f);          // (f < 0: past 2^31, hence past the end)
             mine += __popc(b[u]);
         }
         int incl = mine;
@@ -281,10 +297,10 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
         __syncthreads();
         int at = incl - mine, total = 0;
 #pragma unroll
-        for (int ww = 0; ww < kCopyWarps; ++ww) { if (ww < w) at += s_warp[ww]; total += s_warp[ww]; }
+        for (int ww = 0; ww < NW; ++ww) { if (ww < w) at += s_warp[ww]; total += s_warp[ww]; }
 #pragma unroll
         for (int u = 0; u < WPT; ++u) {
-            if (WHOLE || tid * WPT < words) {
+            if (tid * WPT < words) {
                 s_bits[tid * WPT + u] = b[u];
                 s_pref[tid * WPT + u] = at;
             }
@@ -298,16 +314,16 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
     const bool in_smem = F <= kWarpPrefixMaxF;   // (else the pre-scanned array)
     int k, before = 0, P, T0 = 0, in_window = 0;
     if (WHOLE) P = in_window = load_window(0, 0);      // (no survivor counts needed)
-    else P = in_smem ? frame_prefix_cta(cnt, F, a, acnt, s_frames, s_warp) : __ldcg(gprefix + F);
+    else P = in_smem ? frame_prefix_cta<NW>(cnt, F, a, acnt, s_frames, s_warp) : __ldcg(gprefix + F);
     const int Lp = NA + P;                       // L' = N + P (Eq. Lpre)
     if (blockIdx.x == 0 && tid == 0) *reinterpret_cast<volatile int*>(out_count) = Lp;
-    const int per = (Lp + (int)gridDim.x - 1) / (int)gridDim.x;
+    // rows per CTA: per_magic is 2^32 / gridDim.x rounded up, so that per * gridDim.x > Lp without a division
+    const int per = (int)__umulhi((unsigned)Lp, per_magic) + 1;
     const int j0 = (int)min((long long)Lp, (long long)blockIdx.x * per), j1 = min(Lp, j0 + per);
     // rows per batch: what fits a slot, but no more than leaves every warp of the CTA a batch
-    int R = min(32, kGatherSlot / row_bytes);
-    R = max(1, min(R, (per + kCopyWarps - 1) / kCopyWarps));
+    const int R = max(1, min(batch, (per + NW - 1) / NW));
 
-    unsigned char* buf = stage + (size_t)w * 2 * kGatherSlot;
+    unsigned char* buf = stage + (size_t)w * 2 * slot;
     uint32_t phase = 0;                          // bit h: parity of slot h
     bool gave_up = false;                        // (lane 0 decides; all lanes of the warp know)
     const unsigned long long once = l2_evict_first_policy();
@@ -320,37 +336,50 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
         for (int h = kGatherWords / 2; h > 0; h >>= 1) if ((WHOLE || h < words) && s_pref[lo + h] <= n) lo += h;
         return T0 + lo * 32 + select_bit(s_bits[lo], n - s_pref[lo]);
     };
-    // lanes 0 .. n-1 issue the loads of output rows jb .. jb + n - 1 into slot h and write their positions
-    auto issue = [&](int jb, int n, int h) {
+    // A unit is a row, or a piece of a slot's size of a longer one.  Lanes 0 .. n-1 issue the loads of units ub .. ub + n - 1
+    // behind output row jb into slot h and write the positions.
+    auto unit_row = [&](int jb, int u, int& pc) {
+        if (pieces == 1) { pc = 0; return jb + u; }
+        const int r = u / pieces;
+        pc = u - r * pieces;
+        return jb + r;
+    };
+    auto unit_bytes = [&](int pc) { return (uint32_t)min(row_bytes - (size_t)pc * slot, (size_t)slot); };
+    auto issue = [&](int jb, int ub, int n, int h) {
         if (lane == 0) {
+            int pc;
+            unit_row(jb, ub, pc);
             bulk_wait_read<0>();                 // the store that used this slot has finished reading it
-            mbar_arrive_expect_tx(&bar[w][h], (uint32_t)(n * row_bytes) + (uint32_t)tx_extra);
+            mbar_arrive_expect_tx(&bar[w][h], (uint32_t)n * unit_bytes(pc) + (uint32_t)tx_extra);
         }
         __syncwarp();
         if (lane < n) {
-            const int j = jb + lane, f = source(j);
+            int pc;
+            const int j = unit_row(jb, ub + lane, pc), f = source(j);
             const bool ok = in_bounds(hdr, 4, j, FN) && in_bounds(hdr, 4, f, FN);      // (checked build)
-            unsigned char* d = buf + h * kGatherSlot + lane * row_bytes;
+            unsigned char* d = buf + h * slot + lane * (uint32_t)row_bytes;
             // (a row the checked build refuses is replaced by row 0, so that the batch still completes)
-            const unsigned char* src = X + (size_t)(ok ? f : 0) * row_bytes;
-            if (stream_once) bulk_load_hint(d, src, (uint32_t)row_bytes, &bar[w][h], once);
-            else bulk_load(d, src, (uint32_t)row_bytes, &bar[w][h]);
-            if (ok) {                            // p_{k,i} = (k, y_i, x_i)  (Eq. compress_pos)
+            const unsigned char* src = X + (size_t)(ok ? f : 0) * row_bytes + (size_t)pc * slot;
+            if (stream_once) bulk_load_hint(d, src, unit_bytes(pc), &bar[w][h], once);
+            else bulk_load(d, src, unit_bytes(pc), &bar[w][h]);
+            if (ok && pc == 0) {                 // p_{k,i} = (k, y_i, x_i)  (Eq. compress_pos)
                 const int kk = f / N, i = f - kk * N, yy = i / W;
                 int* p = out_pos + (size_t)j * 3;
                 p[0] = pos_base + kk + t_off; p[1] = pos_base + yy; p[2] = pos_base + i - yy * W;
             }
         }
     };
-    auto finish = [&](int jb, int n, int h) {    // the batch has landed: one store
+    auto finish = [&](int jb, int ub, int n, int h) {            // the batch has landed: one store
         if (lane == 0) {
+            int pc;
+            const int j = unit_row(jb, ub, pc);
             if (!mbar_wait(&bar[w][h], (phase >> h) & 1, wait_limit)) {
                 mbar_wait(&bar[w][h], (phase >> h) & 1, wait_limit);     // one more bounded chance for the copies to land
                 gave_up = true;
-            } else if (in_bounds(hdr, 4, jb + n - 1, FN)) {
-                unsigned char* d = out_tokens + (size_t)jb * row_bytes;
-                if (stream_once == 2) bulk_store_hint(d, buf + h * kGatherSlot, (uint32_t)(n * row_bytes), once);
-                else bulk_store(d, buf + h * kGatherSlot, (uint32_t)(n * row_bytes));
+            } else if (in_bounds(hdr, 4, j + (pieces == 1 ? n - 1 : 0), FN)) {
+                unsigned char* d = out_tokens + (size_t)j * row_bytes + (size_t)pc * slot;
+                if (stream_once == 2) bulk_store_hint(d, buf + h * slot, (uint32_t)n * unit_bytes(pc), once);
+                else bulk_store(d, buf + h * slot, (uint32_t)n * unit_bytes(pc));
                 bulk_commit();
             }
         }
@@ -358,12 +387,13 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, int row_bytes, int F, int H,
         gave_up = __shfl_sync(0xffffffffu, gave_up ? 1 : 0, 0) != 0;
     };
     auto move_rows = [&](int ja, int jb) {       // rows [ja, jb) of the output, by the warps of the CTA in turn
-        int at = ja + w * R, h = 0;
-        if (at < jb && !gave_up) issue(at, min(R, jb - at), 0);
-        for (; at < jb && !gave_up; at += kCopyWarps * R) {
-            const int next = at + kCopyWarps * R;
-            if (next < jb) issue(next, min(R, jb - next), h ^ 1);
-            finish(at, min(R, jb - at), h);
+        const int units = (jb - ja) * pieces;
+        int at = w * R, h = 0;
+        if (at < units && !gave_up) issue(ja, at, min(R, units - at), 0);
+        for (; at < units && !gave_up; at += NW * R) {
+            const int next = at + NW * R;
+            if (next < units) issue(ja, next, min(R, units - next), h ^ 1);
+            finish(ja, at, min(R, units - at), h);
             h ^= 1;
         }
     };
@@ -490,36 +520,44 @@ cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& ou
     // enough warps for one output row each at the usual two-thirds removal, at most three CTAs per SM and clip (a warp
     // loops when there are more)
     const long long want = ((long long)p.F * p.N / 3 + p.N + kCopyWarps - 1) / kCopyWarps;
-    int grid = (int)(want < 3LL * sm_count() ? (want < 1 ? 1 : want) : 3LL * sm_count());
+    const int grid = (int)(want < 3LL * sm_count() ? (want < 1 ? 1 : want) : 3LL * sm_count());
     const dim3 b(kCopyWarps * 32);
     // the pre-scanned prefix of very long clips is read through plain loads: order that case by the stream
     const bool pdl = p.F <= kWarpPrefixMaxF;
-    // Short rows in batches: up to half a slot always, up to a slot where the clip is one window of flags.  Measured, us
-    // per pass with one row per warp at a time / with batches: 128 x 32 x 32 x 64 (128-byte rows) 89.3 / 44.1,
+    // Beside other clips' kernels, short rows in batches: up to half a slot always, up to a slot where the clip is one window of
+    // flags.  Measured, us per pass with one row per warp at a time / with batches: 128 x 32 x 32 x 64 (128-byte rows) 89.3 / 44.1,
     // 128 x 24 x 24 x 256 58.5 / 39.6, 64 x 24 x 24 x 512 43.7 / 35.6, 64 x 32 x 32 x 1024 93.2 / 80.9; 4096-byte rows:
     // 32 x 16 x 16 (one window) 29.3 / 28.5, 128 x 16 x 16 (two windows) 74.6 / 78.4; 2320-byte rows, one window
     // 23.2 / 21.7.  Longer rows keep every warp's slot full by themselves.
-    if (vec && (row_bytes <= kGatherSlot / 2 || (row_bytes <= kGatherSlot && (long long)p.F * p.N <= kGatherWindow))) {
-        constexpr size_t smem = (size_t)kCopyWarps * 2 * kGatherSlot;
-        long long most = 3LL * sm_count() / p.nclips;
-        if (most < 1) most = 1;
-        if (grid > most) grid = (int)most;
-        // Clips beyond one window: windows of sixteen times the tokens that fall to a CTA (a window that holds too few rows
-        // costs another round trip), at least 512.  (Against windows of 16384 tokens and a count prefix per warp, us per pass:
-        // 64 x 24 x 24 x 512 32.3 -> 30.6, 64 x 32 x 32 x 1024 76.8 -> 75.2, 128 x 32 x 32 x 64 31.8 -> 29.8.  Clips of one
-        // window are better off without the counts: 32 x 16 x 16 x 2048 27.0 against 28.0.)
-        const long long FN = (long long)p.F * p.N;
-        int words = 16;
-        while (words < kGatherWords && words * 32LL < 16 * FN / grid) words *= 2;
-        auto launch = [&](auto kernel) {
+    const long long FN = (long long)p.F * p.N;
+    const bool whole = FN <= kGatherWindow;
+    // (a group of clips that has the GPU to itself, one CTA per SM / three: 5 MB in all 16.3 / 17.5 us, 14 MB 13.0 / 14.3, 19 MB
+    // 18.5 / 18.8, 26 MB 20.5 / 20.4, 34 MB 22.3 / 22.1)
+    const bool alone = p.overlapped <= 1 && (p.nclips == 1 || (double)FN * row_bytes * p.nclips <= 24e6);
+    if (vec && (alone || row_bytes <= 2048 || (row_bytes <= 4096 && whole))) {
+        auto launch = [&](auto kernel, int nw, int slot, int per_sm) {
+            const size_t smem = (size_t)nw * 2 * slot;
+            const int ctas = (int)std::min((FN / 3 + p.N + nw - 1) / nw, std::max(1LL, (long long)per_sm * sm_count() / p.nclips));
+            const int pieces = (int)((row_bytes + slot - 1) / slot);
+            const int batch = pieces > 1 ? 1 : (int)std::min((size_t)32, slot / row_bytes);
+            const unsigned per_magic = ctas == 1 ? 0xffffffffu : (unsigned)(((1ULL << 32) + ctas - 1) / ctas);
+            // Clips beyond one window: windows of sixteen times the tokens that fall to a CTA (a window that holds too few rows
+            // costs another round trip), at least 512.  (Against windows of 16384 tokens and a count prefix per warp, us per
+            // pass: 64 x 24 x 24 x 512 32.3 -> 30.6, 64 x 32 x 32 x 1024 76.8 -> 75.2, 128 x 32 x 32 x 64 31.8 -> 29.8.  Clips
+            // of one window are better off without the counts: 32 x 16 x 16 x 2048 27.0 against 28.0.)
+            int words = 16;
+            while (words < kGatherWords && words * 32LL < 16 * FN / ctas) words *= 2;
             cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
             if (e != cudaSuccess) return e;
-            return launch_ex(pdl, smem, kernel, dim3(grid, p.nclips), b, st, p.xs, (int)row_bytes, p.F, p.H, p.W, s.hdr,
+            return launch_ex(pdl, smem, kernel, dim3(ctas, p.nclips), dim3(nw * 32), st, p.xs, row_bytes, p.F, p.H, p.W, s.hdr,
                              (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt,
                              p.pos_t_offset, p.pos_base, p.chain_next, wait_poll_limit(), wait_tx_extra(), p.stream_once,
-                             p.sstride, words);
+                             p.sstride, words, per_magic, pieces, batch, slot);
         };
-        return FN <= kGatherWindow ? launch(k_compact_rows<true>) : launch(k_compact_rows<false>);
+        if (!alone) return whole ? launch(k_compact_rows<true, 8>, 8, 4096, 3) : launch(k_compact_rows<false, 8>, 8, 4096, 3);
+        if (row_bytes <= 128)                    // (32 rows, one per lane, fill no more than half a slot of 8 KB)
+            return whole ? launch(k_compact_rows<true, 16>, 16, 4096, 1) : launch(k_compact_rows<false, 16>, 16, 4096, 1);
+        return whole ? launch(k_compact_rows<true, 8>, 8, 8192, 1) : launch(k_compact_rows<false, 8>, 8, 8192, 1);
     }
     const dim3 g(grid, p.nclips);
     if (vec) {

@@ -12,8 +12,9 @@ constexpr int kScanChunks = 4;       // frame counts per lane fetched at once by
 // (`pref`: [kWarpPrefixMaxF + 4]; pref[F] is the total, which is returned).  The anchor frame counts `acnt` tokens.  By all
 // threads of a CTA of 256.  (Not for the gather with one row per warp at a time: its warps do better without a barrier
 // before their first copy, 37.8 against 38.7 us per pass on 32 x 16 x 16 x 4096, 247 against 255 on 64 x 32 x 32 x 4096.)
+template <int NW>
 __device__ __forceinline__ int frame_prefix_cta(const int* cnt, int F, int a, int acnt, int* pref, int* s_warp) {
-    static_assert(kWarpPrefixMaxF == 4 * kCopyWarps * 32, "four frames per thread");
+    static_assert(kWarpPrefixMaxF <= 4 * NW * 32, "four frames per thread");
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, k = tid * 4;
     // (the counts are 256-byte aligned and followed by other scratch: a load that starts inside may run past their end)
     int4 v = k < F ? __ldcg(reinterpret_cast<const int4*>(cnt + k)) : make_int4(0, 0, 0, 0);
@@ -34,8 +35,8 @@ __device__ __forceinline__ int frame_prefix_cta(const int* cnt, int F, int a, in
     __syncthreads();
     int at = incl - mine, total = 0;
 #pragma unroll
-    for (int ww = 0; ww < kCopyWarps; ++ww) { at += ww < w ? s_warp[ww] : 0; total += s_warp[ww]; }
-    if (k <= F) {
+    for (int ww = 0; ww < NW; ++ww) { at += ww < w ? s_warp[ww] : 0; total += s_warp[ww]; }
+    if (k <= F && k < kWarpPrefixMaxF) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) { pref[k + e] = at; at += c[e]; }
     }

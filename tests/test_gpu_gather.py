@@ -31,3 +31,15 @@ def test_segment_has_no_anchor_block(shape):
     assert n == int(cnt) - N and n > 0
     assert torch.equal(seg[:n], full[N:N + n])
     assert torch.equal(spos[:n], pos[N:N + n] + torch.tensor([10, 0, 0], dtype=torch.int32, device="cuda"))
+
+
+@pytest.mark.parametrize("shape,dtype", [((2, 2, 3, 4096), "bf16"), ((3, 3, 4, 4104), "bf16"), ((5, 4, 5, 6152), "bf16"),      # 1, 2, 2 pieces
+                                         ((4, 3, 3, 2052), "f32"), ((3, 2, 2, 8200), "bf16"),                                   # 2, 3 pieces
+                                         ((70, 16, 15, 2056), "bf16"), ((33, 23, 22, 4104), "bf16"),                            # several windows
+                                         ((40, 3, 4, 64), "bf16"), ((40, 3, 4, 72), "bf16"), ((260, 9, 8, 16), "f32"),          # 128, 144, 64 bytes
+                                         ((1030, 2, 2, 4104), "bf16"), ((1, 1, 1, 4104), "bf16")])
+def test_rows_of_pieces_and_rows_that_fill_no_slot(shape, dtype):
+    """alone: a row of up to three pieces of a slot; windows; the smallest rows; more frames than the shared prefix holds"""
+    X = corr_clip(*shape, seed=sum(shape), dtype=dtype)
+    check_clip(X, 1, 0.6)
+    check_clip(X, 1, 0.6, anchor_mode=2, order=1, pos_base=7)
