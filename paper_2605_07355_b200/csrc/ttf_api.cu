@@ -156,7 +156,7 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
     p->nsl = C % 4 == 0 ? (C + 127) / 128 : (C + 31) / 32;
     p->anchor_mode = 0; p->anchor_arg = 0; p->emit_anchor = 1; p->pos_t_offset = 0; p->pos_base = 0; p->natural_order = 0;
     p->use_tc = choose_match(*p);
-    p->fuse_cnt = nullptr; p->fresh = 0; p->chain = 0; p->chain_next = 0; p->overlapped = 0; p->stream_once = 0;
+    p->fuse_cnt = nullptr; p->match_begins = 0; p->fresh = 0; p->chain = 0; p->chain_next = 0; p->overlapped = 0; p->stream_once = 0;
     return TTF_OK;
 }
 
@@ -258,7 +258,8 @@ static int run_front(const Problem& p, const Scratch& s, int* out_anchor, float*
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e);
 #endif
-    { ProfScope ps(st, PK_NORM_SUM); e = launch_norm_sum(p, s, st); }
+    e = cudaSuccess;
+    if (!p.match_begins) { ProfScope ps(st, PK_NORM_SUM); e = launch_norm_sum(p, s, st); }
     if (e != cudaSuccess) return cuda_fail(e);
     if (p.anchor_mode == 0) {
         ProfScope ps(st, PK_FRAME_STATS);
@@ -276,7 +277,8 @@ static OutPtrs one_out(void* out_tokens, int* out_count, int* out_pos) {
     return o;
 }
 
-static int compress_impl(const Problem& p, void* ws, const OutPtrs& out, cudaStream_t st) {
+static int compress_impl(Problem p, void* ws, const OutPtrs& out, cudaStream_t st) {
+    p.match_begins = match_begins_call(p, out) ? 1 : 0;
     Scratch s;
     carve_scratch(p, ws, &s);
     int rc = run_front(p, s, nullptr, s.shat, s.dst, s.keep, st);

@@ -201,9 +201,6 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
 // 64 x 24 x 24 x 512 23.8 / 26.1).
 // Where other clips' kernels run beside it the CTAs are three per SM, and long rows go one at a time: the waits of one CTA
 // are filled by others (16 clips of 32 x 16 x 16 x 4096 448 us, 457 with one CTA per SM; 8 of 24 x 20 x 20 x 1024 84.6 / 87.4).
-constexpr int kGatherWords = 512;                       // bit words of a window
-constexpr int kGatherWindow = kGatherWords * 32;        // tokens
-
 // 32 keep flags (0 or 1 each) -> one bit each.  (The flags are masked first: a word that reaches past the end of the
 // array holds other bytes, whose higher bits would spill into its neighbours' in the product.)
 __device__ __forceinline__ unsigned pack_flags(const uint4& lo, const uint4& hi) {
@@ -232,7 +229,7 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
                int* __restrict__ hdr, const int* __restrict__ cnt, const int* __restrict__ gprefix,
                const unsigned char* __restrict__ keep, const __grid_constant__ OutPtrs outs, int NA, int acnt, int t_off,
                int pos_base, int late_trigger, int wait_limit, int tx_extra, int stream_once, size_t sstride, int window_words,
-               unsigned per_magic, int pieces, int batch, int slot)
+               unsigned per_magic, int pieces, int batch, int slot, int match_begins)
 {
     constexpr int kThreads = NW * 32;
     const int words = WHOLE ? kGatherWords : window_words;
@@ -261,6 +258,8 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     // ---- window of the walk: bits and prefix of tokens [T0, T0 + 32 words) ------------------------------------------
     constexpr int WPT = (kGatherWords + kThreads - 1) / kThreads;         // consecutive words per thread
     const int a = __ldcg(hdr + HDR_ANCHOR);
+    const bool reporter = blockIdx.x == 0 && tid == 0;
+    const int match_error = reporter && match_begins ? __ldcg(hdr + HDR_MATCH_ERROR) : 0;
     auto load_window = [&](int T0, int first) -> int {          // tokens before `first` do not count; returns the total
         uint4 v[WPT][2];
 #pragma unroll
@@ -429,7 +428,11 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
             __threadfence();
             *reinterpret_cast<volatile int*>(out_count) = -1;
         }
-        if (blockIdx.x == 0 && w == 0) {
+        if (reporter) {
+            if (match_error) {                   // (a matching kernel that began its call)
+                report_give_up(hdr);
+                hdr[HDR_MATCH_ERROR] = 0;
+            }
             __threadfence();
             if (atomicAdd(hdr + HDR_ERROR, 0)) *reinterpret_cast<volatile int*>(out_count) = -1;
         }
@@ -552,7 +555,7 @@ cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& ou
             return launch_ex(pdl, smem, kernel, dim3(ctas, p.nclips), dim3(nw * 32), st, p.xs, row_bytes, p.F, p.H, p.W, s.hdr,
                              (const int*)s.cnt, (const int*)s.prefix, (const unsigned char*)s.keep, out, NA, acnt,
                              p.pos_t_offset, p.pos_base, p.chain_next, wait_poll_limit(), wait_tx_extra(), p.stream_once,
-                             p.sstride, words, per_magic, pieces, batch, slot);
+                             p.sstride, words, per_magic, pieces, batch, slot, p.match_begins);
         };
         if (!alone) return whole ? launch(k_compact_rows<true, 8>, 8, 4096, 3) : launch(k_compact_rows<false, 8>, 8, 4096, 3);
         if (row_bytes <= 128)                    // (32 rows, one per lane, fill no more than half a slot of 8 KB)

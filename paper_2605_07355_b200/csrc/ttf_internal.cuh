@@ -20,6 +20,8 @@ enum { HDR_ANCHOR = 0,          // anchor frame a*
        HDR_ERROR = 2,           // 1: a bounded wait of this call gave up; 2: a checked build caught an index outside its
                                 // array (cleared by the first kernel of every call)
        HDR_BATCH_ERROR = 3,     // the same, kept until the block is cleared: the clips of a batch that share a block report here
+       HDR_MATCH_ERROR = 4,     // a bounded wait of a matching kernel that begins its call gave up (zero between calls: the
+                                // gather of the call moves it to HDR_ERROR)
        HDR_CHECK_SLACK = 8,     // checked build: every limit is lowered by this much (test hook; zero otherwise)
        HDR_CHECK_SITE = 9,      // checked build: kernel site, index (clamped to 31 bits) and limit of the first index
        HDR_CHECK_INDEX = 10,    // that was out of range
@@ -56,6 +58,7 @@ struct Problem {
     int use_tc;         // 1: the matching step runs on tcgen05 (ttf_match_tc.cu)
     int* fuse_cnt;      // [N] the query's counts of tokens fused into each anchor cell, or NULL: zeroed between the
                         // sweep and the matching kernel, which counts (single clips only)
+    int match_begins;   // 1: the matching kernel is the first of the call (see match_begins_call)
     int fresh;          // 1: the scratch blocks may hold anything: the first kernel clears their control words
     int chain;          // 1: the kernel before this call's sweep in the stream is the gather of the library's previous
                         // clip, which works on another scratch block: the sweep may run beside it
@@ -90,6 +93,8 @@ struct AnchorSrc {
     int nsl;
     int fixed;          // >= 0: the anchor is this frame (first / last / explicit rule)
     int from_hdr;       // 1: an earlier kernel left it in hdr[HDR_ANCHOR]
+    int begins;         // 1: no kernel of the call came before: the error word is the reader's to clear, what it has to report
+                        // itself goes into HDR_MATCH_ERROR
     int* hdr;
     int* out_anchor;    // optional user copy (single clips only)
 };
@@ -110,9 +115,28 @@ inline bool uses_f32_match(const Problem& p) {
 cudaError_t launch_match_f32(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                              unsigned char* keep, cudaStream_t st);
 
+// The longest clip whose gather, where the call has the GPU to itself, takes the whole keep mask at once (k_compact_rows).
+constexpr int kGatherWords = 512;                       // bit words of a window
+constexpr int kGatherWindow = kGatherWords * 32;        // tokens
+
 // The sweep stores per-token partial squared norms only for the kernels that read them.
 inline bool needs_sweep_norms(const Problem& p) {
     return !p.use_tc && !uses_f32_match(p) && (!uses_mma_match(p) || p.r == 2);
+}
+
+// A call with a fixed anchor needs nothing of X before its matching kernel.  What is left of a kernel before it is to clear the
+// survivor counters, which the gather of one window of flags does not read, and the error word, which the matching kernel clears
+// itself: then it comes first.  (Not in the checked build, where all CTAs report through the error word from the start, nor for
+// the warp-level kernel.)  Us per pass through the
+// binding 21 x 13 x 19 x 1160 14.3 -> 12.9, 6 x 22 x 24 x 264 14.2 -> 11.6, the 9 x 16 x 16 x 4096 segment 59.7 -> 57.2; in a replayed
+// graph, where the host's part is gone, 12.4 -> 12.5, 8.8 -> 8.4, and 32 x 16 x 16 x 1152 fp32 18.8 -> 18.3.
+inline bool match_begins_call(const Problem& p, const OutPtrs& out) {
+#ifdef TTF_DEBUG
+    return false;
+#else
+    return p.anchor_mode != 0 && p.nclips == 1 && p.overlapped <= 1 && !p.chain && !p.fresh && (p.use_tc || uses_f32_match(p)) && p.vec &&
+           reinterpret_cast<uintptr_t>(out.tokens[0]) % 16 == 0 && (long long)p.F * p.N <= kGatherWindow && p.F <= kWarpPrefixMaxF;
+#endif
 }
 
 // tcgen05 matching (ttf_match_tc.cu)
@@ -158,6 +182,7 @@ inline AnchorSrc make_anchor_src(const Problem& p, const Scratch& s, int* out_an
     AnchorSrc a;
     a.Dp = s.Dp; a.Qp = s.Qp; a.Gp = s.Gp; a.nsl = p.nsl; a.hdr = s.hdr; a.out_anchor = out_anchor;
     a.fixed = p.anchor_mode == 0 ? -1 : (p.anchor_mode == 1 ? 0 : (p.anchor_mode == 2 ? p.F - 1 : p.anchor_arg));
+    a.begins = p.match_begins;
     a.from_hdr = p.anchor_mode == 0 ? 1 : 0;     // the statistics kernel's last CTA left the arg max there
     return a;
 }
@@ -252,7 +277,8 @@ __device__ __forceinline__ void gate_token(float best, int best_j, float t, size
 }
 
 // a bounded wait of this call has run out
-__device__ __forceinline__ void report_give_up(int* hdr) {
+__device__ __forceinline__ void report_give_up(int* hdr, bool begins = false) {
+    if (begins) { atomicExch(hdr + HDR_MATCH_ERROR, 1); return; }    // (HDR_ERROR may still be about to be cleared)
     atomicExch(hdr + HDR_ERROR, 1);
     atomicExch(hdr + HDR_BATCH_ERROR, 1);
 }

@@ -88,6 +88,7 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
     trace_mark(asrc.hdr, 5, false);
     const int a = asrc.fixed >= 0 ? asrc.fixed : __ldcg(asrc.hdr + HDR_ANCHOR);
     if (blockIdx.x == 0 && tid == 0 && asrc.fixed >= 0) {
+        if (asrc.begins) asrc.hdr[HDR_ERROR] = 0;
         asrc.hdr[HDR_ANCHOR] = a;                          // the gather reads it from here
         if (asrc.out_anchor) *asrc.out_anchor = a;
     }
@@ -143,7 +144,7 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
         // copies still land in this CTA's shared memory: wait (bounded again) for the stages issued last
         for (int it = issued > S::STAGES ? issued - S::STAGES : 0; it < issued; ++it)
             mbar_wait(&bar[it % S::STAGES], (it / S::STAGES) & 1, wait_limit);
-        report_give_up(asrc.hdr);
+        report_give_up(asrc.hdr, asrc.begins);
     }
     pdl_launch_dependents();                               // (not at the start: the gather's CTAs would take the place
                                                            // of other clips' kernels while this one runs)

@@ -237,6 +237,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     trace_mark(asrc.hdr, 5, false);
     const int a = asrc.fixed >= 0 ? asrc.fixed : __ldcg(asrc.hdr + HDR_ANCHOR);
     if (blockIdx.x == 0 && tid == 0 && asrc.fixed >= 0) {
+        if (asrc.begins) asrc.hdr[HDR_ERROR] = 0;
         asrc.hdr[HDR_ANCHOR] = a;                // the gather reads it from here
         if (asrc.out_anchor) *asrc.out_anchor = a;
     }
@@ -479,7 +480,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
         tc_fence_after();
         tmem_dealloc(tmem, tmem_cols);
     }
-    if (tid == 0 && s_err) report_give_up(asrc.hdr);
+    if (tid == 0 && s_err) report_give_up(asrc.hdr, asrc.begins);
 }
 
 // ---- host side: tensor maps and launch ------------------------------------------------------------------------
