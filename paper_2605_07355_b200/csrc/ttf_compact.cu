@@ -534,9 +534,7 @@ cudaError_t launch_compact(const Problem& p, const Scratch& s, const OutPtrs& ou
     // 23.2 / 21.7.  Longer rows keep every warp's slot full by themselves.
     const long long FN = (long long)p.F * p.N;
     const bool whole = FN <= kGatherWindow;
-    // (a group of clips that has the GPU to itself, one CTA per SM / three: 5 MB in all 16.3 / 17.5 us, 14 MB 13.0 / 14.3, 19 MB
-    // 18.5 / 18.8, 26 MB 20.5 / 20.4, 34 MB 22.3 / 22.1)
-    const bool alone = p.overlapped <= 1 && (p.nclips == 1 || (double)FN * row_bytes * p.nclips <= 24e6);
+    const bool alone = gather_alone(p);
     if (vec && (alone || row_bytes <= 2048 || (row_bytes <= 4096 && whole))) {
         auto launch = [&](auto kernel, int nw, int slot, int per_sm) {
             const size_t smem = (size_t)nw * 2 * slot;

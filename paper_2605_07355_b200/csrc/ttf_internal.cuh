@@ -124,6 +124,15 @@ inline bool needs_sweep_norms(const Problem& p) {
     return !p.use_tc && !uses_f32_match(p) && (!uses_mma_match(p) || p.r == 2);
 }
 
+// Whether the gather runs with one CTA per SM.  A call that has the GPU to itself does.  Not for groups of clips beyond 24 MB (one
+// CTA per SM / three: 5 MB in all 16.3 / 17.5 us, 14 MB 13.0 / 14.3, 19 MB 18.5 / 18.8, 26 MB 20.5 / 20.4, 34 MB 22.3 / 22.1),
+// nor for a clip of far more than L2 holds (268 MB 126.7 / 132.5 us, 537 MB 242.3 / 240.3 and at r = 2 250.0 / 247.2: the rows
+// come from DRAM).
+inline bool gather_alone(const Problem& p) {
+    const double bytes = (double)p.F * p.N * p.C * (p.dtype == 0 ? 4.0 : 2.0) * p.nclips;
+    return p.overlapped <= 1 && bytes <= (p.nclips == 1 ? 300e6 : 24e6);
+}
+
 // A call with a fixed anchor needs nothing of X before its matching kernel.  What is left of a kernel before it is to clear the
 // survivor counters, which the gather of one window of flags does not read, and the error word, which the matching kernel clears
 // itself: then it comes first.  (Not in the checked build, where all CTAs report through the error word from the start, nor for
@@ -135,7 +144,7 @@ inline bool match_begins_call(const Problem& p, const OutPtrs& out) {
     return false;
 #else
     return p.anchor_mode != 0 && p.nclips == 1 && p.overlapped <= 1 && !p.chain && !p.fresh && (p.use_tc || uses_f32_match(p)) && p.vec &&
-           reinterpret_cast<uintptr_t>(out.tokens[0]) % 16 == 0 && (long long)p.F * p.N <= kGatherWindow && p.F <= kWarpPrefixMaxF;
+           reinterpret_cast<uintptr_t>(out.tokens[0]) % 16 == 0 && (long long)p.F * p.N <= kGatherWindow && p.F <= kWarpPrefixMaxF && gather_alone(p);
 #endif
 }
 
