@@ -17,6 +17,7 @@
 #include "ttf_async.cuh"
 #include "ttf_cluster.cuh"
 
+#include <cstdlib>
 #include <map>
 #include <mutex>
 #include <set>
@@ -367,7 +368,7 @@ k_frame_stats(const float* S, int F, int C, int nsl, float* Dp, float* Qp, float
 // CTAs, 0.9 us; hence sixteen where the kernel runs alone), three block barriers and the cluster barrier.
 // With eight CTAs, two shuffle trees per frame and every warp adding up all channels of g for itself a pass took, in a
 // replayed graph, 39.3 us (32 x 16 x 16 x 4096), 28.9 (2048 channels), 134.7 (128 frames) and 11.3 (4 x 8 x 8 x 64) where it
-// took 38.0, 28.1, 130.2 and 10.2; the order of summation that eight and sixteen CTAs share added nothing (39.8 -> 39.6 and
+// took 38.0, 28.1, 130.2 and 10.2, without the folds of frames that a clip does not have 0.3 - 0.4 less again; the order of summation that eight and sixteen CTAs share added nothing (39.8 -> 39.6 and
 // 28.5 -> 28.3 per call).
 constexpr int kStatClusterMaxF = 256;     // frames the cluster kernel takes (shares of all frames live in shared memory)
 
@@ -444,6 +445,7 @@ k_frame_stats_cluster(const float* S, int F, int C, int nsl, int* hdr, int* out_
         if (!one_chunk) load_chunk(k0);              // (a second round trip per chunk for clips of several chunks)
 #pragma unroll
         for (int j0 = 0; j0 < FB; j0 += FP) {
+            if (k0 + w + j0 * kNormWarps >= F) break;    // (no frames left for this warp: a fold is 450 cycles)
             float part[8];                           // [<S_k, g> or |S_k|^2][unit][frames j0 .. j0 + FP - 1]
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -616,6 +618,15 @@ cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anch
     // its places in one GPC are free at the same moment.
     if (p.C % 4 == 0 && p.nsl <= 32 && p.F <= kStatClusterMaxF) {
         if (p.nsl == 1) return launch_stats_cluster_t<1, 1>(p, s, out_anchor, st);      // nothing to split
+        // Up to four slices of so few frames that one CTA holds their sums (64 KB) at once: what the other CTAs would save is
+        // less than the exchange between them costs (1200 cycles; us per pass with eight CTAs / one: 24 x 20 x 15 x 248
+        // 15.5 / 14.9, 16 x 14 x 14 x 512 13.2 / 12.8, 32 x 14 x 14 x 512 14.4 / 14.2, 52 x 14 x 9 x 208 14.0 / 13.6; eight
+        // slices, 16 x 16 x 16 x 1024 15.2 / 15.4).
+        if (p.nsl == 2 && p.F <= 64) return launch_stats_cluster_t<2, 1>(p, s, out_anchor, st);
+        if (p.nsl <= 4 && p.F <= 32) return launch_stats_cluster_t<4, 1>(p, s, out_anchor, st);
+        static const int lim = getenv("TTF_ST") ? atoi(getenv("TTF_ST")) : 64;
+        if (p.nsl <= 4 && p.nsl * p.F <= lim) return p.nsl == 2 ? launch_stats_cluster_t<2, 1>(p, s, out_anchor, st) : launch_stats_cluster_t<4, 1>(p, s, out_anchor, st);
+        if (p.nsl <= 8 && p.nsl * p.F <= lim) return launch_stats_cluster_t<8, 1>(p, s, out_anchor, st);
         const bool alone = p.overlapped <= 1 && large_clusters();
         if (p.nsl > 16) return alone ? launch_stats_cluster_t<2, 16>(p, s, out_anchor, st)
                                      : launch_stats_cluster_t<4, 8>(p, s, out_anchor, st);

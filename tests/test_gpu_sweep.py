@@ -22,3 +22,11 @@ def test_slice_widths(shape, dtype):
     outs = P.ttf_compress_batch(Xs, 1, 0.6)
     torch.cuda.synchronize()
     assert_same_as_single(Xs, 1, 0.6, outs)
+
+
+@pytest.mark.parametrize("shape,dtype", [((64, 3, 3, 136), "bf16"), ((65, 3, 3, 136), "bf16"), ((32, 3, 4, 264), "bf16"), ((33, 3, 4, 512), "bf16"),
+                                         ((7, 4, 4, 512), "bf16"), ((8, 4, 4, 520), "bf16"), ((64, 2, 3, 256), "f32"), ((33, 2, 3, 388), "f32"),
+                                         ((9, 3, 3, 2056), "bf16"), ((40, 3, 3, 4096), "bf16")])
+def test_statistics_in_one_cta_and_in_a_cluster(shape, dtype):
+    """two to four slices of channels at the frames that one CTA holds and one more; frames that leave warps without any"""
+    test_slice_widths(shape, dtype)
