@@ -4,6 +4,8 @@
 #include "ttf_async.cuh"
 #include "ttf_cluster.cuh"
 
+#include <algorithm>
+
 namespace ttf {
 
 constexpr int kXThreads = 256;
@@ -176,6 +178,125 @@ k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int*
     }
 }
 
+// The same with bulk copies, for rows of whole 16-byte pieces: ONE CTA per SM, whose warps move batches of consecutive output
+// rows (or pieces of long ones) through three slots of 8 KB each, two loads ahead; a batch leaves as one store.  The flags before
+// a CTA's tokens are read by 148 CTAs instead of up to 1184 (they queue on the same lines), short rows move 32 to a batch, and a
+// row that is no multiple of eight loads per lane has no serial rest.  Us per call in a replayed graph, plain loads / bulk:
+// 32 x 16 x 16 x 512 7.2 / 4.9, 64 x 32 x 32 x 64 14.4 / 8.3, 14 x 25 x 14 x 2800 13.9 / 9.8, 48 x 16 x 16 x 1536 21.6 / 12.0,
+// 64 x 32 x 32 x 1024 47.8 / 36.3; from two launches 128 x 32 x 32 x 64 27.8 / 15.9, x 512 53.3 / 38.7, 256 x 32 x 32 x 64 50.1 /
+// 30.0.  (Two slots of 8 KB 10.2 and 12.4 where three take 9.8 and 12.0; four of 4 KB 10.9.)
+// A wait that runs out has nobody to report to here: the warp copies what is left by plain loads and stores.
+constexpr int kRestoreBulk = 1 << 18;
+constexpr int kRestoreSlots = 3, kRestoreSlot = 8192, kRestoreAhead = 2;
+__global__ void __launch_bounds__(kXThreads)
+k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const int* anchor, const unsigned char* keep,
+               const int* dst, int per, unsigned char* out, int* row_index, int pieces, int batch, int wait_limit, int tx_extra)
+{
+    extern __shared__ __align__(128) unsigned char stage[];      // [warps][kRestoreSlots][kRestoreSlot]
+    __shared__ uint64_t bar[kXThreads / 32][kRestoreSlots];
+    __shared__ int s_warp[kXThreads / 32];
+    __shared__ int s_row[kXThreads];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int f0 = blockIdx.x * per, f1 = min(FN, f0 + per);
+    pdl_launch_dependents();
+    if (lane == 0) {
+        for (int h = 0; h < kRestoreSlots; ++h) mbar_init(&bar[w][h], 1);
+        mbar_init_fence();
+    }
+    __syncwarp();
+    pdl_wait();                                  // the caller's kernels before this one
+    unsigned char next_keep = f0 + tid < f1 ? keep[f0 + tid] : (unsigned char)0;
+    int next_dst = f0 + tid < f1 ? dst[f0 + tid] : 0;
+    const int a = __ldcg(anchor);
+    const bool inside = (unsigned)a < (unsigned)(FN / N);
+    const int a0 = inside ? a * N : FN, a1 = inside ? a0 + N : FN;
+    int c = count_flags(keep, 0, (size_t)min(f0, a0), tid);
+    if (f0 > a1) c += count_flags(keep, (size_t)a1, (size_t)f0, tid);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) s_warp[w] = c;
+    __syncthreads();
+    int run = N;
+#pragma unroll
+    for (int ww = 0; ww < kXThreads / 32; ++ww) run += s_warp[ww];
+
+    unsigned char* const buf = stage + (size_t)w * kRestoreSlots * kRestoreSlot;
+    int issued = 0, finished = 0;                // batches of this warp; batch n goes through slot n % kRestoreSlots
+    bool gave_up = false;
+    for (int b0 = f0; b0 < f1; b0 += kXThreads) {
+        const int f = b0 + tid, end = min(f1, b0 + kXThreads);
+        const bool in = f < f1, own = f >= a0 && f < a1;
+        const bool kp = in && !own && next_keep;
+        const int to = next_dst;
+        next_keep = f + kXThreads < f1 ? keep[f + kXThreads] : (unsigned char)0;
+        next_dst = f + kXThreads < f1 ? dst[f + kXThreads] : 0;
+        const unsigned m = __ballot_sync(0xffffffffu, kp);
+        __syncthreads();                         // (the indices of the round before this one, and s_warp, are done with)
+        if (lane == 0) s_warp[w] = __popc(m);
+        __syncthreads();
+        int off = 0, total = 0;
+#pragma unroll
+        for (int ww = 0; ww < kXThreads / 32; ++ww) { off += ww < w ? s_warp[ww] : 0; total += s_warp[ww]; }
+        if (in) {
+            const int r = own ? f - a0 : (kp ? run + off + __popc(m & ((1u << lane) - 1)) : to);
+            s_row[tid] = r;
+            row_index[f] = r;
+        }
+        run += total;
+        __syncthreads();
+        const int R = max(1, min(batch, (end - b0 + kXThreads / 32 - 1) / (kXThreads / 32)));
+        const int units = (end - b0) * pieces, step = kXThreads / 32 * R;
+        auto piece_bytes = [&](int pc) { return (uint32_t)min(row_bytes - (size_t)pc * kRestoreSlot, (size_t)kRestoreSlot); };
+        auto issue = [&](int u) {
+            const int n = min(R, units - u), h = issued % kRestoreSlots;
+            const int r0 = pieces == 1 ? u : u / pieces, pc = pieces == 1 ? 0 : u - r0 * pieces;
+            if (lane == 0) {
+                bulk_wait_read<kRestoreSlots - 1 - kRestoreAhead>();      // the store that used this slot has finished reading it
+                mbar_arrive_expect_tx(&bar[w][h], (uint32_t)n * piece_bytes(pc) + (uint32_t)tx_extra);
+            }
+            __syncwarp();
+            if (lane < n)
+                bulk_load(buf + h * kRestoreSlot + lane * (uint32_t)row_bytes,
+                          comp + (size_t)s_row[r0 + lane] * row_bytes + (size_t)pc * kRestoreSlot, piece_bytes(pc), &bar[w][h]);
+            ++issued;
+        };
+        int ahead = w * R;
+        for (int q = 0; q < kRestoreAhead && ahead < units && !gave_up; ++q, ahead += step) issue(ahead);
+        for (int u = w * R; u < units; u += step) {
+            const int n = min(R, units - u);
+            const int r0 = pieces == 1 ? u : u / pieces, pc = pieces == 1 ? 0 : u - r0 * pieces;
+            unsigned char* d = out + (size_t)(b0 + r0) * row_bytes + (size_t)pc * kRestoreSlot;
+            if (!gave_up) {
+                if (ahead < units) { issue(ahead); ahead += step; }
+                const int h = finished % kRestoreSlots;
+                bool ok = true;
+                if (lane == 0) ok = mbar_wait(&bar[w][h], (finished / kRestoreSlots) & 1, wait_limit);
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (ok) {
+                    if (lane == 0) {
+                        bulk_store(d, buf + h * kRestoreSlot, (uint32_t)n * piece_bytes(pc));
+                        bulk_commit();
+                    }
+                    ++finished;
+                    continue;
+                }
+                gave_up = true;
+            }
+            // a copy that does not arrive: this batch and the rest by plain loads and stores
+            for (int q = 0; q < n; ++q) {
+                const uint4* src = reinterpret_cast<const uint4*>(comp + (size_t)s_row[r0 + q] * row_bytes + (size_t)pc * kRestoreSlot);
+                uint4* to4 = reinterpret_cast<uint4*>(d + (size_t)q * row_bytes);
+                for (int e = lane; e < (int)(piece_bytes(pc) / 16); e += 32) to4[e] = src[e];
+            }
+        }
+    }
+    if (lane == 0) {
+        // copies still on their way into this CTA's shared memory (bounded again)
+        for (; finished < issued; ++finished) mbar_wait(&bar[w][finished % kRestoreSlots], (finished / kRestoreSlots) & 1, wait_limit);
+        bulk_wait<0>();
+    }
+}
+
 template <typename U>
 static cudaError_t launch_restore_t(const unsigned char* c, size_t row_bytes, int F, int N, const int* anchor,
                                     const unsigned char* keep, const int* dst, unsigned char* o, int* row_index,
@@ -194,12 +315,33 @@ static cudaError_t launch_restore_t(const unsigned char* c, size_t row_bytes, in
     return launch_pdl(k_restore_copy<U>, dim3((unsigned)blocks), dim3(kXThreads), st, c, row_bytes, rows, row_index, o);
 }
 
+// Plain loads stay where they are the faster ones: rows of whole 4 KB, which keep eight loads per lane in flight throughout, once
+// the output is more than half of L2 (bulk / plain: 50 MB 15.1 / 15.3 us, 67 MB in rows of 4 KB 19.0 / 18.3, of 8 KB 19.0 / 18.0,
+// 151 MB 41.9 / 37.6), and the smallest clips, whose rows gain nothing from the way through shared memory (131 KB 3.65 / 3.15,
+// 524 KB 3.65 / 3.4, in 4096 rows 3.66 / 4.15, 790 KB 3.65 / 3.65).
+static bool restore_in_bulk(long long FN, size_t row_bytes) {
+    const double mb = (double)FN * row_bytes * 1e-6;
+    if (FN > kRestoreBulk || (FN <= 2048 && mb <= 0.75)) return false;
+    return row_bytes % 4096 != 0 || mb <= 52.0;
+}
+
 cudaError_t launch_restore(const void* comp, size_t row_bytes, int F, int N, const int* anchor,
                            const unsigned char* keep, const int* dst, void* out_full, int* row_index,
                            cudaStream_t st) {
     const unsigned char* c = reinterpret_cast<const unsigned char*>(comp);
     unsigned char* o = reinterpret_cast<unsigned char*>(out_full);
     const uintptr_t al = reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(out_full) | row_bytes;
+    if (al % 16 == 0 && restore_in_bulk((long long)F * N, row_bytes)) {
+        const int FN = F * N, most = sm_count();
+        const int per = std::max(8, (FN + most - 1) / most);
+        const int pieces = (int)((row_bytes + kRestoreSlot - 1) / kRestoreSlot);
+        const int batch = pieces > 1 ? 1 : (int)std::min((size_t)32, kRestoreSlot / row_bytes);
+        constexpr size_t smem = (size_t)(kXThreads / 32) * kRestoreSlots * kRestoreSlot;
+        cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_restore_bulk), smem);
+        if (e != cudaSuccess) return e;
+        return launch_ex(true, smem, k_restore_bulk, dim3((FN + per - 1) / per), dim3(kXThreads), st, c, row_bytes, FN, N, anchor, keep,
+                         dst, per, o, row_index, pieces, batch, wait_poll_limit(), wait_tx_extra());
+    }
     if (al % 16 == 0) return launch_restore_t<uint4>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);
     if (al % 4 == 0) return launch_restore_t<uint32_t>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);
     if (al % 2 == 0) return launch_restore_t<uint16_t>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);

@@ -172,3 +172,30 @@ def test_an_anchor_outside_the_clip_excludes_no_frame(shape, anchor):
     assert (idx.cpu().numpy() == ref).all() and (full[:, 0].cpu().numpy() == ref).all()
     got = P.ttf_stats(dev(sim), dev(keep), a, F, H, W, 0.3, 0.05).tolist()
     assert got == [int(keep.sum()), int(F * N - keep.sum()), int((np.abs(sim.astype(np.float64) - np.float64(np.float32(0.3))) < np.float64(np.float32(0.05))).sum())]
+
+
+@pytest.mark.parametrize("F,N,row_bytes", [(9, 256, 16), (9, 256, 48), (64, 37, 4096), (64, 33, 8192), (33, 71, 8208), (5, 500, 24592), (300, 256, 128),
+                                           (130, 1030, 272), (2, 1024, 1008), (260, 1024, 16), (6, 2187, 4096), (9, 1000, 8192),
+                                           (1, 3000, 320), (2049, 1, 512)])
+@pytest.mark.parametrize("wait", [None, (32, 16)])
+def test_restore_in_bulk_at_the_edges(F, N, row_bytes, wait):
+    """rows of one and several pieces, batches, rounds of 256 tokens that end inside a batch, the sizes next to the lines of the
+    rule; with the test hook that makes every copy's wait run out, after which the rows go by plain loads and stores"""
+    g = torch.Generator().manual_seed(F * N + row_bytes)
+    keep = (torch.rand(F * N, generator=g) < 0.4).to(torch.uint8)
+    a = int(torch.randint(0, F, (1,), generator=g))
+    keep.view(F, N)[a] = 1
+    dst = torch.randint(0, N, (F * N,), generator=g, dtype=torch.int32)
+    source = keep.bool().clone().view(F, N)
+    source[a] = False
+    ref = torch.where(source.view(-1), torch.cumsum(source.view(-1), 0).int() - 1 + N, dst).view(F, N)
+    ref[a] = torch.arange(N, dtype=torch.int32)
+    rows = torch.randint(0, 256, (N + int(source.sum()), row_bytes), generator=g, dtype=torch.uint8).cuda()
+    if wait:
+        P.ttf_debug_set_wait(*wait)
+    try:
+        full, idx = P.ttf_restore(rows, F, 1, N, torch.tensor([a], dtype=torch.int32, device="cuda"), keep.cuda(), dst.cuda())
+        torch.cuda.synchronize()
+    finally:
+        P.ttf_debug_set_wait()
+    assert torch.equal(idx.cpu(), ref.view(-1)) and torch.equal(full, rows[ref.view(-1).long().cuda()])
