@@ -52,7 +52,7 @@ __device__ __forceinline__ float dot4(const float4& a, const float4& b, float ac
     return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
 }
 
-template <int R, int G>
+template <int R, int G, int ST>      // ST: stages of the ring
 __global__ void __launch_bounds__(F32Shape<R>::MAXW * 32)
 k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C, float t, AnchorSrc asrc,
             float* __restrict__ shat, int* __restrict__ dst, unsigned char* __restrict__ keep, int* __restrict__ cnt,
@@ -64,7 +64,7 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
     shat = clip_block(shat, sstride); dst = clip_block(dst, sstride); keep = clip_block(keep, sstride);
     using S = F32Shape<R>;
     extern __shared__ __align__(128) unsigned char f32_ring[];
-    __shared__ uint64_t bar[S::STAGES];
+    __shared__ uint64_t bar[ST];
     __shared__ float s_sum[S::MAXW][S::NG * 32];
     __shared__ int s_err;
     const int N = H * W;
@@ -77,7 +77,7 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
 
     trace_mark(asrc.hdr, 2, false);
     if (tid == 0) {
-        for (int s = 0; s < S::STAGES; ++s) mbar_init(&bar[s], 1);
+        for (int s = 0; s < ST; ++s) mbar_init(&bar[s], 1);
         mbar_init_fence();
         s_err = 0;
         tensormap_prefetch(&mapA);
@@ -93,16 +93,15 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
         if (asrc.out_anchor) *asrc.out_anchor = a;
     }
 
-    auto issue = [&](int it) {                             // thread 0: both tiles of stage it
-        unsigned char* s = f32_ring + (size_t)(it % S::STAGES) * stage_bytes;
-        uint64_t* b = &bar[it % S::STAGES];
-        mbar_arrive_expect_tx(b, stage_bytes + (uint32_t)tx_extra);       // (extra: test hook only)
-        tma_load_4d(s, &mapA, it * kF32KC, x, y, k0, b);
-        tma_load_4d(s + abytes, &mapB, it * kF32KC, x - R, y - R, a, b);
+    auto issue = [&](int it, int slot) {                   // thread 0: both tiles of stage it
+        unsigned char* s = f32_ring + (size_t)slot * stage_bytes;
+        mbar_arrive_expect_tx(&bar[slot], stage_bytes + (uint32_t)tx_extra);      // (extra: test hook only)
+        tma_load_4d(s, &mapA, it * kF32KC, x, y, k0, &bar[slot]);
+        tma_load_4d(s + abytes, &mapB, it * kF32KC, x - R, y - R, a, &bar[slot]);
     };
     int issued = 0;
     if (tid == 0)
-        for (; issued < S::STAGES && issued < nst; ++issued) issue(issued);
+        for (; issued < ST && issued < nst; ++issued) issue(issued, issued);
 
     float acc[S::FW][S::WIN], na[S::FW], nb[S::WIN];
 #pragma unroll
@@ -115,11 +114,12 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
     for (int c = 0; c < S::WIN; ++c) nb[c] = 0.f;
 
     bool ok = true;                                        // (per thread: a thread whose wait ran out stops computing,
-    for (int it = 0; it < nst; ++it) {                     // but takes part in every barrier)
-        const int s = it % S::STAGES;
-        if (ok && !mbar_wait(&bar[s], (it / S::STAGES) & 1, wait_limit)) { ok = false; atomicExch(&s_err, 1); }
+    int slot = 0;                                          // but takes part in every barrier)
+    uint32_t parity = 0;
+    for (int it = 0; it < nst; ++it) {
+        if (ok && !mbar_wait(&bar[slot], parity, wait_limit)) { ok = false; atomicExch(&s_err, 1); }
         if (ok) {
-            const unsigned char* sa = f32_ring + (size_t)s * stage_bytes + lane * 16;
+            const unsigned char* sa = f32_ring + (size_t)slot * stage_bytes + lane * 16;
             const float4* ra = reinterpret_cast<const float4*>(sa + (size_t)w * S::FW * kF32Row);
             const float4* rb = reinterpret_cast<const float4*>(sa + abytes);
             float4 va[S::FW];
@@ -135,15 +135,16 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
                 for (int f = 0; f < S::FW; ++f) acc[f][c] = dot4(va[f], vb, acc[f][c]);
             }
         }
-        if (it + S::STAGES < nst) {                        // the stage is free: refill it
+        if (it + ST < nst) {                               // the stage is free: refill it
             __syncthreads();
-            if (tid == 0 && !*(volatile int*)&s_err) { issue(it + S::STAGES); issued = it + S::STAGES + 1; }
+            if (tid == 0 && !*(volatile int*)&s_err) { issue(it + ST, slot); issued = it + ST + 1; }
         }
+        if (++slot == ST) { slot = 0; parity ^= 1; }
     }
     if (tid == 0 && *(volatile int*)&s_err) {
         // copies still land in this CTA's shared memory: wait (bounded again) for the stages issued last
-        for (int it = issued > S::STAGES ? issued - S::STAGES : 0; it < issued; ++it)
-            mbar_wait(&bar[it % S::STAGES], (it / S::STAGES) & 1, wait_limit);
+        for (int it = issued > ST ? issued - ST : 0; it < issued; ++it)
+            mbar_wait(&bar[it % ST], (it / ST) & 1, wait_limit);
         report_give_up(asrc.hdr, asrc.begins);
     }
     pdl_launch_dependents();                               // (not at the start: the gather's CTAs would take the place
@@ -191,6 +192,32 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
     trace_mark(asrc.hdr, 2, true);
 }
 
+// Stages of the ring.  A ring of four leaves room for two CTAs of 32 frames on an SM, one of three for three, which is better
+// where a launch then fits the GPU at once, or is several times what fits; no more than the channels fill, so that short rows
+// make room for more CTAs.  A launch that fits with the whole ring keeps it (us per pass, replayed graph, whole ring / as here:
+// 98 x 10 x 32 x 352 37.1 / 32.5, 64 x 24 x 24 x 512 46.4 / 43.9, two of 102 x 15 x 12 x 288 40.0 / 37.7, 34 x 15 x 15 x 3312 at
+// r = 0 68.3 / 62.7; with three stages where this takes four, 68 x 13 x 15 x 2520 84.7 / 95.0 and 32 x 16 x 16 x 1152 22.7 / 24.4).
+template <int R> static int ring_stages(const Problem& p, long long units, int FR) {
+    using S = F32Shape<R>;
+    const int nst = (p.C + kF32KC - 1) / kF32KC;
+    auto places = [&](int stages) { return (long long)sm_count() * (220 * 1024 / (stages * (FR + S::WIN) * kF32Row)); };
+    if (units <= places(S::STAGES)) return S::STAGES;
+    if (nst < S::STAGES) return nst < 2 ? 2 : nst;
+    return R < 2 && (units <= places(3) || units > 2 * places(3)) ? 3 : S::STAGES;
+}
+
+template <int R, int G, int ST>
+static cudaError_t launch_f32_ring(const Problem& p, const Scratch& s, const ClipMaps<G>& maps, int FR, unsigned units, int* out_anchor,
+                                   float* shat, int* dst, unsigned char* keep, cudaStream_t st) {
+    using S = F32Shape<R>;
+    const auto kernel = k_match_f32<R, G, ST>;
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), (size_t)ST * (32 + S::WIN) * kF32Row);
+    if (e != cudaSuccess) return e;
+    return launch_ex(true, (size_t)ST * (FR + S::WIN) * kF32Row, kernel, dim3(units, p.nclips), dim3(FR / S::FW * 32), st, maps, p.F, p.H,
+                     p.W, p.C, p.t, make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, wait_poll_limit(), wait_tx_extra(),
+                     p.sstride, p.fuse_cnt);
+}
+
 // Frames per CTA: 32 reads the window rows least often (41 rows per 32 at r = 1, 25 per 16), but a grid of fewer than
 // three CTAs per two SMs leaves SMs idle: then 16, then 8 (at least FW).
 template <int R, int G>
@@ -204,13 +231,12 @@ static cudaError_t launch_f32_t(const Problem& p, const Scratch& s, int* out_anc
         if (!make_tensor_map(&maps.a[n], p.xs.X[n], 0, p.F, p.H, p.W, p.C, kF32KC, 1, 1, FR, false) ||
             !make_tensor_map(&maps.b[n], p.xs.X[n], 0, p.F, p.H, p.W, p.C, kF32KC, S::SIDE, S::SIDE, 1, false))
             return cudaErrorInvalidValue;
-    const size_t smem = (size_t)S::STAGES * (FR + S::WIN) * kF32Row;
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_f32<R, G>), (size_t)S::STAGES * (32 + S::WIN) * kF32Row);
-    if (e != cudaSuccess) return e;
     const long long units = (long long)p.N * ((p.F + FR - 1) / FR);
-    return launch_ex(true, smem, k_match_f32<R, G>, dim3((unsigned)units, p.nclips), dim3(FR / S::FW * 32), st, maps, p.F, p.H,
-                     p.W, p.C, p.t, make_anchor_src(p, s, out_anchor), shat, dst, keep, s.cnt, wait_poll_limit(),
-                     wait_tx_extra(), p.sstride, p.fuse_cnt);
+    const int stages = ring_stages<R>(p, units * p.nclips, FR);
+    if constexpr (R < 2)
+        if (stages == 4) return launch_f32_ring<R, G, 4>(p, s, maps, FR, (unsigned)units, out_anchor, shat, dst, keep, st);
+    return stages == 3 ? launch_f32_ring<R, G, 3>(p, s, maps, FR, (unsigned)units, out_anchor, shat, dst, keep, st)
+                       : launch_f32_ring<R, G, 2>(p, s, maps, FR, (unsigned)units, out_anchor, shat, dst, keep, st);
 }
 
 cudaError_t launch_match_f32(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,

@@ -32,3 +32,10 @@ def test_gives_up_and_recovers():
         P.ttf_debug_set_wait()
     check_clip(X, 1, 0.7)
     assert P.ttf_last_device_status() == B.TTF_OK
+
+
+@pytest.mark.parametrize("r", [0, 1, 2])
+@pytest.mark.parametrize("shape", [(33, 20, 20, 100), (40, 21, 20, 132), (64, 20, 16, 260), (33, 24, 25, 384), (70, 24, 24, 516)])
+def test_rings_of_fewer_stages(shape, r):
+    """more units than fit the GPU with the whole ring, rows of one to five stages"""
+    check_clip(corr_clip(*shape, seed=sum(shape) + r, dtype="f32"), r, 0.6)
