@@ -17,7 +17,6 @@
 #include "ttf_async.cuh"
 #include "ttf_cluster.cuh"
 
-#include <cstdlib>
 #include <map>
 #include <mutex>
 #include <set>
@@ -624,9 +623,6 @@ cudaError_t launch_frame_stats(const Problem& p, const Scratch& s, int* out_anch
         // slices, 16 x 16 x 16 x 1024 15.2 / 15.4).
         if (p.nsl == 2 && p.F <= 64) return launch_stats_cluster_t<2, 1>(p, s, out_anchor, st);
         if (p.nsl <= 4 && p.F <= 32) return launch_stats_cluster_t<4, 1>(p, s, out_anchor, st);
-        static const int lim = getenv("TTF_ST") ? atoi(getenv("TTF_ST")) : 64;
-        if (p.nsl <= 4 && p.nsl * p.F <= lim) return p.nsl == 2 ? launch_stats_cluster_t<2, 1>(p, s, out_anchor, st) : launch_stats_cluster_t<4, 1>(p, s, out_anchor, st);
-        if (p.nsl <= 8 && p.nsl * p.F <= lim) return launch_stats_cluster_t<8, 1>(p, s, out_anchor, st);
         const bool alone = p.overlapped <= 1 && large_clusters();
         if (p.nsl > 16) return alone ? launch_stats_cluster_t<2, 16>(p, s, out_anchor, st)
                                      : launch_stats_cluster_t<4, 8>(p, s, out_anchor, st);
