@@ -147,7 +147,10 @@ int ttf_compress(const void* features, int F, int H, int W, int C, int r, float 
  * (half of the batch, at most 16), and the groups are spread round-robin over two streams ("lanes")
  * that the library keeps per device; these fork from `stream` and join it again through events, so the call is
  * asynchronous, ordered on `stream` like any other, and can be captured in a CUDA graph.  The kernels of one group
- * leave part of the GPU idle while they ramp up and drain; the other lane's fill those gaps
+ * leave part of the GPU idle while they ramp up and drain; the other lane's fill those gaps.  Small batches (up to
+ * eight clips of 64 MB together, 160 MB with a fixed anchor; outside a capture up to sixteen of 16 or 32 MB) run on `stream`
+ * itself instead, in groups of up to eight, on scratch that belongs to the stream; where that cannot be had (a capture
+ * on a stream that has none) they take the lanes
  * (ttf_set_schedule asks for a number of single clips in flight instead; a lane then chains its clips on two scratch
  * blocks used in turn: the sweep of a clip runs beside the gather of the clip before it).  The streams, their events and
  * the scratch are created by the first call on a device: make that call outside any stream capture.  The scratch (the

@@ -23,16 +23,17 @@ static int cuda_fail(cudaError_t e) {
 }
 
 int sm_count() {
-    static std::mutex mu;
-    static std::map<int, int> cache;
+    constexpr int kDevices = 64;
+    static std::atomic<int> cache[kDevices];     // (asked several times per call: no lock)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(dev);
-    if (it != cache.end()) return it->second;
+    if (dev >= 0 && dev < kDevices) {
+        const int n = cache[dev].load(std::memory_order_relaxed);
+        if (n > 0) return n;
+    }
     int n = 148;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 148;
-    cache[dev] = n;
+    if (dev >= 0 && dev < kDevices) cache[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
@@ -1192,7 +1193,7 @@ int ttf_profile_stages(const void* const* features, int nclips, int F, int H, in
         if (n == 0) p0 = p;
         same_layout = same_layout && p.vec == p0.vec && (!p.vec || aligned(n) == aligned(0));
     }
-    const BatchPlan plan = plan_batch(p0, nclips, same_layout);
+    const BatchPlan plan = plan_batch(p0, nclips, same_layout, takes_own_stream(p0, nclips, same_layout, false, st));
     std::vector<GroupLaunch> gs;                 // the launches a batch call of these clips would make
     for (int n0 = 0; n0 < nclips; n0 += plan.group)
         gs.push_back(group_launch(plan, p0, nullptr, stride, features, nclips, n0, out_tokens, out_count, out_pos_thw));
