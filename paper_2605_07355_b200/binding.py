@@ -24,7 +24,7 @@ EXPORTS = [
     "ttf_query", "ttf_query_ws", "ttf_compress_host", "ttf_release", "ttf_profile_begin", "ttf_profile_end",
     "ttf_query_static", "ttf_compress_ex", "ttf_query_ex", "ttf_compress_segment", "ttf_restore",
     "ttf_sim_histogram", "ttf_stats", "ttf_compress_batch", "ttf_compress_batch_ex", "ttf_profile_stages", "ttf_profile_read_floor", "ttf_compress_mean", "ttf_compress_host_batch",
-    "ttf_set_schedule", "ttf_set_match_kernel", "ttf_last_device_status", "ttf_workspace_status", "ttf_debug_set_wait", "ttf_debug_func_attr_needed", "ttf_debug_set_check_slack",
+    "ttf_set_schedule", "ttf_set_match_kernel", "ttf_last_device_status", "ttf_workspace_status", "ttf_debug_set_wait", "ttf_debug_func_attr_needed", "ttf_debug_set_check_slack", "ttf_debug_match_split",
 ]
 TTF_ERR_TIMEOUT, TTF_ERR_STATIC_LIMIT, TTF_ERR_BOUNDS = 5, 6, 7
 TTF_ANCHOR_AUTO, TTF_ANCHOR_FIRST, TTF_ANCHOR_LAST, TTF_ANCHOR_EXPLICIT = 0, 1, 2, 3
@@ -83,6 +83,8 @@ def lib() -> ctypes.CDLL:
         L.ttf_workspace_status.argtypes = [vp, vp, ctypes.POINTER(i)]
         L.ttf_debug_set_check_slack.restype = i
         L.ttf_debug_set_check_slack.argtypes = [i]
+        L.ttf_debug_match_split.restype = i
+        L.ttf_debug_match_split.argtypes = [i] * 6 + [ctypes.POINTER(i)]
         L.ttf_debug_set_wait.restype = i
         L.ttf_debug_set_wait.argtypes = [i, i]
         L.ttf_debug_func_attr_needed.restype = i
@@ -303,6 +305,17 @@ def ttf_debug_set_wait(poll_limit: int = 1 << 18, tx_extra_bytes: int = 0) -> No
 def ttf_debug_set_check_slack(slack: int = 0) -> int:
     """ttf_debug_set_check_slack: returns the status (TTF_ERR_UNSUPPORTED = 2 from the normal build)."""
     return int(lib().ttf_debug_set_check_slack(int(slack)))
+
+
+def ttf_debug_match_split(F: int, H: int, W: int, C: int, r: int, clips: int = 1):
+    """ttf_debug_match_split: (grid rows of a tile, chunks of its channels, CTAs per tile), or None."""
+    split = (ctypes.c_int * 3)()
+    rc = lib().ttf_debug_match_split(F, H, W, C, r, clips, split)
+    if rc == 2:                                  # TTF_ERR_UNSUPPORTED: not a clip of the tcgen05 kernel
+        return None
+    if rc != TTF_OK:
+        raise TTFError(rc, "ttf_debug_match_split")
+    return tuple(split)
 
 
 def ttf_set_match_kernel(which: int = 0) -> None:

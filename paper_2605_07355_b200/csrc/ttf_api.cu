@@ -444,6 +444,18 @@ int ttf_debug_func_attr_needed(const void* key, int device, size_t bytes) {
     return g_func_attr.needs(key, device, bytes) ? 1 : 0;
 }
 
+int ttf_debug_match_split(int F, int H, int W, int C, int r, int clips, int* split) {
+    if (!split || clips < 1 || clips > kMaxGroup) return TTF_ERR_INVALID_ARG;
+    Problem p;
+    int rc = make_problem(reinterpret_cast<const void*>(uintptr_t(256)), F, H, W, C, r, 0.f, TTF_DTYPE_BF16, &p);
+    if (rc != TTF_OK) return rc;
+    if (!tc_match_eligible(p)) return TTF_ERR_UNSUPPORTED;
+    p.nclips = clips;
+    const TcPlan t = tc_plan(p);
+    split[0] = t.rows; split[1] = t.chunks; split[2] = t.pieces;
+    return TTF_OK;
+}
+
 int ttf_workspace_bytes(int F, int H, int W, int C, int r, int dtype, size_t* bytes) {
     if (!bytes) return TTF_ERR_INVALID_ARG;
     Problem p;

@@ -151,6 +151,8 @@ inline bool match_begins_call(const Problem& p, const OutPtrs& out) {
 // tcgen05 matching (ttf_match_tc.cu)
 bool tc_match_eligible(const Problem& p);
 size_t tc_match_tiles(const Problem& p);
+struct TcPlan { int rows; long long tiles; int chunks, pieces; };      // grid rows of a tile, tiles of a clip, parts of a tile's
+TcPlan tc_plan(const Problem& p);                                      // channel range, CTAs that share a tile
 cudaError_t launch_match_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                             unsigned char* keep, cudaStream_t st);
 

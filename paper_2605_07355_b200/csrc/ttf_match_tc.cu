@@ -119,24 +119,33 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int NB) {
 }
 
 // ---- the kernel -------------------------------------------------------------------------------------------
+// MMA N of a tile of `wy` grid rows
+constexpr int tile_columns(int r, int wy) { return ((kTcWB + 2 * r) * (wy + 2 * r) + 15) / 16 * 16; }
+// Chunks of a tile at most: the same whatever its rows, so that no sum in tensor memory has more terms than in tiles of one row
+// (a tensor-memory accumulator truncates: similarities of 8 x 8 x 8 x 4096 at r = 1 against 64 bits 5.4e-7 with eight chunks,
+// 1.3e-6 with four, which took 20.5 us per pass against 17.3; 4 x 12 x 12 x 4096 1.1e-6 -> 4.9e-7 and 20.1 -> 17.1 us).
+constexpr int max_chunks(int r) { return r == 2 ? 4 : 8; }
+// ... and of one CTA (256 columns of tensor memory at most: two CTAs per SM)
+constexpr int own_chunks(int nb) { return nb > 32 ? 4 : 8; }
+
 template <int R, int WY> struct TcShape {
     static constexpr int FR = kTcM / (kTcWB * WY);        // frames per tile
     static constexpr int SIDE = 2 * R + 1;
     static constexpr int BW = kTcWB + 2 * R, BH = WY + 2 * R;      // candidate cells: columns, rows
     static constexpr int NCAND = BW * BH;                 // rows the B box delivers
-    static constexpr int NB = (NCAND + 15) / 16 * 16;     // MMA N
+    static constexpr int NB = tile_columns(R, WY);        // MMA N
     static constexpr int BBYTES = NB * 128;
     static constexpr int BBOX = NCAND * 128;              // bytes one B box copy delivers
     static constexpr int STAGE = kTcABytes + BBYTES;
     static constexpr int STAGES = 4;                      // two CTAs per SM with room left for CTAs of other kernels
     static constexpr int WIN = SIDE * SIDE;               // candidates of one source row
-    static constexpr int MAXCH = NB > 32 ? 4 : 8;         // chunks at most (tensor memory: MAXCH * NB <= 256 columns)
+    static constexpr int MAXCH = max_chunks(R), OWNCH = own_chunks(NB);
     // what one rank sends another (and itself): window sums and squared norms of the rows the other one finishes,
     // squared norms of the candidates
     static constexpr int XBYTES = (kTcM * (WIN + 1) + MAXCH * NCAND) * 4;                 // received by one rank
     static constexpr int RING = STAGES * STAGE;
     static constexpr int NP = NCAND * 8;                  // (candidate row, 16-byte piece column) pairs
-    static constexpr int NORMBYTES = MAXCH * (kTcM + NP) * 4;
+    static constexpr int NORMBYTES = OWNCH * (kTcM + NP) * 4;
 };
 
 // m is all ones or zero: a or b without a branch.  (The window of a row starts at one of four columns; as conditional
@@ -247,7 +256,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     const int m = q * 32 + lane;                           // source row of an epilogue thread: (frame, cell row, cell column)
     const int et = (warp - 2) * 32 + lane;                 // 0..127 among the epilogue threads
     float* const s_na = reinterpret_cast<float*>(dyn + S::RING + S::XBYTES);      // [chunk][row] squared norms
-    float* const s_nbp = s_na + S::MAXCH * kTcM;           // [chunk][candidate row, piece column]
+    float* const s_nbp = s_na + S::OWNCH * kTcM;           // [chunk][candidate row, piece column]
     const int dx = m & 3, dy = (m >> 2) & (WY - 1);
     float win[S::WIN];                                     // this row's window of dot products
     float na = 0.f, nb = 0.f;                              // squared norm of source row m / of candidate row et
@@ -370,7 +379,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
                 tmem_ld<NG>(lanes + (uint32_t)(h * S::NB), x);
                 tmem_ld<NG>(lanes + (uint32_t)((h + 1) * S::NB), z);
                 tmem_add<NG>(x, z);
-                if (S::MAXCH > 4 && h == 4) {
+                if (S::OWNCH > 4 && h == 4) {
                     uint32_t u[NG][8];
                     tmem_ld<NG>(lanes + (uint32_t)(6 * S::NB), u);
                     tmem_ld<NG>(lanes + (uint32_t)(7 * S::NB), z);
@@ -542,7 +551,7 @@ static int tile_rows(const Problem& p) {
 size_t tc_match_tiles(const Problem& p) { return tiles_of(p, tile_rows(p)); }
 
 // Parts of a tile's channel range: the largest power of two with which a launch over one clip still fits the GPU in one
-// wave of two CTAs per SM, at most 8 (4 for r = 2) and at least 2 stages each (4 stages: 16 x 8 x 8 x 512 13.9 us per pass,
+// wave of two CTAs per SM, at most max_chunks and at least 2 stages each (4 stages: 16 x 8 x 8 x 512 13.9 us per pass,
 // 2: 12.9, 1: 13.3; 16 x 14 x 14 x 512 16.7 / 15.3 / 15.3).  (One CTA per SM with a ring twice as deep measured the same
 // alone, 18.8 against 19.2 us on a cold 8B-shaped clip, and slower with other clips' kernels beside it, 34.0 against
 // 32.2 us per clip.)
@@ -582,6 +591,33 @@ static long long cluster_places(int n) {
     return known[{dev, n}] = found;
 }
 
+// How a launch splits its work.  The tile and its chunks depend on the clip's shape alone, the CTAs (= cluster size) of a tile on
+// what is in flight.
+TcPlan tc_plan(const Problem& p) {
+    TcPlan t;
+    t.rows = tile_rows(p);
+    t.tiles = (long long)tiles_of(p, t.rows);
+    t.chunks = split_of(p, t.tiles, max_chunks(p.r));
+    const int own = own_chunks(tile_columns(p.r, t.rows));
+    // (eight parts of 48 columns are not worth a second CTA on an SM: 5 x 29 x 13 x 1016 17.0 us per pass, with four 16.1)
+    if (t.chunks > own && t.tiles * t.chunks > sm_count()) {
+        const int one_row = split_of(p, (long long)tiles_of(p, 1), max_chunks(p.r));
+        t.chunks = one_row > own ? one_row : own;
+    }
+    // Three or more single clips in flight (ttf_set_schedule, clips that cannot share a launch)
+    // fill the GPU together: 16 clips of 32 x 16 x 16 x 4096 on eight lanes 497 -> 445 us, on three 512 -> 506 (on two 530 ->
+    // 507, but three clips, of which two share a launch, 98 -> 102).
+    const int beside = p.nclips == 1 && p.overlapped >= 3 ? p.overlapped : 1;
+    // Not more than run at the same time: the cluster that has to wait for a place costs the whole main loop once more (us per
+    // pass, 32 frames of 2048 channels: 71 tiles in fours 23.4, 72 in fours 30.9, in twos 27.2; 33 in eights 19.6, 34 in
+    // eights 23.8, in fours 20.6; 12 x 24 x 24 x 2048 28.8 -> 26.0).
+    const long long units = t.tiles * p.nclips * beside;
+    t.pieces = split_of(p, units, t.chunks);
+    while (t.pieces > 1 && units > cluster_places(t.pieces)) t.pieces /= 2;
+    if (t.pieces * own < t.chunks) t.pieces = t.chunks / own;
+    return t;
+}
+
 template <int R, int WY, int G>
 static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                unsigned char* keep, cudaStream_t st) {
@@ -595,18 +631,9 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
     const size_t need = (size_t)S::RING + S::XBYTES + S::NORMBYTES + 1024, smem = need < 80 * 1024 ? 80 * 1024 : need;
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R, WY, G>), smem);
     if (e != cudaSuccess) return e;
-    const long long tiles = (long long)tiles_of(p, WY);
-    const int chunks = split_of(p, tiles, S::MAXCH);
-    // CTAs (= cluster size) per tile.  Three or more single clips in flight (ttf_set_schedule, clips that cannot share a launch)
-    // fill the GPU together: 16 clips of 32 x 16 x 16 x 4096 on eight lanes 497 -> 445 us, on three 512 -> 506 (on two 530 ->
-    // 507, but three clips, of which two share a launch, 98 -> 102).
-    const int beside = p.nclips == 1 && p.overlapped >= 3 ? p.overlapped : 1;
-    // Not more than run at the same time: the cluster that has to wait for a place costs the whole main loop once more (us per
-    // pass, 32 frames of 2048 channels: 71 tiles in fours 23.4, 72 in fours 30.9, in twos 27.2; 33 in eights 19.6, 34 in
-    // eights 23.8, in fours 20.6; 12 x 24 x 24 x 2048 28.8 -> 26.0).
-    const long long units = tiles * p.nclips * beside;
-    int pieces = split_of(p, units, chunks);
-    while (pieces > 1 && units > cluster_places(pieces)) pieces /= 2;
+    const TcPlan plan = tc_plan(p);
+    const long long tiles = plan.tiles;
+    const int chunks = plan.chunks, pieces = plan.pieces;
     auto log2_of = [](int n) { int l = 0; while ((1 << l) < n) ++l; return l; };
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles * pieces), p.nclips); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;

@@ -61,3 +61,30 @@ def test_bits_of_tiles_of_fewer_frames(shape, r, clips):
 def test_as_many_clusters_as_run_at_once_and_one_more(tiles):
     X = corr_clip(3, tiles * 4, 4, 256 if tiles < 100 else 128, seed=tiles, dtype="bf16")
     check_clip(X, 1, 0.6)
+
+
+@pytest.mark.parametrize("shape", [(8, 8, 8, 4096), (4, 12, 12, 4096), (8, 10, 10, 4096)])
+def test_error_of_the_similarities_of_short_clips(shape):
+    """Against 64 bits.  A sum in tensor memory loses at most 2^-23 of its value per addition, half of that on average, and half of
+    it again while it grows: n additions n 2^-25.  Eight parts of 4096 channels are 32 additions of 16 channels each."""
+    F, H, W, C = shape
+    X = to_device(corr_clip(*shape, seed=sum(shape), dtype="bf16"))
+    q = P.ttf_query(X, 1, 0.6)
+    x = X.double()
+    x = x / x.norm(dim=-1, keepdim=True)
+    anchor = x[int(q["anchor"])]
+    best = torch.full((F, H, W), -2.0, dtype=torch.float64, device="cuda")
+    for dy in (-1, 0, 1):
+        for dx in (-1, 0, 1):
+            y0, y1, x0, x1 = max(0, -dy), min(H, H - dy), max(0, -dx), min(W, W - dx)
+            sim = (x[:, y0:y1, x0:x1] * anchor[y0 + dy:y1 + dy, x0 + dx:x1 + dx]).sum(-1)
+            best[:, y0:y1, x0:x1] = torch.maximum(best[:, y0:y1, x0:x1], sim)
+    best[int(q["anchor"])] = 1.0
+    assert float((q["best_sim"].view(F, H, W).double() - best).norm() / best.norm()) < 32 * 2.0 ** -25
+
+
+def test_a_cta_never_sums_more_parts_than_its_tensor_memory_holds():
+    """so many tiles that one CTA each would fill the GPU, in eight parts of 48 columns"""
+    shape, clips = (8, 20, 8, 1024), 32
+    assert P.ttf_debug_match_split(*shape, 1, clips=16) == (4, 8, 2) and P.ttf_debug_match_split(*shape, 1) == (4, 8, 8)
+    test_bits_do_not_depend_on_the_split(shape, 1, clips)
