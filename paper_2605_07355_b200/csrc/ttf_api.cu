@@ -165,15 +165,33 @@ static int make_problem(const void* X, int F, int H, int W, int C, int r, float 
 struct CacheEntry {
     void* ptr = nullptr; size_t bytes = 0;
     size_t unit = 0;                             // scratch of the largest clip seen on this stream
-    std::vector<void*> outgrown;                 // smaller blocks of the same clips, which captured graphs may still use
+    std::vector<std::pair<void*, size_t>> outgrown;      // smaller blocks of the same clips, which captured graphs may still use
     std::vector<const int*> status_words;        // header blocks the most recent call on this stream used
     int status_index = HDR_ERROR;                // ... and the word of each that tells how it went
+    int status_kept = 0;                         // what the words of blocks said that have been given back since
 };
 typedef std::map<std::pair<int, cudaStream_t>, CacheEntry> ScratchCache;
 static std::mutex g_mu;
 static ScratchCache g_scratch;
 static ScratchCache g_batch_scratch;             // of small batches (batch_on_stream), apart from the scratch of other calls:
                                                  // batches may be enqueued from several threads
+
+// Gives a block back on which nothing runs any more (g_mu is held).  The words in it that tell how the last call on a stream went
+// (of this stream, or of one whose batch ran on this lane) are read for the last time.
+static void free_block(void* ptr, size_t bytes) {
+    const uintptr_t b = reinterpret_cast<uintptr_t>(ptr);
+    for (auto& kv : g_scratch) {
+        CacheEntry& ce = kv.second;
+        for (size_t i = 0; i < ce.status_words.size();) {
+            if (reinterpret_cast<uintptr_t>(ce.status_words[i]) - b >= bytes) { ++i; continue; }
+            int v = 0;
+            if (cudaMemcpy(&v, ce.status_words[i] + ce.status_index, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) cudaGetLastError();
+            if (v > ce.status_kept) ce.status_kept = v;
+            ce.status_words.erase(ce.status_words.begin() + i);
+        }
+    }
+    cudaFree(ptr);
+}
 
 // `bytes` of scratch for a call on `st`; `unit` is the scratch of one of its clips.  The block moves when a larger clip
 // arrives.  A block that is too small because the call has more clips than those before it is kept beside its successor:
@@ -190,17 +208,16 @@ static int cached_scratch(size_t bytes, size_t unit, cudaStream_t st, void** out
             // earlier calls on this stream may still read the old blocks
             e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) return cuda_fail(e);
-            cudaFree(ce.ptr);
-            for (void* q : ce.outgrown) cudaFree(q);
+            free_block(ce.ptr, ce.bytes);
+            for (auto& q : ce.outgrown) free_block(q.first, q.second);
             ce.ptr = nullptr; ce.bytes = 0;
             ce.outgrown.clear();
-            ce.status_words.clear();
         }
         if (bytes < 2 * ce.bytes) bytes = 2 * ce.bytes;
         void* fresh = nullptr;
         e = cudaMalloc(&fresh, bytes);
         if (e != cudaSuccess) return cuda_fail(e);
-        if (ce.ptr) ce.outgrown.push_back(ce.ptr);
+        if (ce.ptr) ce.outgrown.push_back({ce.ptr, ce.bytes});
         ce.ptr = fresh; ce.bytes = bytes;
         // the arrival counters must start at zero; the kernels leave them at zero after every call
         e = cudaMemsetAsync(ce.ptr, 0, bytes, st);
@@ -210,6 +227,7 @@ static int cached_scratch(size_t bytes, size_t unit, cudaStream_t st, void** out
     *out = ce.ptr;
     ce.status_words.assign(1, reinterpret_cast<const int*>(ce.ptr));
     ce.status_index = HDR_ERROR;
+    ce.status_kept = 0;
     return TTF_OK;
 }
 static size_t scratch_held(cudaStream_t st, ScratchCache& cache = g_scratch) {
@@ -372,8 +390,8 @@ const char* ttf_status_string(int status) {
 
 int ttf_last_cuda_error(void) { return tl_cuda_error; }
 
-static int read_status_words(const std::vector<const int*>& words, int index, int* host_status) {
-    *host_status = TTF_OK;
+static int read_status_words(const std::vector<const int*>& words, int index, int* host_status, int kept = 0) {
+    *host_status = kept == 2 ? TTF_ERR_BOUNDS : (kept ? TTF_ERR_TIMEOUT : TTF_OK);
     for (const int* hdr : words) {
         int v = 0;
         cudaError_t e = cudaMemcpy(&v, hdr + index, sizeof(int), cudaMemcpyDeviceToHost);
@@ -393,13 +411,13 @@ int ttf_last_device_status(ttf_stream_t stream, int* host_status) {
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
     std::vector<const int*> words;
-    int index = HDR_ERROR;
+    int index = HDR_ERROR, kept = 0;
     {
         std::lock_guard<std::mutex> lk(g_mu);
         auto it = g_scratch.find(std::make_pair(dev, st));
-        if (it != g_scratch.end()) { words = it->second.status_words; index = it->second.status_index; }
+        if (it != g_scratch.end()) { words = it->second.status_words; index = it->second.status_index; kept = it->second.status_kept; }
     }
-    return read_status_words(words, index, host_status);     // no call of the library on this stream yet: TTF_OK
+    return read_status_words(words, index, host_status, kept);     // no call of the library on this stream yet: TTF_OK
 }
 
 int ttf_workspace_status(const void* workspace, ttf_stream_t stream, int* host_status) {
@@ -743,6 +761,7 @@ static void report_batch(cudaStream_t st, const std::vector<const int*>& words) 
     CacheEntry& ce = g_scratch[std::make_pair(dev, st)];
     ce.status_words = words;
     ce.status_index = HDR_BATCH_ERROR;           // (groups that use the same blocks in turn clear the other word)
+    ce.status_kept = 0;
 }
 
 // Scratch of the lanes of `plan`.  Where it cannot grow, inside a capture or for lack of memory, the groups become as large as
@@ -1276,7 +1295,7 @@ int ttf_release(void) {
             cudaError_t e = cudaDeviceSynchronize();
             if (e != cudaSuccess && first == cudaSuccess) first = e;
             if (kv.second.ptr) cudaFree(kv.second.ptr);
-            for (void* q : kv.second.outgrown) cudaFree(q);
+            for (auto& q : kv.second.outgrown) cudaFree(q.first);
         }
         cache->clear();
     }

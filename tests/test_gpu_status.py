@@ -146,3 +146,55 @@ def test_a_batch_reports_a_clip_whose_scratch_block_a_later_clip_used():
         assert P.ttf_last_device_status(st) == B.TTF_OK
     finally:
         P.ttf_set_schedule(0)
+
+
+def test_the_status_of_a_batch_outlives_its_scratch():
+    """a batch over the lanes; then a larger clip on another stream takes the place of the lanes' scratch"""
+    Xs = [to_device(corr_clip(4, 5, 5, 64, seed=83, dtype="bf16"))] * 3
+    larger = [to_device(corr_clip(40, 16, 16, 512, seed=84, dtype="bf16"))] * 3
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    P.ttf_release()
+    P.ttf_set_schedule(2)
+    try:
+        for limits, status in (((32, 16), B.TTF_ERR_TIMEOUT), ((), B.TTF_OK)):
+            P.ttf_debug_set_wait(*limits)
+            P.ttf_compress_batch(Xs, 1, 0.7, stream=a)
+            P.ttf_debug_set_wait()
+            P.ttf_compress_batch(larger, 1, 0.7, stream=b)
+            assert P.ttf_last_device_status(b) == B.TTF_OK
+            assert P.ttf_last_device_status(a) == status
+            P.ttf_release()
+    finally:
+        P.ttf_debug_set_wait()
+        P.ttf_set_schedule(0)
+
+
+def test_status_after_a_batch_that_found_no_memory():
+    """small batches on the caller's stream: the block of the first makes room for a larger clip's, for which there is no memory"""
+    Xs = [to_device(corr_clip(4, 5, 5, 64, seed=85, dtype="bf16"))] * 3
+    larger = [to_device(corr_clip(256, 1, 1, 32768, seed=86, dtype="bf16"))] * 3      # (more than 40 MB of scratch each)
+    outs = P.ttf_compress_batch(larger, 1, 0.7)              # (loads the kernels, before memory is short)
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    P.ttf_release()
+    P.ttf_debug_set_wait(32, 16)
+    try:
+        P.ttf_compress_batch(Xs, 1, 0.7, stream=st)
+        torch.cuda.synchronize()
+    finally:
+        P.ttf_debug_set_wait()
+    hold, size = [], 64 << 30
+    while size >= 16 << 20:
+        try:
+            hold.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+        except torch.cuda.OutOfMemoryError:
+            size //= 2
+    try:
+        with pytest.raises(P.TTFError):
+            P.ttf_compress_batch(larger, 1, 0.7, *outs, stream=st)
+        assert P.ttf_last_device_status(st) == B.TTF_ERR_TIMEOUT          # (of the batch before: nothing of the other one ran)
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+    P.ttf_compress_batch(larger, 1, 0.7, *outs, stream=st)
+    assert P.ttf_last_device_status(st) == B.TTF_OK
