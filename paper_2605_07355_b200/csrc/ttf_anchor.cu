@@ -61,13 +61,6 @@ __device__ __forceinline__ float fold8(float (&v)[8], int lane) {
     return r;
 }
 
-// The control words of a block at the start of a call: the error word reports on this call only; a block that may hold anything
-// (fresh) also gets its arrival counter and the error word of its batch cleared.
-__device__ __forceinline__ void clear_words(int* hdr, bool fresh) {
-    hdr[HDR_ERROR] = 0;
-    if (fresh) { hdr[HDR_DONE_ALL] = 0; hdr[HDR_BATCH_ERROR] = 0; }
-}
-
 // LS: lanes across a slice (8, 16 or 32); RG = 256 / LS row groups walk the tokens interleaved.
 // CLS: a thread keeps CLS running sums, of every CLS-th of its tokens.  A sum over all tokens is the same tree whether 32
 // classes of tokens belong to 32 row groups of 8 lanes (CLS = 1), to 16 of 16 (2) or to 8 of 32 (4): class w + 8 J to warp w,

@@ -266,18 +266,23 @@ static std::atomic<int> g_check_slack{0};
 __global__ void k_set_word(int* word, int value, size_t stride) {
     *reinterpret_cast<int*>(reinterpret_cast<uintptr_t>(word) + blockIdx.x * stride) = value;
 }
+// What precedes the first kernel of a call: the slack, and what clear_words leaves to it.
+static cudaError_t begin_checked(const Problem& p, const Scratch& s, cudaStream_t st) {
+    auto set = [&](int word, int value) { k_set_word<<<p.nclips, 1, 0, st>>>(s.hdr + word, value, p.sstride); };
+    set(HDR_CHECK_SLACK, g_check_slack.load());
+    set(HDR_ERROR, 0);
+    if (p.fresh) { set(HDR_BATCH_ERROR, 0); set(HDR_DONE_ALL, 0); }
+    return cudaGetLastError();
+}
+#else
+static cudaError_t begin_checked(const Problem&, const Scratch&, cudaStream_t) { return cudaSuccess; }
 #endif
 
 // steps shared by compress and query: norms + frame sums, anchor, matching + gate
 static int run_front(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                      unsigned char* keep, cudaStream_t st) {
-    cudaError_t e;
-#ifdef TTF_DEBUG
-    k_set_word<<<p.nclips, 1, 0, st>>>(s.hdr + HDR_CHECK_SLACK, g_check_slack.load(), p.sstride);
-    e = cudaGetLastError();
+    cudaError_t e = begin_checked(p, s, st);
     if (e != cudaSuccess) return cuda_fail(e);
-#endif
-    e = cudaSuccess;
     if (!p.match_begins) { ProfScope ps(st, PK_NORM_SUM); e = launch_norm_sum(p, s, st); }
     if (e != cudaSuccess) return cuda_fail(e);
     if (p.anchor_mode == 0) {
@@ -891,7 +896,8 @@ static int batch_on_streams(const void* const* features, int nclips, int F, int 
         // ran in the other lane).
         Scratch sc;
         carve_scratch(p, block, &sc);
-        { ProfScope pr(ls, PK_NORM_SUM); e = launch_norm_sum(p, sc, ls); }
+        e = begin_checked(p, sc, ls);
+        if (e == cudaSuccess) { ProfScope pr(ls, PK_NORM_SUM); e = launch_norm_sum(p, sc, ls); }
         if (e == cudaSuccess) { ProfScope pr(ls, PK_FRAME_STATS); e = launch_frame_stats(p, sc, nullptr, ls); }
         if (e == cudaSuccess && q > 0) e = cudaStreamWaitEvent(ls, L->matched[(q - 1) % kMatchedRing], 0);
         if (e == cudaSuccess) { ProfScope pr(ls, PK_MATCH); e = launch_match(p, sc, nullptr, sc.shat, sc.dst, sc.keep, ls); }

@@ -135,17 +135,11 @@ inline bool gather_alone(const Problem& p) {
 
 // A call with a fixed anchor needs nothing of X before its matching kernel.  What is left of a kernel before it is to clear the
 // survivor counters, which the gather of one window of flags does not read, and the error word, which the matching kernel clears
-// itself: then it comes first.  (Not in the checked build, where all CTAs report through the error word from the start, nor for
-// the warp-level kernel.)  Us per pass through the
-// binding 21 x 13 x 19 x 1160 14.3 -> 12.9, 6 x 22 x 24 x 264 14.2 -> 11.6, the 9 x 16 x 16 x 4096 segment 59.7 -> 57.2; in a replayed
-// graph, where the host's part is gone, 12.4 -> 12.5, 8.8 -> 8.4, and 32 x 16 x 16 x 1152 fp32 18.8 -> 18.3.
+// itself: then it comes first.  (Not for the warp-level kernel.)  Us per pass through the binding 21 x 13 x 19 x 1160 14.3 -> 12.9,
+// 6 x 22 x 24 x 264 14.2 -> 11.6, the 9 x 16 x 16 x 4096 segment 59.7 -> 57.2; in a replayed graph, where the host's part is gone, 12.4 -> 12.5, 8.8 -> 8.4, and 32 x 16 x 16 x 1152 fp32 18.8 -> 18.3.
 inline bool match_begins_call(const Problem& p, const OutPtrs& out) {
-#ifdef TTF_DEBUG
-    return false;
-#else
     return p.anchor_mode != 0 && p.nclips == 1 && p.overlapped <= 1 && !p.chain && !p.fresh && (p.use_tc || uses_f32_match(p)) && p.vec &&
            reinterpret_cast<uintptr_t>(out.tokens[0]) % 16 == 0 && (long long)p.F * p.N <= kGatherWindow && p.F <= kWarpPrefixMaxF && gather_alone(p);
-#endif
 }
 
 // tcgen05 matching (ttf_match_tc.cu)
@@ -292,6 +286,16 @@ __device__ __forceinline__ void report_give_up(int* hdr, bool begins = false) {
     if (begins) { atomicExch(hdr + HDR_MATCH_ERROR, 1); return; }    // (HDR_ERROR may still be about to be cleared)
     atomicExch(hdr + HDR_ERROR, 1);
     atomicExch(hdr + HDR_BATCH_ERROR, 1);
+}
+
+// The control words of a block at the start of a call: the error word reports on this call only; a block that may hold anything
+// (fresh) also gets its arrival counter and the error word of its batch cleared.  (In the checked build any CTA of the first
+// kernel may report before this is done: there the words are cleared before it is launched.)
+__device__ __forceinline__ void clear_words(int* hdr, bool fresh) {
+#ifndef TTF_DEBUG
+    hdr[HDR_ERROR] = 0;
+    if (fresh) { hdr[HDR_DONE_ALL] = 0; hdr[HDR_BATCH_ERROR] = 0; }
+#endif
 }
 
 // Checked build (-DTTF_DEBUG): every global store whose index a kernel computes is guarded by in_bounds().  An

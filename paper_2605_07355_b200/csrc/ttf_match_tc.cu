@@ -246,7 +246,7 @@ k_match_tc(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C,
     trace_mark(asrc.hdr, 5, false);
     const int a = asrc.fixed >= 0 ? asrc.fixed : __ldcg(asrc.hdr + HDR_ANCHOR);
     if (blockIdx.x == 0 && tid == 0 && asrc.fixed >= 0) {
-        if (asrc.begins) asrc.hdr[HDR_ERROR] = 0;
+        if (asrc.begins) clear_words(asrc.hdr, false);
         asrc.hdr[HDR_ANCHOR] = a;                // the gather reads it from here
         if (asrc.out_anchor) *asrc.out_anchor = a;
     }

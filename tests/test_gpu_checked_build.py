@@ -30,6 +30,7 @@ for which in (1, 2):                                              # warp-level a
         X = corr_clip(F, H, W, C, seed=F + H + W + C + r, dtype=dt)
         check_clip(X, r, 0.7)
         check_clip(X, r, 0.5, order=1, pos_base=3)
+        check_clip(X, r, 0.6, anchor_mode=2)                      # (the matching kernel begins the call, where it can)
         assert P.ttf_last_device_status() == 0, (which, F, H, W, C, r, dt)
 P.ttf_set_match_kernel(0)
 s = clips.CONFIGS["vl2b_cal"]
@@ -47,6 +48,28 @@ for which in (1, 2):
     assert P.ttf_debug_set_check_slack(0) == 0
     check_clip(X, 1, 0.7)                                         # the first kernel of a call clears the word
     assert P.ttf_last_device_status() == 0
+P.ttf_set_match_kernel(0)
+
+# a report of the first kernel is not lost to the clearing of the words (a clip of one CTA, whose sums are all reported)
+small = to_device(corr_clip(1, 2, 2, 8, seed=10, dtype="f32"))
+ws = torch.zeros(P.ttf_workspace_bytes(1, 2, 2, 8, 1, 0), dtype=torch.uint8, device="cuda")
+P.ttf_debug_set_check_slack(8)
+P.ttf_query(small, 1, 0.7, workspace=ws)
+assert P.ttf_workspace_status(ws) == P.TTF_ERR_BOUNDS and int(ws.view(torch.int32)[9]) == 1
+P.ttf_debug_set_check_slack(0)
+
+# small batches on the caller's stream, whose blocks hold another shape's data
+st = torch.cuda.Stream()
+for kw in (dict(), dict(anchor_mode=1)):
+    P.ttf_compress_batch([to_device(corr_clip(7, 6, 9, 200, seed=11, dtype="bf16"))] * 3, 1, 0.6, stream=st, **kw)
+    P.ttf_debug_set_check_slack(5)
+    P.ttf_compress_batch([Xd] * 5, 1, 0.7, stream=st, **kw)
+    assert P.ttf_last_device_status(st) == P.TTF_ERR_BOUNDS
+    P.ttf_debug_set_check_slack(0)
+    outs = P.ttf_compress_batch([Xd] * 5, 1, 0.7, stream=st, **kw)
+    assert P.ttf_last_device_status(st) == 0
+    one = P.ttf_compress(Xd, 1, 0.7, **kw)
+    assert all(int(c) == int(one[1]) for c in outs[1])
 print("checked build ok")
 """
 
