@@ -43,7 +43,7 @@
 #include "ttf_cluster.cuh"
 #include "ttf_tensormap.cuh"
 
-#include <map>
+#include <atomic>
 #include <mutex>
 
 namespace ttf {
@@ -567,16 +567,15 @@ static int split_of(const Problem& p, long long tiles, int most) {
 // cluster lie in one GPC: 148 SMs hold 148 clusters of two, 71 of four, 33 of eight.  (The runtime is asked about a kernel of
 // the same shape that uses no tensor memory: for one that does it counts one CTA per SM, although two run.)
 __global__ void __launch_bounds__(kTcThreads) k_cluster_places(int* p) { if (p) *p = 0; }
-static long long cluster_places(int n) {
-    constexpr int kSmem = 100 * 1024;
-    static std::mutex mu;
-    static std::map<std::pair<int, int>, long long> known;
+static long long cluster_places(int n) {                          // n = 1, 2, 4 or 8
+    constexpr int kSmem = 100 * 1024, kDevices = 64;
+    static std::atomic<int> known[kDevices][4];                   // (asked on every launch: no lock)
+    const int level = n == 8 ? 3 : n / 2;
     int dev = 0;
     if (n == 1 || cudaGetDevice(&dev) != cudaSuccess) return 2LL * sm_count() / n;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = known.find({dev, n});
-    if (it != known.end()) return it->second;
-    int found = 0;
+    const bool keep = dev >= 0 && dev < kDevices;
+    int found = keep ? known[dev][level].load(std::memory_order_relaxed) : 0;
+    if (found > 0) return found;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = kSmem;
     cudaLaunchAttribute attr;
@@ -588,7 +587,8 @@ static long long cluster_places(int n) {
         cudaGetLastError();
         found = 2 * sm_count() / n;
     }
-    return known[{dev, n}] = found;
+    if (keep) known[dev][level].store(found, std::memory_order_relaxed);
+    return found;
 }
 
 // How a launch splits its work.  The tile and its chunks depend on the clip's shape alone, the CTAs (= cluster size) of a tile on
