@@ -115,35 +115,20 @@ k_restore_copy(const unsigned char* __restrict__ comp, size_t row_bytes, long lo
     restore_rows<U>(comp, row_bytes, gw, rows, nw, out, threadIdx.x & 31, [&](long long f) { return __ldcg(row_index + f); });
 }
 
-// Both steps in one launch, for clips of up to kRestoreWhole tokens: a CTA owns a contiguous range of tokens, counts the
-// preserved tokens before it (16 flags per load: one round trip), ranks its own 256 at a time, and copies their rows from
-// the indices in shared memory.  What bounds it is the traffic of long rows, and for short ones a chain of round trips.  Us
-// per call / in a replayed graph, with a launch for the indices -> in one: 4 x 16 x 16 x 64 bf16 channels 11.7 / 3.9 -> 8.9 /
-// 2.4, 32 x 16 x 16 x 64 11.7 / 4.9 -> 8.7 / 6.3, 32 x 16 x 16 x 4096 18.5 / 16.9 -> 15.3 / 15.2 (its 90 MB at the copy rate:
-// 13.8), 64 x 32 x 32 x 64 15.4 / 13.0 -> 14.1 / 14.0, x 1024 53.7 / 48.7 -> 45.5 / 45.4: the graph's time alone would draw the
-// line for short rows at 4096 tokens, a call's at 65536.  In longer clips the flags that every CTA reads outweigh the launch.
-constexpr int kRestoreWhole = 1 << 16;
-
-template <typename U>
-__global__ void __launch_bounds__(kXThreads)
-k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int* anchor, const unsigned char* keep,
-          const int* dst, int per, unsigned char* out, int* row_index)
-{
-    __shared__ int s_warp[kXThreads / 32];
-    __shared__ int s_row[kXThreads];
+// The compressed rows of tokens [f0, f1), which belong to this CTA: it counts the preserved tokens before them (16 flags per load:
+// one round trip) and ranks its own, 256 at a time; round(b0, end) finds the rows of tokens [b0, end) in s_row.  The anchor
+// frame's tokens are [a0, a1), none of the clip's for an anchor outside it.
+template <typename Round>
+__device__ __forceinline__ void restore_rounds(int FN, int N, const int* anchor, const unsigned char* keep, const int* dst, int f0, int f1,
+                                               int* row_index, int* s_warp, int* s_row, Round&& round) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int f0 = blockIdx.x * per, f1 = min(FN, f0 + per);
-    pdl_launch_dependents();
-    pdl_wait();                                  // the caller's kernels before this one
     // (what the first round needs of this CTA's tokens is asked for together with the anchor and the flags before them)
     unsigned char next_keep = f0 + tid < f1 ? keep[f0 + tid] : (unsigned char)0;
     int next_dst = f0 + tid < f1 ? dst[f0 + tid] : 0;
-    // the anchor frame's tokens: [a0, a1), none of the clip's for an anchor outside it
     const int a = __ldcg(anchor);
     const bool inside = (unsigned)a < (unsigned)(FN / N);
     const int a0 = inside ? a * N : FN, a1 = inside ? a0 + N : FN;
-    // preserved source tokens before f0 (the anchor frame does not count)
-    int c = count_flags(keep, 0, (size_t)min(f0, a0), tid);
+    int c = count_flags(keep, 0, (size_t)min(f0, a0), tid);      // (the anchor frame does not count)
     if (f0 > a1) c += count_flags(keep, (size_t)a1, (size_t)f0, tid);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
@@ -173,9 +158,32 @@ k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int*
         }
         run += total;
         __syncthreads();
-        restore_rows<U>(comp, row_bytes, b0 + w, min(f1, b0 + kXThreads), kXThreads / 32, out, lane,
-                        [&](long long g) { return s_row[(int)g - b0]; });
+        round(b0, min(f1, b0 + kXThreads));
     }
+}
+
+// Both steps in one launch, for clips of up to kRestoreWhole tokens: a CTA owns a contiguous range of tokens and copies their rows
+// from the indices in shared memory.  What bounds it is the traffic of long rows, and for short ones a chain of round trips.  Us
+// per call / in a replayed graph, with a launch for the indices -> in one: 4 x 16 x 16 x 64 bf16 channels 11.7 / 3.9 -> 8.9 /
+// 2.4, 32 x 16 x 16 x 64 11.7 / 4.9 -> 8.7 / 6.3, 32 x 16 x 16 x 4096 18.5 / 16.9 -> 15.3 / 15.2 (its 90 MB at the copy rate:
+// 13.8), 64 x 32 x 32 x 64 15.4 / 13.0 -> 14.1 / 14.0, x 1024 53.7 / 48.7 -> 45.5 / 45.4: the graph's time alone would draw the
+// line for short rows at 4096 tokens, a call's at 65536.  In longer clips the flags that every CTA reads outweigh the launch.
+constexpr int kRestoreWhole = 1 << 16;
+
+template <typename U>
+__global__ void __launch_bounds__(kXThreads)
+k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int* anchor, const unsigned char* keep,
+          const int* dst, int per, unsigned char* out, int* row_index)
+{
+    __shared__ int s_warp[kXThreads / 32];
+    __shared__ int s_row[kXThreads];
+    const int f0 = blockIdx.x * per, f1 = min(FN, f0 + per);
+    pdl_launch_dependents();
+    pdl_wait();                                  // the caller's kernels before this one
+    restore_rounds(FN, N, anchor, keep, dst, f0, f1, row_index, s_warp, s_row, [&](int b0, int end) {
+        restore_rows<U>(comp, row_bytes, b0 + (threadIdx.x >> 5), end, kXThreads / 32, out, threadIdx.x & 31,
+                        [&](long long g) { return s_row[(int)g - b0]; });
+    });
 }
 
 // The same with bulk copies, for rows of whole 16-byte pieces: ONE CTA per SM, whose warps move batches of consecutive output
@@ -205,45 +213,10 @@ k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const
     }
     __syncwarp();
     pdl_wait();                                  // the caller's kernels before this one
-    unsigned char next_keep = f0 + tid < f1 ? keep[f0 + tid] : (unsigned char)0;
-    int next_dst = f0 + tid < f1 ? dst[f0 + tid] : 0;
-    const int a = __ldcg(anchor);
-    const bool inside = (unsigned)a < (unsigned)(FN / N);
-    const int a0 = inside ? a * N : FN, a1 = inside ? a0 + N : FN;
-    int c = count_flags(keep, 0, (size_t)min(f0, a0), tid);
-    if (f0 > a1) c += count_flags(keep, (size_t)a1, (size_t)f0, tid);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0) s_warp[w] = c;
-    __syncthreads();
-    int run = N;
-#pragma unroll
-    for (int ww = 0; ww < kXThreads / 32; ++ww) run += s_warp[ww];
-
     unsigned char* const buf = stage + (size_t)w * kRestoreSlots * kRestoreSlot;
     int issued = 0, finished = 0;                // batches of this warp; batch n goes through slot n % kRestoreSlots
     bool gave_up = false;
-    for (int b0 = f0; b0 < f1; b0 += kXThreads) {
-        const int f = b0 + tid, end = min(f1, b0 + kXThreads);
-        const bool in = f < f1, own = f >= a0 && f < a1;
-        const bool kp = in && !own && next_keep;
-        const int to = next_dst;
-        next_keep = f + kXThreads < f1 ? keep[f + kXThreads] : (unsigned char)0;
-        next_dst = f + kXThreads < f1 ? dst[f + kXThreads] : 0;
-        const unsigned m = __ballot_sync(0xffffffffu, kp);
-        __syncthreads();                         // (the indices of the round before this one, and s_warp, are done with)
-        if (lane == 0) s_warp[w] = __popc(m);
-        __syncthreads();
-        int off = 0, total = 0;
-#pragma unroll
-        for (int ww = 0; ww < kXThreads / 32; ++ww) { off += ww < w ? s_warp[ww] : 0; total += s_warp[ww]; }
-        if (in) {
-            const int r = own ? f - a0 : (kp ? run + off + __popc(m & ((1u << lane) - 1)) : to);
-            s_row[tid] = r;
-            row_index[f] = r;
-        }
-        run += total;
-        __syncthreads();
+    restore_rounds(FN, N, anchor, keep, dst, f0, f1, row_index, s_warp, s_row, [&](int b0, int end) {
         const int R = max(1, min(batch, (end - b0 + kXThreads / 32 - 1) / (kXThreads / 32)));
         const int units = (end - b0) * pieces, step = kXThreads / 32 * R;
         auto piece_bytes = [&](int pc) { return (uint32_t)min(row_bytes - (size_t)pc * kRestoreSlot, (size_t)kRestoreSlot); };
@@ -289,7 +262,7 @@ k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const
                 for (int e = lane; e < (int)(piece_bytes(pc) / 16); e += 32) to4[e] = src[e];
             }
         }
-    }
+    });
     if (lane == 0) {
         // copies still on their way into this CTA's shared memory (bounded again)
         for (; finished < issued; ++finished) mbar_wait(&bar[w][finished % kRestoreSlots], (finished / kRestoreSlots) & 1, wait_limit);
