@@ -186,21 +186,21 @@ k_restore(const unsigned char* comp, size_t row_bytes, int FN, int N, const int*
     });
 }
 
-// The same with bulk copies, for rows of whole 16-byte pieces: ONE CTA per SM, whose warps move batches of consecutive output
-// rows (or pieces of long ones) through three slots of 8 KB each, two loads ahead; a batch leaves as one store.  The flags before
-// a CTA's tokens are read by 148 CTAs instead of up to 1184 (they queue on the same lines), short rows move 32 to a batch, and a
+// The same with bulk copies, for rows of whole 16-byte pieces: one CTA per SM (see restore_plan), whose warps move batches of
+// consecutive output rows (or pieces of long ones) through three slots, two loads ahead; a batch leaves as one store.  The flags
+// before a CTA's tokens are read by 148 CTAs instead of up to 1184 (they queue on the same lines), short rows move 32 to a batch, and a
 // row that is no multiple of eight loads per lane has no serial rest.  Us per call in a replayed graph, plain loads / bulk:
 // 32 x 16 x 16 x 512 7.2 / 4.9, 64 x 32 x 32 x 64 14.4 / 8.3, 14 x 25 x 14 x 2800 13.9 / 9.8, 48 x 16 x 16 x 1536 21.6 / 12.0,
 // 64 x 32 x 32 x 1024 47.8 / 36.3; from two launches 128 x 32 x 32 x 64 27.8 / 15.9, x 512 53.3 / 38.7, 256 x 32 x 32 x 64 50.1 /
 // 30.0.  (Two slots of 8 KB 10.2 and 12.4 where three take 9.8 and 12.0; four of 4 KB 10.9.)
 // A wait that runs out has nobody to report to here: the warp copies what is left by plain loads and stores.
 constexpr int kRestoreBulk = 1 << 18;
-constexpr int kRestoreSlots = 3, kRestoreSlot = 8192, kRestoreAhead = 2;
+constexpr int kRestoreSlots = 3, kRestoreAhead = 2;
 __global__ void __launch_bounds__(kXThreads)
 k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const int* anchor, const unsigned char* keep,
-               const int* dst, int per, unsigned char* out, int* row_index, int pieces, int batch, int wait_limit, int tx_extra)
+               const int* dst, int per, unsigned char* out, int* row_index, int pieces, int batch, int slots, int slot, int wait_limit, int tx_extra)
 {
-    extern __shared__ __align__(128) unsigned char stage[];      // [warps][kRestoreSlots][kRestoreSlot]
+    extern __shared__ __align__(128) unsigned char stage[];      // [warps][slots][slot]
     __shared__ uint64_t bar[kXThreads / 32][kRestoreSlots];
     __shared__ int s_warp[kXThreads / 32];
     __shared__ int s_row[kXThreads];
@@ -213,13 +213,13 @@ k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const
     }
     __syncwarp();
     pdl_wait();                                  // the caller's kernels before this one
-    unsigned char* const buf = stage + (size_t)w * kRestoreSlots * kRestoreSlot;
+    unsigned char* const buf = stage + (size_t)w * slots * slot;
     int issued = 0, finished = 0;                // batches of this warp; batch n goes through slot n % kRestoreSlots
     bool gave_up = false;
     restore_rounds(FN, N, anchor, keep, dst, f0, f1, row_index, s_warp, s_row, [&](int b0, int end) {
         const int R = max(1, min(batch, (end - b0 + kXThreads / 32 - 1) / (kXThreads / 32)));
         const int units = (end - b0) * pieces, step = kXThreads / 32 * R;
-        auto piece_bytes = [&](int pc) { return (uint32_t)min(row_bytes - (size_t)pc * kRestoreSlot, (size_t)kRestoreSlot); };
+        auto piece_bytes = [&](int pc) { return (uint32_t)min(row_bytes - (size_t)pc * slot, (size_t)slot); };
         auto issue = [&](int u) {
             const int n = min(R, units - u), h = issued % kRestoreSlots;
             const int r0 = pieces == 1 ? u : u / pieces, pc = pieces == 1 ? 0 : u - r0 * pieces;
@@ -229,8 +229,8 @@ k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const
             }
             __syncwarp();
             if (lane < n)
-                bulk_load(buf + h * kRestoreSlot + lane * (uint32_t)row_bytes,
-                          comp + (size_t)s_row[r0 + lane] * row_bytes + (size_t)pc * kRestoreSlot, piece_bytes(pc), &bar[w][h]);
+                bulk_load(buf + h * slot + lane * (uint32_t)row_bytes,
+                          comp + (size_t)s_row[r0 + lane] * row_bytes + (size_t)pc * slot, piece_bytes(pc), &bar[w][h]);
             ++issued;
         };
         int ahead = w * R;
@@ -238,7 +238,7 @@ k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const
         for (int u = w * R; u < units; u += step) {
             const int n = min(R, units - u);
             const int r0 = pieces == 1 ? u : u / pieces, pc = pieces == 1 ? 0 : u - r0 * pieces;
-            unsigned char* d = out + (size_t)(b0 + r0) * row_bytes + (size_t)pc * kRestoreSlot;
+            unsigned char* d = out + (size_t)(b0 + r0) * row_bytes + (size_t)pc * slot;
             if (!gave_up) {
                 if (ahead < units) { issue(ahead); ahead += step; }
                 const int h = finished % kRestoreSlots;
@@ -247,7 +247,7 @@ k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const
                 ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
                 if (ok) {
                     if (lane == 0) {
-                        bulk_store(d, buf + h * kRestoreSlot, (uint32_t)n * piece_bytes(pc));
+                        bulk_store(d, buf + h * slot, (uint32_t)n * piece_bytes(pc));
                         bulk_commit();
                     }
                     ++finished;
@@ -257,7 +257,7 @@ k_restore_bulk(const unsigned char* comp, size_t row_bytes, int FN, int N, const
             }
             // a copy that does not arrive: this batch and the rest by plain loads and stores
             for (int q = 0; q < n; ++q) {
-                const uint4* src = reinterpret_cast<const uint4*>(comp + (size_t)s_row[r0 + q] * row_bytes + (size_t)pc * kRestoreSlot);
+                const uint4* src = reinterpret_cast<const uint4*>(comp + (size_t)s_row[r0 + q] * row_bytes + (size_t)pc * slot);
                 uint4* to4 = reinterpret_cast<uint4*>(d + (size_t)q * row_bytes);
                 for (int e = lane; e < (int)(piece_bytes(pc) / 16); e += 32) to4[e] = src[e];
             }
@@ -288,14 +288,49 @@ static cudaError_t launch_restore_t(const unsigned char* c, size_t row_bytes, in
     return launch_pdl(k_restore_copy<U>, dim3((unsigned)blocks), dim3(kXThreads), st, c, row_bytes, rows, row_index, o);
 }
 
-// Plain loads stay where they are the faster ones: rows of whole 4 KB, which keep eight loads per lane in flight throughout, once
-// the output is more than half of L2 (bulk / plain: 50 MB 15.1 / 15.3 us, 67 MB in rows of 4 KB 19.0 / 18.3, of 8 KB 19.0 / 18.0,
-// 151 MB 41.9 / 37.6), and the smallest clips, whose rows gain nothing from the way through shared memory (131 KB 3.65 / 3.15,
-// 524 KB 3.65 / 3.4, in 4096 rows 3.66 / 4.15, 790 KB 3.65 / 3.65).
-static bool restore_in_bulk(long long FN, size_t row_bytes) {
+// How a call copies, by size.  Calls on other streams of the caller's want room on the SMs too, and with 192 KB of slots in every
+// launch two restores cannot share an SM.  Us per call in a replayed graph, on one / two / four streams:
+//                           plain loads             192 KB of slots         as here
+//   5 x 16 x 16 x  512       2.96   1.67   1.19      3.05   2.40   2.37      (plain)
+//   9 x 16 x 16 x 1024       5.91   3.41   2.63      4.04   3.04   3.04      4.39   2.70   1.85
+//  12 x 16 x 16 x 2048       5.81   3.80   3.16      5.72   4.41   4.43      (plain)
+//  20 x 16 x 16 x 2048       8.36   5.58   4.92      7.24   5.84   5.78      7.36   5.49   5.46
+//  32 x 16 x 16 x 2048      10.74   7.48   7.52      9.93   8.24   7.99     10.13   7.74   7.50
+//  16 x 16 x 16 x 1024       6.76   4.22   4.00      4.88   3.87   3.86      (192 KB)
+//  64 x 16 x 16 x 1024      17.5   12.5   12.5      10.2    8.6    8.4       (192 KB)
+//  - Rows of whole 4 KB keep eight plain loads per lane in flight throughout and gain from bulk copies only between 20 and 52 MB of
+//    output (bulk / plain alone: 50 MB 15.1 / 15.3, 67 MB in rows of 4 KB 19.0 / 18.3, of 8 KB 19.0 / 18.0, 151 MB 41.9 / 37.6);
+//    there two CTAs of 96 KB per SM do as well as one of 192 KB.
+//  - The smallest clips gain nothing from the way through shared memory (131 KB 3.65 / 3.15, 524 KB 3.65 / 3.4, in 4096 rows 3.66 /
+//    4.15).
+//  - Clips of up to 3072 tokens take no more slots, and no larger ones, than their warps fill; from about there on plain loads were
+//    never the faster ones.
+struct RestorePlan { bool bulk; int ctas, per, pieces, batch, slots, slot; size_t smem; };
+static RestorePlan restore_plan(long long FN, size_t row_bytes) {
+    constexpr int warps = kXThreads / 32;
     const double mb = (double)FN * row_bytes * 1e-6;
-    if (FN > kRestoreBulk || (FN <= 2048 && mb <= 0.75)) return false;
-    return row_bytes % 4096 != 0 || mb <= 52.0;
+    const bool whole_4k = row_bytes % 4096 == 0;
+    RestorePlan q = {};
+    q.bulk = FN <= kRestoreBulk && (whole_4k ? mb > 20.0 && mb <= 52.0 : FN > 2048 || mb > 1.5);
+    if (!q.bulk) return q;
+    const size_t most = whole_4k ? 4096 : 8192;              // bytes of a slot
+    const int ctas = sm_count() * (whole_4k ? 2 : 1);
+    q.per = (int)std::max<long long>(warps, (FN + ctas - 1) / ctas);
+    q.ctas = (int)((FN + q.per - 1) / q.per);
+    q.pieces = (int)((row_bytes + most - 1) / most);
+    q.batch = q.pieces > 1 ? 1 : (int)std::min<size_t>(32, most / row_bytes);
+    q.slots = kRestoreSlots;
+    q.slot = (int)most;
+    if (FN <= 3072 && q.per <= kXThreads) {      // (one round)
+        const int rows = (q.per + warps - 1) / warps;
+        if (q.pieces == 1) {
+            q.batch = std::min(q.batch, rows);
+            q.slot = (int)(q.batch * row_bytes);
+        }
+        q.slots = (int)std::min<long long>(kRestoreSlots, ((long long)rows * q.pieces + q.batch - 1) / q.batch);
+    }
+    q.smem = (size_t)warps * q.slots * q.slot;
+    return q;
 }
 
 cudaError_t launch_restore(const void* comp, size_t row_bytes, int F, int N, const int* anchor,
@@ -304,16 +339,12 @@ cudaError_t launch_restore(const void* comp, size_t row_bytes, int F, int N, con
     const unsigned char* c = reinterpret_cast<const unsigned char*>(comp);
     unsigned char* o = reinterpret_cast<unsigned char*>(out_full);
     const uintptr_t al = reinterpret_cast<uintptr_t>(comp) | reinterpret_cast<uintptr_t>(out_full) | row_bytes;
-    if (al % 16 == 0 && restore_in_bulk((long long)F * N, row_bytes)) {
-        const int FN = F * N, most = sm_count();
-        const int per = std::max(8, (FN + most - 1) / most);
-        const int pieces = (int)((row_bytes + kRestoreSlot - 1) / kRestoreSlot);
-        const int batch = pieces > 1 ? 1 : (int)std::min((size_t)32, kRestoreSlot / row_bytes);
-        constexpr size_t smem = (size_t)(kXThreads / 32) * kRestoreSlots * kRestoreSlot;
-        cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_restore_bulk), smem);
+    const RestorePlan q = restore_plan((long long)F * N, row_bytes);
+    if (al % 16 == 0 && q.bulk) {
+        cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_restore_bulk), q.smem);
         if (e != cudaSuccess) return e;
-        return launch_ex(true, smem, k_restore_bulk, dim3((FN + per - 1) / per), dim3(kXThreads), st, c, row_bytes, FN, N, anchor, keep,
-                         dst, per, o, row_index, pieces, batch, wait_poll_limit(), wait_tx_extra());
+        return launch_ex(true, q.smem, k_restore_bulk, dim3(q.ctas), dim3(kXThreads), st, c, row_bytes, F * N, N, anchor, keep,
+                         dst, q.per, o, row_index, q.pieces, q.batch, q.slots, q.slot, wait_poll_limit(), wait_tx_extra());
     }
     if (al % 16 == 0) return launch_restore_t<uint4>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);
     if (al % 4 == 0) return launch_restore_t<uint32_t>(c, row_bytes, F, N, anchor, keep, dst, o, row_index, st);

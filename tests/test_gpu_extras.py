@@ -176,7 +176,8 @@ def test_an_anchor_outside_the_clip_excludes_no_frame(shape, anchor):
 
 @pytest.mark.parametrize("F,N,row_bytes", [(9, 256, 16), (9, 256, 48), (64, 37, 4096), (64, 33, 8192), (33, 71, 8208), (5, 500, 24592), (300, 256, 128),
                                            (130, 1030, 272), (2, 1024, 1008), (260, 1024, 16), (6, 2187, 4096), (9, 1000, 8192),
-                                           (1, 3000, 320), (2049, 1, 512)])
+                                           (1, 3000, 320), (2049, 1, 512), (5, 1000, 4096), (12, 1024, 4096), (3, 1000, 8192),
+                                           (2, 1400, 16384), (47, 65, 1040), (3073, 1, 512), (3, 900, 576)])
 @pytest.mark.parametrize("wait", [None, (32, 16)])
 def test_restore_in_bulk_at_the_edges(F, N, row_bytes, wait):
     """rows of one and several pieces, batches, rounds of 256 tokens that end inside a batch, the sizes next to the lines of the
