@@ -43,3 +43,17 @@ def test_near_ties_fall_the_same_way_alone_and_in_batches(shape, dtype):
             assert anchors_of_batch(Xs[:16]) == alone[:16], schedule
     finally:
         P.ttf_set_schedule(0)
+
+
+@pytest.mark.parametrize("C,slices", [(256, (0, 1)), (384, (0, 2)), (512, (0, 1)), (512, (1, 2)), (640, (0, 4))])
+def test_small_shares_of_one_slice_are_not_lost_in_a_large_one_of_another(C, slices):
+    """One token per frame.  Frame 1 is frame 0 (its square is beyond 2^23, where a step of fp32 in the product with the sum of all
+    frames is 2) and four small channels in another slice of 128, whose four shares of 0.9 each would not count one by one.  They make
+    its cosine the larger one by 2e-7; everything else is exact."""
+    large, small = slices
+    X = torch.zeros((3, 1, 1, C), dtype=torch.float32)
+    X[0, 0, 0, large * 128] = X[1, 0, 0, large * 128] = 2900.0
+    few = slice(small * 128, small * 128 + 4)
+    X[1, 0, 0, few] = 0.9 / 64
+    X[2, 0, 0, few] = 64.0
+    assert int(P.ttf_query(X.cuda(), 0, 0.6, want=("anchor",))["anchor"]) == 1
