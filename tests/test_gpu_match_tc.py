@@ -53,14 +53,20 @@ def test_tiles_of_fewer_frames(shape, r):
 
 @pytest.mark.parametrize("shape,r,clips", [((6, 8, 8, 1024), 1, 24), ((40, 8, 8, 1024), 1, 24), ((16, 16, 16, 1024), 2, 24)])
 def test_bits_of_tiles_of_fewer_frames(shape, r, clips):
-    """a tile as a cluster, and (the second and third) as one CTA that sums all chunks itself"""
+    """a tile as a cluster, and as fewer CTAs (the second two, the third one) that sum several chunks each"""
     test_bits_do_not_depend_on_the_split(shape, r, clips)
 
 
-@pytest.mark.parametrize("tiles", [33, 34, 71, 72, 148, 149])
-def test_as_many_clusters_as_run_at_once_and_one_more(tiles):
-    X = corr_clip(3, tiles * 4, 4, 256 if tiles < 100 else 128, seed=tiles, dtype="bf16")
-    check_clip(X, 1, 0.6)
+@pytest.mark.parametrize("C,ctas", [(1024, 8), (512, 4)])
+def test_as_many_clusters_as_run_at_once_and_one_more(C, ctas):
+    """tiles of one grid row of a clip of 32 frames, as many as run at the same time as clusters of eight and of four CTAs, and one
+    more (33 and 34, 71 and 72 of them on 148 SMs): then a tile has half as many, which sum two parts of its channels each"""
+    fits = max(n for n in range(1, 2 * 148 // ctas + 1) if P.ttf_debug_match_split(32, 1, 4 * n, C, 1) == (1, ctas, ctas))
+    assert P.ttf_debug_match_split(32, 1, 4 * (fits + 1), C, 1) == (1, ctas, ctas // 2)      # (not fewer parts: fewer CTAs)
+    for tiles in (fits, fits + 1):
+        shape = (32, 1, 4 * tiles, C)
+        check_clip(corr_clip(*shape, seed=tiles, dtype="bf16"), 1, 0.6)
+        test_bits_do_not_depend_on_the_split(shape, 1, 24)
 
 
 @pytest.mark.parametrize("shape", [(8, 8, 8, 4096), (4, 12, 12, 4096), (8, 10, 10, 4096)])

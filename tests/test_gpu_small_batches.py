@@ -2,6 +2,7 @@
 Every clip comes out as from the call for it alone, also where the stream's blocks hold another shape's data, where two
 streams work at the same time, where a capture finds no scratch on its stream, and for a stream handle that means another
 stream in every thread."""
+import ctypes
 import threading
 
 import pytest
@@ -41,13 +42,16 @@ def test_every_clip_as_alone_on_dirty_blocks(shape, dtype, n):
 
 
 def test_two_streams_and_two_threads():
-    """single calls and batches on the same stream from two threads, beside a second stream"""
+    """batches on two streams from two threads, each of which also makes single calls on a stream of the two"""
     sets = [clips_of((6, 5, 7, 128), 5, seed=930), clips_of((9, 6, 6, 72), 8, seed=950)]
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
-    results = {}
+    results, alone = {}, {0: [], 1: []}
 
     def work(i):
-        outs = [P.ttf_compress_batch(sets[i], 1, 0.6, stream=st) for _ in range(20) for st in streams]
+        outs = []
+        for n in range(20):
+            outs += [P.ttf_compress_batch(sets[i], 1, 0.6, stream=st) for st in streams]
+            alone[i].append(P.ttf_compress(sets[i][n % 5], 1, 0.6, stream=streams[i]))
         results[i] = outs
     threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
     [t.start() for t in threads]
@@ -56,6 +60,35 @@ def test_two_streams_and_two_threads():
     for i in range(2):
         for outs in (results[i][0], results[i][-2], results[i][-1]):
             assert_same_as_single(sets[i], 1, 0.6, outs)
+        for n, (tok, cnt, pos) in enumerate(alone[i]):
+            ref = results[i][-1]
+            L = int(ref[1][n % 5])
+            assert int(cnt) == L and torch.equal(tok[:L], ref[0][n % 5][:L]) and torch.equal(pos[:L], ref[2][n % 5][:L])
+
+
+def test_more_streams_than_hold_scratch():
+    """64 streams hold scratch of their own; batches on further ones take the lanes, and after ttf_release theirs again"""
+    Xs = clips_of((5, 4, 6, 64), 3, seed=910)
+    streams = []
+    try:
+        for _ in range(66):
+            h = ctypes.c_void_p()
+            assert int(torch.cuda.cudart().cudaStreamCreate(ctypes.addressof(h))) == 0
+            streams.append(h.value)
+        P.ttf_release()
+        for _ in range(2):
+            outs = [P.ttf_compress_batch(Xs, 1, 0.6, stream=st) for st in streams]
+            torch.cuda.synchronize()
+            for o in outs[:2] + outs[-4:]:
+                assert_same_as_single(Xs, 1, 0.6, o)
+            assert P.ttf_last_device_status(streams[-1]) == P.TTF_OK
+        P.ttf_release()
+        assert_same_as_single(Xs, 1, 0.6, P.ttf_compress_batch(Xs, 1, 0.6, stream=streams[-1]))
+    finally:
+        torch.cuda.synchronize()
+        P.ttf_release()
+        for st in streams:
+            torch.cuda.cudart().cudaStreamDestroy(st)
 
 
 def test_capture_on_a_stream_without_scratch_and_with_it():
