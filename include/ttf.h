@@ -153,8 +153,10 @@ int ttf_compress(const void* features, int F, int H, int W, int C, int r, float 
  * asynchronous, ordered on `stream` like any other, and can be captured in a CUDA graph.  The kernels of one group
  * leave part of the GPU idle while they ramp up and drain; the other lane's fill those gaps.  Small batches (up to
  * eight clips of 64 MB together, 160 MB with a fixed anchor; outside a capture up to sixteen of 16 or 32 MB) run on `stream`
- * itself instead, in groups of up to eight, on scratch that belongs to the stream; where that cannot be had (a capture
- * on a stream that has none) they take the lanes
+ * itself instead, in groups of up to eight, on scratch that belongs to the stream.  The first 64 streams that are used so
+ * keep theirs until ttf_release, besides the scratch of the lanes, which such a batch claims too (a later capture may need it):
+ * up to twice the memory.  Where a stream has none and cannot get any (in a capture, beyond 64 streams, without memory) they take
+ * the lanes
  * (ttf_set_schedule asks for a number of single clips in flight instead; a lane then chains its clips on two scratch
  * blocks used in turn: the sweep of a clip runs beside the gather of the clip before it).  The streams, their events and
  * the scratch are created by the first call on a device: make that call outside any stream capture.  The scratch (the
@@ -177,7 +179,7 @@ int ttf_set_match_kernel(int which);
 
 /*
  * Schedule of ttf_compress_batch (the paper has no counterpart).  clips_in_flight: 0 = automatic (two groups of
- * clips in flight, one launch per kernel and group), 1 to 8 = so many lanes of single clips, or TTF_SCHEDULE_PIPELINED.  Eq. (auto_anchor) needs all of X before any token can be matched,
+ * clips in flight, one launch per kernel and group; small batches on the caller's stream, see ttf_compress_batch), 1 to 8 = so many lanes of single clips, or TTF_SCHEDULE_PIPELINED.  Eq. (auto_anchor) needs all of X before any token can be matched,
  * so X is read twice; with few clips in flight the second read finds the clip in L2 but the kernels of one clip leave
  * much of the GPU idle while they ramp up and drain, with many the gaps are filled but the clips displace one another
  * in L2.  Results do not depend on it.  Process-wide; takes effect with the next call.

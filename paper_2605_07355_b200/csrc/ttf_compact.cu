@@ -177,6 +177,26 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     trace_mark(hdr, 3, true);
 }
 
+// 32 keep flags (0 or 1 each) -> one bit each.  (The flags are masked first: a word that reaches past the end of the
+// array holds other bytes, whose higher bits would spill into its neighbours' in the product.)
+__device__ __forceinline__ unsigned pack_flags(const uint4& lo, const uint4& hi) {
+    const unsigned w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    unsigned bits = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) bits |= ((((w[e] & 0x01010101u) * 0x01020408u) >> 24) & 0xfu) << (4 * e);   // byte i -> bit i
+    return bits;
+}
+// position of the n-th (0-based) set bit; n < popcount(bits)
+__device__ __forceinline__ int select_bit(unsigned bits, int n) {
+    int at = 0;
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) {
+        const int c = __popc((bits >> at) & ((1u << h) - 1u));
+        if (n >= c) { n -= c; at += h; }
+    }
+    return at;
+}
+
 // The same with the rows of a CTA found together.  A CTA owns a contiguous range of output rows.  It packs the keep
 // flags of a window of tokens into bit words in shared memory together with the exclusive prefix of their population
 // counts, after which the source row of any output row of the window is found by a binary search and a select in shared
@@ -201,26 +221,7 @@ k_compact_bulk(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
 // 64 x 24 x 24 x 512 23.8 / 26.1).
 // Where other clips' kernels run beside it the CTAs are three per SM, and long rows go one at a time: the waits of one CTA
 // are filled by others (16 clips of 32 x 16 x 16 x 4096 448 us, 457 with one CTA per SM; 8 of 24 x 20 x 20 x 1024 84.6 / 87.4).
-// 32 keep flags (0 or 1 each) -> one bit each.  (The flags are masked first: a word that reaches past the end of the
-// array holds other bytes, whose higher bits would spill into its neighbours' in the product.)
-__device__ __forceinline__ unsigned pack_flags(const uint4& lo, const uint4& hi) {
-    const unsigned w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-    unsigned bits = 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) bits |= ((((w[e] & 0x01010101u) * 0x01020408u) >> 24) & 0xfu) << (4 * e);   // byte i -> bit i
-    return bits;
-}
-// position of the n-th (0-based) set bit; n < popcount(bits)
-__device__ __forceinline__ int select_bit(unsigned bits, int n) {
-    int at = 0;
-#pragma unroll
-    for (int h = 16; h > 0; h >>= 1) {
-        const int c = __popc((bits >> at) & ((1u << h) - 1u));
-        if (n >= c) { n -= c; at += h; }
-    }
-    return at;
-}
-
+//
 // WHOLE: the clip is one window.  Else the windows are `window_words` * 32 tokens.  NW: warps; `slot`: bytes of a staging slot, of
 // which a warp has two; `pieces` of a row, or `batch` rows at most to a slot.
 template <bool WHOLE, int NW>
@@ -316,7 +317,8 @@ k_compact_rows(const __grid_constant__ ClipPtrs xs, size_t row_bytes, int F, int
     else P = in_smem ? frame_prefix_cta<NW>(cnt, F, a, acnt, s_frames, s_warp) : __ldcg(gprefix + F);
     const int Lp = NA + P;                       // L' = N + P (Eq. Lpre)
     if (blockIdx.x == 0 && tid == 0) *reinterpret_cast<volatile int*>(out_count) = Lp;
-    // rows per CTA: per_magic is 2^32 / gridDim.x rounded up, so that per * gridDim.x > Lp without a division
+    // rows per CTA: per_magic is 2^32 / gridDim.x rounded up, so that per * gridDim.x > Lp without a division (for one CTA
+    // 2^32 - 1: per = Lp)
     const int per = (int)__umulhi((unsigned)Lp, per_magic) + 1;
     const int j0 = (int)min((long long)Lp, (long long)blockIdx.x * per), j1 = min(Lp, j0 + per);
     // rows per batch: what fits a slot, but no more than leaves every warp of the CTA a batch

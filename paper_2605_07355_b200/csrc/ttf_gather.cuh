@@ -10,7 +10,7 @@ constexpr int kScanChunks = 4;       // frame counts per lane fetched at once by
 
 // Exclusive prefix of the survivor counts of all frames in shared memory, for clips of up to kWarpPrefixMaxF frames
 // (`pref`: [kWarpPrefixMaxF + 4]; pref[F] is the total, which is returned).  The anchor frame counts `acnt` tokens.  By all
-// threads of a CTA of 256.  (Not for the gather with one row per warp at a time: its warps do better without a barrier
+// threads of a CTA of NW warps.  (Not for the gather with one row per warp at a time: its warps do better without a barrier
 // before their first copy, 37.8 against 38.7 us per pass on 32 x 16 x 16 x 4096, 247 against 255 on 64 x 32 x 32 x 4096.)
 template <int NW>
 __device__ __forceinline__ int frame_prefix_cta(const int* cnt, int F, int a, int acnt, int* pref, int* s_warp) {

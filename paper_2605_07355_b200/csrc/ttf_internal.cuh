@@ -127,7 +127,12 @@ inline bool needs_sweep_norms(const Problem& p) {
 // Whether the gather runs with one CTA per SM.  A call that has the GPU to itself does.  Not for groups of clips beyond 24 MB (one
 // CTA per SM / three: 5 MB in all 16.3 / 17.5 us, 14 MB 13.0 / 14.3, 19 MB 18.5 / 18.8, 26 MB 20.5 / 20.4, 34 MB 22.3 / 22.1),
 // nor for a clip of far more than L2 holds (268 MB 126.7 / 132.5 us, 537 MB 242.3 / 240.3 and at r = 2 250.0 / 247.2: the rows
-// come from DRAM).
+// come from DRAM).  Calls on several streams of the caller's count as alone: the library does not see what else runs, and what
+// this form gains on one stream it gives back in part on four.  Us per clip in a replayed graph on one / two / four streams, three
+// CTAs and one: 32 x 16 x 16 x 4096 37.9 33.9 32.4 and 36.6 34.7 33.3, 16 x 16 x 16 x 4096 29.6 20.7 19.8 and 24.9 20.9 21.0, 20 x 14
+// x 14 x 3584 31.4 21.1 18.4 and 27.0 21.3 19.2, 32 x 16 x 16 x 2048 27.4 20.8 20.3 and 24.4 20.5 20.2, 9 x 16 x 16 x 1024 15.1 11.2
+// 8.5 and 14.0 10.2 9.2, 24 x 20 x 15 x 248 17.5 9.9 6.8 and 15.0 9.0 6.9.  (16 warps of 4 KB slots, two CTAs of 64 KB, batches dealt
+// out over all CTAs in turn: none is better on two and four streams and as good on one.)
 inline bool gather_alone(const Problem& p) {
     const double bytes = (double)p.F * p.N * p.C * (p.dtype == 0 ? 4.0 : 2.0) * p.nclips;
     return p.overlapped <= 1 && bytes <= (p.nclips == 1 ? 300e6 : 24e6);
