@@ -110,14 +110,15 @@ int ttf_workspace_status(const void* workspace, ttf_stream_t stream, int* host_s
  * every limit of those tests by that many elements, so that valid indices at the end of an array are reported and
  * skipped: the reporting path can be exercised with all accesses still in bounds.  The normal build returns
  * TTF_ERR_UNSUPPORTED.
- * ttf_debug_match_split: how the tcgen05 matching kernel would split a launch over `clips` (1 to 16) clips of this shape;
+ * ttf_debug_match_split: how the tcgen05 matching kernel would split a launch over `clips` (1 to 16) clips of this shape in one
+ * of `lanes` lanes (1: nothing beside it);
  * split[0] = grid rows of a tile, split[1] = parts of its channel range that are summed apart, split[2] = CTAs that share a
- * tile.  The first two do not depend on `clips`.  TTF_ERR_UNSUPPORTED for a shape that the kernel does not take.
+ * tile.  The second depends on the shape alone.  TTF_ERR_UNSUPPORTED for a shape that the kernel does not take.
  */
 int ttf_debug_set_wait(int poll_limit, int tx_extra_bytes);
 int ttf_debug_func_attr_needed(const void* key, int device, size_t bytes);
 int ttf_debug_set_check_slack(int slack);
-int ttf_debug_match_split(int F, int H, int W, int C, int r, int clips, int* split);
+int ttf_debug_match_split(int F, int H, int W, int C, int r, int clips, int lanes, int* split);
 
 /*
  * Scratch bytes one call needs for a clip of this shape (per-token inverse norms, per-frame channel sums,

@@ -84,7 +84,7 @@ def lib() -> ctypes.CDLL:
         L.ttf_debug_set_check_slack.restype = i
         L.ttf_debug_set_check_slack.argtypes = [i]
         L.ttf_debug_match_split.restype = i
-        L.ttf_debug_match_split.argtypes = [i] * 6 + [ctypes.POINTER(i)]
+        L.ttf_debug_match_split.argtypes = [i] * 7 + [ctypes.POINTER(i)]
         L.ttf_debug_set_wait.restype = i
         L.ttf_debug_set_wait.argtypes = [i, i]
         L.ttf_debug_func_attr_needed.restype = i
@@ -307,10 +307,10 @@ def ttf_debug_set_check_slack(slack: int = 0) -> int:
     return int(lib().ttf_debug_set_check_slack(int(slack)))
 
 
-def ttf_debug_match_split(F: int, H: int, W: int, C: int, r: int, clips: int = 1):
+def ttf_debug_match_split(F: int, H: int, W: int, C: int, r: int, clips: int = 1, lanes: int = 1):
     """ttf_debug_match_split: (grid rows of a tile, chunks of its channels, CTAs per tile), or None."""
     split = (ctypes.c_int * 3)()
-    rc = lib().ttf_debug_match_split(F, H, W, C, r, clips, split)
+    rc = lib().ttf_debug_match_split(F, H, W, C, r, clips, lanes, split)
     if rc == 2:                                  # TTF_ERR_UNSUPPORTED: not a clip of the tcgen05 kernel
         return None
     if rc != TTF_OK:

@@ -99,6 +99,7 @@ struct ProfScope {
 };
 
 // Schedule of a batch: clips in flight (ttf_set_schedule)
+constexpr int kBatchStreams = 8;                 // lanes at most
 static std::atomic<int> g_sched_lanes{0};        // 0: automatic
 static std::atomic<int> g_match_kernel{0};       // ttf_set_match_kernel: 0 automatic, 1 warp-level MMA, 2 tcgen05
 
@@ -467,13 +468,13 @@ int ttf_debug_func_attr_needed(const void* key, int device, size_t bytes) {
     return g_func_attr.needs(key, device, bytes) ? 1 : 0;
 }
 
-int ttf_debug_match_split(int F, int H, int W, int C, int r, int clips, int* split) {
-    if (!split || clips < 1 || clips > kMaxGroup) return TTF_ERR_INVALID_ARG;
+int ttf_debug_match_split(int F, int H, int W, int C, int r, int clips, int lanes, int* split) {
+    if (!split || clips < 1 || clips > kMaxGroup || lanes < 1 || lanes > kBatchStreams) return TTF_ERR_INVALID_ARG;
     Problem p;
     int rc = make_problem(reinterpret_cast<const void*>(uintptr_t(256)), F, H, W, C, r, 0.f, TTF_DTYPE_BF16, &p);
     if (rc != TTF_OK) return rc;
     if (!tc_match_eligible(p)) return TTF_ERR_UNSUPPORTED;
-    p.nclips = clips;
+    p.nclips = clips; p.overlapped = lanes;
     const TcPlan t = tc_plan(p);
     split[0] = t.rows; split[1] = t.chunks; split[2] = t.pieces;
     return TTF_OK;
@@ -637,7 +638,6 @@ int ttf_compress_mean(const void* features, int F, int H, int W, int C, int r, f
 // The clips of a batch are independent: they go through the kernels in groups (one launch covers a group), and the
 // groups are spread round-robin over up to kBatchStreams internal streams per device that fork from the caller's
 // stream and join it again (events only: the call stays asynchronous and can be captured in a graph).
-constexpr int kBatchStreams = 8;
 constexpr int kMatchedRing = 4;                  // events "clip n has been matched" of the pipelined schedule, used in turn
 struct BatchLanes {
     cudaStream_t s[kBatchStreams] = {}; cudaEvent_t fork = nullptr; cudaEvent_t join[kBatchStreams] = {};

@@ -537,28 +537,26 @@ static size_t tiles_of(const Problem& p, int wy) {
     const int fr = kTcM / (kTcWB * wy);
     return (size_t)((p.F + fr - 1) / fr) * ((p.H + wy - 1) / wy) * ((p.W + kTcWB - 1) / kTcWB);
 }
-// Grid rows of a tile (1, 2 or 4, hence 32, 16 or 8 frames): the one with the fewest rows to fetch, padding and candidates
-// included.  (r = 2 with four rows would need 64 columns of 128 registers.)
-static int tile_rows(const Problem& p) {
+static int rows_per_stage(const Problem& p, int wy) { return kTcM + (kTcWB + 2 * p.r) * (wy + 2 * p.r); }
+static int most_rows(const Problem& p) { return p.r == 2 ? 2 : 4; }       // (r = 2 with four rows would need 64 columns of 128 registers)
+// The tile (1, 2 or 4 grid rows, hence 32, 16 or 8 frames) with the fewest rows to fetch, padding and candidates included.
+static int fewest_rows(const Problem& p) {
     int best = 1;
-    size_t least = 0;
-    for (int wy = 1; wy <= (p.r == 2 ? 2 : 4); wy *= 2) {
-        const size_t rows = tiles_of(p, wy) * (kTcM + (kTcWB + 2 * p.r) * (wy + 2 * p.r));
-        if (wy == 1 || rows < least) { least = rows; best = wy; }
-    }
+    for (int wy = 2; wy <= most_rows(p); wy *= 2)
+        if (tiles_of(p, wy) * rows_per_stage(p, wy) < tiles_of(p, best) * rows_per_stage(p, best)) best = wy;
     return best;
 }
-size_t tc_match_tiles(const Problem& p) { return tiles_of(p, tile_rows(p)); }
+size_t tc_match_tiles(const Problem& p) { return tiles_of(p, fewest_rows(p)); }
 
 // Parts of a tile's channel range: the largest power of two with which a launch over one clip still fits the GPU in one
 // wave of two CTAs per SM, at most max_chunks and at least 2 stages each (4 stages: 16 x 8 x 8 x 512 13.9 us per pass,
 // 2: 12.9, 1: 13.3; 16 x 14 x 14 x 512 16.7 / 15.3 / 15.3).  (One CTA per SM with a ring twice as deep measured the same
 // alone, 18.8 against 19.2 us on a cold 8B-shaped clip, and slower with other clips' kernels beside it, 34.0 against
 // 32.2 us per clip.)
-static int split_of(const Problem& p, long long tiles, int most) {
+static int split_of(const Problem& p, long long tiles, int most, int sms) {
     const int nst = (p.C + kTcKC - 1) / kTcKC;
     int n = 1;
-    while (n * 2 <= most && tiles * (n * 2) <= 2LL * sm_count() && nst / (n * 2) >= 2) n *= 2;
+    while (n * 2 <= most && tiles * (n * 2) <= 2LL * sms && nst / (n * 2) >= 2) n *= 2;
     return n;
 }
 
@@ -591,35 +589,76 @@ static long long cluster_places(int n) {                          // n = 1, 2, 4
     return found;
 }
 
-// How a launch splits its work.  The tile and its chunks depend on the clip's shape alone, the CTAs (= cluster size) of a tile on
-// what is in flight.
+// Chunks of a tile of `wy` rows in a launch over one clip: what split_of gives, but never fewer than tiles of one row have.
+static int chunks_alone(const Problem& p, int wy, int sms) {
+    const int own = own_chunks(tile_columns(p.r, wy)), one_row = split_of(p, (long long)tiles_of(p, 1), max_chunks(p.r), sms);
+    int n = split_of(p, (long long)tiles_of(p, wy), max_chunks(p.r), sms);
+    // (eight parts of 48 columns are not worth a second CTA on an SM: 5 x 29 x 13 x 1016 17.0 us per pass, with four 16.1)
+    if (n > own && (long long)tiles_of(p, wy) * n > sms) n = own;
+    return n > one_row ? n : one_row;
+}
+static int least_pieces(const Problem& p, int wy, int chunks) {           // (a CTA has tensor memory for own_chunks)
+    const int own = own_chunks(tile_columns(p.r, wy));
+    return chunks > own ? chunks / own : 1;
+}
+// Grid rows of a tile in a launch over `clips` clips, beside which nothing runs, whose channels are summed in `chunks` parts (0: as
+// each tile has alone, and without a look at the places of clusters, which are not the same on every device).  The tile with the fewest rows to fetch, but not where its CTAs are more than one per SM and leave places
+// empty that another tile's fill: such a launch takes as long as the SM with the most CTAs, CTAs x stages x rows of a stage.  (A
+// CTA alone on its SM is counted as two: it is hardly faster.)  Us per pass, replayed graph, the fewest rows / as here:
+// 40 x 26 x 20 x 1992 63.2 / 54.5 (175 / 195 CTAs), 23 x 24 x 23 x 3856 63.5 / 58.0 (216 / 288), 24 x 24 x 24 x 2048 37.4 / 35.2,
+// 20 x 20 x 20 x 2048 30.7 / 29.0 (with a fixed anchor 20.2 / 20.9), 67 x 7 x 9 x 3568 30.3 / 28.3, 54 x 30 x 19 x 2432 at r = 0
+// 109.6 / 102.8; three of 24 x 20 x 15 x 248 18.2 / 16.6.
+static int tile_rows(const Problem& p, long long clips, int chunks, int sms) {
+    const int nst = (p.C + kTcKC - 1) / kTcKC, few = fewest_rows(p);
+    auto time = [&](int wy, long long* ctas) {
+        const int n = chunks ? chunks : chunks_alone(p, wy, sms);
+        const long long tiles = (long long)tiles_of(p, wy) * clips;
+        int pieces = split_of(p, tiles, n, sms);
+        while (chunks && pieces > 1 && tiles > cluster_places(pieces)) pieces /= 2;
+        if (pieces < least_pieces(p, wy, n)) pieces = least_pieces(p, wy, n);
+        *ctas = tiles * pieces;
+        const long long per_sm = (*ctas + sms - 1) / sms;
+        return (per_sm < 2 ? 2 : per_sm) * ((nst + pieces - 1) / pieces) * rows_per_stage(p, wy);
+    };
+    long long ctas, t[3] = {}, least = time(few, &ctas);
+    if (ctas <= sms) return few;
+    for (int i = 0; 1 << i <= most_rows(p); ++i) {
+        t[i] = time(1 << i, &ctas);
+        least = t[i] < least ? t[i] : least;
+    }
+    int best = 0;                                // the fewest rows among those that take at most a twentieth longer than the shortest
+    for (int i = 0, wy = 1; wy <= most_rows(p); ++i, wy *= 2)
+        if (t[i] * 20 <= least * 21 && (!best || tiles_of(p, wy) * rows_per_stage(p, wy) < tiles_of(p, best) * rows_per_stage(p, best))) best = wy;
+    return best;
+}
+
+// How a launch splits its work.  The chunks depend on the clip's shape alone, the tile and its CTAs (= cluster size) on what is in
+// flight.
 TcPlan tc_plan(const Problem& p) {
     TcPlan t;
-    t.rows = tile_rows(p);
-    t.tiles = (long long)tiles_of(p, t.rows);
-    t.chunks = split_of(p, t.tiles, max_chunks(p.r));
-    const int own = own_chunks(tile_columns(p.r, t.rows));
-    // (eight parts of 48 columns are not worth a second CTA on an SM: 5 x 29 x 13 x 1016 17.0 us per pass, with four 16.1)
-    if (t.chunks > own && t.tiles * t.chunks > sm_count()) {
-        const int one_row = split_of(p, (long long)tiles_of(p, 1), max_chunks(p.r));
-        t.chunks = one_row > own ? one_row : own;
-    }
     // Three or more single clips in flight (ttf_set_schedule, clips that cannot share a launch)
     // fill the GPU together: 16 clips of 32 x 16 x 16 x 4096 on eight lanes 497 -> 445 us, on three 512 -> 506 (on two 530 ->
     // 507, but three clips, of which two share a launch, 98 -> 102).
     const int beside = p.nclips == 1 && p.overlapped >= 3 ? p.overlapped : 1;
+    const int sms = sm_count();
+    t.chunks = chunks_alone(p, tile_rows(p, 1, 0, sms), sms);
+    // (beside another lane's kernels the fewest rows: 8 clips of 20 x 20 x 20 x 1024 73.4 us, by the rule above 80.4, 4 of
+    // 40 x 16 x 16 x 1024 49.7 / 51.6, 2 of 23 x 24 x 23 x 2048 63.0 / 69.1.  The products of a row and a candidate are the same
+    // whatever tile they are in.)
+    t.rows = p.overlapped > 1 ? fewest_rows(p) : tile_rows(p, p.nclips, t.chunks, sms);
+    t.tiles = (long long)tiles_of(p, t.rows);
     // Not more than run at the same time: the cluster that has to wait for a place costs the whole main loop once more (us per
     // pass, 32 frames of 2048 channels: 71 tiles in fours 23.4, 72 in fours 30.9, in twos 27.2; 33 in eights 19.6, 34 in
     // eights 23.8, in fours 20.6; 12 x 24 x 24 x 2048 28.8 -> 26.0).
     const long long units = t.tiles * p.nclips * beside;
-    t.pieces = split_of(p, units, t.chunks);
+    t.pieces = split_of(p, units, t.chunks, sms);
     while (t.pieces > 1 && units > cluster_places(t.pieces)) t.pieces /= 2;
-    if (t.pieces * own < t.chunks) t.pieces = t.chunks / own;
+    if (t.pieces < least_pieces(p, t.rows, t.chunks)) t.pieces = least_pieces(p, t.rows, t.chunks);
     return t;
 }
 
 template <int R, int WY, int G>
-static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
+static cudaError_t launch_tc_t(const Problem& p, const TcPlan& plan, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                unsigned char* keep, cudaStream_t st) {
     using S = TcShape<R, WY>;
     ClipMaps<G> maps;
@@ -631,7 +670,6 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
     const size_t need = (size_t)S::RING + S::XBYTES + S::NORMBYTES + 1024, smem = need < 80 * 1024 ? 80 * 1024 : need;
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_match_tc<R, WY, G>), smem);
     if (e != cudaSuccess) return e;
-    const TcPlan plan = tc_plan(p);
     const long long tiles = plan.tiles;
     const int chunks = plan.chunks, pieces = plan.pieces;
     auto log2_of = [](int n) { int l = 0; while ((1 << l) < n) ++l; return l; };
@@ -654,10 +692,10 @@ static cudaError_t launch_tc_t(const Problem& p, const Scratch& s, int* out_anch
 template <int R, int G>
 static cudaError_t launch_tc_rows(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,
                                   unsigned char* keep, cudaStream_t st) {
-    const int wy = tile_rows(p);
-    if constexpr (R < 2) if (wy == 4) return launch_tc_t<R, 4, G>(p, s, out_anchor, shat, dst, keep, st);
-    return wy == 2 ? launch_tc_t<R, 2, G>(p, s, out_anchor, shat, dst, keep, st)
-                   : launch_tc_t<R, 1, G>(p, s, out_anchor, shat, dst, keep, st);
+    const TcPlan plan = tc_plan(p);
+    if constexpr (R < 2) if (plan.rows == 4) return launch_tc_t<R, 4, G>(p, plan, s, out_anchor, shat, dst, keep, st);
+    return plan.rows == 2 ? launch_tc_t<R, 2, G>(p, plan, s, out_anchor, shat, dst, keep, st)
+                          : launch_tc_t<R, 1, G>(p, plan, s, out_anchor, shat, dst, keep, st);
 }
 template <int G>
 static cudaError_t launch_tc(const Problem& p, const Scratch& s, int* out_anchor, float* shat, int* dst,

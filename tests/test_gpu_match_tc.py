@@ -92,5 +92,15 @@ def test_error_of_the_similarities_of_short_clips(shape):
 def test_a_cta_never_sums_more_parts_than_its_tensor_memory_holds():
     """so many tiles that one CTA each would fill the GPU, in eight parts of 48 columns"""
     shape, clips = (8, 20, 8, 1024), 32
-    assert P.ttf_debug_match_split(*shape, 1, clips=16) == (4, 8, 2) and P.ttf_debug_match_split(*shape, 1) == (4, 8, 8)
+    assert P.ttf_debug_match_split(*shape, 1, clips=16, lanes=2) == (4, 8, 2) and P.ttf_debug_match_split(*shape, 1) == (4, 8, 8)
     test_bits_do_not_depend_on_the_split(shape, 1, clips)
+
+
+@pytest.mark.parametrize("shape,r,clips,group", [((40, 16, 16, 1024), 1, 16, (8, 2)), ((23, 24, 23, 520), 1, 8, (4, 2)),
+                                                 ((17, 21, 11, 1496), 0, 16, (8, 2)), ((24, 20, 15, 248), 1, 3, (3, 1))])
+def test_bits_do_not_depend_on_the_tile(shape, r, clips, group):
+    """clips whose tile alone has other rows than in a group of the batch"""
+    alone = P.ttf_debug_match_split(*shape, r)
+    grouped = P.ttf_debug_match_split(*shape, r, *group)
+    assert alone[0] != grouped[0] and alone[1] == grouped[1]
+    test_bits_do_not_depend_on_the_split(shape, r, clips)

@@ -79,7 +79,7 @@ def test_tensor_core_pipeline_gives_up_and_recovers(C):
 def test_tiles_of_one_cta_and_several_chunks_give_up_and_recover(r, clips):
     """large launches: every tile is one CTA that sums all chunks of its channels (8 alone, 4 for r = 2) itself"""
     X = corr_clip(32, 8, 8, 1024, seed=82, dtype="bf16")
-    assert P.ttf_debug_match_split(*X.shape, r, clips=clips // 2) == (1, 4 if r == 2 else 8, 1)
+    assert P.ttf_debug_match_split(*X.shape, r, clips=clips // 2, lanes=2) == (1, 4 if r == 2 else 8, 1)
     Xs = [to_device(X)] * clips
     st = torch.cuda.Stream()
     ref = P.ttf_compress(Xs[0], r, 0.7, stream=st)
