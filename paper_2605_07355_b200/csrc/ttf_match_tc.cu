@@ -602,12 +602,11 @@ static int least_pieces(const Problem& p, int wy, int chunks) {           // (a 
     return chunks > own ? chunks / own : 1;
 }
 // Grid rows of a tile in a launch over `clips` clips, beside which nothing runs, whose channels are summed in `chunks` parts (0: as
-// each tile has alone, and without a look at the places of clusters, which are not the same on every device).  The tile with the fewest rows to fetch, but not where its CTAs are more than one per SM and leave places
-// empty that another tile's fill: such a launch takes as long as the SM with the most CTAs, CTAs x stages x rows of a stage.  (A
-// CTA alone on its SM is counted as two: it is hardly faster.)  Us per pass, replayed graph, the fewest rows / as here:
-// 40 x 26 x 20 x 1992 63.2 / 54.5 (175 / 195 CTAs), 23 x 24 x 23 x 3856 63.5 / 58.0 (216 / 288), 24 x 24 x 24 x 2048 37.4 / 35.2,
-// 20 x 20 x 20 x 2048 30.7 / 29.0 (with a fixed anchor 20.2 / 20.9), 67 x 7 x 9 x 3568 30.3 / 28.3, 54 x 30 x 19 x 2432 at r = 0
-// 109.6 / 102.8; three of 24 x 20 x 15 x 248 18.2 / 16.6.
+// each tile has alone, and without a look at the places of clusters, which are not the same on every device).  The tile with the fewest rows to fetch, but not where its CTAs are more than one per SM and another tile's are done
+// sooner: waves of two CTAs per SM x stages x rows of a stage.  Us per pass, replayed graph, the fewest rows / as here (CTAs):
+// 40 x 26 x 20 x 1992 63.2 / 54.5 (175 / 195), 23 x 24 x 23 x 3856 63.5 / 58.0 (216 / 288), 40 x 32 x 32 x 2048 116.5 / 97.6 (320 / 384),
+// 33 x 32 x 32 x 3000 144.3 / 119.7, 65 x 23 x 31 x 2216 131.3 / 114.6 (432 / 480), 20 x 20 x 20 x 2048 30.7 / 29.0 (with a fixed anchor
+// 20.2 / 20.9), 54 x 30 x 19 x 2432 at r = 0 109.6 / 102.8 (300 / 280); three of 24 x 20 x 15 x 248 18.2 / 16.6.
 static int tile_rows(const Problem& p, long long clips, int chunks, int sms) {
     const int nst = (p.C + kTcKC - 1) / kTcKC, few = fewest_rows(p);
     auto time = [&](int wy, long long* ctas) {
@@ -617,8 +616,7 @@ static int tile_rows(const Problem& p, long long clips, int chunks, int sms) {
         while (chunks && pieces > 1 && tiles > cluster_places(pieces)) pieces /= 2;
         if (pieces < least_pieces(p, wy, n)) pieces = least_pieces(p, wy, n);
         *ctas = tiles * pieces;
-        const long long per_sm = (*ctas + sms - 1) / sms;
-        return (per_sm < 2 ? 2 : per_sm) * ((nst + pieces - 1) / pieces) * rows_per_stage(p, wy);
+        return (*ctas + 2 * sms - 1) / (2 * sms) * ((nst + pieces - 1) / pieces) * rows_per_stage(p, wy);
     };
     long long ctas, t[3] = {}, least = time(few, &ctas);
     if (ctas <= sms) return few;
