@@ -153,7 +153,8 @@ int ttf_compress(const void* features, int F, int H, int W, int C, int r, float 
  * that the library keeps per device; these fork from `stream` and join it again through events, so the call is
  * asynchronous, ordered on `stream` like any other, and can be captured in a CUDA graph.  The kernels of one group
  * leave part of the GPU idle while they ramp up and drain; the other lane's fill those gaps.  Small batches (up to
- * eight clips of 64 MB together, 160 MB with a fixed anchor; outside a capture up to sixteen of 16 or 32 MB) run on `stream`
+ * eight clips of some 50 MB together, 160 MB with a fixed anchor; outside a capture up to sixteen of at most 16 or 32 MB, less in
+ * fp32 and for r = 2) run on `stream`
  * itself instead, in groups of up to eight, on scratch that belongs to the stream.  The first 64 streams that are used so
  * keep theirs until ttf_release, besides the scratch of the lanes, which such a batch claims too (a later capture may need it):
  * up to twice the memory.  Where a stream has none and cannot get any (in a capture, beyond 64 streams, without memory) they take

@@ -677,7 +677,11 @@ static int batch_lanes(BatchLanes** out) {
 // 25.7 MB 30.4 / 21.9, 67 MB 54.6 / 49.9 and 40.1 / 35.3, 134 MB 58.3 / 55.3, 157 MB 70.7 / 67.8, 201 MB 81.4 / 79.9, 335 MB
 // 132.6 / 135.7.  Nine to sixteen clips are two launches of each kernel, which do not overlap here: 14 MB 40.2 / 37.2, 28 MB
 // 40.1 / 39.4, 51 MB 49.7 / 62.3 (fixed anchors 32 MB 33.7 / 27.6, 51 MB 40.3 / 45.1), and in a replayed graph, where the
-// host's part is gone, 1.3 MB 18.2 / 23.7: not in a capture.
+// host's part is gone, 1.3 MB 18.2 / 23.7: not in a capture.  Where the matching takes longer per byte the line lies lower: r = 2 and
+// fp32, lanes / own stream: 12 clips of 20 x 14 x 13 in bf16 r = 2 10 MB 37.6 / 39.3, 5 MB 37.1 / 33.1; fp32 15 MB 37.0 / 43.2, 10 MB
+// 37.5 / 33.7; fp32 r = 2 10 MB 38.3 / 44.1; fixed anchors bf16 r = 2 20 MB 33.0 / 36.1, 10 MB 33.1 / 30.8, fp32 30 MB 38.6 / 44.2, 20 MB
+// 35.9 / 36.7, fp32 r = 2 10 MB 33.6 / 35.7, 4 MB 33.1 / 28.0.  More than four clips of 59 MB and r = 2 61.8 / 67.3, 8 of 60 MB
+// 48.0 / 50.2, 30 MB 35.2 / 33.5; six of 96 MB in fp32 with a fixed anchor 52.9 / 54.8.
 constexpr int kInlineClips = 16, kInlineGroup = 8;
 constexpr size_t kInlineStreams = 64;            // streams that hold scratch for it; on further ones the lanes take the batch
 
@@ -685,8 +689,10 @@ static bool takes_own_stream(const Problem& p, int nclips, bool same_layout, boo
     if (st == cudaStreamPerThread) return false;                     // (one handle, another stream in every thread)
     if (g_sched_lanes.load() != 0 || !same_layout || nclips > kInlineClips || (nclips > kInlineGroup && capturing)) return false;
     const double mb = (double)p.F * p.N * p.C * (p.dtype == TTF_DTYPE_F32 ? 4e-6 : 2e-6) * nclips;
-    const bool sweep = p.anchor_mode == 0 || needs_sweep_norms(p);
-    return mb <= (nclips <= kInlineGroup ? (sweep ? 64.0 : 160.0) : (sweep ? 16.0 : 32.0));
+    const bool sweep = p.anchor_mode == 0 || needs_sweep_norms(p), f32 = p.dtype == TTF_DTYPE_F32;
+    if (nclips > kInlineGroup) return mb * (f32 ? 1.6 : 1.0) * (p.r > 2 ? 8.0 : (p.r == 2 ? (f32 ? 2.7 : 2.0) : 1.0)) <= (sweep ? 16.0 : 32.0);
+    if (sweep) return mb <= (nclips > 4 ? 45.0 : 64.0);
+    return mb <= (f32 ? 64.0 : 160.0);
 }
 
 // How a batch is cut into launches: `group` clips per launch, `lanes` groups in flight, `sets` of `group` scratch blocks
