@@ -192,11 +192,13 @@ k_match_f32(const __grid_constant__ ClipMaps<G> maps, int F, int H, int W, int C
     trace_mark(asrc.hdr, 2, true);
 }
 
-// Stages of the ring.  At r <= 1 a ring of four leaves room for two CTAs of 32 frames on an SM, one of three for three, which is
-// better where a launch then fits the GPU at once, or is several times what fits.  (At r = 2 the registers leave room for one CTA
-// of 32 frames whatever its ring.)  No more than the channels fill, so that short rows make room for more CTAs.  A launch that fits with the whole ring keeps it (us per pass, replayed graph, whole ring / as here:
-// 98 x 10 x 32 x 352 37.1 / 32.5, 64 x 24 x 24 x 512 46.4 / 43.9, two of 102 x 15 x 12 x 288 40.0 / 37.7, 34 x 15 x 15 x 3312 at
-// r = 0 68.3 / 62.7; with three stages where this takes four, 68 x 13 x 15 x 2520 84.7 / 95.0 and 32 x 16 x 16 x 1152 22.7 / 24.4).
+// Stages of the ring.  At r <= 1 a ring of four leaves room for two CTAs of 32 frames on an SM, one of three for three,
+// which is better where a launch then fits the GPU at once, or is several times what fits.  (At r = 2 the registers leave
+// room for one CTA of 32 frames whatever its ring.)  No more than the channels fill, so that short rows make room for more
+// CTAs.  A launch that fits with the whole ring keeps it (us per pass, replayed graph, whole ring / as here: 98 x 10 x 32 x
+// 352 37.1 / 32.5, 64 x 24 x 24 x 512 46.4 / 43.9, two of 102 x 15 x 12 x 288 40.0 / 37.7 and, measured again, 39.0 / 38.4,
+// 34 x 15 x 15 x 3312 at r = 0 68.3 / 62.7; with three stages where this takes four, 68 x 13 x 15 x 2520 84.7 / 95.0 and 32
+// x 16 x 16 x 1152 22.7 / 24.4).
 template <int R> static int ring_stages(const Problem& p, long long units, int FR) {
     using S = F32Shape<R>;
     const int nst = (p.C + kF32KC - 1) / kF32KC;

@@ -115,3 +115,20 @@ def test_per_thread_default_stream():
     P.ttf_compress_batch(Xs, 1, 0.6, *outs, stream=2)               # cudaStreamPerThread
     torch.cuda.synchronize()
     assert_same_as_single(Xs, 1, 0.6, outs)
+
+
+@pytest.mark.parametrize("dtype,r,n,channels,launches", [("bf16", 1, 12, 64, 2), ("bf16", 2, 12, 1024, 2), ("f32", 2, 9, 264, 2), ("bf16", 1, 5, 1024, 1),
+                                                         ("bf16", 1, 5, 8192, 2), ("f32", 3, 9, 64, 2)])
+def test_every_clip_as_alone_on_both_sides_of_the_line(dtype, r, n, channels, launches):
+    """batches of 9 to 16 clips that take the caller's stream or the lanes by what their matching costs, and of five below and above
+    45 MB: one launch of each kernel or two"""
+    from bench import count_launches
+    Xs = clips_of((8, 9, 8, channels), 3, dtype, seed=1010)
+    Xs = [Xs[j % 3] for j in range(n)]
+    if channels == 8192:
+        Xs = clips_of((60, 4, 3, channels), 3, dtype, seed=1020)
+        Xs = [Xs[j % 3] for j in range(n)]
+    outs = P.ttf_compress_batch(Xs, r, 0.6)
+    assert P.ttf_last_device_status() == P.TTF_OK
+    assert_same_as_single(Xs, r, 0.6, outs)
+    assert count_launches(lambda: P.ttf_compress_batch(Xs, r, 0.6)) == launches * 4
